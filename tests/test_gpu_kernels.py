@@ -202,6 +202,35 @@ def test_gemm_pair_and_single_cta_tiles_agree(ctx, m, n, k):
     assert torch.equal(res[0][0].view(torch.int32), res[1][0].view(torch.int32))
 
 
+@pytest.mark.parametrize("m,n,k", [(1, 33, 16), (31, 1, 48), (257, 259, 64), (128, 255, 144), (300, 1025, 32), (33, 65, 4608)])
+def test_gemm_row_pitch_without_16_byte_alignment(ctx, m, n, k):
+    """fp32 and raw outputs whose rows TMA cannot write, at the edges of a 32 x 32 piece: bit-exact, and
+    nothing outside the matrix is written."""
+    import ctypes as C
+    import paper_2302_01382_b200 as q
+    rng = np.random.default_rng(m * n + k)
+    ld = (k + 15) // 16 * 16
+    qx, qw = _codes(rng, m, k, ld), _codes(rng, n, k, ld)
+    sw = (10.0 ** rng.uniform(-4, -2, n)).astype(np.float32)
+    sx = np.float32(0.0173)
+    guard = 64
+    y = torch.full((m * n + 2 * guard,), 7.0, device="cuda")
+    acc = torch.full((m * n + 2 * guard,), 7, dtype=torch.int32, device="cuda")
+    qxd, qwd, swd = dev(qx), dev(qw), dev(sw)
+    for out, dst in ((y, "y"), (acc, "acc")):
+        p = C.c_void_p(out.data_ptr() + 4 * guard)
+        rc = ctx.lib.qcfg_gemm_i8(ctx.h, C.c_void_p(qxd.data_ptr()), ld, C.c_void_p(qwd.data_ptr()), ld, m, n, k, float(sx),
+                                  C.c_void_p(swd.data_ptr()), 0, p if dst == "y" else None, p if dst == "acc" else None,
+                                  C.c_void_p(torch.cuda.current_stream().cuda_stream))
+        assert rc == q.OK
+    ctx.check_sync()
+    want = orc.int_gemm(qx[:, :k], qw[:, :k])
+    np.testing.assert_array_equal(host(acc)[guard:-guard].reshape(m, n), want)
+    np.testing.assert_array_equal(host(y)[guard:-guard].reshape(m, n), orc.dequant_output(want, sx, sw))
+    for out in (y, acc):
+        assert (host(out)[:guard] == 7).all() and (host(out)[-guard:] == 7).all()
+
+
 def test_gemm_i8_worst_case_magnitude(ctx):
     k = 4608
     qx = np.full((128, k), 127, np.int8)
