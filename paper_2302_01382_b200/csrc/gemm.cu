@@ -1572,7 +1572,18 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   const GemmArgs* gs = ordered;
   const GemmArgs& g0 = gs[0];
   const int esz = g0.is_bf16 ? 2 : 1;
-  const int bn = tile_n_of(g0.n);
+  // Tile width: by the output's width, then halved while that still leaves every CTA of the launch one
+  // tile at most.
+  int bn = tile_n_of(g0.n);
+  {
+    const int sms = sm_count(ctx);
+    auto ctas = [&](int width) {
+      int64_t cols = 0;
+      for (int i = 0; i < count; ++i) cols += (gs[i].n + width - 1) / width;
+      return cols * ((g0.m + BM - 1) / BM);
+    };
+    while (bn > 32 && ctas(bn / 2) <= sms) bn /= 2;
+  }
   for (int i = 0; i < count; ++i) {
     const GemmArgs& g = gs[i];
     if (g.m <= 0 || g.n <= 0 || g.k <= 0) return set_error(ctx, QCFG_ESHAPE, "gemm: m, n, k must be positive");

@@ -10,19 +10,23 @@
 //   acc = fma(e, e, acc)
 // The clip of Eq. 1 is a no-op here because the scale comes from the row's own maximum.
 //
-// Work distribution: the tensors of one kernel variant form one flat sequence of rows, cut into as
-// many equal pieces as blocks stay resident on the device (three per SM); a piece that crosses a
-// tensor boundary becomes several segments.  Every block therefore starts once, streams the same
-// amount of data and ends with the others: no per-item start-up cost and no ragged last wave.
-// Each segment writes its 7 sums and its maximum to its own slot; one finalize block per tensor
-// adds the tensor's slots in a fixed order, so the result does not depend on timing.
+// Work distribution: the rows of all tensors form one flat sequence, cut into as many pieces of equal
+// cost as blocks stay resident on the device; a piece that crosses a tensor boundary becomes several
+// segments.  Every block therefore starts once, streams the same amount and ends with the others,
+// whatever the mix of row lengths (the 54 tensors of ResNet-50 took one launch per row length and
+// one block for the 147-column stem: 144 us, now 46).
+// Each segment writes its 7 sums and its maximum to its own slot; one block per tensor (the one that
+// finishes its last segment, or a finalize kernel's) adds the tensor's slots in a fixed order, so the
+// result does not depend on timing.
+// Queues were slower: blocks taking items of an eighth of a piece 126 us against 94 for 80 M elements
+// in rows of 768, single warps taking items 125 us.
 //
 // Sums: fp32 in three short stages, then fp64.  A thread's packed accumulators take at most
 // kChainTerms squared errors each; they are then added into a second fp32 accumulator per bit width,
-// which takes at most kChainTerms such sums; that one is reduced over the warp by five pairwise
+// which takes at most kChainSums such sums; that one is reduced over the warp by five pairwise
 // steps and added to the warp's fp64 sum in shared memory.  A sequential fp32 sum of n non-negative
 // terms is within (n-1)*2^-24 relative of the exact sum, so the three stages together stay within
-// (31 + 1 + 31 + 5) * 2^-24 = 4.1e-6, inside the sweep's 1e-5 tolerance; no thread keeps fp64
+// (31 + 1 + 15 + 5) * 2^-24 = 3.1e-6, inside the sweep's 1e-5 tolerance; no thread keeps fp64
 // accumulators in registers.
 #include <cstring>
 
@@ -37,8 +41,9 @@ constexpr int kNB = 7;                       // bit widths 2..8
 constexpr float kMagic = 12582912.0f;        // 1.5 * 2^23
 constexpr int kRing = 3;                     // shared-memory row stages per thread
 constexpr int kBlocksPerSM = 3;
-constexpr int kChainTerms = 32;              // terms per fp32 accumulator at each of the two stages
-constexpr int64_t kMinBlockElems = 16 * 1024;   // do not cut the work of a variant finer than this
+constexpr int kChainTerms = 32;              // terms per fp32 accumulator of the first stage
+constexpr int kChainSums = 16;               // such sums per fp32 accumulator of the second stage
+constexpr int64_t kMinBlockElems = 2 * 1024;   // do not cut the work finer than one round of a block's eight warps at 256 columns
 
 // One run of whole rows of one tensor, processed by one block.
 struct SweepSeg {
@@ -46,12 +51,14 @@ struct SweepSeg {
   int32_t rows;
   int32_t cols;
   int32_t tensor;         // index into the caller's tensor list
-  int32_t team_log2;      // team size = 32 << team_log2 (row variants)
+  int32_t team_log2;      // team size = 32 << team_log2
   int32_t slot;           // partial-result slot
-  int32_t pad;
+  int16_t v;              // float4 per thread and row (1..8); 0: rows too long for the ring
+  int16_t vec;            // rows are 16-byte aligned and whole float4
 };
+static_assert(sizeof(SweepSeg) == 32, "one segment is two 16-byte words");
 struct SweepBlock { int32_t seg0, nseg; };
-struct TensorSlots { int32_t slot0, slot1; };
+struct TensorSlots { int32_t slot0, slot1; unsigned done, pad; };   // done: segments finished; back at 0 after every call
 
 __device__ __forceinline__ void scales_for_lane(float A, int lane, float& s, float& inv) {
   int b = 2 + (lane % kNB);
@@ -67,29 +74,6 @@ __device__ __forceinline__ void err4(float x, float s, float inv, float& acc) {
   acc = fmaf(e, e, acc);
 }
 
-// Writes the block's 7 sums and its maximum to out[0..7].  Ends with a barrier, so the shared
-// buffer may be reused at once.
-__device__ __forceinline__ void block_reduce_store(double (&dacc)[kNB], float amax, double* __restrict__ out) {
-  __shared__ double sred[kThreads / 32][8];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int j = 0; j < kNB; ++j) {
-    double v = warp_sum(dacc[j]);
-    if (lane == 0) sred[warp][j] = v;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-  if (lane == 0) sred[warp][7] = (double)amax;
-  __syncthreads();
-  if (threadIdx.x < 8) {
-    double v = sred[0][threadIdx.x];
-    for (int w = 1; w < kThreads / 32; ++w)
-      v = (threadIdx.x == 7) ? fmax(v, sred[w][7]) : v + sred[w][threadIdx.x];
-    out[threadIdx.x] = v;
-  }
-  __syncthreads();
-}
-
 // Two elements per instruction: the four operations of one (element, b) evaluation as packed
 // fp32 arithmetic (sm_100 fma.rn.f32x2 / add.rn.f32x2), which halves the issue slots they need.
 // ns holds the negated scale in both halves.
@@ -101,231 +85,17 @@ __device__ __forceinline__ void err8(float2 x, float2 ns, float2 inv, float2& ac
   acc = __ffma2_rn(e, e, acc);
 }
 
-// Rows of up to 32*V*team float4; cols % 4 == 0 and 16-byte aligned rows.  All 7 bit widths are
-// always evaluated (a narrower request only selects columns in the finalize kernel).
-template <int V>
-__global__ void __launch_bounds__(kThreads, kBlocksPerSM)
-sweep_rows_kernel(const SweepSeg* __restrict__ segs, const SweepBlock* __restrict__ blocks, int per_tensor,
-                  const float* __restrict__ tensor_absmax, double* __restrict__ partial) {
-  // rows between two first-stage flushes: every row adds 2*V terms to each half of a packed accumulator
-  constexpr int kFlushRows = (kChainTerms / (2 * V)) > 0 ? (kChainTerms / (2 * V)) : 1;
-  // Programmatic dependent launch: the block is scheduled while the previous kernel of the stream
-  // drains and waits here for that kernel's results (result slots, per-tensor maxima, and whatever
-  // produced the weights).
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const SweepBlock blk = blocks[blockIdx.x];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ float smax2[2][kThreads / 32];
-  __shared__ double swarp[kThreads / 32][8];             // per warp: 7 fp64 sums and the maximum
-  extern __shared__ float4 ring[];                       // [kRing][V][kThreads]
-
-  for (int si = blk.seg0; si < blk.seg0 + blk.nseg; ++si) {
-    const SweepSeg d = segs[si];
-    const int T = 32 << d.team_log2;
-    const int nteams = kThreads / T;
-    const int team = threadIdx.x / T;
-    const int tl = threadIdx.x % T;
-    const int c4 = d.cols >> 2;
-    const int n_iter = (d.rows + nteams - 1) / nteams;
-    const float A_tensor = per_tensor ? tensor_absmax[d.tensor] : 0.0f;
-    int row_parity = 0;
-
-    float2 facc[kNB];
-    float f2[kNB];
-#pragma unroll
-    for (int j = 0; j < kNB; ++j) { facc[j] = make_float2(0.0f, 0.0f); f2[j] = 0.0f; }
-    if (lane < 8) swarp[warp][lane] = 0.0;
-    float amax_blk = 0.0f;
-
-    auto process_row = [&](const float4 (&cur)[V]) {
-      float m = 0.0f;
-#pragma unroll
-      for (int v = 0; v < V; ++v)
-        m = fmaxf(fmaxf(fmaxf(m, fabsf(cur[v].x)), fmaxf(fabsf(cur[v].y), fabsf(cur[v].z))), fabsf(cur[v].w));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (T > 32) {
-        // the team's warps exchange their maxima through shared memory; a named barrier per team
-        // keeps other teams running, and alternating slots make one barrier per row enough
-        float* slot = smax2[row_parity];
-        if (lane == 0) slot[warp] = m;
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(T) : "memory");
-        const int w0 = team * (T >> 5);
-        m = slot[w0];
-        for (int w = 1; w < (T >> 5); ++w) m = fmaxf(m, slot[w0 + w]);
-        row_parity ^= 1;
-      }
-      amax_blk = fmaxf(amax_blk, m);
-      if (per_tensor) m = A_tensor;
-
-      // the 7 scale pairs: two IEEE divisions in lanes 0..6, broadcast by shuffles
-      float s_l, inv_l;
-      scales_for_lane(m, lane, s_l, inv_l);
-      float2 ns[kNB], inv[kNB];
-#pragma unroll
-      for (int j = 0; j < kNB; ++j) {
-        const float sj = -__shfl_sync(0xffffffffu, s_l, j), ij = __shfl_sync(0xffffffffu, inv_l, j);
-        ns[j] = make_float2(sj, sj);
-        inv[j] = make_float2(ij, ij);
-      }
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        const float2 lo = make_float2(cur[v].x, cur[v].y), hi = make_float2(cur[v].z, cur[v].w);
-#pragma unroll
-        for (int j = 0; j < kNB; ++j) {
-          err8(lo, ns[j], inv[j], facc[j]);
-          err8(hi, ns[j], inv[j], facc[j]);
-        }
-      }
-    };
-    // second stage -> the warp's fp64 sums
-    auto flush2 = [&]() {
-#pragma unroll
-      for (int j = 0; j < kNB; ++j) {
-        float v = f2[j];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) swarp[warp][j] += (double)v;
-        f2[j] = 0.0f;
-      }
-    };
-
-    // Rows stream through a three-stage ring in shared memory filled by cp.async, two rows ahead
-    // of the one being processed: enough loads in flight to cover HBM latency without holding
-    // future rows in registers.  Every thread copies and reads back only its own 16-byte slots, so
-    // no barrier is needed between the copy and the read.
-    // rowp: this thread's first float4 of the next row its team fetches; fetch_row: that row's index
-    const float4* rowp = reinterpret_cast<const float4*>(d.w + (int64_t)team * d.cols) + tl;
-    const int64_t row_step4 = (int64_t)nteams * c4;
-    int fetch_row = team;
-    const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(ring + threadIdx.x);
-    auto issue_row = [&](int stage) {
-      const uint32_t dst0 = ring0 + (uint32_t)(stage * V) * (kThreads * 16);
-      const bool row_ok = fetch_row < d.rows;
-#pragma unroll
-      for (int v = 0; v < V; ++v) {
-        const uint32_t dst = dst0 + v * (kThreads * 16);
-        if (row_ok && tl + v * T < c4) {
-          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(rowp + v * T) : "memory");
-        } else {
-          asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "f"(0.0f) : "memory");
-        }
-      }
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      rowp += row_step4;
-      fetch_row += nteams;
-    };
-    issue_row(0);
-    issue_row(1);
-    int stage = 0, n1 = 0, n2 = 0;
-    for (int it = 0; it < n_iter; ++it) {
-      int nxt = stage + 2; if (nxt >= kRing) nxt -= kRing;
-      issue_row(nxt);                                                 // zeros past the end
-      asm volatile("cp.async.wait_group 2;" ::: "memory");            // the row of this iteration has landed
-      float4 cur[V];
-#pragma unroll
-      for (int v = 0; v < V; ++v) cur[v] = ring[(stage * V + v) * kThreads + threadIdx.x];
-      process_row(cur);
-      if (++n1 == kFlushRows) {
-#pragma unroll
-        for (int j = 0; j < kNB; ++j) { f2[j] += facc[j].x + facc[j].y; facc[j] = make_float2(0.0f, 0.0f); }
-        n1 = 0;
-        if (++n2 == kChainTerms - 1) { flush2(); n2 = 0; }
-      }
-      if (++stage == kRing) stage = 0;
-    }
-#pragma unroll
-    for (int j = 0; j < kNB; ++j) f2[j] += facc[j].x + facc[j].y;
-    flush2();
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax_blk = fmaxf(amax_blk, __shfl_xor_sync(0xffffffffu, amax_blk, o));
-    if (lane == 0) swarp[warp][7] = (double)amax_blk;
-    __syncthreads();
-    if (threadIdx.x < 8) {                  // the warps' sums in a fixed order
-      double v = swarp[0][threadIdx.x];
-      for (int w = 1; w < kThreads / 32; ++w)
-        v = (threadIdx.x == 7) ? fmax(v, swarp[w][7]) : v + swarp[w][threadIdx.x];
-      partial[(int64_t)d.slot * 8 + threadIdx.x] = v;
-    }
-    __syncthreads();
-  }
-}
-
-// Any shape or alignment: the whole block works on one row at a time and reads it twice
-// (the second read hits L1/L2).
-__global__ void __launch_bounds__(kThreads)
-sweep_generic_kernel(const SweepSeg* __restrict__ segs, const SweepBlock* __restrict__ blocks, int per_tensor,
-                     const float* __restrict__ tensor_absmax, int jlo, int jhi, double* __restrict__ partial) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  const SweepBlock blk = blocks[blockIdx.x];
-  const int lane = threadIdx.x & 31;
-  __shared__ float smax[kThreads / 32];
-  for (int si = blk.seg0; si < blk.seg0 + blk.nseg; ++si) {
-    const SweepSeg d = segs[si];
-    const float A_tensor = per_tensor ? tensor_absmax[d.tensor] : 0.0f;
-    double dacc[kNB];
-#pragma unroll
-    for (int j = 0; j < kNB; ++j) dacc[j] = 0.0;
-    float amax_blk = 0.0f;
-    for (int row = 0; row < d.rows; ++row) {
-      const float* p = d.w + (int64_t)row * d.cols;
-      float m = 0.0f;
-      for (int c = threadIdx.x; c < d.cols; c += kThreads) m = fmaxf(m, fabsf(__ldg(p + c)));
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0) smax[threadIdx.x >> 5] = m;
-      __syncthreads();
-      m = smax[0];
-      for (int w = 1; w < kThreads / 32; ++w) m = fmaxf(m, smax[w]);
-      __syncthreads();
-      amax_blk = fmaxf(amax_blk, m);
-      if (per_tensor) m = A_tensor;
-      float s_l, inv_l;
-      scales_for_lane(m, lane, s_l, inv_l);
-      float s[kNB], inv[kNB], facc[kNB];
-#pragma unroll
-      for (int j = 0; j < kNB; ++j) {
-        s[j] = __shfl_sync(0xffffffffu, s_l, j);
-        inv[j] = __shfl_sync(0xffffffffu, inv_l, j);
-        facc[j] = 0.0f;
-      }
-      int terms = 0;
-      for (int c = threadIdx.x; c < d.cols; c += kThreads) {
-        float x = __ldg(p + c);
-#pragma unroll
-        for (int j = 0; j < kNB; ++j)
-          if (j >= jlo && j <= jhi) err4(x, s[j], inv[j], facc[j]);
-        if (++terms == kChainTerms) {            // very long rows: keep the fp32 chains short
-#pragma unroll
-          for (int j = 0; j < kNB; ++j) { dacc[j] += (double)facc[j]; facc[j] = 0.0f; }
-          terms = 0;
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < kNB; ++j) dacc[j] += (double)facc[j];
-    }
-    block_reduce_store(dacc, amax_blk, partial + (int64_t)d.slot * 8);
-  }
-}
-
-// One block per tensor: 32 groups of 8 threads stride over the tensor's slots (thread j of a group
-// owns column j: 7 sums and the maximum), then thread j < 8 combines the 32 group results in a
-// fixed order.
-__global__ void __launch_bounds__(256)
-sweep_finalize_kernel(const double* __restrict__ partial, const TensorSlots* __restrict__ ts, int jlo, int nb,
-                      double* __restrict__ sse, float* __restrict__ absmax, int write_absmax) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");     // the slots come from the kernels before
-  __shared__ double sm[32][8];
-  const int t = blockIdx.x;
+// The tensor's result from the slots of its segments, written by the block that finished the last of
+// them: 32 groups of 8 threads stride over the slots (thread j of a group owns column j: 7 sums and
+// the maximum), then thread j < 8 combines the 32 group results.  The order is that of the slots,
+// whichever block does it, so the result does not depend on timing.
+__device__ __forceinline__ void finalize_tensor(const double* __restrict__ partial, int slot0, int slot1, int t, int jlo, int nb,
+                                                double* __restrict__ sse, float* __restrict__ absmax, int write_absmax,
+                                                double (*sm)[8]) {
   const int j = threadIdx.x & 7, g = threadIdx.x >> 3;
-  const TensorSlots r = ts[t];
   double v = 0.0;
-  for (int i = r.slot0 + g; i < r.slot1; i += 32) {
-    const double x = partial[(int64_t)i * 8 + j];
+  for (int i = slot0 + g; i < slot1; i += 32) {
+    const double x = __ldcg(partial + (int64_t)i * 8 + j);      // other blocks wrote them: not through L1
     v = (j == 7) ? fmax(v, x) : v + x;
   }
   sm[g][j] = v;
@@ -339,41 +109,341 @@ sweep_finalize_kernel(const double* __restrict__ partial, const TensorSlots* __r
       sse[(int64_t)t * nb + (j - jlo)] = a;
     }
   }
+  __syncthreads();
+}
+
+// One run of rows of up to 4*V*team elements.  All 7 bit widths are always evaluated (a narrower
+// request only selects columns at the end).
+template <int V, bool ALL_VEC>
+__device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor, float A_tensor, float4* ring,
+                                              double* __restrict__ out) {
+  // rows between two first-stage flushes: every row adds 2*V terms to each half of a packed accumulator
+  constexpr int kFlushRows = (kChainTerms / (2 * V)) > 0 ? (kChainTerms / (2 * V)) : 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int T = 32 << d.team_log2;
+  const int nteams = kThreads >> (5 + d.team_log2);
+  const int team = threadIdx.x >> (5 + d.team_log2);
+  const int tl = threadIdx.x & (T - 1);
+  const int n_iter = (d.rows + nteams - 1) / nteams;
+  const int c4 = d.cols >> 2;
+  int row_parity = 0;
+  __shared__ float smax2[2][kThreads / 32];
+  __shared__ double swarp[kThreads / 32][8];             // per warp: 7 fp64 sums and the maximum
+
+  float2 facc[kNB];
+  float f2[kNB];
+#pragma unroll
+  for (int j = 0; j < kNB; ++j) { facc[j] = make_float2(0.0f, 0.0f); f2[j] = 0.0f; }
+  if (lane < 8) swarp[warp][lane] = 0.0;
+  float amax_blk = 0.0f;
+
+  auto process_row = [&](const float4 (&cur)[V]) {
+    float m = 0.0f;
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+      m = fmaxf(fmaxf(fmaxf(m, fabsf(cur[v].x)), fmaxf(fabsf(cur[v].y), fabsf(cur[v].z))), fabsf(cur[v].w));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (T > 32) {
+      // the team's warps exchange their maxima through shared memory; a named barrier per team
+      // keeps other teams running, and alternating slots make one barrier per row enough
+      float* slot = smax2[row_parity];
+      if (lane == 0) slot[warp] = m;
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(T) : "memory");
+      const int w0 = team * (T >> 5);
+      m = slot[w0];
+      for (int w = 1; w < (T >> 5); ++w) m = fmaxf(m, slot[w0 + w]);
+      row_parity ^= 1;
+    }
+    amax_blk = fmaxf(amax_blk, m);
+    if (per_tensor) m = A_tensor;
+
+    // the 7 scale pairs: two IEEE divisions in lanes 0..6, broadcast by shuffles
+    float s_l, inv_l;
+    scales_for_lane(m, lane, s_l, inv_l);
+    float2 ns[kNB], inv[kNB];
+#pragma unroll
+    for (int j = 0; j < kNB; ++j) {
+      const float sj = -__shfl_sync(0xffffffffu, s_l, j), ij = __shfl_sync(0xffffffffu, inv_l, j);
+      ns[j] = make_float2(sj, sj);
+      inv[j] = make_float2(ij, ij);
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const float2 lo = make_float2(cur[v].x, cur[v].y), hi = make_float2(cur[v].z, cur[v].w);
+#pragma unroll
+      for (int j = 0; j < kNB; ++j) {
+        err8(lo, ns[j], inv[j], facc[j]);
+        err8(hi, ns[j], inv[j], facc[j]);
+      }
+    }
+  };
+  // second stage -> the warp's fp64 sums
+  auto flush2 = [&]() {
+#pragma unroll
+    for (int j = 0; j < kNB; ++j) {
+      float v = f2[j];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) swarp[warp][j] += (double)v;
+      f2[j] = 0.0f;
+    }
+  };
+
+  // Rows stream through a three-stage ring in shared memory filled by cp.async, two rows ahead
+  // of the one being processed: enough loads in flight to cover HBM latency without holding
+  // future rows in registers.  Every thread copies and reads back only its own 16-byte slots, so
+  // no barrier is needed between the copy and the read.  Rows that are not whole aligned float4
+  // are copied word by word, consecutive lanes taking consecutive words; which element sits in
+  // which slot does not matter to the sums.
+  const float* rowp = d.w + (int64_t)team * d.cols + (ALL_VEC || d.vec ? 4 * tl : tl);   // this thread's first element of its team's next row
+  const int64_t row_step = (int64_t)nteams * d.cols;
+  int fetch_row = team;
+  const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(ring + threadIdx.x);
+  auto issue_row = [&](int stage) {
+    const uint32_t dst0 = ring0 + (uint32_t)(stage * V) * (kThreads * 16);
+    const bool row_ok = fetch_row < d.rows;
+    if (ALL_VEC || d.vec) {
+#pragma unroll
+      for (int v = 0; v < V; ++v) {
+        const uint32_t dst = dst0 + v * (kThreads * 16);
+        if (row_ok && tl + v * T < c4) {
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(reinterpret_cast<const float4*>(rowp) + v * T) : "memory");
+        } else {
+          asm volatile("st.shared.v4.f32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "f"(0.0f) : "memory");
+        }
+      }
+    } else {
+#pragma unroll 4
+      for (int e = 0; e < 4 * V; ++e) {
+        const uint32_t dst = dst0 + (e >> 2) * (kThreads * 16) + (e & 3) * 4;
+        if (row_ok && tl + e * T < d.cols) {
+          asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(rowp + e * T) : "memory");
+        } else {
+          asm volatile("st.shared.f32 [%0], %1;" ::"r"(dst), "f"(0.0f) : "memory");
+        }
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    rowp += row_step;
+    fetch_row += nteams;
+  };
+  issue_row(0);
+  issue_row(1);
+  int stage = 0, n1 = 0, n2 = 0;
+  for (int it = 0; it < n_iter; ++it) {
+    int nxt = stage + 2; if (nxt >= kRing) nxt -= kRing;
+    issue_row(nxt);                                                 // zeros past the end
+    asm volatile("cp.async.wait_group 2;" ::: "memory");            // the row of this iteration has landed
+    float4 cur[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) cur[v] = ring[(stage * V + v) * kThreads + threadIdx.x];
+    process_row(cur);
+    if (++n1 == kFlushRows) {
+#pragma unroll
+      for (int j = 0; j < kNB; ++j) { f2[j] += facc[j].x + facc[j].y; facc[j] = make_float2(0.0f, 0.0f); }
+      n1 = 0;
+      if (++n2 == kChainSums - 1) { flush2(); n2 = 0; }
+    }
+    if (++stage == kRing) stage = 0;
+  }
+#pragma unroll
+  for (int j = 0; j < kNB; ++j) f2[j] += facc[j].x + facc[j].y;
+  flush2();
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) amax_blk = fmaxf(amax_blk, __shfl_xor_sync(0xffffffffu, amax_blk, o));
+  if (lane == 0) swarp[warp][7] = (double)amax_blk;
+  __syncthreads();
+  if (threadIdx.x < 8) {                  // the warps' sums in a fixed order
+    double v = swarp[0][threadIdx.x];
+    for (int w = 1; w < kThreads / 32; ++w)
+      v = (threadIdx.x == 7) ? fmax(v, swarp[w][7]) : v + swarp[w][threadIdx.x];
+    out[threadIdx.x] = v;
+  }
+}
+
+// Rows longer than the ring holds: the whole block works on one row at a time and reads it twice
+// (the second read hits L1/L2).
+__device__ __forceinline__ void sweep_segment_long(const SweepSeg& d, int per_tensor, float A_tensor, int jlo, int jhi,
+                                                   double* __restrict__ out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ float smax[kThreads / 32];
+  __shared__ double swarp[kThreads / 32][8];
+  double dacc[kNB];
+#pragma unroll
+  for (int j = 0; j < kNB; ++j) dacc[j] = 0.0;
+  float amax_blk = 0.0f;
+  for (int row = 0; row < d.rows; ++row) {
+    const float* p = d.w + (int64_t)row * d.cols;
+    float m = 0.0f;
+    for (int c = threadIdx.x; c < d.cols; c += kThreads) m = fmaxf(m, fabsf(__ldg(p + c)));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) smax[warp] = m;
+    __syncthreads();
+    m = smax[0];
+    for (int w = 1; w < kThreads / 32; ++w) m = fmaxf(m, smax[w]);
+    __syncthreads();
+    amax_blk = fmaxf(amax_blk, m);
+    if (per_tensor) m = A_tensor;
+    float s_l, inv_l;
+    scales_for_lane(m, lane, s_l, inv_l);
+    float s[kNB], inv[kNB], facc[kNB];
+#pragma unroll
+    for (int j = 0; j < kNB; ++j) {
+      s[j] = __shfl_sync(0xffffffffu, s_l, j);
+      inv[j] = __shfl_sync(0xffffffffu, inv_l, j);
+      facc[j] = 0.0f;
+    }
+    int terms = 0;
+    for (int c = threadIdx.x; c < d.cols; c += kThreads) {
+      float x = __ldg(p + c);
+#pragma unroll
+      for (int j = 0; j < kNB; ++j)
+        if (j >= jlo && j <= jhi) err4(x, s[j], inv[j], facc[j]);
+      if (++terms == kChainTerms) {            // very long rows: keep the fp32 chains short
+#pragma unroll
+        for (int j = 0; j < kNB; ++j) { dacc[j] += (double)facc[j]; facc[j] = 0.0f; }
+        terms = 0;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kNB; ++j) dacc[j] += (double)facc[j];
+  }
+#pragma unroll
+  for (int j = 0; j < kNB; ++j) {
+    double v = warp_sum(dacc[j]);
+    if (lane == 0) swarp[warp][j] = v;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) amax_blk = fmaxf(amax_blk, __shfl_xor_sync(0xffffffffu, amax_blk, o));
+  if (lane == 0) swarp[warp][7] = (double)amax_blk;
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    double v = swarp[0][threadIdx.x];
+    for (int w = 1; w < kThreads / 32; ++w)
+      v = (threadIdx.x == 7) ? fmax(v, swarp[w][7]) : v + swarp[w][threadIdx.x];
+    out[threadIdx.x] = v;
+  }
+}
+
+// All segments of a call.  KV: the float4 count per thread of every segment, all of them aligned, or 0
+// when the plan mixes row lengths (the body is then chosen per segment, at the register count of the
+// largest).  FUSED: the block that finishes a tensor's last segment also writes the tensor's result
+// (plans that do not fill the device: 15.6 us for three tensors of 256 columns against 20.5 with a
+// second launch); otherwise a finalize kernel follows (the counting costs every segment a round trip to
+// L2: 110.4 against 106.3 us for 340 MB).
+template <int KV, bool FUSED>
+__global__ void __launch_bounds__(kThreads, kBlocksPerSM)
+sweep_kernel(const SweepSeg* __restrict__ segs, const SweepBlock* __restrict__ blocks, TensorSlots* __restrict__ slots, int per_tensor,
+             const float* __restrict__ tensor_absmax, int jlo, int nb, double* __restrict__ partial, double* __restrict__ sse,
+             float* __restrict__ absmax) {
+  // Programmatic dependent launch: the block is scheduled while the previous kernel of the stream
+  // drains and waits here for that kernel's results (result slots, per-tensor maxima, and whatever
+  // produced the weights).
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  __shared__ double fin[32][8];
+  __shared__ int last;
+  extern __shared__ float4 ring[];                       // [kRing][V][kThreads]
+  const SweepBlock blk = blocks[blockIdx.x];
+  for (int si = blk.seg0; si < blk.seg0 + blk.nseg; ++si) {
+    const SweepSeg d = segs[si];
+    const float A_tensor = per_tensor ? tensor_absmax[d.tensor] : 0.0f;
+    double* out = partial + (int64_t)d.slot * 8;
+    if (KV > 0) sweep_segment<(KV > 0 ? KV : 1), true>(d, per_tensor, A_tensor, ring, out);
+    else switch (d.v) {
+      case 0: sweep_segment_long(d, per_tensor, A_tensor, jlo, jlo + nb - 1, out); break;
+      case 1: sweep_segment<1, false>(d, per_tensor, A_tensor, ring, out); break;
+      case 2: sweep_segment<2, false>(d, per_tensor, A_tensor, ring, out); break;
+      case 3: sweep_segment<3, false>(d, per_tensor, A_tensor, ring, out); break;
+      case 4: sweep_segment<4, false>(d, per_tensor, A_tensor, ring, out); break;
+      case 5: sweep_segment<5, false>(d, per_tensor, A_tensor, ring, out); break;
+      case 6: sweep_segment<6, false>(d, per_tensor, A_tensor, ring, out); break;
+      case 7: sweep_segment<7, false>(d, per_tensor, A_tensor, ring, out); break;
+      default: sweep_segment<8, false>(d, per_tensor, A_tensor, ring, out); break;
+    }
+    if (!FUSED) { __syncthreads(); continue; }
+    // The eight values of the slot become visible before the segment is counted; the counter wraps
+    // to zero with the tensor's last segment, so the next call finds it as this one did.
+    if (threadIdx.x < 8) __threadfence();
+    __syncthreads();
+    const int slot0 = slots[d.tensor].slot0, slot1 = slots[d.tensor].slot1;
+    if (threadIdx.x == 0) {
+      const unsigned n = (unsigned)(slot1 - slot0);
+      last = atomicInc(&slots[d.tensor].done, n - 1) == n - 1;
+      __threadfence();
+    }
+    __syncthreads();
+    if (last) finalize_tensor(partial, slot0, slot1, d.tensor, jlo, nb, sse, absmax, per_tensor ? 0 : 1, fin);
+  }
+}
+__global__ void __launch_bounds__(kThreads)
+sweep_finalize_kernel(const TensorSlots* __restrict__ slots, int write_absmax, int jlo, int nb, const double* __restrict__ partial,
+                      double* __restrict__ sse, float* __restrict__ absmax) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");     // the slots come from the kernel before
+  __shared__ double fin[32][8];
+  const int t = blockIdx.x;
+  finalize_tensor(partial, slots[t].slot0, slots[t].slot1, t, jlo, nb, sse, absmax, write_absmax, fin);
+}
+
+// Per-tensor maxima for the per-tensor grids, over the same segments: integer max of |x| bit patterns.
+__global__ void __launch_bounds__(kThreads)
+sweep_absmax_kernel(const SweepSeg* __restrict__ segs, const SweepBlock* __restrict__ blocks, unsigned* __restrict__ absmax) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  __shared__ unsigned sm[kThreads / 32];
+  const SweepBlock blk = blocks[blockIdx.x];
+  for (int si = blk.seg0; si < blk.seg0 + blk.nseg; ++si) {
+    const SweepSeg d = segs[si];
+    const int64_t n = (int64_t)d.rows * d.cols;
+    unsigned m = 0;
+    auto fold = [&](float x) { const unsigned a = abs_bits(x); m = m > a ? m : a; };
+    if (d.vec) {
+      const float4* p = reinterpret_cast<const float4*>(d.w);
+#pragma unroll 4
+      for (int64_t i = threadIdx.x; i < (n >> 2); i += kThreads) { const float4 x = __ldg(p + i); fold(x.x); fold(x.y); fold(x.z); fold(x.w); }
+    } else {
+#pragma unroll 4
+      for (int64_t i = threadIdx.x; i < n; i += kThreads) fold(__ldg(d.w + i));
+    }
+    m = warp_max_u(m);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      m = warp_max_u(threadIdx.x < kThreads / 32 ? sm[threadIdx.x] : 0u);
+      if (threadIdx.x == 0 && m) atomicMax(absmax + d.tensor, m);
+    }
+    __syncthreads();
+  }
 }
 
 // Launch configuration with programmatic stream serialization: the kernel may start while its
 // predecessor in the stream drains; it orders itself with griddepcontrol.wait.
-cudaLaunchAttribute g_pdl_attr;
-inline cudaLaunchConfig_t pdl_config(int blocks, int threads, size_t smem, cudaStream_t st) {
-  g_pdl_attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  g_pdl_attr.val.programmaticStreamSerializationAllowed = 1;
+inline cudaLaunchConfig_t pdl_config(cudaLaunchAttribute* attr, int blocks, size_t smem, cudaStream_t st) {
+  attr->id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr->val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)blocks);
-  cfg.blockDim = dim3((unsigned)threads);
+  cfg.blockDim = dim3((unsigned)kThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cfg.attrs = &g_pdl_attr;
+  cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cfg;
 }
 
-template <int V>
-void launch_rows(const SweepSeg* segs, const SweepBlock* blocks, int n_blocks, int per_tensor, const float* amax,
-                 double* partial, cudaStream_t st) {
-  constexpr size_t smem = (size_t)kRing * V * kThreads * sizeof(float4);
-  cudaLaunchConfig_t cfg = pdl_config(n_blocks, kThreads, smem, st);
-  cudaLaunchKernelEx(&cfg, sweep_rows_kernel<V>, segs, blocks, per_tensor, amax, partial);
-}
+using SweepKernel = void (*)(const SweepSeg*, const SweepBlock*, TensorSlots*, int, const float*, int, int, double*, double*, float*);
+constexpr SweepKernel kSweepKernels[9] = {sweep_kernel<0, false>, sweep_kernel<1, false>, sweep_kernel<2, false>,
+                                          sweep_kernel<3, false>, sweep_kernel<4, false>, sweep_kernel<5, false>,
+                                          sweep_kernel<6, false>, sweep_kernel<7, false>, sweep_kernel<8, false>};
+constexpr SweepKernel kSweepFused = sweep_kernel<0, true>;
 
-template <int V>
-cudaError_t set_rows_smem() {
-  return cudaFuncSetAttribute(sweep_rows_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)((size_t)kRing * V * kThreads * sizeof(float4)));
-}
+constexpr size_t ring_bytes(int v) { return (size_t)kRing * v * kThreads * sizeof(float4); }
 
 // ------------------------------------------------------------------ planning (host)
-
-constexpr int kClasses = 9;                  // 0 = generic kernel, V = 1..8 = row kernel variants
 
 // Capacity of the tables a plan is written into.  Segments never exceed blocks + tensors.
 struct PlanTables {
@@ -383,125 +453,132 @@ struct PlanTables {
 };
 struct Plan {
   int n_segs = 0, n_blocks = 0;
-  int class_block0[kClasses], class_blocks[kClasses];
+  int max_v = 0;             // largest float4 count per thread and row: sizes the ring
+  int one_v = 0;             // that count if all rows have it and are aligned, else 0
+  bool fused = false;        // fewer blocks than the device keeps resident: one launch
 };
 
-// Kernel variant and team size of a tensor.
-inline int classify(const float* w, int64_t cols, int* team_log2) {
-  *team_log2 = 0;
-  const bool vec = ((uintptr_t)w % 16 == 0) && (cols % 4 == 0) && cols <= 8192 && cols > 0;
-  if (!vec) return 0;
-  const int64_t c4 = cols / 4;
-  int tl = 0;
-  while (tl < 3 && c4 > (int64_t)(32 << tl) * 8) ++tl;
-  *team_log2 = tl;
-  return (int)((c4 + (32 << tl) - 1) / (32 << tl));     // float4 per thread, 1..8
+// How a tensor's rows are processed, and what one row costs (relative).
+struct RowPlan { int v, team_log2, vec; int64_t cost; };
+// A row takes T = 32 << team_log2 threads with V float4 each.  Measured on long runs of one row length
+// (80 M elements, ns per row over the whole device): T = 32 costs 0.14 (V + 0.5) for V = 1..8, and
+// every doubling of the team about 5 % more per warp (barrier between its warps).  V up to 8 fits
+// the ring with two blocks per SM, V up to 6 with three; two are enough where all rows are that
+// long (1024 columns: 1.27 ns as V = 8 against 1.39 as two warps with V = 4), three serve a mixed plan.
+constexpr int kMaxV = 6;
+inline RowPlan plan_rows(const float* w, int64_t cols, int max_v) {
+  RowPlan best{0, 0, 0, 0};
+  best.vec = ((uintptr_t)w % 16 == 0) && (cols % 4 == 0);
+  const int64_t c4 = (cols + 3) / 4;
+  for (int tl = 0; tl <= 3; ++tl) {
+    const int64_t v = (c4 + (32 << tl) - 1) / (32 << tl);
+    if (v > (tl == 3 ? 8 : max_v)) continue;
+    const int64_t cost = ((int64_t)1 << tl) * (2 * v + 1) * (20 + tl);
+    if (best.v == 0 || cost < best.cost) { best.v = (int)v; best.team_log2 = tl; best.cost = cost; }
+  }
+  if (best.v == 0) best.cost = (cols / 128 + 16) * 80;      // whole block per row, read twice
+  else if (!best.vec) best.cost *= 2;                       // word-wise copies (147 columns: 0.46 against 0.21 ns per row of 128)
+  return best;
 }
 
-// Cuts every variant's rows into equal pieces, one per block.  Returns false when a table is too
-// small.  Segments of one tensor get consecutive slots.
+// Cuts the rows of all tensors into pieces of equal cost, one per block.  Returns false when a table is
+// too small.  Segments of one tensor get consecutive slots; a tensor without elements gets one empty
+// segment, whose zeros become its result.
 bool plan_sweep(const float* const* w, const int64_t* rows, const int64_t* cols, int32_t n_tensors, int sms,
                 const PlanTables& T, Plan* P) {
   if (n_tensors > T.max_tensors) return false;
-  const int resident = sms * kBlocksPerSM;
-  for (int t = 0; t < n_tensors; ++t)      // tensors without elements keep an empty slot range
-    T.slots[t].slot0 = T.slots[t].slot1 = 0;
-  for (int c = 0; c < kClasses; ++c) {
-    P->class_block0[c] = P->n_blocks;
-    P->class_blocks[c] = 0;
-    int64_t total = 0;
-    int tl;
-    for (int t = 0; t < n_tensors; ++t)
-      if (classify(w[t], cols[t], &tl) == c) total += rows[t] * cols[t];
-    if (total == 0) continue;
-    int64_t nblk = (total + kMinBlockElems - 1) / kMinBlockElems;
-    if (nblk > resident) nblk = resident;
-    if (P->n_blocks + nblk > T.max_blocks) return false;
-    const int64_t quota = (total + nblk - 1) / nblk;           // elements per block
-    int blk = P->n_blocks;
-    const int blk_last = P->n_blocks + (int)nblk - 1;
-    int64_t room = quota;
-    T.blocks[blk].seg0 = P->n_segs; T.blocks[blk].nseg = 0;
+  int64_t total = 0, elems = 0;
+  int limit = 8;
+  for (int pass = 0; pass < 2; ++pass) {       // rows of one kind only: V up to 8; otherwise plan again with the mixed plan's limit
+    total = elems = 0;
+    P->max_v = 0;
     for (int t = 0; t < n_tensors; ++t) {
-      if (rows[t] * cols[t] == 0 || classify(w[t], cols[t], &tl) != c) continue;
-      T.slots[t].slot0 = P->n_segs;
-      int64_t row = 0;
-      while (row < rows[t]) {
-        int64_t take = (room + cols[t] - 1) / cols[t];         // whole rows filling the block's quota
-        if (c > 0) {                                            // whole rounds of the block's teams
-          const int64_t nt = kThreads / (32 << tl);
-          take = (take + nt - 1) / nt * nt;
-        }
-        if (blk == blk_last) take = rows[t] - row;              // the last block takes what is left
-        if (take < 1) take = 1;
-        if (take > rows[t] - row) take = rows[t] - row;
-        if (take > 0x7fffffff) take = 0x7fffffff;
-        if (P->n_segs >= T.max_segs) return false;
-        SweepSeg& s = T.segs[P->n_segs];
-        s.w = w[t] + row * cols[t]; s.rows = (int32_t)take; s.cols = (int32_t)cols[t]; s.tensor = t;
-        s.team_log2 = tl; s.slot = P->n_segs; s.pad = 0;
-        P->n_segs++;
-        T.blocks[blk].nseg++;
-        row += take;
-        room -= take * cols[t];
-        if (room <= 0 && blk < blk_last) {
-          ++blk;
-          T.blocks[blk].seg0 = P->n_segs; T.blocks[blk].nseg = 0;
-          room = quota;
-        }
-      }
-      T.slots[t].slot1 = P->n_segs;
+      if (rows[t] * cols[t] == 0) continue;
+      const RowPlan r = plan_rows(w[t], cols[t], limit);
+      P->one_v = r.vec && (elems == 0 || r.v == P->one_v) ? r.v : 0;
+      if (r.v > P->max_v) P->max_v = r.v;
+      total += rows[t] * r.cost;
+      elems += rows[t] * cols[t];
     }
-    // blocks left without a segment are not launched
-    const int used = blk - P->n_blocks + (T.blocks[blk].nseg > 0 ? 1 : 0);
-    P->class_blocks[c] = used;
-    P->n_blocks += used;
+    if (P->one_v || P->max_v <= kMaxV) break;
+    limit = kMaxV;
   }
+  if (P->max_v < 1) P->max_v = 1;
+  const int resident = sms * (P->max_v > kMaxV ? 2 : kBlocksPerSM);
+  int64_t nblk = (elems + kMinBlockElems - 1) / kMinBlockElems;
+  if (nblk > resident) nblk = resident;
+  if (nblk < 1) nblk = 1;
+  P->fused = nblk < resident;
+  if (nblk > T.max_blocks) return false;
+  const int64_t quota = (total + nblk - 1) / nblk;             // cost per block
+  int blk = 0;
+  int64_t room = quota;
+  T.blocks[0].seg0 = 0; T.blocks[0].nseg = 0;
+  for (int t = 0; t < n_tensors; ++t) {
+    const bool empty = rows[t] * cols[t] == 0;
+    const RowPlan r = empty ? RowPlan{P->one_v ? P->one_v : 1, 0, 0, 1} : plan_rows(w[t], cols[t], limit);
+    const int64_t nt = r.v ? kThreads / (32 << r.team_log2) : 1;
+    T.slots[t].slot0 = P->n_segs;
+    T.slots[t].done = 0; T.slots[t].pad = 0;
+    const int64_t n_rows = empty ? 0 : rows[t];
+    int64_t row = 0;
+    do {
+      int64_t take = (room + r.cost - 1) / r.cost;              // whole rows filling the block's quota
+      if (take < 8 * nt) take = (take + nt - 1) / nt * nt;      // few rounds of the block's teams: whole ones
+      if (blk == nblk - 1) take = n_rows - row;                 // the last block takes what is left
+      if (take < nt) take = nt;
+      if (take > n_rows - row) take = n_rows - row;
+      if (take > 0x40000000) take = 0x40000000;
+      if (P->n_segs >= T.max_segs) return false;
+      SweepSeg& s = T.segs[P->n_segs];
+      s.w = empty ? nullptr : w[t] + row * cols[t]; s.rows = (int32_t)take; s.cols = empty ? 0 : (int32_t)cols[t]; s.tensor = t;
+      s.team_log2 = r.team_log2; s.slot = P->n_segs; s.v = (int16_t)r.v; s.vec = (int16_t)r.vec;
+      P->n_segs++;
+      T.blocks[blk].nseg++;
+      row += take;
+      room -= take * r.cost;
+      if (room <= 0 && blk < nblk - 1) {
+        ++blk;
+        T.blocks[blk].seg0 = P->n_segs; T.blocks[blk].nseg = 0;
+        room += quota;                                          // what this block took beyond its quota the next one takes less
+        if (room < quota / 2) room = quota / 2;
+      }
+    } while (row < n_rows);
+    T.slots[t].slot1 = P->n_segs;
+  }
+  P->n_blocks = blk + (T.blocks[blk].nseg > 0 ? 1 : 0);        // a last block left without a segment is not launched
   return true;
 }
 
 // Enqueues the sweep's kernels for a plan whose tables are on the device already.
-int run_plan(Ctx* ctx, const Plan& P, const SweepSeg* segs, const SweepBlock* blocks, const TensorSlots* slots,
-             double* partial, const float* const* w, const int64_t* rows, const int64_t* cols, int32_t n_tensors,
-             int per_tensor, int b_lo, int b_hi, double* sse, float* absmax, cudaStream_t st) {
+int run_plan(Ctx* ctx, const Plan& P, const SweepSeg* segs, const SweepBlock* blocks, TensorSlots* slots, double* partial,
+             int32_t n_tensors, int per_tensor, int b_lo, int b_hi, double* sse, float* absmax, cudaStream_t st) {
+  cudaLaunchAttribute attr;
   if (per_tensor) {
-    for (int t = 0; t < n_tensors; ++t) {
-      int rc = launch_absmax(ctx, w[t], rows[t], cols[t], cols[t], QCFG_PER_TENSOR, absmax + t, st);
-      if (rc != QCFG_OK) return rc;
-    }
-  }
-  const int jlo = b_lo - 2, jhi = b_hi - 2, nb = b_hi - b_lo + 1;
-  for (int c = 0; c < kClasses; ++c) {
-    const int n = P.class_blocks[c];
-    if (n == 0) continue;
-    const SweepBlock* b = blocks + P.class_block0[c];
+    cudaError_t e = cudaMemsetAsync(absmax, 0, (size_t)n_tensors * sizeof(float), st);
+    if (e != cudaSuccess) return check_cuda(ctx, e, "memset absmax");
+    cudaLaunchConfig_t cfg = pdl_config(&attr, P.n_blocks, 0, st);
     prof_begin(ctx, 2, st);
-    switch (c) {
-      case 0: {
-        cudaLaunchConfig_t cfg = pdl_config(n, kThreads, 0, st);
-        cudaLaunchKernelEx(&cfg, sweep_generic_kernel, segs, b, per_tensor, (const float*)absmax, jlo, jhi, partial);
-        break;
-      }
-      case 1: launch_rows<1>(segs, b, n, per_tensor, absmax, partial, st); break;
-      case 2: launch_rows<2>(segs, b, n, per_tensor, absmax, partial, st); break;
-      case 3: launch_rows<3>(segs, b, n, per_tensor, absmax, partial, st); break;
-      case 4: launch_rows<4>(segs, b, n, per_tensor, absmax, partial, st); break;
-      case 5: launch_rows<5>(segs, b, n, per_tensor, absmax, partial, st); break;
-      case 6: launch_rows<6>(segs, b, n, per_tensor, absmax, partial, st); break;
-      case 7: launch_rows<7>(segs, b, n, per_tensor, absmax, partial, st); break;
-      default: launch_rows<8>(segs, b, n, per_tensor, absmax, partial, st); break;
-    }
+    e = cudaLaunchKernelEx(&cfg, sweep_absmax_kernel, segs, blocks, reinterpret_cast<unsigned*>(absmax));
     prof_end(ctx, 2, 0.0, st);
+    if (e != cudaSuccess) return check_cuda(ctx, e, "sweep absmax launch");
     count_launch(ctx);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return check_cuda(ctx, e, "sweep launch");
   }
-  {
-    cudaLaunchConfig_t cfg = pdl_config(n_tensors, 256, 0, st);
-    cudaLaunchKernelEx(&cfg, sweep_finalize_kernel, (const double*)partial, slots, jlo, nb, sse, absmax, per_tensor ? 0 : 1);
-  }
+  cudaLaunchConfig_t cfg = pdl_config(&attr, P.n_blocks, ring_bytes(P.max_v), st);
+  prof_begin(ctx, 2, st);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, P.fused ? kSweepFused : kSweepKernels[P.one_v], segs, blocks, slots, per_tensor,
+                                     (const float*)absmax, b_lo - 2, b_hi - b_lo + 1, partial, sse, absmax);
+  prof_end(ctx, 2, 0.0, st);
+  if (e != cudaSuccess) return check_cuda(ctx, e, "sweep launch");
   count_launch(ctx);
-  return check_cuda(ctx, cudaGetLastError(), "sweep finalize launch");
+  if (!P.fused) {
+    cfg = pdl_config(&attr, n_tensors, 0, st);
+    e = cudaLaunchKernelEx(&cfg, sweep_finalize_kernel, (const TensorSlots*)slots, per_tensor ? 0 : 1, b_lo - 2, b_hi - b_lo + 1,
+                           (const double*)partial, sse, absmax);
+    if (e != cudaSuccess) return check_cuda(ctx, e, "sweep finalize launch");
+    count_launch(ctx);
+  }
+  return check_cuda(ctx, cudaGetLastError(), "sweep launch");
 }
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -511,49 +588,44 @@ inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // The shared-memory opt-in of a kernel is a per-device attribute: set for every variant whenever a
 // context is created (the context's device is current then).
 int sweep_init(Ctx* ctx) {
-  cudaError_t e = set_rows_smem<1>();
-  if (e == cudaSuccess) e = set_rows_smem<2>();
-  if (e == cudaSuccess) e = set_rows_smem<3>();
-  if (e == cudaSuccess) e = set_rows_smem<4>();
-  if (e == cudaSuccess) e = set_rows_smem<5>();
-  if (e == cudaSuccess) e = set_rows_smem<6>();
-  if (e == cudaSuccess) e = set_rows_smem<7>();
-  if (e == cudaSuccess) e = set_rows_smem<8>();
+  cudaError_t e = cudaSuccess;
+  for (int v = 0; v <= 8 && e == cudaSuccess; ++v)
+    e = cudaFuncSetAttribute(kSweepKernels[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes(v ? v : 8));
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(kSweepFused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring_bytes(8));
   return check_cuda(ctx, e, "sweep smem attribute");
 }
 
 int launch_sweep(Ctx* ctx, const float* const* w, const int64_t* rows, const int64_t* cols, int32_t n_tensors,
                  int granularity, int b_lo, int b_hi, double* sse, float* absmax, cudaStream_t st) {
   if (n_tensors == 0) return QCFG_OK;
-  const int resident = sm_count(ctx) * kBlocksPerSM;
-  const int max_blocks = kClasses * resident, max_segs = max_blocks + n_tensors;
-  // host tables in one context-owned buffer: segments | blocks | tensor slot ranges
-  const size_t seg_bytes = align_up((size_t)max_segs * sizeof(SweepSeg), 16);
-  const size_t blk_bytes = align_up((size_t)max_blocks * sizeof(SweepBlock), 16);
+  const int max_blocks = sm_count(ctx) * kBlocksPerSM, max_segs = max_blocks + n_tensors;
+  // host tables in one context-owned buffer: tensor slot ranges | blocks | segments
   const size_t slot_bytes = align_up((size_t)n_tensors * sizeof(TensorSlots), 16);
-  const size_t table_bytes = seg_bytes + blk_bytes + slot_bytes;
-  char* host = static_cast<char*>(host_scratch(ctx, table_bytes));
+  const size_t blk_bytes = align_up((size_t)max_blocks * sizeof(SweepBlock), 16);
+  const size_t seg_bytes = (size_t)max_segs * sizeof(SweepSeg);
+  char* host = static_cast<char*>(host_scratch(ctx, slot_bytes + blk_bytes + seg_bytes));
   if (!host) return set_error(ctx, QCFG_ENOMEM, "sweep: host tables");
-  memset(host, 0, table_bytes);
-  PlanTables T{reinterpret_cast<SweepSeg*>(host), max_segs, reinterpret_cast<SweepBlock*>(host + seg_bytes), max_blocks,
-               reinterpret_cast<TensorSlots*>(host + seg_bytes + blk_bytes), n_tensors};
+  memset(host + slot_bytes, 0, blk_bytes);                       // entries of unused blocks take part in the comparison below
+  PlanTables T{reinterpret_cast<SweepSeg*>(host + slot_bytes + blk_bytes), max_segs,
+               reinterpret_cast<SweepBlock*>(host + slot_bytes), max_blocks, reinterpret_cast<TensorSlots*>(host), n_tensors};
   Plan P;
   if (!plan_sweep(w, rows, cols, n_tensors, sm_count(ctx), T, &P)) return set_error(ctx, QCFG_EINVAL, "sweep: planning failed");
+  const size_t used = slot_bytes + blk_bytes + (size_t)P.n_segs * sizeof(SweepSeg);
 
   // device scratch: partials | the same three tables
-  const size_t partial_bytes = align_up((size_t)(max_segs > 0 ? max_segs : 1) * 8 * sizeof(double), 256);
-  char* base = static_cast<char*>(scratch(ctx, partial_bytes + table_bytes));
-  if (!base) return set_error(ctx, QCFG_ENOMEM, "sweep scratch (%zu bytes)", partial_bytes + table_bytes);
+  const size_t partial_bytes = align_up((size_t)max_segs * 8 * sizeof(double), 256);
+  char* base = static_cast<char*>(scratch(ctx, partial_bytes + slot_bytes + blk_bytes + seg_bytes));
+  if (!base) return set_error(ctx, QCFG_ENOMEM, "sweep scratch (%zu bytes)", partial_bytes + slot_bytes + blk_bytes + seg_bytes);
   char* tab = base + partial_bytes;
   // the tables only depend on the tensor list: a repeated sweep of the same tensors (same scratch
-  // buffer) finds them on the device already
-  if (!sweep_tables_cached(ctx, base, st, host, table_bytes, nullptr, 0)) {
-    const cudaError_t e = cudaMemcpyAsync(tab, host, table_bytes, cudaMemcpyHostToDevice, st);
+  // buffer) finds them on the device already, the counters back at zero
+  if (!sweep_tables_cached(ctx, base, st, host, used, nullptr, 0)) {
+    const cudaError_t e = cudaMemcpyAsync(tab, host, used, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return check_cuda(ctx, e, "sweep table upload");
   }
-  return run_plan(ctx, P, reinterpret_cast<const SweepSeg*>(tab), reinterpret_cast<const SweepBlock*>(tab + seg_bytes),
-                  reinterpret_cast<const TensorSlots*>(tab + seg_bytes + blk_bytes), reinterpret_cast<double*>(base), w, rows,
-                  cols, n_tensors, granularity == QCFG_PER_TENSOR, b_lo, b_hi, sse, absmax, st);
+  return run_plan(ctx, P, reinterpret_cast<const SweepSeg*>(tab + slot_bytes + blk_bytes),
+                  reinterpret_cast<const SweepBlock*>(tab + slot_bytes), reinterpret_cast<TensorSlots*>(tab),
+                  reinterpret_cast<double*>(base), n_tensors, granularity == QCFG_PER_TENSOR, b_lo, b_hi, sse, absmax, st);
 }
 
 
@@ -564,7 +636,7 @@ int launch_sweep(Ctx* ctx, const float* const* w, const int64_t* rows, const int
 // (about 0.6 MiB on every GPU that loads the library, until the process exits).
 
 constexpr int kStaticMaxTensors = 1024;
-constexpr int kStaticMaxBlocks = 4096;                                  // 9 variants x 3 blocks x up to 151 SMs
+constexpr int kStaticMaxBlocks = 4096;                                  // 3 per SM
 constexpr int kStaticMaxSegs = kStaticMaxBlocks + kStaticMaxTensors;
 constexpr int64_t kStaticMaxElems = (int64_t)1 << 35;                   // elements per call
 
@@ -597,7 +669,7 @@ int launch_sweep_static(Ctx* ctx, const float* const* w, const int64_t* rows, co
     if (total > kStaticMaxElems)
       return set_error(ctx, QCFG_ENOMEM, "static sweep: more than 2^35 elements in one call; split the tensors over several calls");
   }
-  if (kClasses * sm_count(ctx) * kBlocksPerSM > kStaticMaxBlocks)
+  if (sm_count(ctx) * kBlocksPerSM > kStaticMaxBlocks)
     return set_error(ctx, QCFG_ENOMEM, "static sweep: the device has more SMs than the fixed tables are sized for");
 
   int dev = -1;
@@ -631,7 +703,7 @@ int launch_sweep_static(Ctx* ctx, const float* const* w, const int64_t* rows, co
   if (e == cudaSuccess) e = cudaMemcpyAsync(S->blocks, T.blocks, (size_t)P.n_blocks * sizeof(SweepBlock), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(S->slots, T.slots, (size_t)n_tensors * sizeof(TensorSlots), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return check_cuda(ctx, e, "static sweep: table upload");
-  return run_plan(ctx, P, S->segs, S->blocks, S->slots, S->partial, w, rows, cols, n_tensors,
+  return run_plan(ctx, P, S->segs, S->blocks, S->slots, S->partial, n_tensors,
                   granularity == QCFG_PER_TENSOR, b_lo, b_hi, sse, absmax, st);
 }
 

@@ -141,6 +141,35 @@ def test_sweep_matches_oracle(ctx, granularity):
     _check_sweep(ctx, tensors, granularity)
 
 
+@pytest.mark.parametrize("granularity", [orc.PER_ROW, orc.PER_TENSOR])
+@pytest.mark.parametrize("shapes,offset", [
+    ([(256, 256), (10, 256)], 0),                    # fewer pieces than resident blocks
+    ([(0, 64), (5, 64), (3, 0), (64, 147)], 0),      # empty tensors, rows that are not whole float4
+    ([(1300, 768), (40, 3072)], 0),                  # one row kind, teams of one and of four warps
+    ([(700, 1024), (77, 4096)], 0),                  # one row kind of the widest chunk
+    ([(300, 768), (129, 1024), (2, 8193), (1000, 20)], 0),
+    ([(130, 256), (33, 768)], 1),                    # rows that do not start on 16 bytes
+])
+def test_sweep_plans_match_oracle(ctx, shapes, offset, granularity):
+    rng = np.random.default_rng(len(shapes) + offset)
+    tensors, on_dev = [], []
+    for s in shapes:
+        tensors.append((rng.standard_normal(s) * rng.uniform(0.01, 3, (s[0], 1))).astype(np.float32))
+        buf = torch.zeros(s[0] * s[1] + offset, device="cuda")
+        buf[offset:] = dev(tensors[-1]).reshape(-1)
+        on_dev.append(buf[offset:].view(s))
+    for _ in range(2):                               # the second call reuses the first one's tables
+        sse, amax = ctx.quant_error_sweep(on_dev, granularity)
+        st, at = ctx.quant_error_sweep_static(on_dev, granularity)
+        ctx.check_sync()
+        full = [i for i, t in enumerate(tensors) if t.size]
+        so, ao = np.zeros((len(tensors), 7)), np.zeros(len(tensors), np.float32)      # a tensor without elements: zeros
+        so[full], ao[full] = orc.quant_error_sweep([tensors[i] for i in full], granularity)
+        np.testing.assert_array_equal(host(amax), ao)
+        np.testing.assert_allclose(host(sse), so, rtol=1e-5, atol=0)
+        assert torch.equal(sse, st) and torch.equal(amax, at)
+
+
 def test_sweep_is_deterministic_and_handles_subranges(ctx):
     rng = np.random.default_rng(1)
     ts = [dev((rng.standard_normal((500, 768)) * 0.02).astype(np.float32)) for _ in range(3)]
