@@ -21,13 +21,12 @@
 // Queues were slower: blocks taking items of an eighth of a piece 126 us against 94 for 80 M elements
 // in rows of 768, single warps taking items 125 us.
 //
-// Sums: fp32 in three short stages, then fp64.  A thread's packed accumulators take at most
+// Sums: fp32 in two short stages, then fp64.  A thread's packed accumulators take at most
 // kChainTerms squared errors each; they are then added into a second fp32 accumulator per bit width,
-// which takes at most kChainSums such sums; that one is reduced over the warp by five pairwise
-// steps and added to the warp's fp64 sum in shared memory.  A sequential fp32 sum of n non-negative
-// terms is within (n-1)*2^-24 relative of the exact sum, so the three stages together stay within
-// (31 + 1 + 15 + 5) * 2^-24 = 3.1e-6, inside the sweep's 1e-5 tolerance; no thread keeps fp64
-// accumulators in registers.
+// which takes at most kChainSums such sums; that one is reduced over the warp in fp64 and added to the
+// warp's sum in shared memory.  A sequential fp32 sum of n non-negative terms is within (n-1)*2^-24
+// relative of the exact sum, so the two stages together stay within (23 + 1 + 15) * 2^-24 = 2.3e-6,
+// inside the sweep's 1e-5 tolerance; no thread keeps fp64 accumulators in registers.
 #include <cstring>
 
 #include "common.cuh"
@@ -41,7 +40,7 @@ constexpr int kNB = 7;                       // bit widths 2..8
 constexpr float kMagic = 12582912.0f;        // 1.5 * 2^23
 constexpr int kRing = 3;                     // shared-memory row stages per thread
 constexpr int kBlocksPerSM = 3;
-constexpr int kChainTerms = 32;              // terms per fp32 accumulator of the first stage
+constexpr int kChainTerms = 24;              // terms per fp32 accumulator of the first stage
 constexpr int kChainSums = 16;               // such sums per fp32 accumulator of the second stage
 constexpr int64_t kMinBlockElems = 2 * 1024;   // do not cut the work finer than one round of a block's eight warps at 256 columns
 
@@ -182,10 +181,8 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
   auto flush2 = [&]() {
 #pragma unroll
     for (int j = 0; j < kNB; ++j) {
-      float v = f2[j];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) swarp[warp][j] += (double)v;
+      const double v = warp_sum((double)f2[j]);
+      if (lane == 0) swarp[warp][j] += v;
       f2[j] = 0.0f;
     }
   };
