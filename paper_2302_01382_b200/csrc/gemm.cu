@@ -1572,8 +1572,10 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   const GemmArgs* gs = ordered;
   const GemmArgs& g0 = gs[0];
   const int esz = g0.is_bf16 ? 2 : 1;
-  // Tile width: by the output's width, then halved while that still leaves every CTA of the launch one
-  // tile at most.
+  // Tile width: by the output's width, then halved while every CTA of the launch still has one tile at
+  // most: a launch that fills half of the SMs or fewer is as long as one tile, and half a tile is
+  // shorter (a mixed 4/8/16-bit block of 768 x 3072 at 3072 tokens: 76.6 -> 74.1 us; the results do not
+  // depend on the tile width).
   int bn = tile_n_of(g0.n);
   {
     const int sms = sm_count(ctx);
