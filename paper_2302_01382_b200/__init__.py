@@ -114,6 +114,11 @@ def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else C.c_void_p(t.data_ptr())
 
 
+def _doubles(a) -> List[float]:
+    """A ctypes array of doubles as a list (one conversion of the buffer, not one per element)."""
+    return memoryview(a).cast("B").cast("d").tolist()
+
+
 def _stream(stream) -> C.c_void_p:
     if stream is None:
         stream = torch.cuda.current_stream()
@@ -366,7 +371,7 @@ class Model:
         ps = (C.c_void_p * n)(*[C.addressof(a) for a in bufs_s])
         pi = (C.c_void_p * n)(*[C.addressof(a) for a in bufs_i])
         self.ctx._check(self.ctx.lib.qcfg_scale_gradients(self.ctx.h, self.h, b, _ptr(x), m, dsx, dix, ps, pi, C.byref(loss), _stream(stream)))
-        return loss.value, list(dsx), list(dix), [list(a) for a in bufs_s], [list(a) for a in bufs_i]
+        return loss.value, list(dsx), list(dix), [_doubles(a) for a in bufs_s], [_doubles(a) for a in bufs_i]
 
     def scales(self, layer: int, bits: int):
         """(scale_x, inv_scale_x, scale_w[n_out], inv_scale_w[n_out]) in use for `layer` at `bits`."""

@@ -200,7 +200,9 @@ struct LayerState {
   // activation scales after scale adjustment, by bit width (otherwise derived from act_absmax)
   bool adj_act[17] = {false};
   float adj_sx[17] = {0}, adj_ix[17] = {0};
-  DevBuf ylin, yact, gout, dsw, diw;   // scale adjustment: rescaled accumulators, activated output, dL/d(output), weight scale gradients
+  DevBuf ylin, yact, gout;         // scale adjustment: rescaled accumulators, activated output, dL/d(output)
+  const float* yact_ptr = nullptr; // activated output of the last adjustment pass (ylin itself without activation and shortcut)
+  double *dsw = nullptr, *diw = nullptr;   // weight scale gradients of the last pass, inside the model's adj_grads
   std::vector<int> consumers;      // layers reading this layer's output as GEMM input
   bool feeds_residual = false;
   // per-evaluation state
@@ -228,7 +230,7 @@ struct Model {
   std::vector<int> calib_same_as;  // layer whose calibrated maximum layer l shares (same input tensor), or -1
   DevBuf search_ref, search_out, search_partial;   // buffers of the search drivers
   DevBuf noise_codes, noise_amax;                  // perturbed bf16 weights of one layer and its max|w|
-  DevBuf adj_gs, adj_gt, adj_qxt, adj_qwt, adj_dx, adj_dw, adj_colsum, adj_dscal;   // scale adjustment temporaries
+  DevBuf adj_gs, adj_gt, adj_qxt, adj_qwt, adj_dx, adj_dw, adj_grads, adj_coef;   // scale adjustment temporaries
   int64_t last_m = 0;
   // what the layers' buffers hold after the last evaluation (for prefix reuse)
   bool reuse_valid = false;
@@ -935,14 +937,14 @@ int qcfg_model_destroy(qcfg_model* model) {
   Model* M = &model->m;
   for (auto& S : M->L) {
     S.w_absmax.release(); S.ybuf.release(); S.abuf.release(); S.prebuf.release();
-    S.ylin.release(); S.yact.release(); S.gout.release(); S.dsw.release(); S.diw.release();
+    S.ylin.release(); S.yact.release(); S.gout.release();
     for (auto& W : S.wc) { W.codes.release(); W.scale.release(); W.inv.release(); }
   }
   M->act_absmax_dev.release();
   M->search_ref.release(); M->search_out.release(); M->search_partial.release();
   M->noise_codes.release(); M->noise_amax.release();
   M->adj_gs.release(); M->adj_gt.release(); M->adj_qxt.release(); M->adj_qwt.release();
-  M->adj_dx.release(); M->adj_dw.release(); M->adj_colsum.release(); M->adj_dscal.release();
+  M->adj_dx.release(); M->adj_dw.release(); M->adj_grads.release(); M->adj_coef.release();
   delete model;
   return QCFG_OK;
 }
@@ -1273,12 +1275,14 @@ int qcfg_noise_sensitivity(qcfg_ctx* ctx, qcfg_model* model, const float* x_dev,
 namespace {
 
 // One pass of the adjustment: the forward of the model under `bits` with its current scales, layer
-// by layer with the rescaled accumulators (ylin) and the activated outputs (yact) kept, the loss
+// by layer with the rescaled accumulators (ylin) and the activated outputs kept, the loss
 // against yref, and (want_grads) the backward pass that leaves the gradients of the weight scales
-// in every layer's dsw / diw and those of the activation scales in M->adj_dscal (two doubles per
-// layer: d/d(scale), d/d(inv_scale)).  Linear layers only.  Synchronises the stream.
+// in every layer's dsw / diw and those of the activation scales at the start of M->adj_grads (two
+// doubles per layer: d/d(scale), d/d(inv_scale)); with grads_host these values are also copied
+// there (2 n, then all dsw, then all diw).  Layers the loss does not depend on have zero gradients and no backward
+// work.  Linear layers only.  Synchronises the stream once, at the end.
 int adjust_pass(qcfg_ctx* h, Model* M, const uint8_t* bits, const float* x_dev, int64_t m, const float* yref, double* loss,
-                bool want_grads, cudaStream_t st) {
+                bool want_grads, std::vector<double>* grads_host, cudaStream_t st) {
   Ctx* c = &h->c;
   const int n = (int)M->L.size();
   const int64_t x_ld = ext_ld_of(M);
@@ -1286,38 +1290,46 @@ int adjust_pass(qcfg_ctx* h, Model* M, const uint8_t* bits, const float* x_dev, 
   auto input_of = [&](int l, const float** p, int64_t* ld) {
     const qcfg_layer& d = M->L[l].d;
     if (d.src < 0) { *p = x_dev + d.src_col0; *ld = x_ld; }
-    else { *p = (const float*)M->L[d.src].yact.p + d.src_col0; *ld = M->L[d.src].d.n_out; }
+    else { *p = M->L[d.src].yact_ptr + d.src_col0; *ld = M->L[d.src].d.n_out; }
   };
   int rc = QCFG_OK;
   for (int l = 0; l < n && !rc; ++l) {
     LayerState& S = M->L[l];
     const qcfg_layer& d = S.d;
-    if (d.kh > 0 || d.pool_before != QCFG_POOL_NONE)
-      return set_error(c, QCFG_ESHAPE, "scale adjustment covers linear layers only (layer %d is a convolution or pooled)", l);
     const int b = bits[l];
-    S.rows = m; S.bits = b;
+    S.rows = m; S.bits = b; S.implicit = false;
     rc = ensure_weight_codes(c, S, b, st);
-    if (!rc) rc = S.abuf.ensure(c, (size_t)(m * S.ldk) * 2);
     if (!rc) rc = S.ylin.ensure(c, (size_t)(m * d.n_out) * 4);
-    if (!rc) rc = S.yact.ensure(c, (size_t)(m * d.n_out) * 4);
     if (rc) break;
     const float* xin; int64_t ldx;
     input_of(l, &xin, &ldx);
     float sx = 1.0f, ix = 1.0f;
     if (b != 16) act_scales(S, b, &sx, &ix);
-    rc = launch_quantize(c, xin, m, d.k_in, ldx, nullptr, ix, QCFG_PER_TENSOR, b, S.abuf.p, S.ldk, st);
-    if (rc) break;
-    S.a_ptr = S.abuf.p; S.a_ready = true;
+    S.a_ptr = nullptr;
+    for (int j = 0; j < l && !S.a_ptr; ++j)          // layers that read the same input with the same grid share its codes
+      if (same_input(M->L[j].d, d) && bits[j] == b && (b == 16 || act_inv(M->L[j], b) == ix)) S.a_ptr = M->L[j].a_ptr;
+    if (!S.a_ptr) {
+      rc = S.abuf.ensure(c, (size_t)(m * S.ldk) * 2);
+      if (!rc) rc = launch_quantize(c, xin, m, d.k_in, ldx, nullptr, ix, QCFG_PER_TENSOR, b, S.abuf.p, S.ldk, st);
+      if (rc) break;
+      S.a_ptr = S.abuf.p;
+    }
+    S.a_ready = true;
     GemmArgs g{};
-    g.a = S.abuf.p; g.lda = S.ldk; g.b = S.wc[b].codes.p; g.ldb = S.ldk;
+    g.a = S.a_ptr; g.lda = S.ldk; g.b = S.wc[b].codes.p; g.ldb = S.ldk;
     g.m = m; g.n = d.n_out; g.k = d.k_in; g.is_bf16 = b == 16; g.act = QCFG_ACT_NONE;
     g.scale_x = sx; g.scale_w = b == 16 ? nullptr : (const float*)S.wc[b].scale.p;
     g.y = (float*)S.ylin.p; g.ldy = d.n_out;
     rc = launch_gemm(c, g, st);
-    const float* res = d.residual_from >= 0 ? (const float*)M->L[d.residual_from].yact.p : nullptr;
-    if (!rc) rc = launch_act_apply(c, (const float*)S.ylin.p, res, d.residual_from >= 0 ? M->L[d.residual_from].d.n_out : 0, d.act,
-                                   (float*)S.yact.p, m, d.n_out, st);
-    S.y_ptr = (const float*)S.yact.p; S.y_internal = false;
+    S.yact_ptr = (const float*)S.ylin.p;
+    if (!rc && (d.residual_from >= 0 || d.act != QCFG_ACT_NONE)) {
+      const float* res = d.residual_from >= 0 ? M->L[d.residual_from].yact_ptr : nullptr;
+      rc = S.yact.ensure(c, (size_t)(m * d.n_out) * 4);
+      if (!rc) rc = launch_act_apply(c, (const float*)S.ylin.p, res, d.residual_from >= 0 ? M->L[d.residual_from].d.n_out : 0, d.act,
+                                     (float*)S.yact.p, m, d.n_out, st);
+      S.yact_ptr = (const float*)S.yact.p;
+    }
+    S.y_ptr = S.yact_ptr; S.y_internal = false;
   }
   if (rc) return rc;
   LayerState& Z = M->L[n - 1];
@@ -1325,89 +1337,126 @@ int adjust_pass(qcfg_ctx* h, Model* M, const uint8_t* bits, const float* x_dev, 
   const int blocks = c->sms * 4;
   rc = M->search_partial.ensure(c, (size_t)blocks * 16);
   std::vector<double> partial((size_t)blocks * 2);
-  const float* ref = yref ? yref : (const float*)Z.yact.p;
-  if (!rc) rc = launch_sqdiff(c, (const float*)Z.yact.p, ref, out_elems, (double*)M->search_partial.p, blocks, st);
-  if (!rc) rc = check_cuda(c, cudaMemcpyAsync(partial.data(), M->search_partial.p, (size_t)blocks * 16, cudaMemcpyDeviceToHost, st), "adjust: loss copy");
-  if (!rc) rc = qcfg_sync_status(h, st);
+  if (!rc) rc = launch_sqdiff(c, Z.yact_ptr, yref, out_elems, (double*)M->search_partial.p, blocks, st);
   if (rc) return rc;
+
+  // ---- backward, on the layers the last output depends on
+  if (want_grads) {
+    std::vector<char> live((size_t)n, 0);
+    live[n - 1] = 1;
+    for (int l = n - 1; l >= 0; --l) {
+      if (!live[l]) continue;
+      if (M->L[l].d.src >= 0) live[M->L[l].d.src] = 1;
+      if (M->L[l].d.residual_from >= 0) live[M->L[l].d.residual_from] = 1;
+    }
+    int64_t max_n = 0, max_k = 0, sum_n = 0;
+    for (auto& S : M->L) {
+      max_n = std::max<int64_t>(max_n, S.d.n_out); max_k = std::max<int64_t>(max_k, S.d.k_in);
+      sum_n += S.d.n_out;
+    }
+    // The weight-gradient product reduces over the m rows and its output is a weight's size: cut into
+    // three partial products (one grouped launch, added up by the kernel that reads them) where
+    // that leaves half of the SMs idle.  A row pitch of three equal pieces, zero behind row m.
+    auto parts_of = [&](const qcfg_layer& d) {
+      return m >= 512 && 2 * ((d.n_out + 127) / 128) * ((d.k_in + 255) / 256) <= c->sms ? 3 : 1;
+    };
+    const int64_t piece = round_up((m + 2) / 3, 64), ldm = 3 * piece;
+    rc = M->adj_grads.ensure(c, (size_t)(2 * n + 3 * sum_n) * 8);
+    if (!rc) rc = M->adj_coef.ensure(c, 4);
+    if (!rc) rc = M->adj_gs.ensure(c, (size_t)(m * round_up(max_n, 8)) * 2);
+    if (!rc) rc = M->adj_gt.ensure(c, (size_t)(max_n * ldm) * 2);
+    if (!rc) rc = M->adj_qxt.ensure(c, (size_t)(max_k * ldm) * 2);
+    if (!rc) rc = M->adj_qwt.ensure(c, (size_t)(max_k * round_up(max_n, 8)) * 2);
+    if (!rc) rc = M->adj_dx.ensure(c, (size_t)(m * max_k) * 4);
+    if (!rc) rc = M->adj_dw.ensure(c, (size_t)(3 * max_n * max_k) * 4);
+    if (!rc) rc = check_cuda(c, cudaMemsetAsync(M->adj_grads.p, 0, (size_t)(2 * n + 3 * sum_n) * 8, st), "adjust: memset");
+    double* dscal = (double*)M->adj_grads.p;
+    double* next = dscal + 2 * n;
+    std::vector<double*> colsum((size_t)n);
+    for (int l = 0; l < n; ++l) { M->L[l].dsw = next; M->L[l].diw = next + sum_n; colsum[l] = next + 2 * sum_n; next += M->L[l].d.n_out; }
+    if (!rc) rc = launch_loss_coef(c, (const double*)M->search_partial.p, blocks, (float*)M->adj_coef.p, st);
+    std::vector<char> have((size_t)n, 0);            // the layer's gout holds a contribution already
+    // where a reader's contribution to layer p's gout goes: = for the first one that covers whole rows, else +=
+    auto contribute = [&](int p, bool whole, bool* assign) -> int {
+      LayerState& P = M->L[p];
+      int erc = P.gout.ensure(c, (size_t)(m * P.d.n_out) * 4);
+      *assign = !have[p] && whole;
+      if (!erc && !have[p] && !whole) erc = check_cuda(c, cudaMemsetAsync(P.gout.p, 0, (size_t)(m * P.d.n_out) * 4, st), "adjust: memset");
+      have[p] = 1;
+      return erc;
+    };
+    for (int l = n - 1; l >= 0 && !rc; --l) {
+      if (!live[l]) continue;
+      LayerState& S = M->L[l];
+      const qcfg_layer& d = S.d;
+      const int b = bits[l];
+      const int64_t nn = d.n_out, kk = d.k_in, ldn = round_up(nn, 8);
+      const bool last = l == n - 1, shortcut = d.residual_from >= 0;
+      const bool want_dx = b != 16 || d.src >= 0;    // a 16-bit layer on the external input needs neither product
+      if (!want_dx && !shortcut) continue;
+      if (last || shortcut) rc = S.gout.ensure(c, (size_t)(m * nn) * 4);
+      const float* res = shortcut ? M->L[d.residual_from].yact_ptr : nullptr;
+      const int64_t ldr = shortcut ? M->L[d.residual_from].d.n_out : 0;
+      float sx = 1.0f, ix = 1.0f;
+      if (b != 16) act_scales(S, b, &sx, &ix);
+      const float qm = b == 16 ? 0.0f : qmax_of(b);
+      const float* sw = b == 16 ? nullptr : (const float*)S.wc[b].scale.p;
+      if (!rc) rc = launch_backward_operands(c, (float*)S.gout.p, S.yact_ptr, last ? yref : nullptr, (const float*)M->adj_coef.p, (const float*)S.ylin.p,
+                                             res, ldr, d.act, sw, m, nn, shortcut, want_dx ? M->adj_gs.p : nullptr, ldn,
+                                             b == 16 ? nullptr : M->adj_gt.p, ldm, b == 16 ? nullptr : colsum[l], st);
+      if (!rc && shortcut) {                         // the shortcut passes the gradient on unchanged
+        bool assign = false;
+        rc = contribute(d.residual_from, true, &assign);
+        if (!rc) rc = launch_input_backward(c, (const float*)S.gout.p, nullptr, 0, 1.0f, 1.0f, 0.0f, m, nn, (float*)M->L[d.residual_from].gout.p, ldr, assign, nullptr, st);
+      }
+      if (!rc && b != 16)         // post-rounding scales: d/ds_w[n] = sum_m g*ylin / s_w[n], d/ds_x = sum g*ylin / s_x
+        rc = launch_gamma_finish(c, colsum[l], sw, sx, nn, S.dsw, dscal + 2 * l, st);
+      if (!rc && want_dx) {       // gradient of the input codes: dxq[m][k] = sum_n (g[m][n] s_w[n]) qw[n][k]   (bf16 tensor-core GEMM)
+        rc = launch_transpose_bf16(c, S.wc[b].codes.p, b == 16 ? 2 : 1, nn, kk, S.ldk, M->adj_qwt.p, ldn, st);
+        GemmArgs g{};
+        g.a = M->adj_gs.p; g.lda = ldn; g.b = M->adj_qwt.p; g.ldb = ldn;
+        g.m = m; g.n = kk; g.k = nn; g.is_bf16 = 1; g.act = QCFG_ACT_NONE; g.y = (float*)M->adj_dx.p; g.ldy = kk;
+        if (!rc) rc = launch_gemm(c, g, st);
+        const float* xin; int64_t ldx;
+        input_of(l, &xin, &ldx);
+        bool assign = false;
+        float* gprod = nullptr;
+        if (!rc && d.src >= 0) {
+          rc = contribute(d.src, d.src_col0 == 0 && kk == M->L[d.src].d.n_out, &assign);
+          gprod = (float*)M->L[d.src].gout.p + d.src_col0;
+        }
+        if (!rc) rc = launch_input_backward(c, (const float*)M->adj_dx.p, xin, ldx, sx, ix, qm, m, kk, gprod,
+                                            d.src >= 0 ? M->L[d.src].d.n_out : 0, assign, b == 16 ? nullptr : dscal + 2 * l + 1, st);
+      }
+      if (!rc && b != 16) {       // gradient of the weight codes: dwq[n][k] = sum_m g[m][n] qx[m][k], then the pre-rounding scales
+        rc = launch_transpose_bf16(c, S.a_ptr, 1, m, kk, S.ldk, M->adj_qxt.p, ldm, st);
+        const int parts = parts_of(d);
+        GemmArgs gs[3];
+        for (int p = 0; p < parts; ++p) {
+          GemmArgs& g = gs[p];
+          g = GemmArgs{};
+          g.a = (const char*)M->adj_gt.p + p * piece * 2; g.lda = ldm; g.b = (const char*)M->adj_qxt.p + p * piece * 2; g.ldb = ldm;
+          g.m = nn; g.n = kk; g.k = parts == 1 ? m : piece; g.is_bf16 = 1; g.act = QCFG_ACT_NONE;
+          g.y = (float*)M->adj_dw.p + p * nn * kk; g.ldy = kk;
+        }
+        if (!rc) rc = launch_gemm_group(c, gs, parts, st);
+        if (!rc) rc = launch_weight_alpha(c, (const float*)M->adj_dw.p, parts, d.w_dev, sw, (const float*)S.wc[b].inv.p, sx, qm, nn, kk, S.diw, st);
+      }
+    }
+    if (!rc && grads_host) {
+      grads_host->resize((size_t)(2 * n + 2 * sum_n));
+      rc = check_cuda(c, cudaMemcpyAsync(grads_host->data(), dscal, grads_host->size() * 8, cudaMemcpyDeviceToHost, st), "adjust: gradient copy");
+    }
+  }
+  // a copy to pageable memory waits for the device, so the copies come last
+  if (!rc) rc = check_cuda(c, cudaMemcpyAsync(partial.data(), M->search_partial.p, (size_t)blocks * 16, cudaMemcpyDeviceToHost, st), "adjust: loss copy");
+  const int src = qcfg_sync_status(h, st);
+  if (rc || src) return rc ? rc : src;
   double d2 = 0.0, r2 = 0.0;
   for (int i = 0; i < blocks; ++i) { d2 += partial[2 * i]; r2 += partial[2 * i + 1]; }
   if (loss) *loss = r2 > 0.0 ? d2 / r2 : 0.0;
-  if (!want_grads) return QCFG_OK;
-  if (!(r2 > 0.0)) return set_error(c, QCFG_ESTATE, "scale adjustment: the reference output is all zero");
-
-  // ---- backward
-  int64_t max_n = 0, max_k = 0;
-  for (auto& S : M->L) { max_n = std::max<int64_t>(max_n, S.d.n_out); max_k = std::max<int64_t>(max_k, S.d.k_in); }
-  const int64_t ldm = round_up(m, 8);
-  rc = M->adj_dscal.ensure(c, (size_t)n * 16);
-  if (!rc) rc = M->adj_colsum.ensure(c, (size_t)max_n * 8);
-  if (!rc) rc = M->adj_gs.ensure(c, (size_t)(m * round_up(max_n, 8)) * 2);
-  if (!rc) rc = M->adj_gt.ensure(c, (size_t)(max_n * ldm) * 2);
-  if (!rc) rc = M->adj_qxt.ensure(c, (size_t)(max_k * ldm) * 2);
-  if (!rc) rc = M->adj_qwt.ensure(c, (size_t)(max_k * round_up(max_n, 8)) * 2);
-  if (!rc) rc = M->adj_dx.ensure(c, (size_t)(m * max_k) * 4);
-  if (!rc) rc = M->adj_dw.ensure(c, (size_t)(max_n * max_k) * 4);
-  if (!rc) rc = check_cuda(c, cudaMemsetAsync(M->adj_dscal.p, 0, (size_t)n * 16, st), "adjust: memset");
-  for (int l = 0; l < n && !rc; ++l) {
-    LayerState& S = M->L[l];
-    rc = S.gout.ensure(c, (size_t)(m * S.d.n_out) * 4);
-    if (!rc) rc = S.dsw.ensure(c, (size_t)S.d.n_out * 8);
-    if (!rc) rc = S.diw.ensure(c, (size_t)S.d.n_out * 8);
-    if (!rc) rc = check_cuda(c, cudaMemsetAsync(S.gout.p, 0, (size_t)(m * S.d.n_out) * 4, st), "adjust: memset");
-    if (!rc) rc = check_cuda(c, cudaMemsetAsync(S.dsw.p, 0, (size_t)S.d.n_out * 8, st), "adjust: memset");
-    if (!rc) rc = check_cuda(c, cudaMemsetAsync(S.diw.p, 0, (size_t)S.d.n_out * 8, st), "adjust: memset");
-  }
-  if (!rc) rc = launch_loss_grad(c, (const float*)Z.yact.p, ref, (float)(2.0 / r2), (float*)Z.gout.p, out_elems, st);
-  double* dscal = (double*)M->adj_dscal.p;
-  for (int l = n - 1; l >= 0 && !rc; --l) {
-    LayerState& S = M->L[l];
-    const qcfg_layer& d = S.d;
-    const int b = bits[l];
-    const int64_t nn = d.n_out, kk = d.k_in, ldn = round_up(nn, 8);
-    float* gpre = (float*)S.gout.p;
-    const float* res = d.residual_from >= 0 ? (const float*)M->L[d.residual_from].yact.p : nullptr;
-    const int64_t ldr = d.residual_from >= 0 ? M->L[d.residual_from].d.n_out : 0;
-    rc = launch_act_backward(c, gpre, (const float*)S.ylin.p, res, ldr, d.act, m, nn, st);
-    if (!rc && d.residual_from >= 0)          // the shortcut passes the gradient on unchanged
-      rc = launch_input_backward(c, gpre, nullptr, 0, 1.0f, 1.0f, 0.0f, m, nn, (float*)M->L[d.residual_from].gout.p, ldr, nullptr, st);
-    float sx = 1.0f, ix = 1.0f;
-    if (b != 16) act_scales(S, b, &sx, &ix);
-    const float qm = b == 16 ? 0.0f : qmax_of(b);
-    if (!rc && b != 16) {       // post-rounding scales: d/ds_w[n] = sum_m g*ylin / s_w[n], d/ds_x = sum g*ylin / s_x
-      rc = check_cuda(c, cudaMemsetAsync(M->adj_colsum.p, 0, (size_t)nn * 8, st), "adjust: memset");
-      if (!rc) rc = launch_col_dot(c, gpre, (const float*)S.ylin.p, m, nn, (double*)M->adj_colsum.p, st);
-      if (!rc) rc = launch_gamma_finish(c, (const double*)M->adj_colsum.p, (const float*)S.wc[b].scale.p, sx, nn, (double*)S.dsw.p, dscal + 2 * l, st);
-    }
-    // gradient of the input codes: dxq[m][k] = sum_n (g[m][n] s_w[n]) qw[n][k]   (bf16 tensor-core GEMM)
-    if (!rc) rc = launch_scale_cols_bf16(c, gpre, b == 16 ? nullptr : (const float*)S.wc[b].scale.p, m, nn, M->adj_gs.p, ldn, st);
-    if (!rc) rc = launch_transpose_bf16(c, S.wc[b].codes.p, b == 16 ? 2 : 1, nn, kk, S.ldk, M->adj_qwt.p, ldn, st);
-    if (!rc) {
-      GemmArgs g{};
-      g.a = M->adj_gs.p; g.lda = ldn; g.b = M->adj_qwt.p; g.ldb = ldn;
-      g.m = m; g.n = kk; g.k = nn; g.is_bf16 = 1; g.act = QCFG_ACT_NONE; g.y = (float*)M->adj_dx.p; g.ldy = kk;
-      rc = launch_gemm(c, g, st);
-    }
-    const float* xin; int64_t ldx;
-    input_of(l, &xin, &ldx);
-    float* gprod = d.src >= 0 ? (float*)M->L[d.src].gout.p + d.src_col0 : nullptr;
-    if (!rc) rc = launch_input_backward(c, (const float*)M->adj_dx.p, xin, ldx, sx, ix, qm, m, kk, gprod,
-                                        d.src >= 0 ? M->L[d.src].d.n_out : 0, b == 16 ? nullptr : dscal + 2 * l + 1, st);
-    if (!rc && b != 16) {       // gradient of the weight codes: dwq[n][k] = sum_m g[m][n] qx[m][k], then the pre-rounding scales
-      rc = launch_transpose_bf16(c, gpre, 0, m, nn, nn, M->adj_gt.p, ldm, st);
-      if (!rc) rc = launch_transpose_bf16(c, S.abuf.p, 1, m, kk, S.ldk, M->adj_qxt.p, ldm, st);
-      if (!rc) {
-        GemmArgs g{};
-        g.a = M->adj_gt.p; g.lda = ldm; g.b = M->adj_qxt.p; g.ldb = ldm;
-        g.m = nn; g.n = kk; g.k = m; g.is_bf16 = 1; g.act = QCFG_ACT_NONE; g.y = (float*)M->adj_dw.p; g.ldy = kk;
-        rc = launch_gemm(c, g, st);
-      }
-      if (!rc) rc = launch_weight_alpha(c, (const float*)M->adj_dw.p, d.w_dev, (const float*)S.wc[b].scale.p, (const float*)S.wc[b].inv.p,
-                                        sx, qm, nn, kk, (double*)S.diw.p, st);
-    }
-  }
-  if (!rc) rc = qcfg_sync_status(h, st);
-  return rc;
+  if (want_grads && !(r2 > 0.0)) return set_error(c, QCFG_ESTATE, "scale adjustment: the reference output is all zero");
+  return QCFG_OK;
 }
 
 int adjust_check(Ctx* c, Model* M, const uint8_t* bits, const float* x_dev, int64_t m, const char* who) {
@@ -1419,15 +1468,18 @@ int adjust_check(Ctx* c, Model* M, const uint8_t* bits, const float* x_dev, int6
   return QCFG_OK;
 }
 
-// reference output: the 16-bit model's last layer, kept in M->search_ref
+// reference output: the 16-bit model's last layer, written to M->search_ref by an ordinary evaluation
 int adjust_reference(qcfg_ctx* h, Model* M, const float* x_dev, int64_t m, cudaStream_t st) {
   Ctx* c = &h->c;
   const int n = (int)M->L.size();
+  for (int l = 0; l < n; ++l)
+    if (M->L[l].d.kh > 0 || M->L[l].d.pool_before != QCFG_POOL_NONE)
+      return set_error(c, QCFG_ESHAPE, "scale adjustment covers linear layers only (layer %d is a convolution or pooled)", l);
   std::vector<uint8_t> b16((size_t)n, 16);
-  int rc = adjust_pass(h, M, b16.data(), x_dev, m, nullptr, nullptr, false, st);
-  const size_t bytes = (size_t)(m * M->L[n - 1].d.n_out) * 4;
-  if (!rc) rc = M->search_ref.ensure(c, bytes);
-  if (!rc) rc = check_cuda(c, cudaMemcpyAsync(M->search_ref.p, M->L[n - 1].yact.p, bytes, cudaMemcpyDeviceToDevice, st), "adjust: reference copy");
+  std::vector<float*> ys((size_t)n, nullptr);
+  int rc = M->search_ref.ensure(c, (size_t)(m * M->L[n - 1].d.n_out) * 4);
+  ys[n - 1] = (float*)M->search_ref.p;
+  if (!rc) rc = forward(c, M, b16.data(), x_dev, ext_ld_of(M), m, ys.data(), false, st);
   return rc;
 }
 
@@ -1443,17 +1495,21 @@ int qcfg_scale_gradients(qcfg_ctx* ctx, qcfg_model* model, const uint8_t* bits, 
   if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   const int n = (int)M->L.size();
+  std::vector<double> g;
+  double value = 0.0;
   rc = adjust_reference(ctx, M, x_dev, m, st);
-  if (!rc) rc = adjust_pass(ctx, M, bits, x_dev, m, (const float*)M->search_ref.p, loss, true, st);
+  if (!rc) rc = adjust_pass(ctx, M, bits, x_dev, m, (const float*)M->search_ref.p, &value, true, &g, st);
   if (rc) return rc;
-  std::vector<double> ds((size_t)2 * n);
-  rc = check_cuda(c, cudaMemcpy(ds.data(), M->adj_dscal.p, ds.size() * 8, cudaMemcpyDeviceToHost), "scale_gradients: copy");
-  for (int l = 0; l < n && !rc; ++l) {
-    if (d_scale_x) d_scale_x[l] = bits[l] == 16 ? 0.0 : ds[2 * l];
-    if (d_inv_scale_x) d_inv_scale_x[l] = bits[l] == 16 ? 0.0 : ds[2 * l + 1];
+  if (loss) *loss = value;
+  int64_t sum_n = 0, at = 2 * n;
+  for (auto& S : M->L) sum_n += S.d.n_out;
+  for (int l = 0; l < n; ++l) {
+    if (d_scale_x) d_scale_x[l] = bits[l] == 16 ? 0.0 : g[2 * l];
+    if (d_inv_scale_x) d_inv_scale_x[l] = bits[l] == 16 ? 0.0 : g[2 * l + 1];
     const size_t bytes = (size_t)M->L[l].d.n_out * 8;
-    if (d_scale_w && d_scale_w[l]) rc = check_cuda(c, cudaMemcpy(d_scale_w[l], M->L[l].dsw.p, bytes, cudaMemcpyDeviceToHost), "scale_gradients: copy");
-    if (!rc && d_inv_scale_w && d_inv_scale_w[l]) rc = check_cuda(c, cudaMemcpy(d_inv_scale_w[l], M->L[l].diw.p, bytes, cudaMemcpyDeviceToHost), "scale_gradients: copy");
+    if (d_scale_w && d_scale_w[l]) memcpy(d_scale_w[l], g.data() + at, bytes);
+    if (d_inv_scale_w && d_inv_scale_w[l]) memcpy(d_inv_scale_w[l], g.data() + at + sum_n, bytes);
+    at += M->L[l].d.n_out;
   }
   M->evaluated = true; M->last_m = m;
   return rc;
@@ -1480,26 +1536,25 @@ int qcfg_adjust_scales(qcfg_ctx* ctx, qcfg_model* model, const uint8_t* bits, co
     S.wc[b].adjusted = true;
     if (!S.adj_act[b]) { host_scales(S.act_absmax, b, &S.adj_sx[b], &S.adj_ix[b]); S.adj_act[b] = true; }
   }
-  std::vector<double> ds((size_t)2 * n);
+  std::vector<double> ds;
   for (int step = 0; step < steps && !rc; ++step) {
     double loss = 0.0;
-    rc = adjust_pass(ctx, M, bits, x_dev, m, (const float*)M->search_ref.p, &loss, true, st);
+    rc = adjust_pass(ctx, M, bits, x_dev, m, (const float*)M->search_ref.p, &loss, true, &ds, st);
     if (rc) break;
     if (losses_host) losses_host[step] = loss;
-    rc = check_cuda(c, cudaMemcpy(ds.data(), M->adj_dscal.p, ds.size() * 8, cudaMemcpyDeviceToHost), "adjust_scales: copy");
     for (int l = 0; l < n && !rc; ++l) {
       const int b = bits[l];
       if (b == 16) continue;
       LayerState& S = M->L[l];
       S.adj_sx[b] = (float)((double)S.adj_sx[b] - lr * ds[2 * l]);
       S.adj_ix[b] = (float)((double)S.adj_ix[b] - lr * ds[2 * l + 1]);
-      rc = launch_sgd(c, (float*)S.wc[b].scale.p, (const double*)S.dsw.p, lr, S.d.n_out, st);
-      if (!rc) rc = launch_sgd(c, (float*)S.wc[b].inv.p, (const double*)S.diw.p, lr, S.d.n_out, st);
+      rc = launch_sgd(c, (float*)S.wc[b].scale.p, S.dsw, lr, S.d.n_out, st);
+      if (!rc) rc = launch_sgd(c, (float*)S.wc[b].inv.p, S.diw, lr, S.d.n_out, st);
       S.wc[b].ready = false;                    // the weight codes follow the new pre-rounding scales
     }
   }
   double loss = 0.0;
-  if (!rc) rc = adjust_pass(ctx, M, bits, x_dev, m, (const float*)M->search_ref.p, &loss, false, st);
+  if (!rc) rc = adjust_pass(ctx, M, bits, x_dev, m, (const float*)M->search_ref.p, &loss, false, nullptr, st);
   if (!rc && losses_host) losses_host[steps] = loss;
   M->evaluated = true; M->last_m = m;
   M->reuse_valid = false;

@@ -79,24 +79,26 @@ int launch_sweep_static(Ctx* ctx, const float* const* w, const int64_t* rows, co
 // ----- adjust.cu (scale adjustment, Section 3.1 second step) --------------------------
 // y = act(ylin + res) elementwise over [rows x n] (res may be null; ldr its row pitch)
 int launch_act_apply(Ctx* ctx, const float* ylin, const float* res, int64_t ldr, int act, float* y, int64_t rows, int64_t n, cudaStream_t st);
-// g = coef * (y - yref)
-int launch_loss_grad(Ctx* ctx, const float* y, const float* yref, float coef, float* g, int64_t count, cudaStream_t st);
-// g *= act'(ylin + res) in place
-int launch_act_backward(Ctx* ctx, float* g, const float* ylin, const float* res, int64_t ldr, int act, int64_t rows, int64_t n, cudaStream_t st);
-// out[c] += sum_r a[r][c] * b[r][c]   (out must be zeroed by the caller)
-int launch_col_dot(Ctx* ctx, const float* a, const float* b, int64_t rows, int64_t n, double* out, cudaStream_t st);
+// dL/d(output) of a layer -> what its backward products need, in one pass: g = gout * act'(ylin + res), or with
+// yref set g = *coef * (y - yref) * act'(...); gs[r][c] = bf16(g * (s_w ? s_w[c] : 1)) (columns n..ld_gs-1 zero),
+// gt[c][r] = bf16(g) (columns rows..ld_gt-1 zero), colsum[c] += sum_r g * ylin (zeroed by the caller); gs, gt
+// and colsum may be null; keep_g stores g back to gout
+int launch_backward_operands(Ctx* ctx, float* gout, const float* y, const float* yref, const float* coef, const float* ylin,
+                             const float* res, int64_t ldr, int act, const float* s_w, int64_t rows, int64_t n, bool keep_g, void* gs, int64_t ld_gs,
+                             void* gt, int64_t ld_gt, double* colsum, cudaStream_t st);
+// *coef = 2 / sum of squares of the reference, from sqdiff's partial sums
+int launch_loss_coef(Ctx* ctx, const double* partial, int blocks, float* coef, cudaStream_t st);
 // d_sw[c] = colsum[c] / s_w[c];  *d_sx += sum_c colsum[c] / s_x
 int launch_gamma_finish(Ctx* ctx, const double* colsum, const float* s_w, float s_x, int64_t n, double* d_sw, double* d_sx, cudaStream_t st);
-// out[r][c] = bf16(g[r][c] * (col_scale ? col_scale[c] : 1)), columns n..ld-1 zero
-int launch_scale_cols_bf16(Ctx* ctx, const float* g, const float* col_scale, int64_t rows, int64_t n, void* out, int64_t ld, cudaStream_t st);
-// dst[c][r] = bf16(src[r][c]); kind 0 fp32, 1 int8, 2 bf16 source; dst row pitch ld_dst (columns rows..ld_dst-1 zero)
+// dst[c][r] = bf16(src[r][c]); kind 1 int8, 2 bf16 source, rows on 16-byte boundaries; dst row pitch ld_dst, a
+// multiple of 8 (columns rows..ld_dst-1 zero)
 int launch_transpose_bf16(Ctx* ctx, const void* src, int kind, int64_t rows, int64_t cols, int64_t ld_src, void* dst, int64_t ld_dst, cudaStream_t st);
 // integer layer: mask = |x*inv_x| <= qmax;  *d_ix += s_x * sum dxq*mask*x;  gprod[r][c] += dxq*(s_x*inv_x)*mask
-// 16-bit layer (qmax == 0): gprod += dxq.  gprod may be null (external input).
+// 16-bit layer (qmax == 0): gprod += dxq.  gprod may be null (external input); assign: = instead of +=.
 int launch_input_backward(Ctx* ctx, const float* dxq, const float* x, int64_t ldx, float s_x, float inv_x, float qmax,
-                          int64_t rows, int64_t k, float* gprod, int64_t ldg, double* d_ix, cudaStream_t st);
-// d_iw[r] = s_x * s_w[r] * sum_c dwq[r][c] * w[r][c] * (|w[r][c]*inv_w[r]| <= qmax)
-int launch_weight_alpha(Ctx* ctx, const float* dwq, const float* w, const float* s_w, const float* inv_w, float s_x, float qmax,
+                          int64_t rows, int64_t k, float* gprod, int64_t ldg, bool assign, double* d_ix, cudaStream_t st);
+// d_iw[r] = s_x * s_w[r] * sum_c dwq[r][c] * w[r][c] * (|w[r][c]*inv_w[r]| <= qmax), dwq the sum of `parts` (1 or 3) matrices
+int launch_weight_alpha(Ctx* ctx, const float* dwq, int parts, const float* w, const float* s_w, const float* inv_w, float s_x, float qmax,
                         int64_t n, int64_t k, double* d_iw, cudaStream_t st);
 // s[i] = float(double(s[i]) - lr * g[i])
 int launch_sgd(Ctx* ctx, float* s, const double* g, double lr, int64_t n, cudaStream_t st);

@@ -32,7 +32,7 @@ def _gpu_scales(model, layers, bits):
     return out
 
 
-@pytest.mark.parametrize("kind", ["tiny_mlp", "bert_block", "residual"])
+@pytest.mark.parametrize("kind", ["tiny_mlp", "bert_block", "residual", "split_reduction", "odd_sizes"])
 def test_gradients_update_and_evaluation_match_the_oracle(kind):
     import paper_2302_01382_b200 as q
     if kind == "tiny_mlp":
@@ -41,6 +41,12 @@ def test_gradients_update_and_evaluation_match_the_oracle(kind):
     elif kind == "bert_block":
         w = wl.bert_stack(41, 320, 128, 512, 1, bit_choices=None)
         bits = [8, 4, 6, 16, 8, 4]
+    elif kind == "split_reduction":      # enough rows for the weight gradients' three partial products
+        w = wl.tiny_mlp(seed=43, m=577, dims=(132, 260, 96, 20), bits=(8, 4, 8))
+        bits = [8, 6, 8]
+    elif kind == "odd_sizes":            # nothing is a multiple of four
+        w = wl.tiny_mlp(seed=44, m=67, dims=(45, 131, 63, 9), bits=(8, 4, 8))
+        bits = [8, 16, 6]
     else:
         L = wl.Layer
         layers = [L("a", 96, 64, src=-1, act=orc.ACT_RELU), L("b", 96, 96, src=0, act=orc.ACT_RELU),
