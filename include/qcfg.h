@@ -125,8 +125,9 @@ int qcfg_set_gemm_chains(qcfg_ctx* ctx, int enabled);
  * other layers launch nothing.  This is what consecutive configurations of the searches allow:
  * Algorithm 2 changes one layer per evaluation, Algorithm 1 a slice of the ordering.  The CALLER
  * guarantees that the contents of x_dev did not change between such calls.  Results are
- * bit-identical to a full evaluation.  qcfg_calibrate_model, qcfg_latency_table and
- * qcfg_noise_sensitivity always run every layer.                                              */
+ * bit-identical to a full evaluation.  qcfg_calibrate_model and qcfg_latency_table always run every
+ * layer.  qcfg_search and qcfg_noise_sensitivity reuse in this way among their own forwards whatever
+ * the switch says (the input stays the same within a call), starting from a full one.           */
 int qcfg_set_prefix_reuse(qcfg_ctx* ctx, int enabled);
 
 /* Per-launch timing, off by default.  Mode 1: CUDA events recorded around every launch on the
@@ -295,8 +296,8 @@ int qcfg_config_cost(qcfg_model* model, const uint8_t* bits, const uint8_t* bs, 
  * like the clean ones).  The second argument of N(0, .) is read as the standard deviation.
  * noise_dev is a HOST array of n_layers DEVICE pointers to the caller's standard-normal draws,
  * [n_out x k_in] row-major like the weights (the generator is the caller's); a NULL entry skips
- * the layer (E_N = 0).  e_n_host receives n_layers doubles.  Costs one forward per perturbed layer
- * plus one; synchronises the stream after each.  No calibration needed.                        */
+ * the layer (E_N = 0).  e_n_host receives n_layers doubles.  Costs one forward plus, per perturbed
+ * layer, the layers its output reaches; synchronises the stream at the end.  No calibration needed. */
 int qcfg_noise_sensitivity(qcfg_ctx* ctx, qcfg_model* model, const float* x_dev, int64_t m,
                            const float* const* noise_dev, float lambda, double* e_n_host, void* stream);
 

@@ -52,6 +52,23 @@ def test_noise_sensitivity_matches_oracle(ctx, make):
             assert got[b] > got[a]
 
 
+def test_noise_sensitivity_runs_only_what_a_perturbation_reaches(ctx):
+    """Parallel branches: the layers an earlier perturbation reached and the next one does not are run again, so
+    every E_N equals that of a call which perturbs this layer alone, bit for bit; with the switch for reuse
+    between calls on, a changed input gives the changed input's result."""
+    w = wl.resnet50(seed=8, batch=2, in_hw=32, width=16, n_classes=10, blocks=(2, 1, 1, 1))
+    nus = wl.standard_normal_like(w.weights, 5)
+    both = _run(ctx, w, nus, 0.05)
+    for l in (1, 2, 3, 4, 7, len(nus) - 1):
+        alone = _run(ctx, w, [n if i == l else None for i, n in enumerate(nus)], 0.05)
+        assert alone[l] == both[l] and np.count_nonzero(alone) <= 1
+    ctx.set_prefix_reuse(True)
+    try:
+        assert np.array_equal(_run(ctx, w, nus, 0.05), both)
+    finally:
+        ctx.set_prefix_reuse(False)
+
+
 def test_noise_sensitivity_zero_lambda_and_errors(ctx):
     import paper_2302_01382_b200 as q
     w = wl.tiny_mlp()

@@ -83,3 +83,24 @@ def test_search_argument_errors(setup):
     assert e.value.status == q.EBITS
     bits, vis, acc, n_evals = model.search(1, order, [16], 0.9, x, w.m)     # nothing to lower
     assert bits == [16] * len(order) and n_evals == 0
+
+
+@pytest.mark.parametrize("algorithm", [0, 1])
+def test_search_reuses_within_a_call_only(setup, algorithm):
+    """Evaluations of a search restart where the configuration changed; the fidelities are those of full
+    evaluations, and a second call sees the input as it is then."""
+    q, ctx, model, w, x, order, evaluate = setup
+    n = len(order)
+    for inp in (x, x.flip(0).contiguous()):
+        x2 = x.clone()
+        model.search(algorithm, order, [16, 8, 4], 0.97, x2, w.m)
+        x2.copy_(inp)                                  # same buffer, other contents
+        bits, vis, acc, _ = model.search(algorithm, order, [16, 8, 4], 0.97, x2, w.m)
+        out = [torch.empty((w.m, w.layers[-1].n_out), device="cuda") for _ in range(2)]
+        for i, c in enumerate([[16] * n] + vis):
+            ys = [None] * (n - 1) + [out[min(i, 1)]]
+            model.eval_config(c, inp, w.m, ys)
+            if i:
+                ref, y = out[0].double(), out[1].double()
+                full = 1.0 - float(torch.linalg.norm(y - ref) / torch.linalg.norm(ref))
+                assert acc[i - 1] == pytest.approx(full, rel=1e-12, abs=1e-12)
