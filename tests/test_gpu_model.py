@@ -343,3 +343,26 @@ def test_calibration_maxima_do_not_depend_on_fusion_or_chaining(ctx):
         ctx.set_fusion(True)
         ctx.set_gemm_chains(True)
         model.close()
+
+
+@pytest.mark.parametrize("m,n", [(1, 32), (127, 36), (130, 100), (257, 128), (300, 132), (1200, 388), (40000, 256)])
+def test_shortcut_layers_at_tile_edges(ctx, m, n):
+    """Layers with an fp32 shortcut whose result goes to the caller and, as codes of two grids, to two readers:
+    rows and columns at the edges of tiles and of 32 x 32 blocks, one to many tiles per CTA."""
+    L = wl.Layer
+    layers = [L("a", n, 48, src=-1), L("b", n, n, src=0, act=orc.ACT_RELU, residual_from=0), L("c", 16, n, src=1), L("d", 24, n, src=1),
+              L("e", n, 24, src=3, residual_from=1)]
+    rng = np.random.default_rng(m + n)
+    x = rng.standard_normal((m, 48)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("shortcut", 1, layers, m, x, ws)
+    model, xd = build(ctx, w)
+    act_g, w_amax = check_calibration(model, w)
+    for bits in ([8, 6, 8, 4, 8], [8, 8, 4, 4, 16]):
+        ys = run_eval(ctx, model, w, xd, bits)
+        teacher_forced_check(ctx, model, w, xd, bits, ys, act_g, w_amax, sample_rows=300)
+        only = [None] * 4 + [torch.full_like(ys[4], float("nan"))]        # shortcuts and readers inside the model
+        model.eval_config(bits, xd, m, only)
+        ctx.check_sync()
+        assert torch.equal(only[4], ys[4])
+    model.close()
