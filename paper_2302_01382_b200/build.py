@@ -20,7 +20,7 @@ def _newest(paths):
 def build_library(force: bool = False, verbose: bool = False) -> str:
     """Compiles the CUDA sources into libqcfg.so next to this file and returns its path."""
     srcs = [os.path.join(CSRC, s) for s in SOURCES]
-    deps = srcs + [os.path.join(CSRC, "common.cuh"),
+    deps = srcs + [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "ptx.cuh"),
                    os.path.join(os.path.dirname(PKG), "include", "qcfg.h")]
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _newest(deps):
         return LIB

@@ -28,6 +28,7 @@
 #include <unordered_map>
 
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace qcfg {
 
@@ -49,7 +50,6 @@ constexpr int kResBarOffset = 512;    // in the header: two barriers per epilogu
 constexpr int kShortcutBytes = 2 * 4096 + 1024;   // per epilogue warp: two 32 x 32 fp32 blocks and one of codes
 constexpr int kCsBytes = kEpiWarps * 64 * 4;   // per epilogue warp: rescale factors of its 64 columns
 constexpr int kSmemMax = 232448;      // 227 KB
-constexpr uint64_t kWaitLimitNs = 2000000000ull;
 
 constexpr int kNumOuts = 2 + kMaxSlots;   // raw accumulators, fp32 output, consumer code slots
 
@@ -95,6 +95,11 @@ struct GroupDesc {
 // Implicit-GEMM convolution: the A operand is not a matrix in memory but the NHWC code tensor of the
 // layer's input; row (b, oh, ow) of the k-block (tap, channel chunk) is gathered from pixel
 // (b, oh*stride - pad + dy, ow*stride - pad + dx), zero outside the image.
+// How the operand gets into shared memory: gather warps (any multiple of 16 bytes of channels), or TMA in its
+// im2col mode, where one load brings a chunk of channels of 128 consecutive output pixels at one tap:
+// 128-byte chunks (channels a multiple of 128 bytes; the usual 128B-swizzled tile), or two 64-byte chunks
+// per k-block (a multiple of 64 bytes; two half tiles of 64-byte rows, 64B swizzle).
+enum : int32_t { CONV_NONE = 0, CONV_GATHER = 1, CONV_TMA128 = 2, CONV_TMA64 = 3 };
 struct ConvDesc {
   int32_t on, H, W, C, kh, kw, stride, pad, OH, OW, esz, K;
   int64_t img_bytes;          // bytes of one image (H * W * C * esz)
@@ -128,50 +133,6 @@ template <bool CHAIN> struct LaunchArgs {
 static_assert(sizeof(LaunchArgs<true>) <= 32764, "kernel parameters are limited to 32764 bytes");
 
 // ---------------------------------------------------------------------------- PTX wrappers
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ uint64_t global_timer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-// Bounded wait.  Returns false when the CTA should give up (this or another wait timed out).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned* err,
-                                          uint64_t limit_ns = kWaitLimitNs) {
-  uint64_t t0 = 0;
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 1023u) == 0) {
-      if (*abort_flag) return false;
-      uint64_t now = global_timer();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > limit_ns) {
-        atomicOr(err, ERR_TIMEOUT);
-        *abort_flag = 1;
-        return false;
-      }
-    }
-  }
-}
 
 // Chains: waits until a counter of finished tiles has reached `need`.  Bounded like every other wait.
 __device__ __forceinline__ bool flag_wait(const unsigned* flag, uint32_t need, volatile int* abort_flag, unsigned* err,
@@ -239,41 +200,18 @@ __device__ __forceinline__ bool reported_wait(uint32_t rep0, uint32_t need, int 
   }
 }
 
-// The same wait for a whole converged warp, written so that the compiler sees warp-uniform control
-// flow (the spin is inside one asm statement, the outcome is a vote): the producer and the MMA
-// issuer run their loops on all 32 lanes, which keeps their address and descriptor arithmetic on
-// the uniform datapath, and elect one lane only for the TMA / MMA instructions themselves.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, unsigned* err) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .u32 n;\n\t"
-      "mov.u32 n, 64;\n\t"
-      "SPIN:\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "@p bra DONE;\n\t"
-      "sub.u32 n, n, 1;\n\t"
-      "setp.ne.u32 p, n, 0;\n\t"
-      "@p bra SPIN;\n\t"
-      "mov.u32 %0, 0;\n\t"
-      "bra OUT;\n\t"
-      "DONE:\n\t"
-      "mov.u32 %0, 1;\n\t"
-      "OUT:\n\t}"
-      : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-  if (__all_sync(0xffffffffu, done != 0)) return true;
-  const bool ok = mbar_wait(bar, parity, abort_flag, err);
-  return __all_sync(0xffffffffu, ok);
-}
-__device__ __forceinline__ bool elect_one() {
-  uint32_t e;
-  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(e));
-  return e != 0;
-}
-
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t x, int32_t y) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
+}
+
+// im2col loads: (w, h) is the first pixel's corner of the filter window, (dx, dy) the tap
+__device__ __forceinline__ void tma_load_im2col(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t c, int32_t w, int32_t h, int32_t n,
+                                                int dx, int dy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"((uint16_t)dx), "h"((uint16_t)dy) : "memory");
 }
 
 // Pair flavour (two CTAs of a cluster work on one 256-row tile, cta_group::2): the load of either
@@ -284,6 +222,12 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(dst), "l"(map), "r"(bar & kPeerBitMask), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void tma_load_im2col_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t c, int32_t w, int32_t h,
+                                                     int32_t n, int dx, int dy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};"
+      ::"r"(dst), "l"(map), "r"(bar & kPeerBitMask), "r"(c), "r"(w), "r"(h), "r"(n), "h"((uint16_t)dx), "h"((uint16_t)dy) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_leader(uint32_t bar) {   // arrive on the first CTA's copy of the barrier
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar & kPeerBitMask) : "memory");
@@ -302,13 +246,6 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
 template <bool BF16>
 __device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
   if (BF16) {
@@ -324,32 +261,6 @@ __device__ __forceinline__ void tc_mma_pair(uint32_t d_tmem, uint64_t a_desc, ui
   }
 }
 
-template <bool BF16>
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  if (BF16) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-  } else {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-  }
-}
-
-__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-        "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-        "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr));
-}
 __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
@@ -358,8 +269,6 @@ __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&v)[16
         "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
       : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
 // Shared-memory matrix descriptors used by the MMA issuer: K-major tile of 128-byte rows, 128B
 // swizzle, groups of 8 rows 1024 bytes apart (the layout a 128B-swizzled TMA box produces).
 // Bits 0-13 start address in 16-byte units, bit 16 leading byte offset (unused for swizzled
@@ -387,10 +296,6 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t sr
                ::"l"(map), "r"(src), "r"(x), "r"(y) : "memory");
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
-__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-
 // Writes one warp's 32-row x 32-column piece of an output.  Each thread holds its row's 32
 // elements packed into WORDS 32-bit words (32: fp32 / int32, 16: bf16, 8: int8).
 // Staged path: the warp lays the piece out in one of its two shared-memory slots and one lane
@@ -855,15 +760,44 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   int ld_tm = tm0, ld_tn = tn0;
   const CUtensorMap* ld_map_a = &mp[q->mi[0][MAP_A]];
   const CUtensorMap* ld_map_b = &mp[q->mi[0][MAP_B]];
+  constexpr bool kConv = !GROUPED && !CHAIN;
+  const bool conv_tma = kConv && p.conv.on >= CONV_TMA128;
+  int cv_n = 0, cv_h = 0, cv_w = 0;              // TMA convolutions: corner of the tile's first pixel
+  int cv_c = 0, cv_dx = 0, cv_dy = 0;            // channel and tap of the next chunk
   auto set_tile_coords = [&]() {
     const int g = group_of(ld_tn);
     if (GROUPED) { ld_map_a = &mp[q->mi[g][MAP_A]]; ld_map_b = &mp[q->mi[g][MAP_B]]; }
     ld_ya = ld_tm * rows_per_tile + rank * BM;
     ld_yb = tile_in_group(ld_tn, g) * p.bn + rank * b_rows;
+    if (conv_tma) {
+      const int opix = p.conv.OH * p.conv.OW;
+      cv_n = ld_ya / opix;
+      const int pix = ld_ya - cv_n * opix, oh = pix / p.conv.OW;
+      cv_h = oh * p.conv.stride - p.conv.pad;
+      cv_w = (pix - oh * p.conv.OW) * p.conv.stride - p.conv.pad;
+      cv_c = 0; cv_dx = 0; cv_dy = 0;
+    }
   };
-  set_tile_coords();
+  if (warp == 0) set_tile_coords();
   const bool elected = elect_one();    // the lane of a converged warp that issues TMA / MMA instructions
-  const bool conv_on = p.conv.on != 0;
+  const bool conv_on = p.conv.on == CONV_GATHER;
+  // one 128-row column of patches per call; chunks behind the last tap repeat the first one (the B tile is zero there)
+  auto load_patches = [&]() {
+    const int chunk = (p.conv.on == CONV_TMA64 ? 64 : 128) / (BF16 ? 2 : 1);
+    const int loads = p.conv.on == CONV_TMA64 ? 2 : 1;
+    for (int h = 0; h < loads; ++h) {
+      const bool past = cv_dy == p.conv.kh;
+      if (elected) {
+        const uint32_t dst = ld_dst + h * (BM * 64);
+        if (PAIR) tma_load_im2col_pair(dst, ld_map_a, ld_bar, past ? 0 : cv_c, cv_w, cv_h, cv_n, past ? 0 : cv_dx, past ? 0 : cv_dy);
+        else tma_load_im2col(dst, ld_map_a, ld_bar, past ? 0 : cv_c, cv_w, cv_h, cv_n, past ? 0 : cv_dx, past ? 0 : cv_dy);
+      }
+      if (!past) {
+        cv_c += chunk;
+        if (cv_c >= p.conv.C) { cv_c = 0; if (++cv_dx == p.conv.kw) { cv_dx = 0; ++cv_dy; } }
+      }
+    }
+  };
   // bytes the TMA loads of one CTA put into a stage (the A tile is gathered in convolution launches)
   const uint32_t tma_bytes = conv_on ? (uint32_t)b_rows * kStageKBytes : stage_bytes;
   auto issue_load = [&]() {   // whole warp 0; the stage's empty barrier must already have been passed
@@ -871,14 +805,15 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     if (PAIR) {
       // the first CTA's barrier collects the bytes of both CTAs' loads
       if (rank == 0) mbar_expect_tx(ld_bar, 2 * tma_bytes);
-      if (!conv_on) tma_load_2d_pair(ld_dst, ld_map_a, ld_bar, ld_x, ld_ya);
+      if (!kConv || !(conv_on || conv_tma)) tma_load_2d_pair(ld_dst, ld_map_a, ld_bar, ld_x, ld_ya);
       tma_load_2d_pair(ld_dst + BM * kStageKBytes, ld_map_b, ld_bar, ld_x, ld_yb);
     } else {
       mbar_expect_tx(ld_bar, tma_bytes);
-      if (!conv_on) tma_load_2d(ld_dst, ld_map_a, ld_bar, ld_x, ld_ya);
+      if (!kConv || !(conv_on || conv_tma)) tma_load_2d(ld_dst, ld_map_a, ld_bar, ld_x, ld_ya);
       tma_load_2d(ld_dst + BM * kStageKBytes, ld_map_b, ld_bar, ld_x, ld_yb);
     }
     }
+    if (kConv && conv_tma) load_patches();
     ld_dst += stage_bytes; ld_bar += 8; ld_x += k_elems;
     if (++ld_s == p.stages) { ld_s = 0; ld_ph ^= 1; ld_dst = stage0; ld_bar = full0; }
     if (++ld_kb == q->k_blocks) {
@@ -892,7 +827,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   if (threadIdx.x == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mp[q->mi[0][MAP_A]]) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mp[q->mi[0][MAP_B]]) : "memory");
-    const uint32_t full_count = 1 + (p.conv.on ? kGatherWarps * (PAIR ? 2 : 1) : 0);   // the TMA thread, plus one arrival per gather warp
+    const uint32_t full_count = 1 + (conv_on ? kGatherWarps * (PAIR ? 2 : 1) : 0);   // the TMA thread, plus one arrival per gather warp
     for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, full_count); mbar_init(empty0 + 8 * s, 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, PAIR ? 2 * kEpiWarps : kEpiWarps); }
     if (!PAIR && !BF16) for (int a = 0; a < 2 * kEpiWarps; ++a) mbar_init(smem_u32(smem + kResBarOffset) + 8 * a, 1);
@@ -989,12 +924,17 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
       int s = 0; uint32_t ph = 0;
       bool ok = true;
       int t = 0;
+      // A tiles of two 64-byte halves: 64B swizzle (layout type 4), 8-row groups 512 bytes apart, the
+      // second half BM * 64 bytes behind the first
+      const bool halves = kConv && p.conv.on == CONV_TMA64;
+      const uint32_t a_hi = halves ? (uint32_t)(512 >> 4) | (1u << 14) | (4u << 29) : kDescHi;
+      const uint32_t a_half = halves ? (uint32_t)((BM * 64) >> 4) - 4u : 0u;
       auto mma4 = [&](uint32_t d_tmem, uint32_t first_acc) {
         if (!elected) return;
 #pragma unroll
         for (int k4 = 0; k4 < kStageKBytes / kUmmaKBytes; ++k4) {
           // advancing the start address by 32 bytes (2 units) steps along K inside the swizzle atom
-          const uint64_t da = ((uint64_t)kDescHi << 32) | (uint64_t)(lo + 2u * k4);
+          const uint64_t da = ((uint64_t)(kConv ? a_hi : kDescHi) << 32) | (uint64_t)(lo + 2u * k4 + (kConv && k4 >= 2 ? a_half : 0u));
           const uint64_t db = ((uint64_t)kDescHi << 32) | (uint64_t)(lo + kBOff + 2u * k4);
           const uint32_t acc = k4 == 0 ? first_acc : 1u;
           if (PAIR) tc_mma_pair<BF16>(d_tmem, da, db, p.idesc, acc);
@@ -1341,6 +1281,10 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn g_encode = nullptr;
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const int*,
+                                   const int*, cuuint32_t, cuuint32_t, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeIm2colFn g_encode_im2col = nullptr;
 
 // A two-dimensional tiled tensor map.  Encoding one costs a driver call of a microsecond or two and
 // an evaluation needs a couple of hundred, always the same ones (a map depends only on address,
@@ -1378,6 +1322,39 @@ bool encode_2d(CUtensorMap* map, CUtensorMapDataType dt, const void* ptr, uint64
   cuuint32_t estr[2] = {1, 1};
   const CUresult r = g_encode(map, dt, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz, promo,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return false;
+  std::lock_guard<std::mutex> lock(g_map_mutex);
+  if (g_map_cache.size() >= kMapCacheMax) g_map_cache.clear();
+  g_map_cache.emplace(key, *map);
+  return true;
+}
+
+// Tensor map of a convolution's NHWC code tensor for im2col loads of `chunk_bytes` of channels and 128 output
+// pixels (kept in the same table as the tiled ones).  False: the driver does not take this geometry.
+bool make_im2col_map(CUtensorMap* map, const GemmArgs& g, int64_t images, int chunk_bytes) {
+  const int esz = g.is_bf16 ? 2 : 1;
+  const CUtensorMapDataType dt = g.is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8;
+  const CUtensorMapSwizzle swz = chunk_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
+  const int lower = -g.conv_pad, upper_w = g.conv_pad - (g.conv_kw - 1), upper_h = g.conv_pad - (g.conv_kh - 1);
+  if (!g_encode_im2col || g.conv_kh != g.conv_kw || lower < -128 || upper_w < -128 || upper_h < -128 || g.conv_pad > 127 || g.conv_stride > 8 || g.conv_kw > 128 ||
+      g.conv_kh > 128 || images > 0x7fffffff || g.conv_h >= 0x10000 || g.conv_w >= 0x10000)
+    return false;
+  const MapKey key{g.a, (uint64_t)g.conv_c | ((uint64_t)g.conv_w << 32), (uint64_t)g.conv_h | ((uint64_t)images << 32),
+                   (uint64_t)g.conv_kh | ((uint64_t)g.conv_kw << 16) | ((uint64_t)g.conv_stride << 32) | ((uint64_t)g.conv_pad << 48),
+                   (uint32_t)chunk_bytes, (uint32_t)BM, (uint32_t)dt, 0x100u | (uint32_t)swz, 0u};
+  {
+    std::lock_guard<std::mutex> lock(g_map_mutex);
+    auto it = g_map_cache.find(key);
+    if (it != g_map_cache.end()) { *map = it->second; return true; }
+  }
+  cuuint64_t dims[4] = {(cuuint64_t)g.conv_c, (cuuint64_t)g.conv_w, (cuuint64_t)g.conv_h, (cuuint64_t)images};
+  const cuuint64_t px = (cuuint64_t)g.conv_c * esz;
+  cuuint64_t strides[3] = {px, px * g.conv_w, px * g.conv_w * g.conv_h};
+  int lo[2] = {lower, lower}, up[2] = {upper_w, upper_h};
+  cuuint32_t estr[4] = {1, (cuuint32_t)g.conv_stride, (cuuint32_t)g.conv_stride, 1};
+  const CUresult r = g_encode_im2col(map, dt, 4, const_cast<void*>(g.a), dims, strides, lo, up, (cuuint32_t)(chunk_bytes / esz), (cuuint32_t)BM,
+                                     estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return false;
   std::lock_guard<std::mutex> lock(g_map_mutex);
   if (g_map_cache.size() >= kMapCacheMax) g_map_cache.clear();
@@ -1468,6 +1445,10 @@ int gemm_init(Ctx* ctx) {
     cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
     if (e != cudaSuccess || qres != cudaDriverEntryPointSuccess || !fn)
       return set_error(ctx, QCFG_ECUDA, "cuTensorMapEncodeTiled entry point not found");
+    void* fi = nullptr;
+    e = cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &fi, cudaEnableDefault, &qres);
+    if (e == cudaSuccess && qres == cudaDriverEntryPointSuccess) g_encode_im2col = reinterpret_cast<EncodeIm2colFn>(fi);
+    else (void)cudaGetLastError();        // convolutions then keep the gather warps
     g_encode = reinterpret_cast<EncodeTiledFn>(fn);
   }
   cudaError_t e = cudaSuccess;
@@ -1779,7 +1760,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   const bool conv = g0.conv_kh > 0;
   if (conv) {
     ConvDesc& cv = p.conv;
-    cv.on = 1; cv.H = g0.conv_h; cv.W = g0.conv_w; cv.C = g0.conv_c; cv.kh = g0.conv_kh; cv.kw = g0.conv_kw;
+    cv.on = CONV_GATHER; cv.H = g0.conv_h; cv.W = g0.conv_w; cv.C = g0.conv_c; cv.kh = g0.conv_kh; cv.kw = g0.conv_kw;
     cv.stride = g0.conv_stride; cv.pad = g0.conv_pad; cv.esz = esz; cv.K = (int32_t)g0.k;
     cv.OH = (cv.H + 2 * cv.pad - cv.kh) / cv.stride + 1;
     cv.OW = (cv.W + 2 * cv.pad - cv.kw) / cv.stride + 1;
@@ -1787,6 +1768,10 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
     cv.src = reinterpret_cast<const uint8_t*>(g0.a);
     if (cv.OH < 1 || cv.OW < 1 || g0.m % ((int64_t)cv.OH * cv.OW))
       return set_error(ctx, QCFG_ESHAPE, "gemm: convolution rows are not a whole number of images");
+    // TMA in its im2col mode where the channels come in whole 64-byte chunks, gather warps otherwise
+    const int64_t images = g0.m / ((int64_t)cv.OH * cv.OW), cbytes = (int64_t)cv.C * esz;
+    if (cbytes % 128 == 0 && make_im2col_map(&maps[MAP_A], g0, images, 128)) cv.on = CONV_TMA128;
+    else if (cbytes % 64 == 0 && make_im2col_map(&maps[MAP_A], g0, images, 64)) cv.on = CONV_TMA64;
   }
   // Launches that may join a chain all take the larger staging size, so any sequence of them
   // shares one shared-memory layout.
@@ -1947,7 +1932,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   // touching global memory.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(conv ? kGemmThreadsConv : kGemmThreads);
+  cfg.blockDim = dim3(p.conv.on == CONV_GATHER ? kGemmThreadsConv : kGemmThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];

@@ -366,3 +366,33 @@ def test_shortcut_layers_at_tile_edges(ctx, m, n):
         ctx.check_sync()
         assert torch.equal(only[4], ys[4])
     model.close()
+
+
+@pytest.mark.parametrize("c,n,hw,k,stride,pad,batch", [(64, 64, 9, 3, 1, 1, 3), (64, 256, 13, 3, 1, 1, 5), (128, 128, 14, 3, 2, 1, 4),
+                                                       (192, 48, 7, 3, 2, 1, 7), (128, 512, 8, 1, 2, 0, 33), (64, 32, 11, 5, 1, 2, 2),
+                                                       (64, 64, 130, 3, 1, 0, 1), (256, 256, 4, 3, 1, 1, 40)])
+def test_convolution_operand_through_tma_matches_the_patch_matrix(ctx, c, n, hw, k, stride, pad, batch):
+    """Channels in whole 64- and 128-byte chunks: TMA brings the patches.  Filters of one, nine and 25 taps (odd chunk
+    counts leave half a k-block), strides, tiles that cross rows and images, a ragged last tile, CTA pairs."""
+    L = wl.Layer
+    oh = (hw + 2 * pad - k) // stride + 1
+    layers = [L("in", c, 16, src=-1, kh=1, kw=1, stride=1, in_h=hw, in_w=hw, in_c=16, src_h=hw, src_w=hw),
+              L("conv", n, k * k * c, src=0, act=orc.ACT_RELU, kh=k, kw=k, stride=stride, pad=pad, in_h=hw, in_w=hw, in_c=c, src_h=hw, src_w=hw),
+              L("out", 16, n, src=1, kh=1, kw=1, stride=1, in_h=oh, in_w=oh, in_c=n, src_h=oh, src_w=oh)]
+    rng = np.random.default_rng(c + n + hw)
+    x = rng.standard_normal((batch, hw, hw, 16)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("conv", 1, layers, batch, x, ws)
+    model, xd = build(ctx, w)
+    act_g, w_amax = check_calibration(model, w)
+    for bits in ([8, 8, 8], [8, 5, 16], [8, 16, 4]):
+        outs = []
+        for implicit in (True, False):
+            ctx.set_implicit_conv(implicit)
+            outs.append(run_eval(ctx, model, w, xd, bits))
+            if implicit:
+                teacher_forced_check(ctx, model, w, xd, bits, outs[0], act_g, w_amax)
+        ctx.set_implicit_conv(True)
+        for a, b in zip(*outs):
+            assert torch.equal(a, b)
+    model.close()
