@@ -73,11 +73,11 @@ constexpr int kPoolAll = kMaxGroups * kMapsPerGroup;   // a launch of its own: e
 constexpr int kPoolChain = 8;                          // a record of a chain: the (distinct) maps it really uses
 // Epilogue bodies.  The general one handles any combination of outputs with run-time branches; the
 // two common combinations have straight-line bodies (same arithmetic, same order).
-enum : int32_t { EPI_GENERAL = 0, EPI_CODES1 = 1, EPI_Y = 2, EPI_SHORTCUT = 3 };
+enum : int32_t { EPI_GENERAL = 0, EPI_CODES1 = 1, EPI_Y = 2, EPI_SHORTCUT = 3, EPI_CODES32 = 4 };
 // Fast bodies (256-column tiles only): EPI_CODES1 writes each warp's 32 x 64 int8 block with one
 // TMA store (64-byte rows, 64B swizzle), EPI_Y each 32 x 32 fp32 block with one (128-byte rows,
 // 128B swizzle).  EPI_SHORTCUT (int8, one CTA per tile, at most 128 columns): fp32 shortcut in, fp32 matrix and
-// up to two int8 code matrices out.
+// up to two int8 code matrices out.  EPI_CODES32 (one CTA per tile, fewer than 256 columns): one int8 code matrix.
 struct GroupDesc {
   int32_t n, tn_begin;        // columns; first column-tile index of the group in the launch's numbering
   int32_t act;
@@ -108,7 +108,8 @@ struct ConvDesc {
 constexpr int kMaxDeps = 4;
 struct GemmParams {
   int32_t m, k_blocks, bn, tiles_m, tiles_n, stages, is_bf16;   // tiles_n: column tiles of all groups together
-  int32_t epi_bytes;          // staging bytes per epilogue warp (2048 or 4096)
+  int32_t epi_bytes;          // staging bytes per epilogue warp
+  int32_t alternate;          // tiles of 64 columns: half of the epilogue warps take the even tiles, half the odd ones
   uint32_t idesc;
   GroupDesc grp[kMaxGroups];  // unused groups have tn_begin = INT32_MAX
   unsigned* err;
@@ -598,6 +599,45 @@ __device__ __forceinline__ void epilogue_chunk(const GroupDesc& p, const CUtenso
   }
 }
 
+// One warp's 32 x 32 block of a layer whose only output is one int8 code matrix, in tiles narrower than 256
+// columns (the convolutions of 64 and 128 channels and the 1x1 layers in front of them).  One accumulator
+// load, broadcast scales, one TMA store of 32-byte rows; tiles of 64 columns are taken by one half of the epilogue
+// warps or the other in turn.  401408 x 64 x 256: 40.7 us in the general body, 25.1 us here; 100352 x 128 x 512:
+// 20.0 -> 16.8 us.
+template <bool BF16>
+__device__ __forceinline__ void epilogue_codes32(const GroupDesc& G, const CUtensorMap* map, uint32_t tbase, const float* cs, uint32_t stage,
+                                                 int row0, int col0, bool inside, int lane, uint32_t tempty_bar) {
+  uint32_t v[32];
+  tmem_ld32_issue(tbase, v);
+  tmem_ld_wait();
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) mbar_arrive(tempty_bar);
+  const float2 inv2 = make_float2(G.outs[2].inv_scale, G.outs[2].inv_scale);
+  const float qmax = G.outs[2].qmax;
+  uint32_t w[8];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t part[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) part[i] = v[16 * h + i];
+    float2 y[8];
+    sub_values<BF16>(y, part, cs + 16 * h, G.act);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float2 a = code_words2(y[2 * j], inv2, qmax), b = code_words2(y[2 * j + 1], inv2, qmax);
+      w[4 * h + j] = pack4(__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(b.x), __float_as_uint(b.y));
+    }
+  }
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the last tile's store has read the slot
+  __syncwarp();
+  st_shared_v4(stage + lane * 32, w[0], w[1], w[2], w[3]);
+  st_shared_v4(stage + lane * 32 + 16, w[4], w[5], w[6], w[7]);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  if (lane == 0 && inside) tma_store_2d(map, stage, col0, row0);
+}
+
 // One warp's 32 x 32 block of a shortcut layer.  The shortcut block has been brought into `block` by TMA (128-byte
 // rows, 128B swizzle) while the previous tile was worked on; the sum goes back to the same place and out
 // from there, so the block is both the staging of the load and of the store, and no global load sits on the
@@ -675,8 +715,12 @@ __device__ __forceinline__ void epilogue_shortcut(const GroupDesc& G, const CUte
 // Waits only ever point at earlier tiles of the sequence and the launch is cooperative (all CTAs
 // resident), so the first unfinished tile can always proceed.  The records of a chain share tile
 // shape, operand type, stage count, staging size, rows and grid.
-template <bool BF16, bool PAIR, bool GROUPED, bool CHAIN>
-__global__ void __launch_bounds__(kGemmThreadsConv, 1)
+// FL: what the single-GEMM flavours carry besides the plain matrix product.  Convolutions and shortcut layers have
+// instantiations of their own: their code inside the plain kernel slowed its short launches by a tenth to a fifth
+// (100352 x 128 x 512: 20.0 -> 24.5 us).
+enum : int { FL_PLAIN = 0, FL_CONV = 1, FL_SHORTCUT = 2 };
+template <bool BF16, bool PAIR, bool GROUPED, bool CHAIN, int FL = FL_PLAIN>
+__global__ void __launch_bounds__(FL == FL_CONV || CHAIN ? kGemmThreadsConv : kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   const GemmParams& p = L.rec[0].p;        // what all records of the launch have in common is read here
   const GemmParams* q = &L.rec[0].p;       // the record this thread's role is working on
@@ -760,7 +804,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   int ld_tm = tm0, ld_tn = tn0;
   const CUtensorMap* ld_map_a = &mp[q->mi[0][MAP_A]];
   const CUtensorMap* ld_map_b = &mp[q->mi[0][MAP_B]];
-  constexpr bool kConv = !GROUPED && !CHAIN;
+  constexpr bool kConv = FL == FL_CONV;
   const bool conv_tma = kConv && p.conv.on >= CONV_TMA128;
   int cv_n = 0, cv_h = 0, cv_w = 0;              // TMA convolutions: corner of the tile's first pixel
   int cv_c = 0, cv_dx = 0, cv_dy = 0;            // channel and tap of the next chunk
@@ -780,7 +824,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   };
   if (warp == 0) set_tile_coords();
   const bool elected = elect_one();    // the lane of a converged warp that issues TMA / MMA instructions
-  const bool conv_on = p.conv.on == CONV_GATHER;
+  const bool conv_on = kConv && p.conv.on == CONV_GATHER;
   // one 128-row column of patches per call; chunks behind the last tap repeat the first one (the B tile is zero there)
   auto load_patches = [&]() {
     const int chunk = (p.conv.on == CONV_TMA64 ? 64 : 128) / (BF16 ? 2 : 1);
@@ -829,8 +873,8 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mp[q->mi[0][MAP_B]]) : "memory");
     const uint32_t full_count = 1 + (conv_on ? kGatherWarps * (PAIR ? 2 : 1) : 0);   // the TMA thread, plus one arrival per gather warp
     for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, full_count); mbar_init(empty0 + 8 * s, 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, PAIR ? 2 * kEpiWarps : kEpiWarps); }
-    if (!PAIR && !BF16) for (int a = 0; a < 2 * kEpiWarps; ++a) mbar_init(smem_u32(smem + kResBarOffset) + 8 * a, 1);
+    for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, PAIR ? 2 * kEpiWarps : p.alternate ? kEpiWarps / 2 : kEpiWarps); }
+    if (FL == FL_SHORTCUT) for (int a = 0; a < 2 * kEpiWarps; ++a) mbar_init(smem_u32(smem + kResBarOffset) + 8 * a, 1);
     if (CHAIN) for (int a = 0; a < kEpiWarps; ++a) *reinterpret_cast<volatile uint32_t*>(smem + 320 + 4 * a) = 0u;
     *abort_flag = 0;
     *reinterpret_cast<volatile uint32_t*>(smem + 264) = 0u;
@@ -1003,7 +1047,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
         }
       }
     }
-  } else if (warp >= 2 + kEpiWarps) {
+  } else if (kConv && warp >= 2 + kEpiWarps) {
     // ------------------------------------------------------------------ gather warps (convolutions)
     // Each lane owns two rows of the CTA's 128-row A tile.  Per k-block it copies the rows' eight
     // 16-byte chunks from the NHWC source (cp.async with zero fill outside the image, beyond the
@@ -1075,7 +1119,8 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     // ------------------------------------------------------------------ epilogue
     const int ew = warp - 2;
     const int quad = warp & 3;                 // TMEM lanes 32*quad .. 32*quad+31 belong to this warp
-    const int colgrp = ew >> 2;                // four warp sets share the tile's columns
+    const bool alternate = !PAIR && !GROUPED && !CHAIN && FL != FL_SHORTCUT && p.alternate;
+    const int colgrp = alternate ? (ew >> 2) & 1 : ew >> 2;    // four warp sets share the tile's columns (alternate: two, on every other tile)
     const int chunks = p.bn >> 5;
     const int cpg = chunks >= 4 ? (chunks >> 2) : 1;
     const int c_begin = colgrp * cpg;
@@ -1085,7 +1130,17 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     uint32_t cursor = 0;
     bool prev_fast = false;
     bool ok = true;
-    int t = 0;
+    // this warp's walk through the CTA's tiles: all of them, or every other one
+    int t = 0, tile = tile0, tm = tm0, tn = tn0;
+    int e_step = tile_step, e_tm = step_tm, e_tn = step_tn;
+    if (alternate) {
+      if (ew >> 3) {
+        t = 1; tile += tile_step; tm += step_tm; tn += step_tn;
+        if (tm >= q->tiles_m) { tm -= q->tiles_m; ++tn; }
+      }
+      e_step = 2 * tile_step; e_tm = 2 * step_tm; e_tn = 2 * step_tn;
+      if (e_tm >= q->tiles_m) { e_tm -= q->tiles_m; ++e_tn; }
+    }
     // Weight scales of this warp's chunks, one column per lane and chunk.  They are fetched one
     // tile ahead: when the epilogue is the longer phase the accumulator is already waiting at
     // the top of the loop, and a load issued there would put its whole latency on the tile.
@@ -1103,9 +1158,8 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
       }
     };
     float sw_next[2];
-    int tm = tm0, tn = tn0;
     // shortcut blocks: brought in one tile ahead, into the two blocks in turn
-    const bool shortcut = !PAIR && !BF16 && !GROUPED && p.grp[0].mode == EPI_SHORTCUT && c_begin < c_end;
+    const bool shortcut = FL == FL_SHORTCUT && c_begin < c_end;
     const uint32_t res_bar0 = smem_u32(smem + kResBarOffset) + 16 * ew;
     auto fetch_shortcut = [&](int which, int ftm, int ftn) {      // lane 0
       const uint32_t bar = res_bar0 + 8 * which;
@@ -1121,9 +1175,9 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
         load_scales(cur.q, true, tn_0, sw_next);
       }
     } else {
-      load_scales(q, tile0 < num_tiles, tn0, sw_next);
+      load_scales(q, tile < num_tiles, tn, sw_next);
     }
-    for (int tile = tile0; tile < total_tiles && ok; tile += tile_step, ++t) {
+    for (; tile < total_tiles && ok; tile += e_step, t += alternate ? 2 : 1) {
       if (CHAIN) {     // record of this tile, column tile fastest inside it
         cur_seek(cur, tile); q = cur.q; mp = cur.mp;
         int gi_;
@@ -1135,7 +1189,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
       const GroupDesc& G = q->grp[g];
       const int col_base = tile_in_group(tn, g) * p.bn + c_begin * 32;
       const float cs[2] = {__fmul_rn(G.scale_x, sw_next[0]), __fmul_rn(G.scale_x, sw_next[1])};
-      int tm_next = tm + step_tm, tn_next = tn + step_tn;
+      int tm_next = tm + e_tm, tn_next = tn + e_tn;
       if (CHAIN) {
         const int nt = tile + tile_step;
         Cur c2 = cur;
@@ -1145,7 +1199,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
         load_scales(c2.q, nt < total_tiles, tn2, sw_next);
       } else {
         if (tm_next >= q->tiles_m) { tm_next -= q->tiles_m; ++tn_next; }
-        load_scales(q, tile + tile_step < num_tiles, tn_next, sw_next);
+        load_scales(q, tile + e_step < num_tiles, tn_next, sw_next);
       }
       // Chains: the previous tile is reported once its stores have completed.  When this tile's
       // accumulator is already there the check is left to the body (after its first piece, when
@@ -1174,7 +1228,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
       const int nch = c_end - c_begin;           // 0, 1 or 2
       const int64_t row = (int64_t)row0 + lane;
       const uint32_t tempty_bar = tempty0 + 8 * a;
-      if (!PAIR && !BF16 && !GROUPED && G.mode == EPI_SHORTCUT) {
+      if (FL == FL_SHORTCUT) {
         if (nch == 0) {
           __syncwarp();
           if (lane == 0) mbar_arrive(tempty_bar);
@@ -1183,6 +1237,17 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
           __syncwarp();
           epilogue_shortcut(G, mp, q->mi[0], tbase, cs_tab, stage + (t & 1) * 4096, stage + 2 * 4096, row0, col_base, lane, tempty_bar,
                             res_bar0 + 8 * (t & 1), (uint32_t)(t >> 1) & 1u, row0 < q->m && col_base < G.n, abort_flag, p.err, ok);
+        }
+      } else if (!PAIR && !GROUPED && !CHAIN && G.mode == EPI_CODES32) {
+        if (nch == 0) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty_bar);
+        } else {
+          if (!BF16) {
+            cs_tab[lane] = cs[0];
+            __syncwarp();
+          }
+          epilogue_codes32<BF16>(G, &mp[q->mi[0][MAP_OUT + 2]], tbase, cs_tab, stage, row0, col_base, row0 < q->m && col_base < G.n, lane, tempty_bar);
         }
       } else if (G.mode != EPI_GENERAL) {
         // fast bodies: 256-column tiles, so this warp owns 64 columns starting at col_base
@@ -1452,13 +1517,16 @@ int gemm_init(Ctx* ctx) {
     g_encode = reinterpret_cast<EncodeTiledFn>(fn);
   }
   cudaError_t e = cudaSuccess;
-  const void* kernels[10] = {
+  const void* kernels[15] = {
       (const void*)gemm_kernel<false, false, false, false>, (const void*)gemm_kernel<false, false, true, false>,
       (const void*)gemm_kernel<false, true, false, false>,  (const void*)gemm_kernel<false, true, true, false>,
       (const void*)gemm_kernel<true, false, false, false>,  (const void*)gemm_kernel<true, false, true, false>,
       (const void*)gemm_kernel<true, true, false, false>,   (const void*)gemm_kernel<true, true, true, false>,
-      (const void*)gemm_kernel<false, true, true, true>,    (const void*)gemm_kernel<true, true, true, true>};
-  for (int i = 0; i < 10 && e == cudaSuccess; ++i)
+      (const void*)gemm_kernel<false, true, true, true>,    (const void*)gemm_kernel<true, true, true, true>,
+      (const void*)gemm_kernel<false, false, false, false, FL_CONV>, (const void*)gemm_kernel<false, true, false, false, FL_CONV>,
+      (const void*)gemm_kernel<true, false, false, false, FL_CONV>,  (const void*)gemm_kernel<true, true, false, false, FL_CONV>,
+      (const void*)gemm_kernel<false, false, false, false, FL_SHORTCUT>};
+  for (int i = 0; i < 15 && e == cudaSuccess; ++i)
     e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
   if (e != cudaSuccess) return check_cuda(ctx, e, "gemm smem attribute");
   ChainState* cs = new (std::nothrow) ChainState();
@@ -1663,9 +1731,9 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   // Shortcut layers at integer widths whose matrices TMA can reach: a body of its own, which keeps two fp32
   // blocks per epilogue warp in shared memory and therefore works on 128 columns at most.
   bool shortcut = false;
-  if (count == 1 && !g0.is_bf16 && g0.residual && g0.y && !g0.acc && !g0.amax && g0.conv_kh == 0 && !g0.slots[2].kind) {
+  if (count == 1 && !g0.is_bf16 && g0.residual && (g0.y || g0.slots[0].kind) && !g0.acc && !g0.amax && g0.conv_kh == 0 && !g0.slots[2].kind) {
     auto aligned = [](const void* q, int64_t ld_bytes) { return ((uintptr_t)q & 15) == 0 && (ld_bytes & 15) == 0; };
-    shortcut = aligned(g0.residual, g0.ldr * 4) && aligned(g0.y, g0.ldy * 4);
+    shortcut = aligned(g0.residual, g0.ldr * 4) && (!g0.y || aligned(g0.y, g0.ldy * 4));
     for (int i = 0; i < 2; ++i)
       if (g0.slots[i].kind) shortcut = shortcut && g0.slots[i].kind == 1 && aligned(g0.slots[i].ptr, g0.slots[i].ld);
     if (shortcut && bn > 128) bn = 128;
@@ -1738,6 +1806,9 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
     // staging per epilogue warp: two slots of 1 KB when only int8 codes are written, else of 2 KB
     for (int j = 0; j < kNumOuts; ++j) if (G.outs[j].kind >= 3 || (G.outs[j].kind == 2 && G.outs[j].tma)) wide = true;
     G.mode = EPI_GENERAL;
+    if (bn < 256 && count == 1 && !G.residual && !G.amax && !G.outs[0].kind && !G.outs[1].kind && G.outs[2].kind == 1 && G.outs[2].tma &&
+        !G.outs[3].kind && !G.outs[4].kind)
+      G.mode = EPI_CODES32;
     if (bn == 256 && !G.residual && !G.amax && !G.outs[0].kind && !G.outs[3].kind && !G.outs[4].kind) {
       if (!G.outs[1].kind && G.outs[2].kind == 1 && make_fast_map(&maps[i * kMapsPerGroup + MAP_FAST], G.outs[2], g.m, g.n)) G.mode = EPI_CODES1;
       else if (G.outs[1].kind && !G.outs[2].kind && make_fast_map(&maps[i * kMapsPerGroup + MAP_FAST], G.outs[1], g.m, g.n)) { G.mode = EPI_Y; wide = true; }
@@ -1745,7 +1816,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
     if (shortcut) {      // MAP_OUT, the raw accumulators' place, holds the shortcut's map
       OutDesc in{};
       in.kind = 3; in.ptr = const_cast<float*>(g.residual); in.ld = g.ldr;
-      if (!make_fast_map(&maps[MAP_FAST], G.outs[1], g.m, g.n) || !make_fast_map(&maps[MAP_OUT], in, g.m, g.n))
+      if ((g.y && !make_fast_map(&maps[MAP_FAST], G.outs[1], g.m, g.n)) || !make_fast_map(&maps[MAP_OUT], in, g.m, g.n))
         return set_error(ctx, QCFG_ECUDA, "cuTensorMapEncodeTiled failed");
       for (int j = 2; j < 4; ++j)
         if (G.outs[j].kind && !G.outs[j].tma) return set_error(ctx, QCFG_ECUDA, "cuTensorMapEncodeTiled failed");
@@ -1780,6 +1851,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   // producer's rows would cost more than the launch boundary it saves)
   const bool chainable = cs && cs->open && ctx_chain_enabled(ctx) && pair && !conv && bn == 256 && prof_mode(ctx) != 1 && p.tiles_m <= kChainMaxTilesM &&
                          2 * p.tiles_m * p.tiles_n >= sm_count(ctx);
+  p.alternate = !pair && bn == 64 && p.grp[0].mode == EPI_CODES32;
   p.epi_bytes = shortcut ? kShortcutBytes : (wide || chainable) ? 4096 : 2048;
   int stages = (kSmemMax - kSmemHeader - kCsBytes - 1024 - kEpiWarps * p.epi_bytes) / stage_bytes;
   if (stages > kMaxStages) stages = kMaxStages;
@@ -1947,7 +2019,12 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
       gemm_kernel<false, false, false, false>, gemm_kernel<false, false, true, false>, gemm_kernel<false, true, false, false>,
       gemm_kernel<false, true, true, false>,   gemm_kernel<true, false, false, false>,  gemm_kernel<true, false, true, false>,
       gemm_kernel<true, true, false, false>,   gemm_kernel<true, true, true, false>};
-  const Kern kern = kernels[(g0.is_bf16 ? 4 : 0) + (pair ? 2 : 0) + (count > 1 ? 1 : 0)];
+  static const Kern conv_kernels[4] = {
+      gemm_kernel<false, false, false, false, FL_CONV>, gemm_kernel<false, true, false, false, FL_CONV>,
+      gemm_kernel<true, false, false, false, FL_CONV>,  gemm_kernel<true, true, false, false, FL_CONV>};
+  const Kern kern = shortcut ? gemm_kernel<false, false, false, false, FL_SHORTCUT>
+                    : conv   ? conv_kernels[(g0.is_bf16 ? 2 : 0) + (pair ? 1 : 0)]
+                             : kernels[(g0.is_bf16 ? 4 : 0) + (pair ? 2 : 0) + (count > 1 ? 1 : 0)];
   p.stamp = prof_stamp(ctx, g0.is_bf16 ? 1 : 0, ops);
   static thread_local LaunchArgs<false> one;
   memcpy(one.rec[0].m, maps, sizeof(maps));

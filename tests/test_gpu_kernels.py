@@ -392,3 +392,21 @@ def test_second_context_sweeps_wide_rows():
         np.testing.assert_allclose(host(sse), so, rtol=1e-5)
         np.testing.assert_array_equal(host(amax), ao)
         c.close()
+
+
+@pytest.mark.parametrize("m,n,k", [(1, 64, 32), (33, 16, 48), (300, 40, 64), (19000, 64, 64), (19072, 64, 256), (38001, 48, 96), (40000, 128, 64),
+                                   (25000, 100, 160)])
+def test_narrow_code_outputs_match_the_oracle(ctx, m, n, k):
+    """One int8 code matrix of fewer than 256 columns: one to several tiles per CTA, odd and even tile counts (the 64-column
+    tiles are shared out between two halves of the epilogue warps), ragged rows and columns; every code is checked."""
+    import paper_2302_01382_b200 as q
+    rng = np.random.default_rng(m + n + k)
+    qx = rng.integers(-127, 128, (m, k), dtype=np.int8)
+    qw = rng.integers(-127, 128, (n, k), dtype=np.int8)
+    sw = (10.0 ** rng.uniform(-4, -2, n)).astype(np.float32)
+    y = orc.activation(orc.dequant_output(orc.int_gemm(qx, qw), np.float32(0.0173), sw), orc.ACT_RELU)
+    _, inv = orc.scales_from_absmax(np.float32(np.abs(y).max() * 0.6), 6)
+    out = ctx.gemm_i8_requant(dev(qx), dev(qw), k, 0.0173, dev(sw), q.ACT_RELU, float(inv), 6)
+    ctx.check_sync()
+    np.testing.assert_array_equal(host(out)[:, :n], orc.quantize(y, inv, 6))
+    assert not host(out)[:, n:].any()
