@@ -278,6 +278,12 @@ bool reads_rows_directly(const qcfg_layer& d) {
 // A convolution whose operand the GEMM can gather from the NHWC codes of its input: not a plain
 // row read, and channels in whole 16-byte chunks at either operand width.
 bool implicit_capable(const qcfg_layer& d) { return d.kh > 0 && !reads_rows_directly(d) && d.in_c % 16 == 0 && !(d.kh == 1 && d.kw == 1 && d.stride == 1 && d.pad == 0); }
+// A 16-bit convolution of an image with few channels: its own kernel, which never builds a patch matrix and can
+// write its max-pooled output directly.  Depends on the geometry alone, so a layer gives the same bits in
+// every pass, whatever the pass writes and whatever the switches say.
+bool is_stem(const qcfg_layer& d, int bits) {
+  return bits == 16 && d.kh > 0 && d.residual_from < 0 && stem_capable(d.n_out, d.in_h, d.in_w, d.in_c, d.kh, d.kw, d.stride, d.pad, d.act);
+}
 bool same_input(const qcfg_layer& a, const qcfg_layer& b) {
   return a.src == b.src && a.src_col0 == b.src_col0 && a.k_in == b.k_in && a.kh == b.kh && a.kw == b.kw &&
          a.stride == b.stride && a.pad == b.pad && a.pool_before == b.pool_before && a.in_h == b.in_h &&
@@ -467,7 +473,6 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
         srows = d.kh > 0 || d.pool_before != QCFG_POOL_NONE ? m * (int64_t)d.src_h * d.src_w : m;
       } else {
         LayerState& P = M->L[d.src];
-        if (!P.y_ptr) return set_error(ctx, QCFG_ESTATE, "layer %d: producer %d output not materialised", l, d.src);
         sp = P.y_ptr; sld = P.d.n_out; srows = P.rows;
       }
       if (d.pool_before != QCFG_POOL_NONE) {
@@ -481,6 +486,7 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
           if (T.pre_ptr && T.d.src == d.src && T.d.pool_before == d.pool_before && T.d.src_h == d.src_h && T.d.src_w == d.src_w)
             S.pre_ptr = T.pre_ptr;
         }
+        if (!S.pre_ptr && !sp) return set_error(ctx, QCFG_ESTATE, "layer %d: producer %d output not materialised", l, d.src);
         if (!S.pre_ptr) {
           rc = S.prebuf.ensure(ctx, (size_t)(prows * sld) * 4);
           if (rc) return rc;
@@ -493,6 +499,7 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
         }
         sp = S.pre_ptr; srows = prows;
       }
+      if (!sp) return set_error(ctx, QCFG_ESTATE, "layer %d: producer %d output not materialised", l, d.src);
       const bool direct = d.kh == 0 || (d.kh == 1 && d.kw == 1 && d.stride == 1 && d.pad == 0);
       if (d.kh > 0) {
         if (sld != d.in_c || srows != m * (int64_t)d.in_h * d.in_w)
@@ -511,6 +518,43 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
         rc = launch_absmax(ctx, tp, srows, width, sld, QCFG_PER_TENSOR, (float*)M->act_absmax_dev.p + l, st);
         if (rc) return rc;
         range_pending = false;
+      }
+      if (is_stem(d, b)) {
+        // outputs: the max-pooled tensor goes straight to the first layer that reads it so; the full one is
+        // written only if somebody asks for it or reads it in another way
+        LayerState* pooled = nullptr;
+        bool all_pooled = !S.consumers.empty() && !S.feeds_residual;
+        const int64_t oh = (d.in_h + 2 * d.pad - d.kh) / 2 + 1, ow = (d.in_w + 2 * d.pad - d.kw) / 2 + 1;
+        for (int c : S.consumers) {
+          LayerState& C = M->L[c];
+          if (C.d.pool_before != QCFG_POOL_MAX3S2 || C.d.src_h != oh || C.d.src_w != ow) { all_pooled = false; continue; }
+          if (!pooled && dirty[c]) pooled = &C;
+        }
+        float* y_out = (y_dev && y_dev[l]) ? y_dev[l] : nullptr;
+        float* tmp = nullptr;                       // an output pointer the kernel's 16-byte stores cannot take
+        const bool odd_ptr = ((uintptr_t)y_out & 15) != 0;
+        if (!all_pooled || odd_ptr) {
+          rc = S.ybuf.ensure(ctx, (size_t)(S.rows * d.n_out) * 4);
+          if (rc) return rc;
+          if (odd_ptr) { tmp = y_out; y_out = (float*)S.ybuf.p; }
+          else if (!y_out) y_out = (float*)S.ybuf.p;
+        }
+        if (pooled) {
+          rc = pooled->prebuf.ensure(ctx, (size_t)(m * ((oh - 1) / 2 + 1) * ((ow - 1) / 2 + 1) * d.n_out) * 4);
+          if (rc) return rc;
+          pooled->pre_ptr = (const float*)pooled->prebuf.p;
+        }
+        if (y_out || pooled)
+          rc = launch_stem(ctx, sp, m, d.in_h, d.in_w, d.in_c, S.wc[16].codes.p, S.ldk, d.n_out, d.kh, d.kw, d.pad, d.act, y_out,
+                           pooled ? (float*)pooled->prebuf.p : nullptr, st);
+        if (!rc && tmp)
+          rc = check_cuda(ctx, cudaMemcpyAsync(tmp, y_out, (size_t)(S.rows * d.n_out) * 4, cudaMemcpyDeviceToDevice, st), "stem output copy");
+        if (rc) return rc;
+        S.y_ptr = tmp ? tmp : y_out;
+        S.y_internal = S.y_ptr && S.y_ptr == (const float*)S.ybuf.p;
+        S.a_ready = false; S.a_ptr = nullptr;
+        if (layer_ev && cudaEventRecord(layer_ev[2 * l + 1], st) != cudaSuccess) return check_cuda(ctx, cudaGetLastError(), "event record");
+        continue;
       }
       // reuse the codes of an earlier layer that reads the same input with the same grid
       int share = -1;
@@ -677,6 +721,7 @@ int qcfg_create(qcfg_ctx** out, int device) {
   int rc = pinned(&h->c, 16384) ? QCFG_OK : QCFG_ENOMEM;
   if (!rc) rc = gemm_init(&h->c);
   if (!rc) rc = sweep_init(&h->c);
+  if (!rc) rc = stem_init(&h->c);
   if (rc) { gemm_destroy(&h->c); if (h->c.pin_buf) cudaFreeHost(h->c.pin_buf); cudaFree(h->c.err_dev); delete h; return rc; }
   *out = h;
   return QCFG_OK;

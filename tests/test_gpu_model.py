@@ -396,3 +396,45 @@ def test_convolution_operand_through_tma_matches_the_patch_matrix(ctx, c, n, hw,
         for a, b in zip(*outs):
             assert torch.equal(a, b)
     model.close()
+
+
+@pytest.mark.parametrize("c,n,h,wd,k,pad,batch,act", [(3, 64, 32, 32, 7, 3, 3, 1), (3, 32, 33, 47, 7, 3, 2, 1), (1, 16, 20, 9, 5, 2, 40, 0),
+                                                      (4, 48, 17, 255, 3, 1, 2, 1), (2, 64, 7, 8, 7, 0, 5, 0), (3, 64, 65, 224, 7, 3, 4, 1),
+                                                      (3, 16, 16, 64, 8, 3, 2, 1), (3, 64, 16, 260, 7, 3, 1, 1), (5, 64, 16, 16, 3, 1, 2, 1)])
+def test_stem_and_its_pool_match_the_oracle(ctx, c, n, h, wd, k, pad, batch, act):
+    """Stride-2 convolutions of few channels at 16 bit with max-pooled readers: odd and even sizes and paddings, one to
+    four channels, rows up to the widest, many images, and geometries the stem kernel leaves to the general path.  The
+    pooled values must be the maxima of the very outputs the layer returns (its readers' integer outputs are checked
+    bit for bit), and the readers' results must not depend on whether the full output is returned."""
+    L = wl.Layer
+    oh, ow = (h + 2 * pad - k) // 2 + 1, (wd + 2 * pad - k) // 2 + 1
+    ph, pw = (oh + 2 - 3) // 2 + 1, (ow + 2 - 3) // 2 + 1
+    layers = [L("stem", n, k * k * c, src=-1, act=act, kh=k, kw=k, stride=2, pad=pad, in_h=h, in_w=wd, in_c=c, src_h=h, src_w=wd),
+              L("a", 24, n, src=0, kh=1, kw=1, stride=1, in_h=ph, in_w=pw, in_c=n, pool_before=wl.POOL_MAX3S2, src_h=oh, src_w=ow),
+              L("b", 16, n, src=0, kh=1, kw=1, stride=1, in_h=ph, in_w=pw, in_c=n, pool_before=wl.POOL_MAX3S2, src_h=oh, src_w=ow)]
+    rng = np.random.default_rng(h * wd + n)
+    x = rng.standard_normal((batch, h, wd, c)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("stem", 1, layers, batch, x, ws)
+    model, xd = build(ctx, w)
+    act_g, w_amax = check_calibration(model, w)
+    bits = [16, 8, 5]
+    ys = run_eval(ctx, model, w, xd, bits)
+    teacher_forced_check(ctx, model, w, xd, bits, ys, act_g, w_amax)
+    # fp32 sums of exact bf16 products: each within K rounding steps of the magnitude sum
+    ref = orc.bf16_gemm(orc.im2col(x, k, k, 2, pad), ws[0])
+    mag = orc.bf16_gemm(np.abs(orc.im2col(x, k, k, 2, pad)), np.abs(ws[0]))
+    assert np.all(np.abs(host(ys[0]) - orc.activation(ref, act)) <= k * k * c * 2.0 ** -23 * mag + 1e-30)
+    only = [None, torch.full_like(ys[1], float("nan")), torch.full_like(ys[2], float("nan"))]
+    model.eval_config(bits, xd, batch, only)
+    ctx.check_sync()
+    assert torch.equal(only[1], ys[1]) and torch.equal(only[2], ys[2])
+    ctx.set_prefix_reuse(True)
+    try:
+        for b2 in ([16, 8, 5], [16, 4, 5], [16, 4, 8], [16, 8, 5]):       # a changed reader brings the pooled input back
+            model.eval_config(b2, xd, batch, only)
+        ctx.check_sync()
+        assert torch.equal(only[1], ys[1]) and torch.equal(only[2], ys[2])
+    finally:
+        ctx.set_prefix_reuse(False)
+    model.close()
