@@ -410,3 +410,44 @@ def test_narrow_code_outputs_match_the_oracle(ctx, m, n, k):
     ctx.check_sync()
     np.testing.assert_array_equal(host(out)[:, :n], orc.quantize(y, inv, 6))
     assert not host(out)[:, n:].any()
+
+
+@pytest.mark.parametrize("m,n,act", [(4099, 1000, 0), (9000, 520, 2), (2600, 2056, 1)])
+def test_wide_bf16_outputs_match_the_oracle(ctx, m, n, act):
+    """16-bit operands for the next layer out of 256-column tiles, ragged rows and columns, several tiles per CTA."""
+    rng = np.random.default_rng(m + n)
+    k = 96
+    qx, qw = _codes(rng, m, k, k), _codes(rng, n, k, k)
+    sw = (10.0 ** rng.uniform(-4, -2, n)).astype(np.float32)
+    y = orc.activation(orc.dequant_output(orc.int_gemm(qx, qw), np.float32(0.0173), sw), act)
+    out = ctx.gemm_i8_requant(dev(qx), dev(qw), k, 0.0173, dev(sw), act, 1.0, 16)
+    ctx.check_sync()
+    got, want = host(out.float())[:, :n], orc.bf16_round(y)
+    if act == 2:      # GELU outputs are within 1e-6 relative plus 1e-6 * max|y| of the oracle's: rounded, between the bounds' roundings
+        d = (1e-6 * np.abs(y) + 1e-6 * np.abs(y).max()).astype(np.float32)
+        assert np.all(got >= orc.bf16_round(y - d)) and np.all(got <= orc.bf16_round(y + d))
+    else:
+        np.testing.assert_array_equal(got.view(np.uint32), want.view(np.uint32))
+    assert not host(out.float())[:, n:].any()
+
+
+def test_calibration_ranges_do_not_depend_on_the_route(ctx):
+    """Maxima taken in the epilogue that writes the 16-bit operand equal those of separate passes, at sizes whose GEMMs
+    run in 256-column tiles and in chains."""
+    import paper_2302_01382_b200 as q
+    import qcfg_workloads as wl
+    w = wl.bert_stack(6, 9001, 392, 1544, 2, bit_choices=None)
+    weights, x = [dev(a) for a in w.weights], dev(w.x)
+    tables = []
+    for fuse, chains in ((True, True), (True, False), (False, False)):
+        ctx.set_fusion(fuse)
+        ctx.set_gemm_chains(chains)
+        try:
+            model = q.Model(ctx, w.layers, weights)
+            model.calibrate_model(x, w.m)
+            tables.append(model.act_absmax())
+            model.close()
+        finally:
+            ctx.set_fusion(True)
+            ctx.set_gemm_chains(True)
+    assert tables[0] == tables[1] == tables[2]
