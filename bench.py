@@ -40,7 +40,7 @@ WORKLOAD = "bert_base_x12_sweep_calibrate_greedy72"
 # profiles/gemm_int8_bert_base_block.md, taken with one launch per GEMM (ncu cannot launch the
 # cooperative chain kernel); a chained launch is charged this figure times the GEMMs it runs.
 # Set to None whenever the GEMM kernel changes.
-GEMM_TRAFFIC_BYTES = 27.1e6
+GEMM_TRAFFIC_BYTES = 26.4e6
 GEMMS_PER_EVAL = 48          # 12 blocks x (q+k+v grouped, o, ffn1, ffn2)
 DATASHEET_INT8_TOPS = 4500.0      # B200 dense int8, vendor datasheet (an outside figure)
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
