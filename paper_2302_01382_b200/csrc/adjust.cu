@@ -31,6 +31,7 @@ __device__ __forceinline__ float act_derivative(float y, int act) {
 template <bool VEC>
 __global__ void __launch_bounds__(256) act_apply_kernel(const float* __restrict__ ylin, const float* __restrict__ res,
                                                         int64_t ldr, int act, float* __restrict__ y, int64_t rows, int64_t n) {
+  pdl_entry();
   const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
   if (i >= rows * n) return;
   if (VEC) {
@@ -67,6 +68,7 @@ __global__ void __launch_bounds__(256) backward_operands_kernel(
     const float* __restrict__ ylin, const float* __restrict__ res, int64_t ldr, int act, const float* __restrict__ s_w, int64_t rows, int64_t n, int keep_g,
     __nv_bfloat16* __restrict__ gs, int64_t ld_gs, __nv_bfloat16* __restrict__ gt, int64_t ld_gt, double* __restrict__ colsum,
     int tiles_per_block) {
+  pdl_entry();
   __shared__ uint32_t turn[kTile][kTile / 2 + 1];          // [column][row], bf16 pairs; the odd pitch keeps both directions off each other's banks
   __shared__ double csum[16][kTile + 1];
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -149,6 +151,7 @@ __global__ void __launch_bounds__(256) backward_operands_kernel(
 // *coef = 2 / sum of the reference's squares, from the per-block partial sums {difference, reference} of the
 // loss; 0 for an all-zero reference (the call then ends with an error)
 __global__ void __launch_bounds__(256) loss_coef_kernel(const double* __restrict__ partial, int blocks, float* __restrict__ coef) {
+  pdl_entry();
   double v = 0.0;
   for (int i = threadIdx.x; i < blocks; i += 256) v += partial[2 * i + 1];
   v = warp_sum(v);
@@ -163,6 +166,7 @@ __global__ void __launch_bounds__(256) loss_coef_kernel(const double* __restrict
 
 __global__ void __launch_bounds__(256) gamma_finish_kernel(const double* __restrict__ colsum, const float* __restrict__ s_w,
                                                            float s_x, int64_t n, double* __restrict__ d_sw, double* __restrict__ d_sx) {
+  pdl_entry();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   double v = 0.0;
   if (i < n) {
@@ -178,6 +182,7 @@ __global__ void __launch_bounds__(256) gamma_finish_kernel(const double* __restr
 template <typename T>
 __global__ void __launch_bounds__(256) transpose_bf16_kernel(const T* __restrict__ src, int64_t rows, int64_t cols, int64_t ld_src,
                                                              __nv_bfloat16* __restrict__ dst, int64_t ld_dst) {
+  pdl_entry();
   __shared__ uint32_t turn[kTile][kTile / 2 + 1];
   const int64_t r0 = (int64_t)blockIdx.x * kTile, c0 = (int64_t)blockIdx.y * kTile;
   {
@@ -214,6 +219,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(256) input_backward_kernel(const float* __restrict__ dxq, const float* __restrict__ x, int64_t ldx,
                                                              float s_x, float inv_x, float qmax, int64_t rows, int64_t k,
                                                              float* __restrict__ gprod, int64_t ldg, int assign, double* __restrict__ d_ix) {
+  pdl_entry();
   double part = 0.0;
   const float pass = __fmul_rn(s_x, inv_x);
   const int lane = threadIdx.x & 31;
@@ -274,6 +280,7 @@ template <bool VEC, int PARTS>
 __global__ void __launch_bounds__(256) weight_alpha_kernel(const float* __restrict__ dwq, const float* __restrict__ w,
                                                            const float* __restrict__ s_w, const float* __restrict__ inv_w, float s_x,
                                                            float qmax, int64_t n, int64_t k, double* __restrict__ d_iw) {
+  pdl_entry();
   const int64_t row = blockIdx.x;
   const float iw = inv_w[row];
   const float* wr = w + row * k;
@@ -318,6 +325,7 @@ __global__ void __launch_bounds__(256) weight_alpha_kernel(const float* __restri
 }
 
 __global__ void __launch_bounds__(256) sgd_kernel(float* __restrict__ s, const double* __restrict__ g, double lr, int64_t n) {
+  pdl_entry();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) s[i] = (float)__dsub_rn((double)s[i], __dmul_rn(lr, g[i]));     // two roundings, as written
 }
@@ -331,8 +339,8 @@ static inline bool vec4(const void* p, int64_t n, int64_t ld) { return !p || ((u
 int launch_act_apply(Ctx* ctx, const float* ylin, const float* res, int64_t ldr, int act, float* y, int64_t rows, int64_t n, cudaStream_t st) {
   if (rows * n == 0) return QCFG_OK;
   const unsigned blocks = blocks_for((rows * n + 3) / 4);
-  if (vec4(ylin, n, n) && vec4(res, n, ldr) && vec4(y, n, n)) act_apply_kernel<true><<<blocks, 256, 0, st>>>(ylin, res, ldr, act, y, rows, n);
-  else act_apply_kernel<false><<<blocks, 256, 0, st>>>(ylin, res, ldr, act, y, rows, n);
+  if (vec4(ylin, n, n) && vec4(res, n, ldr) && vec4(y, n, n)) launch_pdl(act_apply_kernel<true>, dim3(blocks), dim3(256), 0, st, ylin, res, ldr, act, y, rows, n);
+  else launch_pdl(act_apply_kernel<false>, dim3(blocks), dim3(256), 0, st, ylin, res, ldr, act, y, rows, n);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "activation launch");
 }
@@ -350,20 +358,20 @@ int launch_backward_operands(Ctx* ctx, float* gout, const float* y, const float*
   __nv_bfloat16* s16 = reinterpret_cast<__nv_bfloat16*>(gs);
   __nv_bfloat16* t16 = reinterpret_cast<__nv_bfloat16*>(gt);
   if (vec4(gout, n, n) && vec4(y, n, n) && vec4(yref, n, n) && vec4(ylin, n, n))
-    backward_operands_kernel<true><<<grid, 256, 0, st>>>(gout, y, yref, coef, ylin, res, ldr, act, s_w, rows, n, keep_g, s16, ld_gs, t16, ld_gt, colsum, (int)per);
+    launch_pdl(backward_operands_kernel<true>, dim3(grid), dim3(256), 0, st, gout, y, yref, coef, ylin, res, ldr, act, s_w, rows, n, keep_g, s16, ld_gs, t16, ld_gt, colsum, (int)per);
   else
-    backward_operands_kernel<false><<<grid, 256, 0, st>>>(gout, y, yref, coef, ylin, res, ldr, act, s_w, rows, n, keep_g, s16, ld_gs, t16, ld_gt, colsum, (int)per);
+    launch_pdl(backward_operands_kernel<false>, dim3(grid), dim3(256), 0, st, gout, y, yref, coef, ylin, res, ldr, act, s_w, rows, n, keep_g, s16, ld_gs, t16, ld_gt, colsum, (int)per);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "backward operand launch");
 }
 int launch_loss_coef(Ctx* ctx, const double* partial, int blocks, float* coef, cudaStream_t st) {
-  loss_coef_kernel<<<1, 256, 0, st>>>(partial, blocks, coef);
+  launch_pdl(loss_coef_kernel, dim3(1), dim3(256), 0, st, partial, blocks, coef);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "loss coefficient launch");
 }
 int launch_gamma_finish(Ctx* ctx, const double* colsum, const float* s_w, float s_x, int64_t n, double* d_sw, double* d_sx, cudaStream_t st) {
   if (n == 0) return QCFG_OK;
-  gamma_finish_kernel<<<blocks_for(n), 256, 0, st>>>(colsum, s_w, s_x, n, d_sw, d_sx);
+  launch_pdl(gamma_finish_kernel, dim3(blocks_for(n)), dim3(256), 0, st, colsum, s_w, s_x, n, d_sw, d_sx);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "scale gradient launch");
 }
@@ -371,8 +379,8 @@ int launch_transpose_bf16(Ctx* ctx, const void* src, int kind, int64_t rows, int
   if (cols == 0 || ld_dst == 0) return QCFG_OK;
   const dim3 grid((unsigned)((ld_dst + kTile - 1) / kTile), (unsigned)((cols + kTile - 1) / kTile));
   __nv_bfloat16* d = reinterpret_cast<__nv_bfloat16*>(dst);
-  if (kind == 1) transpose_bf16_kernel<int8_t><<<grid, 256, 0, st>>>(reinterpret_cast<const int8_t*>(src), rows, cols, ld_src, d, ld_dst);
-  else transpose_bf16_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(reinterpret_cast<const __nv_bfloat16*>(src), rows, cols, ld_src, d, ld_dst);
+  if (kind == 1) launch_pdl(transpose_bf16_kernel<int8_t>, dim3(grid), dim3(256), 0, st, reinterpret_cast<const int8_t*>(src), rows, cols, ld_src, d, ld_dst);
+  else launch_pdl(transpose_bf16_kernel<__nv_bfloat16>, dim3(grid), dim3(256), 0, st, reinterpret_cast<const __nv_bfloat16*>(src), rows, cols, ld_src, d, ld_dst);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "transpose launch");
 }
@@ -384,9 +392,9 @@ int launch_input_backward(Ctx* ctx, const float* dxq, const float* x, int64_t ld
   if (by > (rows + 7) / 8) by = (rows + 7) / 8;
   const dim3 grid((unsigned)bx, (unsigned)by);
   if (vec4(dxq, k, k) && vec4(x, k, ldx) && vec4(gprod, k, ldg))
-    input_backward_kernel<true><<<grid, 256, 0, st>>>(dxq, x, ldx, s_x, inv_x, qmax, rows, k, gprod, ldg, assign, d_ix);
+    launch_pdl(input_backward_kernel<true>, dim3(grid), dim3(256), 0, st, dxq, x, ldx, s_x, inv_x, qmax, rows, k, gprod, ldg, assign, d_ix);
   else
-    input_backward_kernel<false><<<grid, 256, 0, st>>>(dxq, x, ldx, s_x, inv_x, qmax, rows, k, gprod, ldg, assign, d_ix);
+    launch_pdl(input_backward_kernel<false>, dim3(grid), dim3(256), 0, st, dxq, x, ldx, s_x, inv_x, qmax, rows, k, gprod, ldg, assign, d_ix);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "input backward launch");
 }
@@ -397,13 +405,13 @@ int launch_weight_alpha(Ctx* ctx, const float* dwq, int parts, const float* w, c
   using Kern = void (*)(const float*, const float*, const float*, const float*, float, float, int64_t, int64_t, double*);
   const Kern kern = parts == 1 ? (v4 ? weight_alpha_kernel<true, 1> : weight_alpha_kernel<false, 1>)
                                : (v4 ? weight_alpha_kernel<true, 3> : weight_alpha_kernel<false, 3>);
-  kern<<<(unsigned)n, 256, 0, st>>>(dwq, w, s_w, inv_w, s_x, qmax, n, k, d_iw);
+  launch_pdl(kern, dim3((unsigned)n), dim3(256), 0, st, dwq, w, s_w, inv_w, s_x, qmax, n, k, d_iw);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "weight scale gradient launch");
 }
 int launch_sgd(Ctx* ctx, float* s, const double* g, double lr, int64_t n, cudaStream_t st) {
   if (n == 0) return QCFG_OK;
-  sgd_kernel<<<blocks_for(n), 256, 0, st>>>(s, g, lr, n);
+  launch_pdl(sgd_kernel, dim3(blocks_for(n)), dim3(256), 0, st, s, g, lr, n);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "scale update launch");
 }

@@ -9,6 +9,7 @@ namespace qcfg {
 
 __global__ void __launch_bounds__(256) maxpool3s2_kernel(const float* __restrict__ src, int64_t B, int H, int W, int C,
                                                          int OH, int OW, float* __restrict__ dst, int vec) {
+  pdl_entry();
   const int cg = vec ? (C >> 2) : C;
   const int64_t total = B * OH * OW * cg;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -56,7 +57,7 @@ int launch_maxpool3s2(Ctx* ctx, const float* src, int64_t B, int H, int W, int C
   const int64_t total = B * OH * OW * (vec ? C / 4 : C);
   if (total == 0) return QCFG_OK;
   prof_begin(ctx, 2, st);
-  maxpool3s2_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(src, B, H, W, C, OH, OW, dst, vec);
+  launch_pdl(maxpool3s2_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, src, B, H, W, C, OH, OW, dst, vec);
   prof_end(ctx, 2, 0.0, st);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "maxpool launch");
@@ -67,6 +68,7 @@ int launch_maxpool3s2(Ctx* ctx, const float* src, int64_t B, int H, int W, int C
 // One thread per (image, channel): fp64 sum over the H*W positions, divided once.
 __global__ void __launch_bounds__(256) avgpool_kernel(const float* __restrict__ src, int64_t B, int HW, int C,
                                                       float* __restrict__ dst) {
+  pdl_entry();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= B * C) return;
   const int c = (int)(idx % C);
@@ -80,7 +82,7 @@ __global__ void __launch_bounds__(256) avgpool_kernel(const float* __restrict__ 
 int launch_avgpool(Ctx* ctx, const float* src, int64_t B, int HW, int C, float* dst, cudaStream_t st) {
   if (B * C == 0) return QCFG_OK;
   prof_begin(ctx, 2, st);
-  avgpool_kernel<<<(unsigned)((B * C + 255) / 256), 256, 0, st>>>(src, B, HW, C, dst);
+  launch_pdl(avgpool_kernel, dim3((unsigned)((B * C + 255) / 256)), dim3(256), 0, st, src, B, HW, C, dst);
   prof_end(ctx, 2, 0.0, st);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "avgpool launch");
@@ -128,6 +130,7 @@ __device__ __forceinline__ uint32_t conv_pack4(uint32_t a, uint32_t b, uint32_t 
 template <bool BF16>
 __global__ void __launch_bounds__(256) im2col_quantize_kernel(const float* __restrict__ src, ConvGeom g, float inv_scale,
                                                               float qmax, void* __restrict__ q, int64_t ldq, int vec) {
+  pdl_entry();
   const int boh = blockIdx.x;
   const int b = boh / g.OH, oh = boh - b * g.OH;
   const int ow = blockIdx.y * blockDim.y + threadIdx.y;
@@ -203,6 +206,7 @@ __global__ void __launch_bounds__(256) im2col_quantize_kernel(const float* __res
 template <bool BF16>
 __global__ void __launch_bounds__(256) im2col_rows_kernel(const float* __restrict__ src, ConvGeom g, float inv_scale, float qmax,
                                                           void* __restrict__ q, int64_t ldq) {
+  pdl_entry();
   extern __shared__ float srows[];                 // [kh][rowlen] then int koff[ldq]
   const int rowlen = (g.W + 2 * g.pad) * g.C;
   int* koff = reinterpret_cast<int*>(srows + g.kh * rowlen);
@@ -264,8 +268,8 @@ int launch_im2col_quantize(Ctx* ctx, const float* src, int64_t B, int H, int W, 
   const size_t rows_smem = ((size_t)kh * (W + 2 * pad) * C + (size_t)ldq) * 4;
   if (!vec && rows_smem <= 48 * 1024) {          // few channels: the row-staged kernel
     prof_begin(ctx, 2, st);
-    if (bits == 16) im2col_rows_kernel<true><<<(unsigned)(B * g.OH), 256, rows_smem, st>>>(src, g, 1.0f, 0.0f, q, ldq);
-    else im2col_rows_kernel<false><<<(unsigned)(B * g.OH), 256, rows_smem, st>>>(src, g, inv_scale, qmax_of(bits), q, ldq);
+    if (bits == 16) launch_pdl(im2col_rows_kernel<true>, dim3((unsigned)(B * g.OH)), dim3(256), rows_smem, st, src, g, 1.0f, 0.0f, q, ldq);
+    else launch_pdl(im2col_rows_kernel<false>, dim3((unsigned)(B * g.OH)), dim3(256), rows_smem, st, src, g, inv_scale, qmax_of(bits), q, ldq);
     prof_end(ctx, 2, 0.0, st);
     count_launch(ctx);
     return check_cuda(ctx, cudaGetLastError(), "im2col launch");
@@ -277,8 +281,8 @@ int launch_im2col_quantize(Ctx* ctx, const float* src, int64_t B, int H, int W, 
   const dim3 grid((unsigned)(B * g.OH), (unsigned)((g.OW + by - 1) / by));
   if (grid.y > 65535) return set_error(ctx, QCFG_ESHAPE, "im2col: output row too wide");
   prof_begin(ctx, 2, st);
-  if (bits == 16) im2col_quantize_kernel<true><<<grid, block, 0, st>>>(src, g, 1.0f, 0.0f, q, ldq, vec);
-  else im2col_quantize_kernel<false><<<grid, block, 0, st>>>(src, g, inv_scale, qmax_of(bits), q, ldq, vec);
+  if (bits == 16) launch_pdl(im2col_quantize_kernel<true>, dim3(grid), dim3(block), 0, st, src, g, 1.0f, 0.0f, q, ldq, vec);
+  else launch_pdl(im2col_quantize_kernel<false>, dim3(grid), dim3(block), 0, st, src, g, inv_scale, qmax_of(bits), q, ldq, vec);
   prof_end(ctx, 2, 0.0, st);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "im2col launch");
@@ -290,6 +294,7 @@ int launch_im2col_quantize(Ctx* ctx, const float* src, int64_t B, int H, int W, 
 __global__ void __launch_bounds__(256) im2col_codes_kernel(const int8_t* __restrict__ src, int64_t rows, int H, int W, int C, int kh,
                                                            int kw, int stride, int pad, int OH, int OW, int8_t* __restrict__ dst,
                                                            int64_t ldd) {
+  pdl_entry();
   const int cpr = kh * kw * C / 16;                 // 16-code chunks per output row
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= rows * cpr) return;
@@ -315,7 +320,7 @@ int launch_im2col_codes(Ctx* ctx, const int8_t* src, int64_t B, int H, int W, in
   const int OH = (H + 2 * pad - kh) / stride + 1, OW = (W + 2 * pad - kw) / stride + 1;
   const int64_t rows = B * OH * OW, total = rows * (kh * kw * C / 16);
   if (total == 0) return QCFG_OK;
-  im2col_codes_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(src, rows, H, W, C, kh, kw, stride, pad, OH, OW, dst, ldd);
+  launch_pdl(im2col_codes_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, src, rows, H, W, C, kh, kw, stride, pad, OH, OW, dst, ldd);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "code patch launch");
 }

@@ -18,6 +18,7 @@ __device__ __forceinline__ unsigned max4(float4 v) {
 __global__ void __launch_bounds__(256) absmax_tensor_kernel(const float* __restrict__ x, int64_t rows,
                                                             int64_t cols, int64_t ld, int vec,
                                                             unsigned* __restrict__ out) {
+  pdl_entry();
   unsigned m = 0;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t nth = (int64_t)gridDim.x * blockDim.x;
@@ -60,6 +61,7 @@ __global__ void __launch_bounds__(256) absmax_tensor_kernel(const float* __restr
 __global__ void __launch_bounds__(256) absmax_rows_kernel(const float* __restrict__ x, int64_t rows,
                                                           int64_t cols, int64_t ld, int vec,
                                                           float* __restrict__ out) {
+  pdl_entry();
   const int lane = threadIdx.x & 31;
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (row >= rows) return;
@@ -98,14 +100,14 @@ int launch_absmax(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_t 
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     prof_begin(ctx, 2, st);
-    absmax_tensor_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, rows, cols, ld, vec,
+    launch_pdl(absmax_tensor_kernel, dim3((unsigned)blocks), dim3(256), 0, st, x, rows, cols, ld, vec,
                                                             reinterpret_cast<unsigned*>(absmax));
     prof_end(ctx, 2, 0.0, st);
   } else {
     if (rows == 0) return QCFG_OK;
     int64_t blocks = (rows + 7) / 8;
     prof_begin(ctx, 2, st);
-    absmax_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(x, rows, cols, ld, vec, absmax);
+    launch_pdl(absmax_rows_kernel, dim3((unsigned)blocks), dim3(256), 0, st, x, rows, cols, ld, vec, absmax);
     prof_end(ctx, 2, 0.0, st);
   }
   count_launch(ctx);
@@ -116,6 +118,7 @@ int launch_absmax(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_t 
 
 __global__ void scales_kernel(const float* __restrict__ absmax, int64_t n, float qmax,
                               float* __restrict__ scale, float* __restrict__ inv_scale) {
+  pdl_entry();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   float A = absmax[i];
@@ -132,7 +135,7 @@ int launch_scales(Ctx* ctx, const float* absmax, int64_t n, int bits, float* sca
                   cudaStream_t st) {
   if (n == 0) return QCFG_OK;
   prof_begin(ctx, 2, st);
-  scales_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(absmax, n, qmax_of(bits), scale, inv_scale);
+  launch_pdl(scales_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, absmax, n, qmax_of(bits), scale, inv_scale);
   prof_end(ctx, 2, 0.0, st);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "scales launch");
@@ -157,6 +160,7 @@ __global__ void __launch_bounds__(256) quantize_kernel(const float* __restrict__
                                                        float inv_scale_val, int per_row, float qmax,
                                                        void* __restrict__ q, int64_t ldq, int vec,
                                                        unsigned* __restrict__ amax) {
+  pdl_entry();
   const int64_t gpr = ldq >> 3;  // groups of 8 per output row
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   unsigned m = 0;
@@ -228,12 +232,12 @@ int launch_quantize(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_
   const unsigned blocks = (unsigned)((total + 255) / 256);
   if (bits == 16) {
     prof_begin(ctx, 2, st);
-    quantize_kernel<true><<<blocks, 256, 0, st>>>(x, rows, cols, ld, nullptr, 1.0f, 0, 0.0f, q, ldq, vec,
+    launch_pdl(quantize_kernel<true>, dim3(blocks), dim3(256), 0, st, x, rows, cols, ld, nullptr, 1.0f, 0, 0.0f, q, ldq, vec,
                                                   reinterpret_cast<unsigned*>(absmax));
     prof_end(ctx, 2, 0.0, st);
   } else {
     prof_begin(ctx, 2, st);
-    quantize_kernel<false><<<blocks, 256, 0, st>>>(x, rows, cols, ld, inv_scale_ptr, inv_scale_val,
+    launch_pdl(quantize_kernel<false>, dim3(blocks), dim3(256), 0, st, x, rows, cols, ld, inv_scale_ptr, inv_scale_val,
                                                    granularity == QCFG_PER_ROW, qmax_of(bits), q, ldq, vec, nullptr);
     prof_end(ctx, 2, 0.0, st);
   }
@@ -250,6 +254,7 @@ int launch_quantize(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_
 __global__ void __launch_bounds__(256) perturb_bf16_kernel(const float* __restrict__ w, const float* __restrict__ nu,
                                                            const float* __restrict__ amax, float lambda, int64_t rows,
                                                            int64_t cols, __nv_bfloat16* __restrict__ q, int64_t ldq) {
+  pdl_entry();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= rows * ldq) return;
   const int64_t r = idx / ldq, c = idx - r * ldq;
@@ -266,7 +271,7 @@ int launch_perturb_bf16(Ctx* ctx, const float* w, const float* nu, const float* 
   const int64_t total = rows * ldq;
   if (total == 0) return QCFG_OK;
   prof_begin(ctx, 2, st);
-  perturb_bf16_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(w, nu, amax_dev, lambda, rows, cols,
+  launch_pdl(perturb_bf16_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, w, nu, amax_dev, lambda, rows, cols,
                                                                       reinterpret_cast<__nv_bfloat16*>(q), ldq);
   prof_end(ctx, 2, 0.0, st);
   count_launch(ctx);
@@ -278,6 +283,7 @@ int launch_perturb_bf16(Ctx* ctx, const float* w, const float* nu, const float* 
 // Per-block partial sums of (y - ref)^2 and ref^2 in fp64 (fixed grid, fixed order: deterministic).
 __global__ void __launch_bounds__(256) sqdiff_kernel(const float* __restrict__ y, const float* __restrict__ ref,
                                                      int64_t n, double* __restrict__ partial) {
+  pdl_entry();
   double d2 = 0.0, r2 = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const double r = (double)__ldg(ref + i), d = (double)__ldg(y + i) - r;
@@ -298,7 +304,7 @@ __global__ void __launch_bounds__(256) sqdiff_kernel(const float* __restrict__ y
 
 int launch_sqdiff(Ctx* ctx, const float* y, const float* ref, int64_t n, double* partial, int blocks, cudaStream_t st) {
   prof_begin(ctx, 2, st);
-  sqdiff_kernel<<<blocks, 256, 0, st>>>(y, ref, n, partial);
+  launch_pdl(sqdiff_kernel, dim3(blocks), dim3(256), 0, st, y, ref, n, partial);
   prof_end(ctx, 2, 0.0, st);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "fidelity launch");
