@@ -1789,7 +1789,17 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   p.bn = bn;
   // pair flavour (two CTAs per 256-row tile, cta_group::2) for wide outputs with at least two
   // row tiles: it halves the B bytes each SM stages per k-block
-  const bool pair = ctx_pair_enabled(ctx) && bn == 256 && g0.m > BM && sm_count(ctx) >= 2;
+  bool pair = ctx_pair_enabled(ctx) && bn == 256 && g0.m > BM && sm_count(ctx) >= 2;
+  // ... and for wide outputs whose tiles were narrowed to 128 columns, while the pairs still have one tile each: a
+  // stage is 24 KB instead of 32 and the ring one or two stages deeper (noise table of the block above:
+  // 360 -> 345 us; its evaluation 66.5 -> 66.2).  A lone int8 code matrix stays with one CTA per tile, where its own body
+  // is.  Four SMs are left out of the count: some may have no partner.
+  if (ctx_pair_enabled(ctx) && bn == 128 && tile_n_of(g0.n) == 256 && !shortcut && g0.conv_kh == 0 && g0.m > BM) {
+    int64_t cols = 0;
+    for (int i = 0; i < count; ++i) cols += (gs[i].n + bn - 1) / bn;
+    const bool codes = count == 1 && !g0.residual && !g0.amax && !g0.acc && !g0.y && g0.slots[0].kind == 1 && !g0.slots[1].kind && !g0.slots[2].kind;
+    pair = !codes && 2 * cols * ((g0.m + 2 * BM - 1) / (2 * BM)) <= sm_count(ctx) - 4;
+  }
   const int tile_rows = pair ? 2 * BM : BM;
   p.tiles_m = (int32_t)((g0.m + tile_rows - 1) / tile_rows);
   const int stage_bytes = (BM + (pair ? bn / 2 : bn)) * kStageKBytes;
@@ -1835,7 +1845,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
     // staging per epilogue warp: two slots of 1 KB when only int8 codes are written, else of 2 KB
     for (int j = 0; j < kNumOuts; ++j) if (G.outs[j].kind >= 3 || (G.outs[j].kind == 2 && G.outs[j].tma)) wide = true;
     G.mode = EPI_GENERAL;
-    if (bn < 256 && count == 1 && !G.residual && !G.amax && !G.outs[0].kind && !G.outs[1].kind && G.outs[2].kind == 1 && G.outs[2].tma &&
+    if (bn < 256 && !pair && count == 1 && !G.residual && !G.amax && !G.outs[0].kind && !G.outs[1].kind && G.outs[2].kind == 1 && G.outs[2].tma &&
         !G.outs[3].kind && !G.outs[4].kind)
       G.mode = EPI_CODES32;
     if (bn == 256 && !G.residual && !G.outs[0].kind && !G.outs[1].kind && G.outs[2].kind == 2 && !G.outs[3].kind && !G.outs[4].kind &&

@@ -231,6 +231,33 @@ def test_gemm_pair_and_single_cta_tiles_agree(ctx, m, n, k):
     assert torch.equal(res[0][0].view(torch.int32), res[1][0].view(torch.int32))
 
 
+@pytest.mark.parametrize("m,n,k", [(3072, 768, 144), (2945, 641, 48), (257, 4600, 80), (129, 9000, 16), (3072, 768, 1552)])
+def test_gemm_pairs_on_narrowed_tiles_match_the_reference(ctx, m, n, k):
+    """Wide outputs whose tiles were narrowed to 128 columns run on pairs while each has one tile: integer sums
+    are exact, and the 16-bit products give the same bits as one CTA per tile."""
+    import paper_2302_01382_b200 as q
+    rng = np.random.default_rng(m * 3 + n)
+    ld = (k + 15) // 16 * 16
+    qx, qw = _codes(rng, m, k, ld), _codes(rng, n, k, ld)
+    sw = (10.0 ** rng.uniform(-4, -2, n)).astype(np.float32)
+    y, acc = ctx.gemm_i8(dev(qx), dev(qw), k, 0.0173, dev(sw), q.ACT_NONE, want_y=True, want_acc=True)
+    ctx.check_sync()
+    ref = orc.int_gemm(qx[:, :k], qw[:, :k])
+    np.testing.assert_array_equal(host(acc), ref)
+    np.testing.assert_array_equal(host(y).view(np.uint32), orc.dequant_output(ref, np.float32(0.0173), sw).view(np.uint32))
+    xq = ctx.quantize(dev(rng.standard_normal((m, k)).astype(np.float32)), None, q.PER_TENSOR, 16)
+    wq = ctx.quantize(dev(rng.standard_normal((n, k)).astype(np.float32)), None, q.PER_TENSOR, 16)
+    res = []
+    for pair in (True, False):
+        ctx.set_pair_tiles(pair)
+        try:
+            res.append(ctx.gemm_bf16(xq, wq, k))
+            ctx.check_sync()
+        finally:
+            ctx.set_pair_tiles(True)
+    assert torch.equal(res[0].view(torch.int32), res[1].view(torch.int32))
+
+
 @pytest.mark.parametrize("m,n,k", [(1, 33, 16), (31, 1, 48), (257, 259, 64), (128, 255, 144), (300, 1025, 32), (33, 65, 4608)])
 def test_gemm_row_pitch_without_16_byte_alignment(ctx, m, n, k):
     """fp32 and raw outputs whose rows TMA cannot write, at the edges of a 32 x 32 piece: bit-exact, and
