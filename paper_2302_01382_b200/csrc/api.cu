@@ -391,14 +391,34 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
       if (!codes_kept && !(P.y_ptr && P.y_internal)) dirty[d.src] = 1;
     }
   }
+  auto codes_kept = [&](int l) {                     // a recomputed layer whose operand is still in its own buffer
+    const LayerState& S = M->L[l];
+    return reuse && S.bits == bits[l] && S.a_ready && S.a_ptr && S.a_ptr == S.abuf.p && (S.d.src < 0 || !dirty[S.d.src]);
+  };
+  // A skipped layer may read its codes out of the buffer of a layer that is about to put others there (layers on one
+  // input, of which one changes its width).  It takes that buffer over, with the codes in it, so that they stay what the
+  // layer ran with: qcfg_debug_dump reads them after the evaluation.
+  if (reuse) {
+    std::vector<int> guests;
+    for (int j = 0; j < n; ++j)
+      if (!dirty[j] && M->L[j].a_ptr && M->L[j].a_ptr != M->L[j].abuf.p) guests.push_back(j);
+    for (int l = 0; l < n && !guests.empty(); ++l) {
+      if (!dirty[l] || codes_kept(l)) continue;
+      for (size_t g = 0; g < guests.size();) {       // again from the front: the buffer it gets in return may have a guest too
+        LayerState& G = M->L[guests[g]];
+        if (G.a_ptr != M->L[l].abuf.p) { ++g; continue; }
+        std::swap(G.abuf, M->L[l].abuf);
+        guests.erase(guests.begin() + (ptrdiff_t)g);
+        g = 0;
+      }
+    }
+  }
   for (int l = 0; l < n; ++l) {
     LayerState& S = M->L[l];
     S.rows = layer_rows(M, l, m);
     if (!dirty[l]) continue;                         // buffers and pointers stay as they are
     S.implicit = ctx->implicit && !calibrate && implicit_capable(S.d);
-    const bool codes_kept = reuse && S.bits == bits[l] && S.a_ready && S.a_ptr && S.a_ptr == S.abuf.p &&
-                            (S.d.src < 0 || !dirty[S.d.src]);
-    if (!codes_kept) { S.a_ready = false; S.a_ptr = nullptr; }
+    if (!codes_kept(l)) { S.a_ready = false; S.a_ptr = nullptr; }
     S.y_ptr = nullptr; S.pre_ptr = nullptr; S.y_internal = false;
     S.bits = calibrate ? 16 : bits[l];
   }

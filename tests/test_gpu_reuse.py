@@ -80,3 +80,72 @@ def test_reuse_is_bit_identical_on_search_sequences(kind):
         model.close()
     finally:
         ctx.close()
+
+
+def _taps(model, w, bits):
+    """Operand codes and accumulators of every integer layer after the last evaluation."""
+    out = []
+    for l, layer in enumerate(w.layers):
+        if bits[l] == 16:
+            out.append(None)
+            continue
+        rows = wl.layer_rows(w.layers, l, w.m)
+        qx = torch.empty((rows, layer.k_in), dtype=torch.int8, device="cuda")
+        acc = torch.empty((rows, layer.n_out), dtype=torch.int32, device="cuda")
+        model.debug_dump(l, qx, None, acc)
+        out.append((qx, acc))
+    return out
+
+
+@pytest.mark.parametrize("kind", ["fan", "bert", "bert_wide_qkv", "resnet"])
+def test_taps_after_partial_forwards(kind):
+    """debug_dump reads what every layer ran with, also where the last evaluation skipped the layer and layers
+    that shared its codes have changed their width since: under prefix reuse and after a search."""
+    import paper_2302_01382_b200 as q
+    rng = np.random.default_rng(12)
+    if kind == "fan":            # layers on one input, which share one operand at equal widths
+        w = wl.bert_stack(24, 300, 128, 512, 1, bit_choices=None)
+    elif kind == "bert":
+        w = wl.bert_stack(21, 200, 128, 512, 3, bit_choices=None)
+    elif kind == "bert_wide_qkv":
+        w = wl.bert_stack_wide_qkv(22, 200, 128, 512, 2)
+    else:
+        w = wl.resnet50(seed=23, batch=2, in_hw=64, width=16, n_classes=24, blocks=(2, 1, 1, 1))
+    n = len(w.layers)
+    ctx, full = q.Context(0), q.Context(0)
+    try:
+        weights = [torch.from_numpy(a).cuda() for a in w.weights]
+        x = torch.from_numpy(w.x).cuda()
+        model, plain = q.Model(ctx, w.layers, weights), q.Model(full, w.layers, weights)
+        for mod in (model, plain):
+            mod.calibrate_model(x, w.m)
+        y = torch.empty((wl.layer_rows(w.layers, n - 1, w.m), w.layers[-1].n_out), device="cuda")
+        ys = [None] * (n - 1) + [y]
+
+        def same_taps(bits, what):
+            plain.eval_config(bits, x, w.m, ys)
+            for l, (got, want) in enumerate(zip(_taps(model, w, bits), _taps(plain, w, bits))):
+                if want is not None:
+                    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1]), f"{kind}, {what}: tap of layer {l}"
+
+        if kind == "fan":
+            seq = [[8] * n, [4] + [8] * (n - 1), [4, 4] + [8] * (n - 2), [8, 4] + [8] * (n - 2), [16, 4, 2] + [8] * (n - 3), [8] * n]
+        else:
+            seq = [list(map(int, b)) for b in _sequences(n, rng)[::4]]
+        ctx.set_prefix_reuse(True)
+        for i, bits in enumerate(seq):
+            model.eval_config(bits, x, w.m, ys)
+            same_taps(bits, f"configuration {i}")
+        ctx.set_prefix_reuse(False)
+        for algorithm in (0, 1):
+            order = [int(i) for i in rng.permutation(n)]
+            _, visited, _, n_evals = model.search(algorithm, order, [8, 4], 0.9, x, w.m)
+            assert n_evals > 0
+            same_taps(list(visited[-1]), f"search {algorithm}")
+        ctx.check_sync()
+        full.check_sync()
+        model.close()
+        plain.close()
+    finally:
+        ctx.close()
+        full.close()
