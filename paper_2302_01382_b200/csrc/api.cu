@@ -1607,6 +1607,7 @@ int adjust_reference(qcfg_ctx* h, Model* M, const float* x_dev, int64_t m, cudaS
   std::vector<float*> ys((size_t)n, nullptr);
   int rc = M->search_ref.ensure(c, (size_t)(m * M->L[n - 1].d.n_out) * 4);
   ys[n - 1] = (float*)M->search_ref.p;
+  M->reuse_valid = false;      // the input may have other contents than at the last evaluation: every layer runs
   if (!rc) rc = forward(c, M, b16.data(), x_dev, ext_ld_of(M), m, ys.data(), false, st);
   return rc;
 }

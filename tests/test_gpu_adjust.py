@@ -137,6 +137,37 @@ def test_gradients_update_and_evaluation_match_the_oracle(kind):
         ctx.close()
 
 
+def test_gradients_see_the_input_as_it_is():
+    """The reference of the loss is computed from the input of the call, not from what an evaluation under
+    prefix reuse left for the same buffer."""
+    import paper_2302_01382_b200 as q
+    w = wl.tiny_mlp()
+    bits = [8, 4, 8]
+    ctx = q.Context(0)
+    try:
+        weights = [torch.from_numpy(a).cuda() for a in w.weights]
+        x, other = torch.from_numpy(w.x).cuda(), torch.from_numpy(-0.5 * w.x[::-1].copy()).cuda()
+        model = q.Model(ctx, w.layers, weights)
+        model.calibrate_model(x, w.m)
+        y = torch.empty((w.m, w.layers[-1].n_out), device="cuda")
+        want = model.scale_gradients(bits, other, w.m)
+        ctx.set_prefix_reuse(True)
+        for losses in (False, True):
+            x.copy_(torch.from_numpy(w.x).cuda())
+            model.eval_config([16] * len(bits), x, w.m, [None] * (len(bits) - 1) + [y])
+            x.copy_(other)
+            if losses:
+                assert model.adjust_scales(bits, x, w.m, steps=0)[0] == pytest.approx(want[0], rel=1e-12)
+            else:
+                got = model.scale_gradients(bits, x, w.m)
+                assert got[0] == pytest.approx(want[0], rel=1e-12)
+                assert _close(got[1], want[1], tol=1e-9) and _close(got[2], want[2], tol=1e-9)
+        ctx.check_sync()
+        model.close()
+    finally:
+        ctx.close()
+
+
 def test_adjust_argument_errors():
     import paper_2302_01382_b200 as q
     ctx = q.Context(0)
