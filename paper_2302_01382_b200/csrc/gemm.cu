@@ -852,7 +852,8 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   if (warp == 0) set_tile_coords();
   const bool elected = elect_one();    // the lane of a converged warp that issues TMA / MMA instructions
   const bool conv_on = kConv && p.conv.on == CONV_GATHER;
-  // one 128-row column of patches per call; chunks behind the last tap repeat the first one (the B tile is zero there)
+  // one 128-row column of patches per call; chunks behind the last tap come from behind the last channel, which reads as
+  // zeros (the B tile is zero there too, but zero times an infinity would not be)
   auto load_patches = [&]() {
     const int chunk = (p.conv.on == CONV_TMA64 ? 64 : 128) / (BF16 ? 2 : 1);
     const int loads = p.conv.on == CONV_TMA64 ? 2 : 1;
@@ -860,8 +861,8 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
       const bool past = cv_dy == p.conv.kh;
       if (elected) {
         const uint32_t dst = ld_dst + h * (BM * 64);
-        if (PAIR) tma_load_im2col_pair(dst, ld_map_a, ld_bar, past ? 0 : cv_c, cv_w, cv_h, cv_n, past ? 0 : cv_dx, past ? 0 : cv_dy);
-        else tma_load_im2col(dst, ld_map_a, ld_bar, past ? 0 : cv_c, cv_w, cv_h, cv_n, past ? 0 : cv_dx, past ? 0 : cv_dy);
+        if (PAIR) tma_load_im2col_pair(dst, ld_map_a, ld_bar, past ? p.conv.C : cv_c, cv_w, cv_h, cv_n, past ? 0 : cv_dx, past ? 0 : cv_dy);
+        else tma_load_im2col(dst, ld_map_a, ld_bar, past ? p.conv.C : cv_c, cv_w, cv_h, cv_n, past ? 0 : cv_dx, past ? 0 : cv_dy);
       }
       if (!past) {
         cv_c += chunk;

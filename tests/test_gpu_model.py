@@ -398,6 +398,39 @@ def test_convolution_operand_through_tma_matches_the_patch_matrix(ctx, c, n, hw,
     model.close()
 
 
+@pytest.mark.parametrize("c,k,hw", [(32, 3, 9), (32, 5, 11), (64, 3, 10), (48, 3, 9)])
+def test_non_finite_convolution_inputs_reach_only_their_windows(ctx, c, k, hw):
+    """16-bit convolutions of an input with infinities and NaN, gathered and from a patch matrix: the same outputs, where
+    an odd number of 64-byte chunks leaves half a k-block empty (32 channels) and where it does not."""
+    L = wl.Layer
+    pad, batch = k // 2, 3
+    geo = dict(kh=k, kw=k, stride=1, pad=pad, in_h=hw, in_w=hw, src_h=hw, src_w=hw)
+    layers = [L("in", c, 16, src=-1, kh=1, kw=1, stride=1, in_h=hw, in_w=hw, in_c=16, src_h=hw, src_w=hw),
+              L("conv", 48, k * k * c, src=0, in_c=c, **geo)]
+    rng = np.random.default_rng(c + k)
+    x = rng.standard_normal((batch, hw, hw, 16)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    ws[0][:] = 0.0
+    ws[0][:, 0] = 1.0                                     # every channel is the input's first one
+    ws[1] = np.abs(ws[1])                                 # an infinity in a window stays one
+    w = wl.Workload("conv", 1, layers, batch, x, ws)
+    model, xd = build(ctx, w)
+    check_calibration(model, w)
+    xd[0, 0, 0, 0], xd[1, hw // 2, 3, 0], xd[2, hw - 1, hw - 1, 0] = float("inf"), float("nan"), float("-inf")
+    outs = []
+    for implicit in (True, False):
+        ctx.set_implicit_conv(implicit)
+        outs.append(host(run_eval(ctx, model, w, xd, [16, 16])[1]).reshape(batch, hw, hw, 48))
+    ctx.set_implicit_conv(True)
+    np.testing.assert_array_equal(outs[0], outs[1])
+    assert np.isinf(outs[0]).any()
+    oy, ox = np.mgrid[:hw, :hw]
+    for b, y, z in ((0, 0, 0), (1, hw // 2, 3), (2, hw - 1, hw - 1)):
+        touched = (abs(oy - y) <= pad) & (abs(ox - z) <= pad)
+        assert np.isfinite(outs[0][b][~touched]).all() and not np.isfinite(outs[0][b][touched]).any()
+    model.close()
+
+
 @pytest.mark.parametrize("c,n,h,wd,k,pad,batch,act", [(3, 64, 32, 32, 7, 3, 3, 1), (3, 32, 33, 47, 7, 3, 2, 1), (1, 16, 20, 9, 5, 2, 40, 0),
                                                       (4, 48, 17, 255, 3, 1, 2, 1), (2, 64, 7, 8, 7, 0, 5, 0), (3, 64, 65, 224, 7, 3, 4, 1),
                                                       (3, 16, 16, 64, 8, 3, 2, 1), (3, 64, 16, 260, 7, 3, 1, 1), (5, 64, 16, 16, 3, 1, 2, 1)])
