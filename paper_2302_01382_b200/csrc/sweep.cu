@@ -111,10 +111,18 @@ __device__ __forceinline__ void finalize_tensor(const double* __restrict__ parti
   __syncthreads();
 }
 
+// What the bodies below keep in shared memory besides the ring, declared once by the kernel: with arrays of their own
+// the nine bodies of a mixed plan took 5 KB, and where the ring is 72 KB only two of the three blocks per SM that the
+// plan counts on were resident (four blocks of hidden size 701: 67 us, 59 this way).
+struct SweepShared {
+  float smax2[2][kThreads / 32];
+  double swarp[kThreads / 32][8];             // per warp: 7 fp64 sums and the maximum
+};
+
 // One run of rows of up to 4*V*team elements.  All 7 bit widths are always evaluated (a narrower
 // request only selects columns at the end).
 template <int V, bool ALL_VEC>
-__device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor, float A_tensor, float4* ring,
+__device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor, float A_tensor, float4* ring, SweepShared& sh,
                                               double* __restrict__ out) {
   // rows between two first-stage flushes: every row adds 2*V terms to each half of a packed accumulator
   constexpr int kFlushRows = (kChainTerms / (2 * V)) > 0 ? (kChainTerms / (2 * V)) : 1;
@@ -126,8 +134,7 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
   const int n_iter = (d.rows + nteams - 1) / nteams;
   const int c4 = d.cols >> 2;
   int row_parity = 0;
-  __shared__ float smax2[2][kThreads / 32];
-  __shared__ double swarp[kThreads / 32][8];             // per warp: 7 fp64 sums and the maximum
+  double (*swarp)[8] = sh.swarp;
 
   float2 facc[kNB];
   float f2[kNB];
@@ -146,7 +153,7 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
     if (T > 32) {
       // the team's warps exchange their maxima through shared memory; a named barrier per team
       // keeps other teams running, and alternating slots make one barrier per row enough
-      float* slot = smax2[row_parity];
+      float* slot = sh.smax2[row_parity];
       if (lane == 0) slot[warp] = m;
       asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(T) : "memory");
       const int w0 = team * (T >> 5);
@@ -262,11 +269,11 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
 
 // Rows longer than the ring holds: the whole block works on one row at a time and reads it twice
 // (the second read hits L1/L2).
-__device__ __forceinline__ void sweep_segment_long(const SweepSeg& d, int per_tensor, float A_tensor, int jlo, int jhi,
+__device__ __forceinline__ void sweep_segment_long(const SweepSeg& d, int per_tensor, float A_tensor, int jlo, int jhi, SweepShared& sh,
                                                    double* __restrict__ out) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ float smax[kThreads / 32];
-  __shared__ double swarp[kThreads / 32][8];
+  float* smax = sh.smax2[0];
+  double (*swarp)[8] = sh.swarp;
   double dacc[kNB];
 #pragma unroll
   for (int j = 0; j < kNB; ++j) dacc[j] = 0.0;
@@ -343,23 +350,24 @@ sweep_kernel(const SweepSeg* __restrict__ segs, const SweepBlock* __restrict__ b
   asm volatile("griddepcontrol.wait;" ::: "memory");
   __shared__ double fin[32][8];
   __shared__ int last;
+  __shared__ SweepShared sh;
   extern __shared__ float4 ring[];                       // [kRing][V][kThreads]
   const SweepBlock blk = blocks[blockIdx.x];
   for (int si = blk.seg0; si < blk.seg0 + blk.nseg; ++si) {
     const SweepSeg d = segs[si];
     const float A_tensor = per_tensor ? tensor_absmax[d.tensor] : 0.0f;
     double* out = partial + (int64_t)d.slot * 8;
-    if (KV > 0) sweep_segment<(KV > 0 ? KV : 1), true>(d, per_tensor, A_tensor, ring, out);
+    if (KV > 0) sweep_segment<(KV > 0 ? KV : 1), true>(d, per_tensor, A_tensor, ring, sh, out);
     else switch (d.v) {
-      case 0: sweep_segment_long(d, per_tensor, A_tensor, jlo, jlo + nb - 1, out); break;
-      case 1: sweep_segment<1, false>(d, per_tensor, A_tensor, ring, out); break;
-      case 2: sweep_segment<2, false>(d, per_tensor, A_tensor, ring, out); break;
-      case 3: sweep_segment<3, false>(d, per_tensor, A_tensor, ring, out); break;
-      case 4: sweep_segment<4, false>(d, per_tensor, A_tensor, ring, out); break;
-      case 5: sweep_segment<5, false>(d, per_tensor, A_tensor, ring, out); break;
-      case 6: sweep_segment<6, false>(d, per_tensor, A_tensor, ring, out); break;
-      case 7: sweep_segment<7, false>(d, per_tensor, A_tensor, ring, out); break;
-      default: sweep_segment<8, false>(d, per_tensor, A_tensor, ring, out); break;
+      case 0: sweep_segment_long(d, per_tensor, A_tensor, jlo, jlo + nb - 1, sh, out); break;
+      case 1: sweep_segment<1, false>(d, per_tensor, A_tensor, ring, sh, out); break;
+      case 2: sweep_segment<2, false>(d, per_tensor, A_tensor, ring, sh, out); break;
+      case 3: sweep_segment<3, false>(d, per_tensor, A_tensor, ring, sh, out); break;
+      case 4: sweep_segment<4, false>(d, per_tensor, A_tensor, ring, sh, out); break;
+      case 5: sweep_segment<5, false>(d, per_tensor, A_tensor, ring, sh, out); break;
+      case 6: sweep_segment<6, false>(d, per_tensor, A_tensor, ring, sh, out); break;
+      case 7: sweep_segment<7, false>(d, per_tensor, A_tensor, ring, sh, out); break;
+      default: sweep_segment<8, false>(d, per_tensor, A_tensor, ring, sh, out); break;
     }
     if (!FUSED) { __syncthreads(); continue; }
     // The eight values of the slot become visible before the segment is counted; the counter wraps

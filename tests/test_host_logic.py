@@ -74,3 +74,21 @@ def test_reference_arm_other_ranks_do_no_work():
     out = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--impl", "reference", "--steps", "1"],
                          env=env, capture_output=True, text=True, timeout=120)
     assert out.returncode == 0 and out.stdout.strip() == ""
+
+
+def test_sweep_blocks_a_plan_counts_on_fit_an_sm():
+    """Plans cut the work for three resident blocks per SM with up to six float4 per thread and row: their static
+    shared memory (as the toolkit lists it, the kilobyte the system keeps per block included), the ring of three
+    stages and the registers have to leave room for them."""
+    cuobjdump = "/usr/local/cuda/bin/cuobjdump"
+    lib = os.path.join(ROOT, "paper_2302_01382_b200", "libqcfg.so")
+    if not (os.path.exists(cuobjdump) and os.path.exists(lib)):
+        pytest.skip("needs the CUDA toolkit and the built library")
+    out = subprocess.run([cuobjdump, "--dump-resource-usage", lib], capture_output=True, text=True, check=True).stdout
+    found = re.findall(r"sweep_kernelILi(\d)ELb([01])E\S*:\s*REG:(\d+) STACK:\d+ SHARED:(\d+)", out)
+    assert len(found) == 10                                # eight row lengths, mixed, mixed with its own finish
+    for v, fused, regs, shared in ((int(a), int(b), int(c), int(d)) for a, b, c, d in found):
+        if v <= 6 and not fused:
+            ring = 3 * (v or 6) * 256 * 16
+            assert 3 * (shared + ring) <= 228 * 1024, (v, shared)
+            assert 3 * 256 * regs <= 65536, (v, regs)
