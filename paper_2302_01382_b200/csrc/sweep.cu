@@ -26,8 +26,12 @@
 // which takes at most kChainSums such sums; that one is reduced over the warp in fp64 and added to the
 // warp's sum in shared memory.  A sequential fp32 sum of n non-negative terms is within (n-1)*2^-24
 // relative of the exact sum, so the two stages together stay within (23 + 1 + 15) * 2^-24 = 2.3e-6,
-// inside the sweep's 1e-5 tolerance; no thread keeps fp64 accumulators in registers.
+// inside the sweep's 1e-5 tolerance; no thread of these rows keeps fp64 accumulators in registers.
+// Rows that are not whole aligned float4 go from the first stage to fp64, after one squared error below 512 columns and
+// one per 256 columns beyond (64 x 147: mean error 4.5e-10 of the sum; through both fp32 stages 1.7e-9.  Four blocks of
+// hidden size 701: 69.7 us against 59.3).
 #include <cstring>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -119,9 +123,9 @@ struct SweepShared {
   double swarp[kThreads / 32][8];             // per warp: 7 fp64 sums and the maximum
 };
 
-// One run of rows of up to 4*V*team elements.  All 7 bit widths are always evaluated (a narrower
-// request only selects columns at the end).
-template <int V, bool ALL_VEC>
+// One run of rows of up to 4*V*team elements, VEC: whole aligned float4, otherwise copied word by word.
+// All 7 bit widths are always evaluated (a narrower request only selects columns at the end).
+template <int V, bool VEC>
 __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor, float A_tensor, float4* ring, SweepShared& sh,
                                               double* __restrict__ out) {
   // rows between two first-stage flushes: every row adds 2*V terms to each half of a packed accumulator
@@ -137,9 +141,12 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
   double (*swarp)[8] = sh.swarp;
 
   float2 facc[kNB];
-  float f2[kNB];
+  float f2[kNB];                              // VEC: the second fp32 stage
+  double dacc[kNB];                           // otherwise: fp64 behind a first stage of `chain` terms
 #pragma unroll
-  for (int j = 0; j < kNB; ++j) { facc[j] = make_float2(0.0f, 0.0f); f2[j] = 0.0f; }
+  for (int j = 0; j < kNB; ++j) { facc[j] = make_float2(0.0f, 0.0f); f2[j] = 0.0f; dacc[j] = 0.0; }
+  const int chain = d.cols < 2 * kThreads ? 1 : d.cols / kThreads < kChainTerms ? d.cols / kThreads : kChainTerms;
+  int terms = 0;
   if (lane < 8) swarp[warp][lane] = 0.0;
   float amax_blk = 0.0f;
 
@@ -174,21 +181,36 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
       ns[j] = make_float2(sj, sj);
       inv[j] = make_float2(ij, ij);
     }
+    auto flush1 = [&]() {                       // !VEC
+      if (++terms < chain) return;
+      terms = 0;
+#pragma unroll
+      for (int j = 0; j < kNB; ++j) { dacc[j] += (double)facc[j].x + (double)facc[j].y; facc[j] = make_float2(0.0f, 0.0f); }
+    };
 #pragma unroll
     for (int v = 0; v < V; ++v) {
       const float2 lo = make_float2(cur[v].x, cur[v].y), hi = make_float2(cur[v].z, cur[v].w);
+      if (VEC) {
 #pragma unroll
-      for (int j = 0; j < kNB; ++j) {
-        err8(lo, ns[j], inv[j], facc[j]);
-        err8(hi, ns[j], inv[j], facc[j]);
+        for (int j = 0; j < kNB; ++j) {
+          err8(lo, ns[j], inv[j], facc[j]);
+          err8(hi, ns[j], inv[j], facc[j]);
+        }
+      } else {
+#pragma unroll
+        for (int j = 0; j < kNB; ++j) err8(lo, ns[j], inv[j], facc[j]);
+        flush1();
+#pragma unroll
+        for (int j = 0; j < kNB; ++j) err8(hi, ns[j], inv[j], facc[j]);
+        flush1();
       }
     }
   };
-  // second stage -> the warp's fp64 sums
+  // second stage, or the thread's fp64 sums -> the warp's fp64 sums
   auto flush2 = [&]() {
 #pragma unroll
     for (int j = 0; j < kNB; ++j) {
-      const double v = warp_sum((double)f2[j]);
+      const double v = warp_sum(VEC ? (double)f2[j] : dacc[j]);
       if (lane == 0) swarp[warp][j] += v;
       f2[j] = 0.0f;
     }
@@ -200,14 +222,14 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
   // no barrier is needed between the copy and the read.  Rows that are not whole aligned float4
   // are copied word by word, consecutive lanes taking consecutive words; which element sits in
   // which slot does not matter to the sums.
-  const float* rowp = d.w + (int64_t)team * d.cols + (ALL_VEC || d.vec ? 4 * tl : tl);   // this thread's first element of its team's next row
+  const float* rowp = d.w + (int64_t)team * d.cols + (VEC ? 4 * tl : tl);   // this thread's first element of its team's next row
   const int64_t row_step = (int64_t)nteams * d.cols;
   int fetch_row = team;
   const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(ring + threadIdx.x);
   auto issue_row = [&](int stage) {
     const uint32_t dst0 = ring0 + (uint32_t)(stage * V) * (kThreads * 16);
     const bool row_ok = fetch_row < d.rows;
-    if (ALL_VEC || d.vec) {
+    if (VEC) {
 #pragma unroll
       for (int v = 0; v < V; ++v) {
         const uint32_t dst = dst0 + v * (kThreads * 16);
@@ -243,7 +265,7 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
 #pragma unroll
     for (int v = 0; v < V; ++v) cur[v] = ring[(stage * V + v) * kThreads + threadIdx.x];
     process_row(cur);
-    if (++n1 == kFlushRows) {
+    if (VEC && ++n1 == kFlushRows) {
 #pragma unroll
       for (int j = 0; j < kNB; ++j) { f2[j] += facc[j].x + facc[j].y; facc[j] = make_float2(0.0f, 0.0f); }
       n1 = 0;
@@ -252,7 +274,10 @@ __device__ __forceinline__ void sweep_segment(const SweepSeg& d, int per_tensor,
     if (++stage == kRing) stage = 0;
   }
 #pragma unroll
-  for (int j = 0; j < kNB; ++j) f2[j] += facc[j].x + facc[j].y;
+  for (int j = 0; j < kNB; ++j) {
+    if (VEC) f2[j] += facc[j].x + facc[j].y;
+    else dacc[j] += (double)facc[j].x + (double)facc[j].y;
+  }
   flush2();
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
@@ -357,17 +382,21 @@ sweep_kernel(const SweepSeg* __restrict__ segs, const SweepBlock* __restrict__ b
     const SweepSeg d = segs[si];
     const float A_tensor = per_tensor ? tensor_absmax[d.tensor] : 0.0f;
     double* out = partial + (int64_t)d.slot * 8;
+    auto run = [&](auto v) {
+      if (d.vec) sweep_segment<decltype(v)::value, true>(d, per_tensor, A_tensor, ring, sh, out);
+      else sweep_segment<decltype(v)::value, false>(d, per_tensor, A_tensor, ring, sh, out);
+    };
     if (KV > 0) sweep_segment<(KV > 0 ? KV : 1), true>(d, per_tensor, A_tensor, ring, sh, out);
     else switch (d.v) {
       case 0: sweep_segment_long(d, per_tensor, A_tensor, jlo, jlo + nb - 1, sh, out); break;
-      case 1: sweep_segment<1, false>(d, per_tensor, A_tensor, ring, sh, out); break;
-      case 2: sweep_segment<2, false>(d, per_tensor, A_tensor, ring, sh, out); break;
-      case 3: sweep_segment<3, false>(d, per_tensor, A_tensor, ring, sh, out); break;
-      case 4: sweep_segment<4, false>(d, per_tensor, A_tensor, ring, sh, out); break;
-      case 5: sweep_segment<5, false>(d, per_tensor, A_tensor, ring, sh, out); break;
-      case 6: sweep_segment<6, false>(d, per_tensor, A_tensor, ring, sh, out); break;
-      case 7: sweep_segment<7, false>(d, per_tensor, A_tensor, ring, sh, out); break;
-      default: sweep_segment<8, false>(d, per_tensor, A_tensor, ring, sh, out); break;
+      case 1: run(std::integral_constant<int, 1>()); break;
+      case 2: run(std::integral_constant<int, 2>()); break;
+      case 3: run(std::integral_constant<int, 3>()); break;
+      case 4: run(std::integral_constant<int, 4>()); break;
+      case 5: run(std::integral_constant<int, 5>()); break;
+      case 6: run(std::integral_constant<int, 6>()); break;
+      case 7: run(std::integral_constant<int, 7>()); break;
+      default: run(std::integral_constant<int, 8>()); break;
     }
     if (!FUSED) { __syncthreads(); continue; }
     // The eight values of the slot become visible before the segment is counted; the counter wraps

@@ -170,6 +170,25 @@ def test_sweep_plans_match_oracle(ctx, shapes, offset, granularity):
         assert torch.equal(sse, st) and torch.equal(amax, at)
 
 
+@pytest.mark.parametrize("cols,offset,terms", [(147, 0, 1), (256, 1, 1), (511, 0, 1), (513, 0, 2), (771, 0, 3)])
+def test_sweep_of_ragged_rows_sums_in_64_bits(ctx, cols, offset, terms):
+    """Rows that are not whole aligned float4: at most `terms` squared errors meet in fp32, so the sum is within terms * 2^-24
+    of the exact sum of the rounded errors.  One row in 48 has a few errors of 0.45, all others are 7e-5: the square of
+    such an error vanishes when fp32 adds it to that of a large one, so long fp32 chains lose more than that."""
+    rows = 20000
+    x = np.full((rows, cols), 7e-5, np.float32)
+    x[::48, 1:64] = 0.45
+    x[:, 0] = 1.0                                     # the row maximum: at 2 bit the grid is -1, 0, 1 and x its own error
+    buf = torch.zeros(rows * cols + offset, device="cuda")
+    buf[offset:] = dev(x).reshape(-1)
+    e = x[:, 1:].astype(np.float64)
+    want = float((e * e).sum())
+    for sweep in (ctx.quant_error_sweep, ctx.quant_error_sweep_static):
+        sse, _ = sweep([buf[offset:].view(rows, cols)])
+        ctx.check_sync()
+        assert abs(float(sse[0, 0]) - want) <= (terms * 2.0 ** -24 + 1e-12) * want
+
+
 def test_sweep_is_deterministic_and_handles_subranges(ctx):
     rng = np.random.default_rng(1)
     ts = [dev((rng.standard_normal((500, 768)) * 0.02).astype(np.float32)) for _ in range(3)]
