@@ -1477,11 +1477,7 @@ int adjust_pass(qcfg_ctx* h, Model* M, const uint8_t* bits, const float* x_dev, 
       if (M->L[l].d.src >= 0) live[M->L[l].d.src] = 1;
       if (M->L[l].d.residual_from >= 0) live[M->L[l].d.residual_from] = 1;
     }
-    int64_t max_n = 0, max_k = 0, sum_n = 0;
-    for (auto& S : M->L) {
-      max_n = std::max<int64_t>(max_n, S.d.n_out); max_k = std::max<int64_t>(max_k, S.d.k_in);
-      sum_n += S.d.n_out;
-    }
+    int64_t max_n = 0, max_k = 0, max_dw = 0, sum_n = 0;
     // The weight-gradient product reduces over the m rows and its output is a weight's size: cut into
     // three partial products (one grouped launch, added up by the kernel that reads them) where
     // that leaves half of the SMs idle.  A row pitch of three equal pieces, zero behind row m.
@@ -1489,6 +1485,11 @@ int adjust_pass(qcfg_ctx* h, Model* M, const uint8_t* bits, const float* x_dev, 
       return m >= 512 && 2 * ((d.n_out + 127) / 128) * ((d.k_in + 255) / 256) <= c->sms ? 3 : 1;
     };
     const int64_t piece = round_up((m + 2) / 3, 64), ldm = 3 * piece;
+    for (auto& S : M->L) {
+      max_n = std::max<int64_t>(max_n, S.d.n_out); max_k = std::max<int64_t>(max_k, S.d.k_in);
+      max_dw = std::max<int64_t>(max_dw, parts_of(S.d) * S.d.n_out * S.d.k_in);
+      sum_n += S.d.n_out;
+    }
     rc = M->adj_grads.ensure(c, (size_t)(2 * n + 3 * sum_n) * 8);
     if (!rc) rc = M->adj_coef.ensure(c, 4);
     if (!rc) rc = M->adj_gs.ensure(c, (size_t)(m * round_up(max_n, 8)) * 2);
@@ -1496,7 +1497,7 @@ int adjust_pass(qcfg_ctx* h, Model* M, const uint8_t* bits, const float* x_dev, 
     if (!rc) rc = M->adj_qxt.ensure(c, (size_t)(max_k * ldm) * 2);
     if (!rc) rc = M->adj_qwt.ensure(c, (size_t)(max_k * round_up(max_n, 8)) * 2);
     if (!rc) rc = M->adj_dx.ensure(c, (size_t)(m * max_k) * 4);
-    if (!rc) rc = M->adj_dw.ensure(c, (size_t)(3 * max_n * max_k) * 4);
+    if (!rc) rc = M->adj_dw.ensure(c, (size_t)max_dw * 4);
     if (!rc) rc = check_cuda(c, cudaMemsetAsync(M->adj_grads.p, 0, (size_t)(2 * n + 3 * sum_n) * 8, st), "adjust: memset");
     double* dscal = (double*)M->adj_grads.p;
     double* next = dscal + 2 * n;

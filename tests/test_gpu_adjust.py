@@ -168,6 +168,31 @@ def test_gradients_see_the_input_as_it_is():
         ctx.close()
 
 
+def test_gradients_of_a_large_layer_take_one_copy_of_its_weight_gradient():
+    """Only layers whose reduction is cut have partial products; a weight that fills the device has one."""
+    import paper_2302_01382_b200 as q
+    n, k, m = 8192, 4096, 600
+    layers = [wl.Layer("a", 96, 64), wl.Layer("b", k, 96, src=0), wl.Layer("c", n, k, src=1)]
+    ctx = q.Context(0)
+    try:
+        g = torch.Generator(device="cuda").manual_seed(5)
+        weights = [torch.randn((l.n_out, l.k_in), generator=g, device="cuda") / l.k_in ** 0.5 for l in layers]
+        x = torch.randn((m, 64), generator=g, device="cuda")
+        model = q.Model(ctx, layers, weights)
+        model.calibrate_model(x, m)
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        loss, _, dix, _, diw = model.scale_gradients([8, 8, 8], x, m)
+        torch.cuda.synchronize()
+        used = before - torch.cuda.mem_get_info()[0]
+        assert np.isfinite(loss) and all(np.isfinite(dix)) and np.isfinite(diw[2]).all()
+        # fp32 gradient, bf16 transpose and int8 codes of the weight, and activations of every kind
+        assert used <= (4 + 2 + 1) * n * k + 40 * (m + 200) * (n + k), used
+        model.close()
+    finally:
+        ctx.close()
+
+
 def test_adjust_argument_errors():
     import paper_2302_01382_b200 as q
     ctx = q.Context(0)
