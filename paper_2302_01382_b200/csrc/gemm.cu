@@ -1716,6 +1716,21 @@ bool gemm_groupable(const GemmArgs& a, const GemmArgs& b) {
   return a.m == b.m && a.k == b.k && a.is_bf16 == b.is_bf16 && tile_n_of(a.n) == tile_n_of(b.n);
 }
 
+// The body for shortcut layers leaves room for a ring of two stages, stages twice the operand bytes of a 256-column pair
+// tile and joins no chain, so it pays while the reduction is short against the blocks it moves.  us for such a
+// layer between two small ones, this body / the general one:
+//   12288 x 768    k = 768 50.5 / 57.2    1280 68.9 / 69.2    1536 77.1 / 73.7
+//   25088 x 1024   k = 768 104 / 119      1024 121 / 127      1280 138 / 134
+//   50176 x 512    k = 768 131 / 139      1024 155 / 152      (the left operand no longer stays in L2 between column tiles)
+//   3072 x 768     k = 1536 28.6 / 31.5   2048 30.7 / 33.0    3072 38.6 / 37.5     (one tile per CTA: no ring to keep full)
+// Twelve transformer blocks of 768 with shortcuts (k = 768 and 3072) at 12288 rows: 1875 us with every shortcut in this body.
+static bool shortcut_body_pays(const GemmArgs& g, int bn, int sms) {
+  const int64_t width = bn > 128 ? 128 : bn;
+  if (g.k <= 768) return true;
+  if (g.k <= 2048 && ((g.m + BM - 1) / BM) * ((g.n + width - 1) / width) <= sms) return true;
+  return g.k <= 1280 && g.m * g.k <= (g.k <= 1024 ? (int64_t)32 << 20 : (int64_t)16 << 20);
+}
+
 int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t st) {
   if (count < 1 || count > kMaxGroups) return set_error(ctx, QCFG_EINVAL, "gemm: %d groups", count);
   // While launches are being chained a record's tiles run group after group.  Of three groups,
@@ -1761,7 +1776,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   // Shortcut layers at integer widths whose matrices TMA can reach: a body of its own, which keeps two fp32
   // blocks per epilogue warp in shared memory and therefore works on 128 columns at most.
   bool shortcut = false;
-  if (count == 1 && !g0.is_bf16 && g0.residual && (g0.y || g0.slots[0].kind) && !g0.acc && !g0.amax && g0.conv_kh == 0 && !g0.slots[2].kind) {
+  if (count == 1 && !g0.is_bf16 && g0.residual && shortcut_body_pays(g0, bn, sm_count(ctx)) && (g0.y || g0.slots[0].kind) && !g0.acc && !g0.amax && g0.conv_kh == 0 && !g0.slots[2].kind) {
     auto aligned = [](const void* q, int64_t ld_bytes) { return ((uintptr_t)q & 15) == 0 && (ld_bytes & 15) == 0; };
     shortcut = aligned(g0.residual, g0.ldr * 4) && (!g0.y || aligned(g0.y, g0.ldy * 4));
     for (int i = 0; i < 2; ++i)

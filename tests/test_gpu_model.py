@@ -368,6 +368,48 @@ def test_shortcut_layers_at_tile_edges(ctx, m, n):
     model.close()
 
 
+@pytest.mark.parametrize("m,n,k,act", [(300, 200, 768, 2), (300, 200, 784, 2), (257, 132, 2064, 2), (9000, 260, 1280, 2), (9000, 260, 1296, 1),
+                                       (33000, 36, 1024, 2), (130, 48, 64, 2)])
+def test_shortcut_layers_of_long_reductions(ctx, m, n, k, act):
+    """Short reductions have a shortcut body of their own, long ones the general one (the line depends on the reduction and
+    on the number of tiles): both sides of it, with GELU behind the shortcut."""
+    L = wl.Layer
+    layers = [L("a", n, 32, src=-1), L("b", n, k, src=-1, act=act, residual_from=0), L("c", 16, n, src=1), L("d", 24, n, src=1)]
+    rng = np.random.default_rng(m + n + k)
+    x = rng.standard_normal((m, k)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("shortcut", 1, layers, m, x, ws)
+    model, xd = build(ctx, w)
+    act_g, w_amax = check_calibration(model, w)
+    bits = [8, 8, 6, 4]
+    ys = run_eval(ctx, model, w, xd, bits)
+    teacher_forced_check(ctx, model, w, xd, bits, ys, act_g, w_amax, sample_rows=200)
+    model.close()
+
+
+def test_shortcut_behind_a_long_reduction_stays_in_its_chain(ctx):
+    """A wide layer with a shortcut and a reduction of 1536 runs in the same chained launch as its producers; one that
+    does not, takes a launch of its own."""
+    L = wl.Layer
+    m, n = 4992, 1536
+    weights = [torch.randn((n, n), device="cuda") / n ** 0.5 for _ in range(3)]
+    x = torch.randn((m, n), device="cuda")
+    y = torch.empty((m, n), device="cuda")
+    launches = []
+    for residual in (-1, 0):
+        import paper_2302_01382_b200 as q
+        layers = [L("a", n, n, src=-1), L("b", n, n, src=0), L("c", n, n, src=1, residual_from=residual)]
+        model = q.Model(ctx, layers, weights)
+        model.calibrate_model(x, m)
+        model.eval_config([8] * 3, x, m, [None, None, y])
+        before = ctx.launch_count()
+        model.eval_config([8] * 3, x, m, [None, None, y])
+        launches.append(ctx.launch_count() - before)
+        ctx.check_sync()
+        model.close()
+    assert launches[0] == launches[1]
+
+
 @pytest.mark.parametrize("c,n,hw,k,stride,pad,batch", [(64, 64, 9, 3, 1, 1, 3), (64, 256, 13, 3, 1, 1, 5), (128, 128, 14, 3, 2, 1, 4),
                                                        (192, 48, 7, 3, 2, 1, 7), (128, 512, 8, 1, 2, 0, 33), (64, 32, 11, 5, 1, 2, 2),
                                                        (64, 64, 130, 3, 1, 0, 1), (256, 256, 4, 3, 1, 1, 40)])
