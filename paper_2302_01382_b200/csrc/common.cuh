@@ -160,14 +160,18 @@ int launch_wait_timeout(Ctx* ctx, uint64_t limit_ns, cudaStream_t st);
 // the stream: a mixed BERT-base block at 3072 tokens 68.0 -> 60.2 us, one ragged linear layer 34.9 -> 32.3 us,
 // the 51 launches of a scale-gradient call 1116 -> 1067 us.
 template <typename... KArgs, typename... Args>
-inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+inline void launch_pdl_if(bool early, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cfg.attrs = &attr; cfg.numAttrs = 1;
+  cfg.attrs = &attr; cfg.numAttrs = early ? 1 : 0;
   (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);      // an error is picked up by the caller's cudaGetLastError
+}
+template <typename... KArgs, typename... Args>
+inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+  launch_pdl_if(true, kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 __device__ __forceinline__ void pdl_entry() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -96,6 +96,23 @@ def test_quantize_codes_bit_exact(ctx, b, shape):
     assert np.abs(want).max() == orc.qmax(b)
 
 
+@pytest.mark.parametrize("bits", [8, 16])
+@pytest.mark.parametrize("rows", [4096, 4097])
+def test_quantize_behind_other_work(ctx, rows, bits):
+    """A quantize launch up to 64 MB of input is scheduled while its predecessor drains, a longer one is not: both wait
+    for the kernel that writes their input."""
+    import paper_2302_01382_b200 as q
+    base = torch.randn((rows, 4096), device="cuda")
+    inv = torch.tensor([31.0], device="cuda")
+    x = torch.empty_like(base)
+    for scale in (1.0, 0.25):
+        torch.mul(base, scale, out=x)
+        y = ctx.quantize(x, None if bits == 16 else inv, q.PER_TENSOR, bits)
+        want = x.bfloat16() if bits == 16 else torch.round(x * inv).clamp(-127, 127).to(torch.int8)
+        assert torch.equal(y, want)
+    ctx.check_sync()
+
+
 def test_quantize_bf16_bit_exact(ctx):
     import paper_2302_01382_b200 as q
     rng = np.random.default_rng(0)
