@@ -388,7 +388,9 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
       if (d.src < 0 || dirty[d.src]) continue;
       LayerState& P = M->L[d.src];
       const bool codes_kept = !changed[l] && S.a_ready && S.a_ptr && S.a_ptr == S.abuf.p;
-      if (!codes_kept && !(P.y_ptr && P.y_internal)) dirty[d.src] = 1;
+      // a pooled reader goes on from its pooled input, which is there as long as its source is not run again (the stem of
+      // a convolutional table writes nothing else)
+      if (!codes_kept && !S.pre_ptr && !(P.y_ptr && P.y_internal)) dirty[d.src] = 1;
     }
   }
   auto codes_kept = [&](int l) {                     // a recomputed layer whose operand is still in its own buffer
@@ -419,7 +421,8 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
     if (!dirty[l]) continue;                         // buffers and pointers stay as they are
     S.implicit = ctx->implicit && !calibrate && implicit_capable(S.d);
     if (!codes_kept(l)) { S.a_ready = false; S.a_ptr = nullptr; }
-    S.y_ptr = nullptr; S.pre_ptr = nullptr; S.y_internal = false;
+    S.y_ptr = nullptr; S.y_internal = false;
+    if (!reuse || S.d.src < 0 || dirty[S.d.src]) S.pre_ptr = nullptr;
     S.bits = calibrate ? 16 : bits[l];
   }
   M->reuse_valid = false;                            // until this evaluation has been enqueued completely

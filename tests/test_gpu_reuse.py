@@ -149,3 +149,42 @@ def test_taps_after_partial_forwards(kind):
     finally:
         ctx.close()
         full.close()
+
+
+def test_a_changed_reader_of_a_pooled_stem_does_not_run_the_stem_again():
+    """Under reuse a layer that reads the max-pooled stem goes on from the pooled tensor: one launch builds its operand and
+    one multiplies it.  A change of the stem itself runs everything again."""
+    import paper_2302_01382_b200 as q
+    L = wl.Layer
+    layers = [L("stem", 32, 147, src=-1, act=wl.ACT_RELU, kh=7, kw=7, stride=2, pad=3, in_h=32, in_w=32, in_c=3, src_h=32, src_w=32)]
+    for name, n in (("a", 24), ("b", 16)):
+        layers.append(L(name, n, 32, src=0, kh=1, kw=1, stride=1, in_h=8, in_w=8, in_c=32, pool_before=wl.POOL_MAX3S2, src_h=16, src_w=16))
+    g = torch.Generator(device="cuda").manual_seed(3)
+    weights = [torch.randn((l.n_out, l.k_in), generator=g, device="cuda") for l in layers]
+    x = torch.randn((5, 32, 32, 3), generator=g, device="cuda")
+    ctx, full = q.Context(0), q.Context(0)
+    try:
+        model, plain = q.Model(ctx, layers, weights), q.Model(full, layers, weights)
+        ys = [None] + [torch.empty((5 * 64, n), device="cuda") for n in (24, 16)]
+        want = [None] + [torch.empty_like(y) for y in ys[1:]]
+        for mod in (model, plain):
+            mod.calibrate_model(x, 5)
+        ctx.set_prefix_reuse(True)
+        for bits, changed in (([16, 8, 5], 0), ([16, 4, 5], 0), ([16, 4, 8], 0), ([16, 8, 8], 1), ([16, 8, 5], 2), ([8, 8, 5], 0),
+                              ([16, 8, 5], 0), ([16, 4, 5], 1)):
+            before = ctx.launch_count()
+            model.eval_config(bits, x, 5, [y if changed in (0, i) else None for i, y in enumerate(ys)])
+            launches = ctx.launch_count() - before
+            if changed:
+                assert launches == 2, (bits, launches)
+            plain.eval_config(bits, x, 5, want)
+            ctx.check_sync()
+            full.check_sync()
+            for i in (1, 2):
+                if changed in (0, i):
+                    assert torch.equal(ys[i], want[i]), (bits, i)
+        model.close()
+        plain.close()
+    finally:
+        ctx.close()
+        full.close()
