@@ -133,13 +133,12 @@ int check_cuda(Ctx* ctx, cudaError_t e, const char* what) {
   if (e == cudaSuccess) return QCFG_OK;
   return set_error(ctx, e == cudaErrorMemoryAllocation ? QCFG_ENOMEM : QCFG_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
-bool sweep_tables_cached(Ctx* ctx, const void* dev_base, cudaStream_t st, const void* a, size_t na, const void* b, size_t nb) {
-  if (ctx->sweep_base == dev_base && ctx->sweep_stream == st && ctx->sweep_tables.size() == na + nb &&
-      memcmp(ctx->sweep_tables.data(), a, na) == 0 && (nb == 0 || memcmp(ctx->sweep_tables.data() + na, b, nb) == 0))
+bool sweep_tables_cached(Ctx* ctx, const void* dev_base, cudaStream_t st, const void* tables, size_t bytes) {
+  if (ctx->sweep_base == dev_base && ctx->sweep_stream == st && ctx->sweep_tables.size() == bytes &&
+      memcmp(ctx->sweep_tables.data(), tables, bytes) == 0)
     return true;
-  ctx->sweep_tables.resize(na + nb);
-  memcpy(ctx->sweep_tables.data(), a, na);
-  if (nb) memcpy(ctx->sweep_tables.data() + na, b, nb);
+  ctx->sweep_tables.resize(bytes);
+  memcpy(ctx->sweep_tables.data(), tables, bytes);
   ctx->sweep_base = dev_base;
   ctx->sweep_stream = st;
   return false;

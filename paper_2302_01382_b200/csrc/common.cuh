@@ -31,9 +31,9 @@ int prof_mode(Ctx* ctx);
 void* scratch(Ctx* ctx, size_t bytes);
 // grows (never shrinks) a host buffer owned by the context; returns nullptr on failure
 void* host_scratch(Ctx* ctx, size_t bytes);
-// true when the same two host tables were the last ones uploaded to this scratch address on
-// this context in this stream (the caller may then skip the upload); records them otherwise
-bool sweep_tables_cached(Ctx* ctx, const void* dev_base, cudaStream_t st, const void* a, size_t na, const void* b, size_t nb);
+// true when the same host table was the last one uploaded to this scratch address on
+// this context in this stream (the caller may then skip the upload); records it otherwise
+bool sweep_tables_cached(Ctx* ctx, const void* dev_base, cudaStream_t st, const void* tables, size_t bytes);
 // optional per-launch timing of one kernel class (0 = int8 GEMM, 1 = bf16 GEMM) with CUDA events
 void prof_begin(Ctx* ctx, int cls, cudaStream_t st);
 void prof_end(Ctx* ctx, int cls, double ops, cudaStream_t st);

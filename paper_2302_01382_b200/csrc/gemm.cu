@@ -341,8 +341,8 @@ __device__ __forceinline__ void store_piece(const OutDesc& o, const CUtensorMap*
     }
     return;
   }
-  if (WORDS == 32 && stage_bytes >= 4096) {
-    // A 4-byte output TMA cannot write (row pitch not a multiple of 16 bytes).  The lanes hold one
+  if constexpr (WORDS == 32) {
+    // A 4-byte output TMA cannot write (row pitch not a multiple of 16 bytes); every launch with one has 4 KB of staging.  The lanes hold one
     // row each, so stores straight from registers would touch 32 rows per instruction; instead the
     // piece is turned in the warp's staging buffer (16-byte chunks swizzled by the row, no bank
     // conflicts either way) and goes out row by row, 32 consecutive words per instruction.
@@ -363,21 +363,20 @@ __device__ __forceinline__ void store_piece(const OutDesc& o, const CUtensorMap*
       out += o.ld;
     }
     __syncwarp();
-    return;
-  }
-  if (!row_ok) return;
-  uint8_t* dst = reinterpret_cast<uint8_t*>(o.ptr) + (row * o.ld + col0) * kElemBytes;
-  if (ncols >= 32 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
-#pragma unroll
-    for (int j = 0; j < WORDS / 4; ++j)
-      reinterpret_cast<uint4*>(dst)[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
   } else {
+    if (!row_ok) return;
+    uint8_t* dst = reinterpret_cast<uint8_t*>(o.ptr) + (row * o.ld + col0) * kElemBytes;
+    if (ncols >= 32 && (reinterpret_cast<uintptr_t>(dst) & 15) == 0) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      if (i < ncols) {
-        if (kElemBytes == 4) reinterpret_cast<uint32_t*>(dst)[i] = w[i * WORDS / 32];
-        else if (kElemBytes == 2) reinterpret_cast<uint16_t*>(dst)[i] = (uint16_t)(w[i >> 1] >> (16 * (i & 1)));
-        else dst[i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+      for (int j = 0; j < WORDS / 4; ++j)
+        reinterpret_cast<uint4*>(dst)[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        if (i < ncols) {
+          if (kElemBytes == 2) reinterpret_cast<uint16_t*>(dst)[i] = (uint16_t)(w[i >> 1] >> (16 * (i & 1)));
+          else dst[i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+        }
       }
     }
   }

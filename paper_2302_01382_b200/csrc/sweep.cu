@@ -653,7 +653,7 @@ int launch_sweep(Ctx* ctx, const float* const* w, const int64_t* rows, const int
   char* tab = base + partial_bytes;
   // the tables only depend on the tensor list: a repeated sweep of the same tensors (same scratch
   // buffer) finds them on the device already, the counters back at zero
-  if (!sweep_tables_cached(ctx, base, st, host, used, nullptr, 0)) {
+  if (!sweep_tables_cached(ctx, base, st, host, used)) {
     const cudaError_t e = cudaMemcpyAsync(tab, host, used, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return check_cuda(ctx, e, "sweep table upload");
   }
