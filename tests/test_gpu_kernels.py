@@ -228,6 +228,24 @@ GEMM_SHAPES = [(64, 16, 32), (128, 32, 128), (64, 10, 256), (300, 200, 150), (70
                (1000, 768, 768), (260, 2304, 144), (3, 5, 7), (2048, 64, 64), (512, 512, 4608)]
 
 
+# ragged in rows and columns and large enough that the tiles stay 256 columns wide
+WIDE = [(4993, 1000), (5000, 1000), (257, 19300)]
+
+
+def tile_columns(m, n):
+    """Width of a single GEMM's tiles: by the output's columns, halved while every CTA still has one tile at most."""
+    width = 256 if n > 128 else 128 if n > 64 else 64 if n > 32 else 32
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    while width > 32 and -(-n // (width // 2)) * -(-m // 128) <= sms:
+        width //= 2
+    return width
+
+
+@pytest.mark.parametrize("m,n", WIDE)
+def test_wide_shapes_keep_whole_tiles(m, n):
+    assert tile_columns(m, n) == 256 and n % 256 and m % 256
+
+
 @pytest.mark.parametrize("m,n,k", GEMM_SHAPES)
 def test_gemm_i8_accumulators_and_rescale_bit_exact(ctx, m, n, k):
     import paper_2302_01382_b200 as q
@@ -243,7 +261,7 @@ def test_gemm_i8_accumulators_and_rescale_bit_exact(ctx, m, n, k):
     np.testing.assert_array_equal(host(y).view(np.uint32), orc.dequant_output(ref, sx, sw).view(np.uint32))
 
 
-@pytest.mark.parametrize("m,n,k", [(5000, 1024, 272), (257, 300, 1040), (129, 2304, 64)])
+@pytest.mark.parametrize("m,n,k", [(5000, 1024, 272), (257, 300, 1040), (129, 2304, 64), (4993, 1000, 272), (257, 19300, 80)])
 def test_gemm_pair_and_single_cta_tiles_agree(ctx, m, n, k):
     """Outputs wider than 128 columns run on CTA pairs (256-row tiles); the single-CTA path must
     give the same bits, also when a pair works through several tiles and when the second CTA's
@@ -333,10 +351,10 @@ def test_gemm_i8_worst_case_magnitude(ctx):
     np.testing.assert_array_equal(host(acc), orc.int_gemm(qx, qw))
 
 
+@pytest.mark.parametrize("m,n,k", [(513, 384, 256), (5000, 1000, 256)])
 @pytest.mark.parametrize("act", [1, 2])
-def test_gemm_i8_activations(ctx, act):
+def test_gemm_i8_activations(ctx, act, m, n, k):
     rng = np.random.default_rng(act)
-    m, n, k = 513, 384, 256
     qx, qw = _codes(rng, m, k, k), _codes(rng, n, k, k)
     sw = (10.0 ** rng.uniform(-3.5, -2.5, n)).astype(np.float32)
     sx = np.float32(0.011)
@@ -352,7 +370,8 @@ def test_gemm_i8_activations(ctx, act):
 
 
 @pytest.mark.parametrize("next_bits", [2, 4, 8, 16])
-@pytest.mark.parametrize("m,n,k,act", [(300, 200, 150, 0), (1000, 768, 768, 1), (515, 1000, 256, 0), (260, 330, 144, 1)])
+@pytest.mark.parametrize("m,n,k,act", [(300, 200, 150, 0), (1000, 768, 768, 1), (515, 1000, 256, 0), (260, 330, 144, 1),
+                                       (5000, 1000, 150, 1)])
 def test_gemm_i8_requant_codes_bit_exact(ctx, m, n, k, act, next_bits):
     rng = np.random.default_rng(m + n + k + next_bits)
     ld = (k + 15) // 16 * 16
@@ -375,7 +394,7 @@ def test_gemm_i8_requant_codes_bit_exact(ctx, m, n, k, act, next_bits):
         assert np.abs(want).max() == orc.qmax(next_bits)
 
 
-@pytest.mark.parametrize("m,n,k", [(64, 16, 16), (300, 200, 150), (1000, 768, 768), (129, 1000, 3072), (128, 1000, 2048)])
+@pytest.mark.parametrize("m,n,k", [(64, 16, 16), (300, 200, 150), (1000, 768, 768), (129, 1000, 3072), (128, 1000, 2048), (4993, 1000, 200)])
 def test_gemm_bf16_matches_fp64_reference(ctx, m, n, k):
     import paper_2302_01382_b200 as q
     rng = np.random.default_rng(m * n + k)

@@ -412,10 +412,12 @@ def test_shortcut_behind_a_long_reduction_stays_in_its_chain(ctx):
 
 @pytest.mark.parametrize("c,n,hw,k,stride,pad,batch", [(64, 64, 9, 3, 1, 1, 3), (64, 256, 13, 3, 1, 1, 5), (128, 128, 14, 3, 2, 1, 4),
                                                        (192, 48, 7, 3, 2, 1, 7), (128, 512, 8, 1, 2, 0, 33), (64, 32, 11, 5, 1, 2, 2),
-                                                       (64, 64, 130, 3, 1, 0, 1), (256, 256, 4, 3, 1, 1, 40)])
+                                                       (64, 64, 130, 3, 1, 0, 1), (256, 256, 4, 3, 1, 1, 40),
+                                                       (64, 264, 27, 3, 1, 1, 9), (128, 264, 28, 3, 1, 1, 9)])
 def test_convolution_operand_through_tma_matches_the_patch_matrix(ctx, c, n, hw, k, stride, pad, batch):
     """Channels in whole 64- and 128-byte chunks: TMA brings the patches.  Filters of one, nine and 25 taps (odd chunk
-    counts leave half a k-block), strides, tiles that cross rows and images, a ragged last tile, CTA pairs."""
+    counts leave half a k-block), strides, tiles that cross rows and images, a ragged last tile; 264 columns on more than 6400
+    rows: CTA pairs, whose tiles stay 256 columns wide and whose last one is ragged."""
     L = wl.Layer
     oh = (hw + 2 * pad - k) // stride + 1
     layers = [L("in", c, 16, src=-1, kh=1, kw=1, stride=1, in_h=hw, in_w=hw, in_c=16, src_h=hw, src_w=hw),
