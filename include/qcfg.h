@@ -125,9 +125,10 @@ int qcfg_set_gemm_chains(qcfg_ctx* ctx, int enabled);
  * other layers launch nothing.  This is what consecutive configurations of the searches allow:
  * Algorithm 2 changes one layer per evaluation, Algorithm 1 a slice of the ordering.  The CALLER
  * guarantees that the contents of x_dev did not change between such calls.  Results are
- * bit-identical to a full evaluation.  qcfg_calibrate_model and qcfg_latency_table always run every
- * layer.  qcfg_search and qcfg_noise_sensitivity reuse in this way among their own forwards whatever
- * the switch says (the input stays the same within a call), starting from a full one.           */
+ * bit-identical to a full evaluation.  qcfg_calibrate_model, qcfg_latency_table and the reference
+ * forward of the scale adjustment always run every layer.  qcfg_search and qcfg_noise_sensitivity
+ * reuse in this way among their own forwards whatever the switch says (the input stays the same
+ * within a call), starting from a full one.                                                     */
 int qcfg_set_prefix_reuse(qcfg_ctx* ctx, int enabled);
 
 /* Per-launch timing, off by default.  Mode 1: CUDA events recorded around every launch on the
@@ -178,7 +179,8 @@ int qcfg_quantize(qcfg_ctx* ctx, const float* x_dev, int64_t rows, int64_t cols,
  * sse_dev[t*(b_hi-b_lo+1) + (b-b_lo)] = sum over the tensor of (x - Q_b(x))^2 (double) and
  * absmax_dev[t] = max|x| over the tensor, so that
  * E_QE(t, b) = sqrt(sse / (rows*cols)) / absmax.  Per-tensor granularity takes a second
- * read of the tensor (the maximum must be known first).                                   */
+ * read of the tensor (the maximum must be known first).  Partial sums and work tables are in
+ * the context's scratch memory: sweeps of one context must not overlap on the GPU.         */
 int qcfg_quant_error_sweep(qcfg_ctx* ctx, const float* const* w_dev, const int64_t* rows,
                            const int64_t* cols, int32_t n_tensors, int granularity, int b_lo,
                            int b_hi, double* sse_dev, float* absmax_dev, void* stream);
@@ -333,7 +335,7 @@ int qcfg_search(qcfg_ctx* ctx, qcfg_model* model, int algorithm, const int32_t* 
  * every step and after the last.  From then on qcfg_eval_config uses the adapted scales wherever a
  * layer runs at the width it was adapted at; qcfg_calibrate_model and qcfg_model_reset_scales go
  * back to max calibration.  Linear layers only (QCFG_ESHAPE for a convolutional table).
- * Synchronises the stream several times per step.                                              */
+ * Synchronises the stream once per step and once at the end.                                   */
 int qcfg_adjust_scales(qcfg_ctx* ctx, qcfg_model* model, const uint8_t* bits, const float* x_dev,
                        int64_t m, int32_t steps, double lr, double* losses_host, void* stream);
 /* The gradients one step of qcfg_adjust_scales would use, at the model's current scales (HOST
