@@ -487,8 +487,8 @@ def run_gpu(args):
         dt = time.perf_counter() - t0
         search = {"algorithm": "greedy", "bs": [8, 4], "target_fidelity": 0.9, "evals": int(n_s), "ms": 1e3 * dt,
                   "evals_per_s": n_s / dt, "layers_at_4_bit": int(sum(1 for b in bits_s if b == 4))}
-        # the same search with prefix reuse: every evaluation restarts at the first layer whose
-        # width changed (reported beside the full-recompute figures, never instead of them)
+        # the same search with the prefix-reuse switch on (the evaluations of one search restart at the
+        # first layer whose width changed either way; the switch carries that over to the next call)
         ctx.set_prefix_reuse(True)
         l0 = ctx.launch_count()
         t0 = time.perf_counter()
