@@ -99,13 +99,29 @@ struct GroupDesc {
 // How the operand gets into shared memory: gather warps (any multiple of 16 bytes of channels), or TMA in its
 // im2col mode, where one load brings a chunk of channels of 128 consecutive output pixels at one tap:
 // 128-byte chunks (channels a multiple of 128 bytes; the usual 128B-swizzled tile), or two 64-byte chunks
-// per k-block (a multiple of 64 bytes; two half tiles of 64-byte rows, 64B swizzle).
-enum : int32_t { CONV_NONE = 0, CONV_GATHER = 1, CONV_TMA128 = 2, CONV_TMA64 = 3 };
+// per k-block (a multiple of 64 bytes; two half tiles of 64-byte rows, 64B swizzle).  CONV_SLAB: see SlabDesc.
+enum : int32_t { CONV_NONE = 0, CONV_GATHER = 1, CONV_TMA128 = 2, CONV_TMA64 = 3, CONV_SLAB = 4 };
 struct ConvDesc {
   int32_t on, H, W, C, kh, kw, stride, pad, OH, OW, esz, K;
   int64_t img_bytes;          // bytes of one image (H * W * C * esz)
   const uint8_t* src;
 };
+// Stride-1 3x3 convolutions whose only output is one int8 code matrix read their input once per tile, not once per tap: a
+// tile is tw x rows output pixels of `imgs` images, and one tiled TMA load per channel chunk brings all input pixels
+// its taps touch (a slab of `pitch` pixels per row, zeros outside the image).  The A operand of tap (dy, dx) is
+// then simply the 128 slab pixels from dy * pitch + dx on: row r of the tile is the output pixel at linear slab position r, and
+// positions that are no output pixel (the halo at the right of a row, the rows between two images) are
+// computed and not stored.  A whole-width tile shares the halo: the zeros left of a row stand right of the row before
+// (right of the last row: zeros the kernel puts behind each slab once).
+struct SlabDesc {
+  int32_t pitch, tw, rows, imgs;        // slab pixels per row; output columns, rows and images of a tile
+  int32_t img_pitch;                    // slab pixels per image
+  int32_t tiles_w, tiles_h, images;
+  int32_t chunk, chunks;                // channel bytes per load (64 or 128), loads per tile
+  int32_t bytes, tx_bytes, count;       // slab size in the ring (whole 1024 bytes, also what the last tap reads), bytes loaded, slabs in the ring
+  int32_t resident;                     // one chunk, one column tile: all weights stay in shared memory, a stage (and barrier) per tap
+};
+constexpr int kMaxSlabs = 4;
 constexpr int kMaxDeps = 4;
 struct GemmParams {
   int32_t m, k_blocks, bn, tiles_m, tiles_n, stages, is_bf16;   // tiles_n: column tiles of all groups together
@@ -116,6 +132,7 @@ struct GemmParams {
   unsigned* err;
   unsigned long long* stamp;  // optional [2]: earliest start / latest end of the launch's CTAs (%globaltimer, ns)
   ConvDesc conv;              // conv.on: A comes from the gather warps (single-group launches only)
+  SlabDesc slab;
   // chains: records of the same launch whose output rows this record reads (-1: none), and
   // whether a later record of the launch reads this one's
   uint8_t mi[kMaxGroups][kMapsPerGroup];   // pool indices of the groups' tensor maps
@@ -208,6 +225,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
 }
 
+__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t c, int32_t w, int32_t h, int32_t n) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+      ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n) : "memory");
+}
 // im2col loads: (w, h) is the first pixel's corner of the filter window, (dx, dy) the tap
 __device__ __forceinline__ void tma_load_im2col(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t c, int32_t w, int32_t h, int32_t n,
                                                 int dx, int dy) {
@@ -224,6 +246,11 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(dst), "l"(map), "r"(bar & kPeerBitMask), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t c, int32_t w, int32_t h, int32_t n) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+      ::"r"(dst), "l"(map), "r"(bar & kPeerBitMask), "r"(c), "r"(w), "r"(h), "r"(n) : "memory");
 }
 __device__ __forceinline__ void tma_load_im2col_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int32_t c, int32_t w, int32_t h,
                                                      int32_t n, int dx, int dy) {
@@ -728,6 +755,41 @@ __device__ __forceinline__ void epilogue_shortcut(const GroupDesc& G, const CUte
   }
 }
 
+// One warp's 32 rows x (32 * nch) columns of a slab convolution: codes go from the registers to the rows' pixels, 32 bytes
+// per lane and chunk (whole sectors), because the 32 rows are no box of the output matrix.  dst: this lane's row at
+// the warp's first column, or null where the row is no output pixel.
+template <bool PAIR>
+__device__ __forceinline__ void epilogue_slab(const GroupDesc& G, uint32_t tbase, const float* cs, int nch, uint8_t* dst, int lane, uint32_t tempty_bar) {
+  const float2 inv2 = make_float2(G.outs[2].inv_scale, G.outs[2].inv_scale);
+  const float qmax = G.outs[2].qmax;
+  const int act = G.act;
+  uint32_t v[32];
+#pragma unroll 1
+  for (int c = 0; c < nch; ++c) {
+    tmem_ld32_issue(tbase + 32 * c, v);
+    tmem_ld_wait();
+    if (c == nch - 1) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) { if (PAIR) mbar_arrive_leader(tempty_bar); else mbar_arrive(tempty_bar); }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      uint32_t part[16], w[4];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) part[i] = v[16 * h + i];
+      float2 y[8];
+      sub_values<false>(y, part, cs + 32 * c + 16 * h, act);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 a = code_words2(y[2 * j], inv2, qmax), b = code_words2(y[2 * j + 1], inv2, qmax);
+        w[j] = pack4(__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(b.x), __float_as_uint(b.y));
+      }
+      if (dst) *reinterpret_cast<uint4*>(dst + 32 * c + 16 * h) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------- the kernel
 
 // One launch runs one GEMM record or, in the CHAIN flavour, up to kChainMax records one after the
@@ -745,7 +807,7 @@ __device__ __forceinline__ void epilogue_shortcut(const GroupDesc& G, const CUte
 // FL: what the single-GEMM flavours carry besides the plain matrix product.  Convolutions and shortcut layers have
 // instantiations of their own: their code inside the plain kernel slowed its short launches by a tenth to a fifth
 // (100352 x 128 x 512: 20.0 -> 24.5 us).
-enum : int { FL_PLAIN = 0, FL_CONV = 1, FL_SHORTCUT = 2 };
+enum : int { FL_PLAIN = 0, FL_CONV = 1, FL_SHORTCUT = 2, FL_SLAB = 3, FL_SLAB64 = 4 };
 template <bool BF16, bool PAIR, bool GROUPED, bool CHAIN, int FL = FL_PLAIN>
 __global__ void __launch_bounds__(FL == FL_CONV || CHAIN ? kGemmThreadsConv : kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
@@ -771,7 +833,9 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   // counts 256-row tiles.
   const int rank = PAIR ? (int)cluster_ctarank() : 0;
   const int b_rows = PAIR ? (p.bn >> 1) : p.bn;                  // B rows held per stage by this CTA
-  const uint32_t stage_bytes = (uint32_t)(BM + b_rows) * kStageKBytes;
+  constexpr bool kSlab = FL == FL_SLAB || FL == FL_SLAB64;       // stages hold weights only, the input's slabs have a ring of their own
+  constexpr int kChunk = FL == FL_SLAB64 ? 64 : 128;             // ... and the slab's channel bytes
+  const uint32_t stage_bytes = kSlab ? (uint32_t)(b_rows * kChunk) : (uint32_t)(BM + b_rows) * kStageKBytes;
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kMaxStages;
   const uint32_t tfull0 = empty0 + 8 * kMaxStages, tempty0 = tfull0 + 16;
   // chains: per epilogue warp, the number of its tiles whose stores have completed (counters, not
@@ -825,7 +889,9 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   int ld_tile = tile0, ld_kb = 0, ld_s = 0;
   uint32_t ld_ph = 0;
   const int k_elems = BF16 ? kStageKBytes / 2 : kStageKBytes;
-  const uint32_t stage0 = smem_u32(stage_base);
+  const uint32_t slab0 = smem_u32(stage_base);                   // kSlab: the slabs, then the stages
+  const uint32_t stage0 = slab0 + (kSlab ? (uint32_t)(p.slab.count * p.slab.bytes) : 0u);
+  const uint32_t sfull0 = smem_u32(smem + kResBarOffset), sempty0 = sfull0 + 8 * kMaxSlabs;
   uint32_t ld_dst = stage0, ld_bar = full0;      // stage address and its full barrier
   int ld_x = 0, ld_ya = 0, ld_yb = 0;            // TMA coordinates of the next k-block
   int ld_tm = tm0, ld_tn = tn0;
@@ -900,6 +966,10 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mp[q->mi[0][MAP_A]]) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&mp[q->mi[0][MAP_B]]) : "memory");
     const uint32_t full_count = 1 + (conv_on ? kGatherWarps * (PAIR ? 2 : 1) : 0);   // the TMA thread, plus one arrival per gather warp
+    if (kSlab) {
+      for (int s = 0; s < 2 * kMaxStages; ++s) mbar_init(full0 + 8 * s, 1);     // ring, or one per resident k-block
+      for (int s = 0; s < 2 * kMaxSlabs; ++s) mbar_init(sfull0 + 8 * s, 1);
+    } else
     for (int s = 0; s < p.stages; ++s) { mbar_init(full0 + 8 * s, full_count); mbar_init(empty0 + 8 * s, 1); }
     for (int a = 0; a < 2; ++a) { mbar_init(tfull0 + 8 * a, 1); mbar_init(tempty0 + 8 * a, PAIR ? 2 * kEpiWarps : p.alternate ? kEpiWarps / 2 : kEpiWarps); }
     if (FL == FL_SHORTCUT) for (int a = 0; a < 2 * kEpiWarps; ++a) mbar_init(smem_u32(smem + kResBarOffset) + 8 * a, 1);
@@ -907,6 +977,12 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     *abort_flag = 0;
     *reinterpret_cast<volatile uint32_t*>(smem + 264) = 0u;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (kSlab) {      // behind what the loads write: zeros
+    const int quads = (p.slab.bytes - p.slab.tx_bytes) >> 4;
+    for (int i = threadIdx.x; i < quads * p.slab.count; i += kGemmThreads)
+      st_shared_v4(slab0 + (uint32_t)((i / quads) * p.slab.bytes + p.slab.tx_bytes + (i % quads) * 16), 0u, 0u, 0u, 0u);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
     if (PAIR) {   // the same warp of both CTAs allocates for the pair
@@ -927,7 +1003,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
   if (p.stamp && threadIdx.x == 32) atomicMin(p.stamp, (unsigned long long)global_timer());
   if (warp == 0) {
     // the ring is empty: fill it before the block-wide barrier so the first tiles are in flight
-    if (!CHAIN) for (int i = 0; i < p.stages && ld_tile < num_tiles; ++i) issue_load();
+    if (!CHAIN && !kSlab) for (int i = 0; i < p.stages && ld_tile < num_tiles; ++i) issue_load();
   }
   tc_fence_before();
   __syncthreads();
@@ -964,6 +1040,65 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
           if (++ld_s == p.stages) { ld_s = 0; ld_ph ^= 1; ld_dst = stage0; ld_bar = full0; }
         }
       }
+    } else if (kSlab) {
+      // Slabs run one ahead of the weights, so that the next chunk's pixels are under way while the ring waits for the
+      // tensor core; with resident weights the ring of slabs is all there is to keep full.
+      const SlabDesc& sd = p.slab;
+      int f_tile = tile0, f_chunk = 0, f_s = 0, f_w = 0, f_h = 0, f_n = 0;
+      uint32_t f_ph = 0;
+      auto fetch_slab = [&]() -> bool {
+        if (f_tile >= num_tiles) return true;
+        if (!mbar_wait_warp(sempty0 + 8 * f_s, f_ph ^ 1, abort_flag, p.err)) return false;
+        if (f_chunk == 0) {
+          const int tm = f_tile % p.tiles_m, mt = PAIR ? 2 * tm + rank : tm;
+          const int wh = sd.tiles_w * sd.tiles_h, ng = mt / wh, q2 = mt - ng * wh, th = q2 / sd.tiles_w;
+          f_n = ng * sd.imgs;
+          f_h = th * sd.rows - p.conv.pad;
+          f_w = (q2 - th * sd.tiles_w) * sd.tw - p.conv.pad;
+        }
+        if (elected) {
+          const uint32_t dst = slab0 + (uint32_t)(f_s * sd.bytes), bar = sfull0 + 8 * f_s;
+          if (rank == 0) mbar_expect_tx(bar, (uint32_t)((PAIR ? 2 : 1) * sd.tx_bytes));
+          if (PAIR) tma_load_4d_pair(dst, ld_map_a, bar, f_chunk * kChunk, f_w, f_h, f_n);
+          else tma_load_4d(dst, ld_map_a, bar, f_chunk * kChunk, f_w, f_h, f_n);
+        }
+        if (++f_s == sd.count) { f_s = 0; f_ph ^= 1; }
+        if (++f_chunk == sd.chunks) { f_chunk = 0; f_tile += tile_step; }
+        return true;
+      };
+      ok = fetch_slab();
+      if (sd.resident) {
+        for (int t = 0; t < 9; ++t, ld_bar += 8, ld_dst += stage_bytes)
+          if (elected) {
+            mbar_expect_tx(ld_bar, stage_bytes);
+            tma_load_2d(ld_dst, ld_map_b, ld_bar, t * p.conv.C, 0);
+          }
+        while (ok && f_tile < num_tiles) ok = fetch_slab();
+      } else {
+        for (int tile = tile0; tile < num_tiles && ok; tile += tile_step) {
+          const int yb = tile / p.tiles_m * p.bn + rank * b_rows;
+          for (int c = 0; c < sd.chunks && ok; ++c) {
+            ok = fetch_slab();
+            int x = c * kChunk;
+            for (int t = 0; t < 9 && ok; ++t, x += p.conv.C) {
+              if (!mbar_wait_warp(ld_bar + 8 * kMaxStages, ld_ph ^ 1, abort_flag, p.err)) { ok = false; break; }
+              if (elected) {
+                if (rank == 0) mbar_expect_tx(ld_bar, (PAIR ? 2 : 1) * stage_bytes);
+                if (PAIR) tma_load_2d_pair(ld_dst, ld_map_b, ld_bar, x, yb);
+                else tma_load_2d(ld_dst, ld_map_b, ld_bar, x, yb);
+              }
+              ld_dst += stage_bytes; ld_bar += 8;
+              if (++ld_s == p.stages) { ld_s = 0; ld_ph ^= 1; ld_dst = stage0; ld_bar = full0; }
+            }
+          }
+        }
+      }
+      // as below for the stages: the pair's first CTA still releases this CTA's slabs
+      if (PAIR)
+        for (int i = 0; i < sd.count && ok; ++i) {
+          if (!mbar_wait_warp(sempty0 + 8 * f_s, f_ph ^ 1, abort_flag, p.err)) ok = false;
+          if (++f_s == sd.count) { f_s = 0; f_ph ^= 1; }
+        }
     } else {
       while (ld_tile < num_tiles) {
         if (!mbar_wait_warp(ld_bar + 8 * kMaxStages, ld_ph ^ 1, abort_flag, p.err)) { ok = false; break; }
@@ -985,7 +1120,83 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (rank == 0) {
+    if (kSlab && rank == 0) {
+      // Per channel chunk one slab and one block of weights per tap; a tap moves the A operand's start by whole slab pixels.
+      // The swizzle pattern stays where the TMA load put it (it follows the address), so the start may be any row.
+      // The taps are written out: an instruction for 64 columns keeps the tensor core for 48 cycles only, and with the taps
+      // in loops issuing one took 240 (56 x 56 x 64, 128 images: 69 us, 32 this way).
+      const SlabDesc& sd = p.slab;
+      constexpr uint32_t kPx = (uint32_t)kChunk >> 4;                  // one slab pixel, in the descriptor's 16-byte units
+      constexpr uint32_t kHi = kChunk == 64 ? (uint32_t)(512 >> 4) | (1u << 14) | (4u << 29) : (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);
+      const uint32_t pitch = (uint32_t)sd.pitch * kPx;
+      const uint32_t alo0 = ((slab0 >> 4) & 0x3FFFu) | (1u << 16), a_step = (uint32_t)sd.bytes >> 4;
+      const uint32_t blo0 = ((stage0 >> 4) & 0x3FFFu) | (1u << 16), b_step = stage_bytes >> 4;
+      uint32_t alo = alo0, sfb = sfull0, sph = 0;
+      int ss = 0, t = 0;
+      bool ok = true;
+      auto mma_tap = [&](uint32_t d_tmem, int tap, uint32_t bl, uint32_t acc) {      // elected lane
+        const uint32_t al = alo + (uint32_t)(tap / 3) * pitch + (uint32_t)(tap % 3) * kPx;
+#pragma unroll
+        for (int k = 0; k < kChunk / kUmmaKBytes; ++k) {
+          const uint64_t da = ((uint64_t)kHi << 32) | (uint64_t)(al + 2u * k), db = ((uint64_t)kHi << 32) | (uint64_t)(bl + 2u * k);
+          if (PAIR) tc_mma_pair<BF16>(d_tmem, da, db, p.idesc, k == 0 ? acc : 1u);
+          else tc_mma<BF16>(d_tmem, da, db, p.idesc, k == 0 ? acc : 1u);
+        }
+      };
+      auto acc_wait = [&](int at) { return mbar_wait_warp(tempty0 + 8 * (at & 1), ((at >> 1) & 1) ^ 1, abort_flag, p.err); };
+      auto next_slab = [&]() {
+        alo += a_step; sfb += 8;
+        if (++ss == sd.count) { ss = 0; sph ^= 1; alo = alo0; sfb = sfull0; }
+      };
+      if (!PAIR && sd.resident) {
+        // one chunk, all weights in shared memory: no wait and no branch between a tile's taps
+        for (int tile = tile0; tile < num_tiles && ok; tile += tile_step, ++t) {
+          if (!acc_wait(t) || !mbar_wait_warp(sfb, sph, abort_flag, p.err)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t d_tmem = tmem_base + (uint32_t)(t & 1) * kAccCols;
+          if (t == 0) {                                    // the weights arrive tap by tap
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) {
+              if (ok && !mbar_wait_warp(full0 + 8 * tap, 0, abort_flag, p.err)) ok = false;
+              tc_fence_after();
+              if (ok && elected) mma_tap(d_tmem, tap, blo0 + (uint32_t)tap * b_step, tap > 0);
+            }
+            if (!ok) break;
+          } else if (elected) {
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) mma_tap(d_tmem, tap, blo0 + (uint32_t)tap * b_step, tap > 0);
+          }
+          if (elected) { tc_commit(sfb + 8 * kMaxSlabs); tc_commit(tfull0 + 8 * (t & 1)); }
+          next_slab();
+        }
+      } else {
+        uint32_t blo = blo0, fb = full0, ph = 0;
+        int s = 0;
+        for (int tile = tile0; tile < num_tiles && ok; tile += tile_step, ++t) {
+          if (!acc_wait(t)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t d_tmem = tmem_base + (uint32_t)(t & 1) * kAccCols;
+          for (int c = 0; c < sd.chunks && ok; ++c) {
+            if (!mbar_wait_warp(sfb, sph, abort_flag, p.err)) { ok = false; break; }
+            tc_fence_after();
+#pragma unroll
+            for (int tap = 0; tap < 9; ++tap) {
+              if (!ok || !mbar_wait_warp(fb, ph, abort_flag, p.err)) { ok = false; break; }
+              tc_fence_after();
+              if (elected) {
+                mma_tap(d_tmem, tap, blo, c + tap > 0);
+                if (PAIR) tc_commit_pair(fb + 8 * kMaxStages); else tc_commit(fb + 8 * kMaxStages);
+              }
+              blo += b_step; fb += 8;
+              if (++s == p.stages) { s = 0; ph ^= 1; blo = blo0; fb = full0; }
+            }
+            if (ok && elected) { if (PAIR) tc_commit_pair(sfb + 8 * kMaxSlabs); else tc_commit(sfb + 8 * kMaxSlabs); }
+            next_slab();
+          }
+          if (ok && elected) { if (PAIR) tc_commit_pair(tfull0 + 8 * (t & 1)); else tc_commit(tfull0 + 8 * (t & 1)); }
+        }
+      }
+    } else if (!kSlab && rank == 0) {
       // Descriptor low words (start address field, 16-byte units) of the four K steps of the
       // current stage's A and B tiles; the high word is the same for all.
       constexpr uint32_t kDescHi = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);
@@ -1195,6 +1406,16 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
       tma_load_2d(stage + which * 4096, &mp[q->mi[0][MAP_OUT]], bar, ftn * p.bn + c_begin * 32, ftm * BM + quad * 32);
     };
     if (shortcut && lane == 0 && tile0 < num_tiles) fetch_shortcut(0, tm0, tn0);
+    // slabs: where this lane's tile row lies among the tile's images, rows and columns (pix_ok: an output pixel at all)
+    int pix_i = 0, pix_h = 0, pix_w = 0;
+    bool pix_ok = false;
+    if (kSlab) {
+      const int r = quad * 32 + lane;
+      pix_i = r / p.slab.img_pitch;
+      pix_h = (r - pix_i * p.slab.img_pitch) / p.slab.pitch;
+      pix_w = r - pix_i * p.slab.img_pitch - pix_h * p.slab.pitch;
+      pix_ok = pix_i < p.slab.imgs && pix_h < p.slab.rows && pix_w < p.slab.tw;
+    }
     if (CHAIN) {
       if (tile0 < total_tiles) {
         cur_seek(cur, tile0);
@@ -1211,7 +1432,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
         int gi_;
         locate(q, tile - cur.first, gi_, tm, tn);
       }
-      const int a = t & 1;
+      const int a = t & 1, a_ph = (t >> 1) & 1;
       const int row0 = tm * rows_per_tile + rank * BM + quad * 32;
       const int g = group_of(tn);
       const GroupDesc& G = q->grp[g];
@@ -1235,7 +1456,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
       // rows other CTAs produce, and they for the report, so the report goes out now.
       uint32_t rep_addr = (CHAIN && t > 0) ? rep0 + 4 * ew : 0u;
       const bool fast_inside = G.mode != EPI_GENERAL && !(row0 >= q->m || col_base >= G.n);
-      if (rep_addr && !(fast_inside && __all_sync(0xffffffffu, mbar_try_wait(tfull0 + 8 * a, (t >> 1) & 1)))) {
+      if (rep_addr && !(fast_inside && __all_sync(0xffffffffu, mbar_try_wait(tfull0 + 8 * a, a_ph)))) {
         if (lane == 0) {
           asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
           asm volatile("st.release.cta.shared::cta.u32 [%0], %1;" ::"r"(rep_addr), "r"((uint32_t)t) : "memory");
@@ -1250,13 +1471,34 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
         }
         __syncwarp();
       }
-      if (!mbar_wait(tfull0 + 8 * a, (t >> 1) & 1, abort_flag, p.err)) { ok = false; break; }
+      uint8_t* slab_dst = nullptr;     // slabs: this lane's output pixel
+      if (kSlab) {
+        const SlabDesc& sd = p.slab;
+        const int mt = PAIR ? 2 * tm + rank : tm;
+        const int wh = sd.tiles_w * sd.tiles_h, ng = mt / wh, q2 = mt - ng * wh, th = q2 / sd.tiles_w;
+        const int img = ng * sd.imgs + pix_i, oh = th * sd.rows + pix_h, ow = (q2 - th * sd.tiles_w) * sd.tw + pix_w;
+        if (pix_ok && img < sd.images && oh < p.conv.OH && ow < p.conv.OW)
+          slab_dst = reinterpret_cast<uint8_t*>(G.outs[2].ptr) + (((int64_t)img * p.conv.OH + oh) * p.conv.OW + ow) * G.outs[2].ld + col_base;
+        cs_tab[lane] = cs[0];
+        cs_tab[32 + lane] = cs[1];
+        __syncwarp();
+      }
+      if (!mbar_wait(tfull0 + 8 * a, a_ph, abort_flag, p.err)) { ok = false; break; }
       tc_fence_after();
       const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(a * kAccCols + c_begin * 32);
       const int nch = c_end - c_begin;           // 0, 1 or 2
       const int64_t row = (int64_t)row0 + lane;
       const uint32_t tempty_bar = tempty0 + 8 * a;
-      if (FL == FL_SHORTCUT) {
+      if (kSlab) {
+        if (nch == 0 || col_base >= G.n) {
+          __syncwarp();
+          if (lane == 0) { if (PAIR) mbar_arrive_leader(tempty_bar); else mbar_arrive(tempty_bar); }
+        } else {
+          const int left = (G.n - col_base) >> 5;         // whole chunks (n is a multiple of 32)
+          epilogue_slab<PAIR>(G, tbase, cs_tab, nch < left ? nch : left, slab_dst, lane, tempty_bar);
+          __syncwarp();
+        }
+      } else if (FL == FL_SHORTCUT) {
         if (nch == 0) {
           __syncwarp();
           if (lane == 0) mbar_arrive(tempty_bar);
@@ -1457,10 +1699,67 @@ bool make_im2col_map(CUtensorMap* map, const GemmArgs& g, int64_t images, int ch
   return true;
 }
 
-int make_map(Ctx* ctx, CUtensorMap* map, const void* ptr, int is_bf16, int64_t k, int64_t rows, int64_t ld, int box_rows) {
+// How a stride-1 convolution is cut into slab tiles: the cut with the fewest tiles, of those the one that loads least.
+// False: some limit of the load (256 pixels or rows per box dimension) is in the way of every cut.
+bool slab_plan(const GemmArgs& g, int64_t images, int OH, int OW, SlabDesc* best) {
+  int64_t best_tiles = 0, best_px = 0;
+  for (int tw = 1; tw <= OW && tw <= BM; ++tw) {
+    SlabDesc d{};
+    d.tw = tw;
+    d.pitch = tw + 2 - (tw < OW ? 0 : g.conv_pad < 2 ? g.conv_pad : 2);
+    d.rows = (BM - tw) / d.pitch + 1;
+    if (d.rows > OH) d.rows = OH;
+    d.tiles_w = (OW + tw - 1) / tw;
+    d.tiles_h = (OH + d.rows - 1) / d.rows;
+    d.img_pitch = (d.rows + 2) * d.pitch;
+    d.imgs = 1;
+    if (tw == OW && d.rows == OH) d.imgs = (BM - ((OH - 1) * d.pitch + tw)) / d.img_pitch + 1;
+    if (d.imgs > images) d.imgs = (int32_t)images;
+    if (d.pitch > 256 || d.rows + 2 > 256 || d.imgs > 256) continue;
+    const int64_t tiles = (int64_t)d.tiles_w * d.tiles_h * ((images + d.imgs - 1) / d.imgs), px = (int64_t)d.img_pitch * d.imgs;
+    if (best_tiles == 0 || tiles < best_tiles || (tiles == best_tiles && px < best_px)) {
+      best_tiles = tiles; best_px = px; *best = d;
+    }
+  }
+  if (best_tiles == 0 || best_tiles > 0x3fffffff) return false;
+  best->images = (int32_t)images;
+  best->chunk = g.conv_c % 128 ? 64 : 128;
+  best->chunks = g.conv_c / best->chunk;
+  best->tx_bytes = (int32_t)(best_px * best->chunk);
+  const int64_t reach = (int64_t)2 * best->pitch + 2 + BM;      // pixels the last tap's operand ends at
+  best->bytes = (int32_t)(((reach > best_px ? reach : best_px) * best->chunk + 1023) / 1024 * 1024);
+  return true;
+}
+
+// Tensor map of a convolution's NHWC code tensor for slab loads.
+bool make_slab_map(CUtensorMap* map, const GemmArgs& g, int64_t images, const SlabDesc& d) {
+  const MapKey key{g.a, (uint64_t)g.conv_c | ((uint64_t)g.conv_w << 32), (uint64_t)g.conv_h | ((uint64_t)images << 32),
+                   (uint64_t)d.pitch | ((uint64_t)(d.rows + 2) << 16) | ((uint64_t)d.imgs << 32), (uint32_t)d.chunk, 0u, 0u, 0x200u, 0u};
+  {
+    std::lock_guard<std::mutex> lock(g_map_mutex);
+    auto it = g_map_cache.find(key);
+    if (it != g_map_cache.end()) { *map = it->second; return true; }
+  }
+  const cuuint64_t px = (cuuint64_t)g.conv_c;
+  cuuint64_t dims[4] = {px, (cuuint64_t)g.conv_w, (cuuint64_t)g.conv_h, (cuuint64_t)images};
+  cuuint64_t strides[3] = {px, px * g.conv_w, px * g.conv_w * g.conv_h};
+  cuuint32_t box[4] = {(cuuint32_t)d.chunk, (cuuint32_t)d.pitch, (cuuint32_t)(d.rows + 2), (cuuint32_t)d.imgs}, estr[4] = {1, 1, 1, 1};
+  const CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(g.a), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                              d.chunk == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return false;
+  std::lock_guard<std::mutex> lock(g_map_mutex);
+  if (g_map_cache.size() >= kMapCacheMax) g_map_cache.clear();
+  g_map_cache.emplace(key, *map);
+  return true;
+}
+
+// chunk_bytes: bytes of the reduction per row of a box, and its swizzle span
+int make_map(Ctx* ctx, CUtensorMap* map, const void* ptr, int is_bf16, int64_t k, int64_t rows, int64_t ld, int box_rows, int chunk_bytes = kStageKBytes) {
   const int esz = is_bf16 ? 2 : 1;
   if (!encode_2d(map, is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, ptr, (uint64_t)k, (uint64_t)rows,
-                 (uint64_t)(ld * esz), (uint32_t)(kStageKBytes / esz), (uint32_t)box_rows, CU_TENSOR_MAP_SWIZZLE_128B,
+                 (uint64_t)(ld * esz), (uint32_t)(chunk_bytes / esz), (uint32_t)box_rows,
+                 chunk_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B))
     return set_error(ctx, QCFG_ECUDA, "cuTensorMapEncodeTiled failed");
   return QCFG_OK;
@@ -1547,7 +1846,7 @@ int gemm_init(Ctx* ctx) {
     g_encode = reinterpret_cast<EncodeTiledFn>(fn);
   }
   cudaError_t e = cudaSuccess;
-  const void* kernels[15] = {
+  const void* kernels[18] = {
       (const void*)gemm_kernel<false, false, false, false>, (const void*)gemm_kernel<false, false, true, false>,
       (const void*)gemm_kernel<false, true, false, false>,  (const void*)gemm_kernel<false, true, true, false>,
       (const void*)gemm_kernel<true, false, false, false>,  (const void*)gemm_kernel<true, false, true, false>,
@@ -1555,8 +1854,10 @@ int gemm_init(Ctx* ctx) {
       (const void*)gemm_kernel<false, true, true, true>,    (const void*)gemm_kernel<true, true, true, true>,
       (const void*)gemm_kernel<false, false, false, false, FL_CONV>, (const void*)gemm_kernel<false, true, false, false, FL_CONV>,
       (const void*)gemm_kernel<true, false, false, false, FL_CONV>,  (const void*)gemm_kernel<true, true, false, false, FL_CONV>,
-      (const void*)gemm_kernel<false, false, false, false, FL_SHORTCUT>};
-  for (int i = 0; i < 15 && e == cudaSuccess; ++i)
+      (const void*)gemm_kernel<false, false, false, false, FL_SHORTCUT>,
+      (const void*)gemm_kernel<false, false, false, false, FL_SLAB>, (const void*)gemm_kernel<false, true, false, false, FL_SLAB>,
+      (const void*)gemm_kernel<false, false, false, false, FL_SLAB64>};
+  for (int i = 0; i < 18 && e == cudaSuccess; ++i)
     e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
   if (e != cudaSuccess) return check_cuda(ctx, e, "gemm smem attribute");
   ChainState* cs = new (std::nothrow) ChainState();
@@ -1731,6 +2032,27 @@ static bool shortcut_body_pays(const GemmArgs& g, int bn, int sms) {
   return g.k <= 1280 && g.m * g.k <= (g.k <= 1024 ? (int64_t)32 << 20 : (int64_t)16 << 20);
 }
 
+// Whether a convolution goes by slabs (and how it is cut).  Integer widths only: the reduction runs chunk by chunk, tap by
+// tap inside, and only integer sums do not depend on the order.
+// By slabs / by im2col loads, us of a launch between two small ones, channels x channels, side, images:
+//   weights resident   64 56 128: 128 / 163   128 28 128: 52 / 61   64 8 128: 10.5 / 11.3   128 8 128: 12.9 / 14.0   128 28 8: 13.9 / 12.5 (56 tiles)
+//   weights streamed   256 14 128: 28.4 / 31.2   512 7 128: 25 / 27.7   512 6 128: 24.2 / 25.4 (64 tiles, 36 runs)   256 9 128: 21.3 / 21.7
+//                      256 8 128: 19.0 / 18.3 (128 tiles, 64 runs)   256 12 128: 26.2 / 21.7 (two rounds of CTA pairs in place of one)   256 14 8: 16.0 / 14.4
+static bool slab_pays(const GemmArgs& g, int sms, SlabDesc* sd) {
+  if (g.conv_kh != 3 || g.conv_kw != 3 || g.conv_stride != 1 || g.is_bf16 || g.conv_c % 64 || g.n % 32 || g.residual || g.amax || g.acc || g.y ||
+      g.slots[0].kind != 1 || g.slots[1].kind || g.slots[2].kind || ((uintptr_t)g.slots[0].ptr & 15) || g.slots[0].ld % 16)
+    return false;
+  const int OH = g.conv_h + 2 * g.conv_pad - 2, OW = g.conv_w + 2 * g.conv_pad - 2;
+  if (OH < 1 || OW < 1 || g.m % ((int64_t)OH * OW) || g.conv_pad > 127 || g.m > 0x7fffffff) return false;
+  if (!slab_plan(g, g.m / ((int64_t)OH * OW), OH, OW, sd)) return false;
+  const int64_t tiles = (int64_t)sd->tiles_w * sd->tiles_h * ((sd->images + sd->imgs - 1) / sd->imgs), runs = (g.m + BM - 1) / BM;
+  if (sd->bytes > 40 * 1024) return false;
+  if (sd->chunks == 1 && g.n <= 128) return 2 * tiles > sms && tiles <= 2 * runs;
+  const int64_t cols = (g.n + 255) / 256;
+  auto rounds = [&](int64_t t) { return ((t + 1) / 2 * cols + sms / 2 - 1) / (sms / 2); };
+  return g.n > 128 && sms > 1 && tiles * ((g.n + 127) / 128) > sms && rounds(tiles) <= rounds(runs) && 5 * tiles <= 9 * runs;
+}
+
 int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t st) {
   if (count < 1 || count > kMaxGroups) return set_error(ctx, QCFG_EINVAL, "gemm: %d groups", count);
   // While launches are being chained a record's tiles run group after group.  Of three groups,
@@ -1764,12 +2086,17 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   // shorter (a mixed 4/8/16-bit block of 768 x 3072 at 3072 tokens: 76.6 -> 74.1 us; the results do not
   // depend on the tile width).
   int bn = tile_n_of(g0.n);
+  // Slab tiles of a convolution in place of runs of 128 output pixels
+  SlabDesc sd{};
+  CUtensorMap slab_map;
+  const bool slab = count == 1 && slab_pays(g0, sm_count(ctx), &sd) && make_slab_map(&slab_map, g0, sd.images, sd);
+  const int64_t row_tiles = slab ? (int64_t)sd.tiles_w * sd.tiles_h * ((sd.images + sd.imgs - 1) / sd.imgs) : (g0.m + BM - 1) / BM;
   {
     const int sms = sm_count(ctx);
     auto ctas = [&](int width) {
       int64_t cols = 0;
       for (int i = 0; i < count; ++i) cols += (gs[i].n + width - 1) / width;
-      return cols * ((g0.m + BM - 1) / BM);
+      return cols * row_tiles;
     };
     while (bn > 32 && ctas(bn / 2) <= sms) bn /= 2;
   }
@@ -1805,7 +2132,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   p.bn = bn;
   // pair flavour (two CTAs per 256-row tile, cta_group::2) for wide outputs with at least two
   // row tiles: it halves the B bytes each SM stages per k-block
-  bool pair = ctx_pair_enabled(ctx) && bn == 256 && g0.m > BM && sm_count(ctx) >= 2;
+  bool pair = ctx_pair_enabled(ctx) && bn == 256 && (slab ? row_tiles > 1 && sd.chunk == 128 : g0.m > BM) && sm_count(ctx) >= 2;
   // ... and for wide outputs whose tiles were narrowed to 128 columns, while the pairs still have one tile each: a
   // stage is 24 KB instead of 32 and the ring one or two stages deeper (noise table of the block above:
   // 360 -> 345 us; its evaluation 66.5 -> 66.2).  A lone int8 code matrix stays with one CTA per tile, where its own body
@@ -1817,8 +2144,8 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
     pair = !codes && 2 * cols * ((g0.m + 2 * BM - 1) / (2 * BM)) <= sm_count(ctx) - 4;
   }
   const int tile_rows = pair ? 2 * BM : BM;
-  p.tiles_m = (int32_t)((g0.m + tile_rows - 1) / tile_rows);
-  const int stage_bytes = (BM + (pair ? bn / 2 : bn)) * kStageKBytes;
+  p.tiles_m = slab ? (int32_t)(pair ? (row_tiles + 1) / 2 : row_tiles) : (int32_t)((g0.m + tile_rows - 1) / tile_rows);
+  const int stage_bytes = slab ? (pair ? bn / 2 : bn) * sd.chunk : (BM + (pair ? bn / 2 : bn)) * kStageKBytes;
   p.is_bf16 = g0.is_bf16;
   // instruction descriptor: D format (F32 = 1, S32 = 2) at bit 4, A/B format (BF16 = 1, S8 = 1)
   // at bits 7 and 10, both operands K-major, N/8 at bit 17, M/16 at bit 24
@@ -1881,7 +2208,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
       G.mode = EPI_SHORTCUT;
     }
     int rc = g.conv_kh > 0 ? QCFG_OK : make_map(ctx, &maps[i * kMapsPerGroup + MAP_A], g.a, g.is_bf16, g.k, g.m, g.lda, BM);
-    if (rc == QCFG_OK) rc = make_map(ctx, &maps[i * kMapsPerGroup + MAP_B], g.b, g.is_bf16, g.k, g.n, g.ldb, pair ? bn / 2 : bn);
+    if (rc == QCFG_OK) rc = make_map(ctx, &maps[i * kMapsPerGroup + MAP_B], g.b, g.is_bf16, g.k, g.n, g.ldb, pair ? bn / 2 : bn, slab ? sd.chunk : kStageKBytes);
     if (rc != QCFG_OK) return rc;
     ops += 2.0 * (double)g.m * (double)g.n * (double)g.k;
   }
@@ -1899,7 +2226,10 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
       return set_error(ctx, QCFG_ESHAPE, "gemm: convolution rows are not a whole number of images");
     // TMA in its im2col mode where the channels come in whole 64-byte chunks, gather warps otherwise
     const int64_t images = g0.m / ((int64_t)cv.OH * cv.OW), cbytes = (int64_t)cv.C * esz;
-    if (cbytes % 128 == 0 && make_im2col_map(&maps[MAP_A], g0, images, 128)) cv.on = CONV_TMA128;
+    if (slab) {
+      maps[MAP_A] = slab_map;
+      cv.on = CONV_SLAB;
+    } else if (cbytes % 128 == 0 && make_im2col_map(&maps[MAP_A], g0, images, 128)) cv.on = CONV_TMA128;
     else if (cbytes % 64 == 0 && make_im2col_map(&maps[MAP_A], g0, images, 64)) cv.on = CONV_TMA64;
   }
   // Launches that may join a chain all take the larger staging size, so any sequence of them
@@ -1909,10 +2239,20 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   // producer's rows would cost more than the launch boundary it saves)
   const bool chainable = cs && cs->open && ctx_chain_enabled(ctx) && pair && !conv && bn == 256 && prof_mode(ctx) != 1 && p.tiles_m <= kChainMaxTilesM &&
                          2 * p.tiles_m * p.tiles_n >= sm_count(ctx);
-  p.alternate = !pair && bn == 64 && p.grp[0].mode == EPI_CODES32;
-  p.epi_bytes = shortcut ? kShortcutBytes : (wide || chainable) ? 4096 : 2048;
-  int stages = (kSmemMax - kSmemHeader - kCsBytes - 1024 - kEpiWarps * p.epi_bytes) / stage_bytes;
+  p.alternate = !pair && bn == 64 && (slab || p.grp[0].mode == EPI_CODES32);
+  p.epi_bytes = slab ? 0 : shortcut ? kShortcutBytes : (wide || chainable) ? 4096 : 2048;
+  if (slab) {
+    // three slabs, all weights if they fit beside them (they are then loaded once per CTA), else a ring of stages
+    const int room = kSmemMax - kSmemHeader - kCsBytes - 1024, blocks = 9 * sd.chunks;
+    sd.count = 3;
+    sd.resident = !pair && p.tiles_n == 1 && sd.chunks == 1 && 3 * sd.bytes + blocks * stage_bytes <= room;
+    if (sd.resident && 4 * sd.bytes + blocks * stage_bytes <= room) sd.count = kMaxSlabs;
+    p.slab = sd;
+    p.k_blocks = blocks;
+  }
+  int stages = (kSmemMax - kSmemHeader - kCsBytes - 1024 - kEpiWarps * p.epi_bytes - (slab ? sd.count * sd.bytes : 0)) / stage_bytes;
   if (stages > kMaxStages) stages = kMaxStages;
+  if (slab && sd.resident) stages = p.k_blocks;
   if (stages <= (shortcut ? 1 : kGatherDepth)) return set_error(ctx, QCFG_ESHAPE, "gemm: too few pipeline stages");
   p.stages = stages;
 
@@ -1939,7 +2279,8 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
     grid = 2 * (*cached);
     if (grid > 2 * num_tiles && !chainable) grid = 2 * num_tiles;
   } else if (grid > num_tiles) grid = num_tiles;
-  const size_t smem = (size_t)kSmemHeader + kCsBytes + 1024 + (size_t)kEpiWarps * p.epi_bytes + (size_t)stages * stage_bytes;
+  const size_t smem = (size_t)kSmemHeader + kCsBytes + 1024 + (size_t)kEpiWarps * p.epi_bytes + (size_t)stages * stage_bytes +
+                      (slab ? (size_t)sd.count * sd.bytes : 0);
   // a chain record carries only the distinct maps it uses; one that needs more runs on its own
   CUtensorMap pool[kPoolChain];
   bool fits = true;
@@ -2080,7 +2421,9 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   static const Kern conv_kernels[4] = {
       gemm_kernel<false, false, false, false, FL_CONV>, gemm_kernel<false, true, false, false, FL_CONV>,
       gemm_kernel<true, false, false, false, FL_CONV>,  gemm_kernel<true, true, false, false, FL_CONV>};
-  const Kern kern = shortcut ? gemm_kernel<false, false, false, false, FL_SHORTCUT>
+  static const Kern slab_kernels[3] = {gemm_kernel<false, false, false, false, FL_SLAB64>, gemm_kernel<false, false, false, false, FL_SLAB>,
+                                       gemm_kernel<false, true, false, false, FL_SLAB>};
+  const Kern kern = slab ? slab_kernels[sd.chunk == 64 ? 0 : pair ? 2 : 1] : shortcut ? gemm_kernel<false, false, false, false, FL_SHORTCUT>
                     : conv   ? conv_kernels[(g0.is_bf16 ? 2 : 0) + (pair ? 1 : 0)]
                              : kernels[(g0.is_bf16 ? 4 : 0) + (pair ? 2 : 0) + (count > 1 ? 1 : 0)];
   p.stamp = prof_stamp(ctx, g0.is_bf16 ? 1 : 0, ops);

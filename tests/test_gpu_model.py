@@ -515,3 +515,41 @@ def test_stem_and_its_pool_match_the_oracle(ctx, c, n, h, wd, k, pad, batch, act
     finally:
         ctx.set_prefix_reuse(False)
     model.close()
+
+
+@pytest.mark.parametrize("c,n,h,wd,pad,batch", [
+    (64, 64, 56, 56, 1, 4), (64, 64, 9, 9, 1, 80), (64, 32, 11, 7, 1, 90), (128, 128, 28, 28, 1, 13), (128, 96, 5, 5, 2, 230), (64, 64, 130, 6, 1, 13),
+    (64, 32, 8, 8, 0, 160), (256, 256, 14, 14, 1, 128), (256, 256, 14, 14, 1, 77), (512, 512, 7, 7, 1, 129), (192, 288, 13, 17, 0, 30), (64, 320, 6, 140, 1, 8),
+    (128, 160, 28, 28, 1, 11), (64, 256, 64, 64, 1, 5), (256, 224, 14, 14, 2, 70), (128, 128, 28, 28, 1, 2)])
+def test_convolution_by_slabs_matches_the_patch_matrix(ctx, c, n, h, wd, pad, batch):
+    """Stride-1 3x3 convolutions whose only output is their reader's int8 codes load their input once per tile.  Tiles that
+    are whole rows, parts of rows and whole images, halos shared and not, 64- and 128-byte chunks, weights resident and
+    streamed, one and several column tiles, CTA pairs with an odd last tile; few tiles stay with the other kernel: codes
+    bit for bit."""
+    L = wl.Layer
+    kh = kw = 3
+    oh, ow = h + 2 * pad - kh + 1, wd + 2 * pad - kw + 1
+    layers = [L("in", c, 16, src=-1, kh=1, kw=1, stride=1, in_h=h, in_w=wd, in_c=16, src_h=h, src_w=wd),
+              L("conv", n, kh * kw * c, src=0, act=orc.ACT_RELU, kh=kh, kw=kw, stride=1, pad=pad, in_h=h, in_w=wd, in_c=c, src_h=h, src_w=wd),
+              L("out", 16, n, src=1, kh=1, kw=1, stride=1, in_h=oh, in_w=ow, in_c=n, src_h=oh, src_w=ow)]
+    rng = np.random.default_rng(c + n + h)
+    x = rng.standard_normal((batch, h, wd, 16)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("conv", 1, layers, batch, x, ws)
+    model, xd = build(ctx, w)
+    rows = batch * oh * ow
+    for bits in ([8, 8, 8], [8, 5, 4]):
+        outs, codes = [], []
+        for implicit in (True, False):
+            ctx.set_implicit_conv(implicit)
+            y = torch.full((rows, 16), float("nan"), device="cuda")
+            model.eval_config(bits, xd, batch, [None, None, y])
+            qx = torch.zeros((rows, n), dtype=torch.int8, device="cuda")
+            model.debug_dump(2, qx, None, None)
+            ctx.check_sync()
+            outs.append(y)
+            codes.append(qx)
+        ctx.set_implicit_conv(True)
+        assert torch.equal(codes[0], codes[1]) and torch.equal(outs[0], outs[1])
+        assert codes[0].any()
+    model.close()
