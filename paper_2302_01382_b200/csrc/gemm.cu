@@ -849,16 +849,30 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     return GROUPED ? (int)(tn >= q->grp[1].tn_begin) + (int)(tn >= q->grp[2].tn_begin) : 0;
   };
   auto tile_in_group = [&](int tn, int g) -> int { return GROUPED ? tn - q->grp[g].tn_begin : tn; };
-  // Tiles are numbered with the row-tile index fastest.  Each role walks its tiles by adding the
+  // Tiles are numbered with the row-tile index fastest, in shortcut layers with the column tile fastest: they are bound by
+  // what they move, and the column tiles of a row tile then read and write whole rows together (ResNet-50 at batch 128,
+  // sixteen such layers: 2397 us per evaluation with the row tile fastest, 2288 this way; plain and convolution launches
+  // do not differ).  Each role walks its tiles by adding the
   // stride split into (row tiles, column tiles) once here: a division per tile would sit on the
   // epilogue's and the producer's path.
+  constexpr bool kColFast = FL == FL_SHORTCUT;
   int num_tiles, step_tn, step_tm, tm0, tn0;
   auto set_record = [&](int li) {
     q = &L.rec[CHAIN ? li : 0].p;
     mp = L.rec[CHAIN ? li : 0].m;
     num_tiles = q->tiles_m * q->tiles_n;
+    if (kColFast) {
+      step_tm = tile_step / q->tiles_n; step_tn = tile_step - step_tm * q->tiles_n;
+      tn0 = tile0 % q->tiles_n; tm0 = tile0 / q->tiles_n;
+      return;
+    }
     step_tn = tile_step / q->tiles_m; step_tm = tile_step - step_tn * q->tiles_m;
     tm0 = tile0 % q->tiles_m; tn0 = tile0 / q->tiles_m;
+  };
+  // after both coordinates have been advanced by their shares of a step
+  auto wrap = [&](int& tm_, int& tn_) {
+    if (kColFast) { if (tn_ >= q->tiles_n) { tn_ -= q->tiles_n; ++tm_; } }
+    else if (tm_ >= q->tiles_m) { tm_ -= q->tiles_m; ++tn_; }
   };
   set_record(0);
   // chains: position in the launch's tile sequence
@@ -957,7 +971,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     if (++ld_kb == q->k_blocks) {
       ld_kb = 0; ld_x = 0; ld_tile += tile_step;
       ld_tm += step_tm; ld_tn += step_tn;
-      if (ld_tm >= q->tiles_m) { ld_tm -= q->tiles_m; ++ld_tn; }
+      wrap(ld_tm, ld_tn);
       set_tile_coords();
     }
   };
@@ -1350,7 +1364,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
         }
       }
       tm += step_tm; tn += step_tn;
-      if (tm >= p.tiles_m) { tm -= p.tiles_m; ++tn; }
+      wrap(tm, tn);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     while (inflight > 0) landed();
@@ -1375,10 +1389,10 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     if (alternate) {
       if (ew >> 3) {
         t = 1; tile += tile_step; tm += step_tm; tn += step_tn;
-        if (tm >= q->tiles_m) { tm -= q->tiles_m; ++tn; }
+        wrap(tm, tn);
       }
       e_step = 2 * tile_step; e_tm = 2 * step_tm; e_tn = 2 * step_tn;
-      if (e_tm >= q->tiles_m) { e_tm -= q->tiles_m; ++e_tn; }
+      wrap(e_tm, e_tn);
     }
     // Weight scales of this warp's chunks, one column per lane and chunk.  They are fetched one
     // tile ahead: when the epilogue is the longer phase the accumulator is already waiting at
@@ -1447,7 +1461,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
         if (nt < total_tiles) locate(c2.q, nt - c2.first, gi2, tm2, tn2);
         load_scales(c2.q, nt < total_tiles, tn2, sw_next);
       } else {
-        if (tm_next >= q->tiles_m) { tm_next -= q->tiles_m; ++tn_next; }
+        wrap(tm_next, tn_next);
         load_scales(q, tile + e_step < num_tiles, tn_next, sw_next);
       }
       // Chains: the previous tile is reported once its stores have completed.  When this tile's
