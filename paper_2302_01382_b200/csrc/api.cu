@@ -243,7 +243,7 @@ struct Model {
   DevBuf act_absmax_dev;           // fp32 [n_layers], filled by calibration
   std::vector<int> calib_same_as;  // layer whose calibrated maximum layer l shares (same input tensor), or -1
   DevBuf search_ref, search_out, search_partial;   // buffers of the search drivers
-  DevBuf noise_codes, noise_amax;                  // perturbed bf16 weights of one layer and its max|w|
+  DevBuf noise_codes;                              // perturbed bf16 weights of one layer
   DevBuf adj_gs, adj_gt, adj_qxt, adj_qwt, adj_dx, adj_dw, adj_grads, adj_coef;   // scale adjustment temporaries
   int64_t last_m = 0;
   // what the layers' buffers hold after the last evaluation (for prefix reuse)
@@ -1031,7 +1031,7 @@ int qcfg_model_destroy(qcfg_model* model) {
   }
   M->act_absmax_dev.release();
   M->search_ref.release(); M->search_out.release(); M->search_partial.release();
-  M->noise_codes.release(); M->noise_amax.release();
+  M->noise_codes.release();
   M->adj_gs.release(); M->adj_gt.release(); M->adj_qxt.release(); M->adj_qwt.release();
   M->adj_dx.release(); M->adj_dw.release(); M->adj_grads.release(); M->adj_coef.release();
   delete model;
@@ -1338,7 +1338,6 @@ int qcfg_noise_sensitivity(qcfg_ctx* ctx, qcfg_model* model, const float* x_dev,
   if (!rc) rc = M->search_out.ensure(c, (size_t)out_elems * 4);
   if (!rc) rc = M->search_partial.ensure(c, (size_t)(n + 1) * blocks * 16);     // sums of every layer's run, and of none
   if (!rc) rc = M->noise_codes.ensure(c, code_bytes);
-  if (!rc) rc = M->noise_amax.ensure(c, 4);
   if (rc) return rc;
   double* partial_dev = (double*)M->search_partial.p;
   std::vector<uint8_t> bits((size_t)n, 16);
@@ -1368,9 +1367,7 @@ int qcfg_noise_sensitivity(qcfg_ctx* ctx, qcfg_model* model, const float* x_dev,
     if (!noise_dev[i] || !reach[i][n - 1]) continue;      // an output it does not reach keeps distance L(x, W) - L(x, W)
     LayerState& S = M->L[i];
     // the tensor's maximum is that of its rows' maxima, which the model holds
-    rc = launch_absmax(c, (const float*)S.w_absmax.p, 1, S.d.n_out, S.d.n_out, QCFG_PER_TENSOR, (float*)M->noise_amax.p, st);
-    if (!rc) rc = launch_perturb_bf16(c, S.d.w_dev, noise_dev[i], (const float*)M->noise_amax.p, lambda, S.d.n_out, S.d.k_in,
-                                      M->noise_codes.p, S.ldk, st);
+    rc = launch_perturb_bf16(c, S.d.w_dev, noise_dev[i], (const float*)S.w_absmax.p, lambda, S.d.n_out, S.d.k_in, M->noise_codes.p, S.ldk, st);
     if (rc) break;
     M->reuse_force.assign((size_t)n, 0);
     for (int l = 0; l < n; ++l) M->reuse_force[l] = l == i || (stale[l] && !reach[i][l]);

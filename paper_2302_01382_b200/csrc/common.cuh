@@ -52,7 +52,7 @@ int launch_quantize(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_
                     const float* inv_scale_ptr, float inv_scale_val, int granularity, int bits,
                     void* q, int64_t ldq, cudaStream_t st, float* absmax = nullptr);
 
-int launch_perturb_bf16(Ctx* ctx, const float* w, const float* nu, const float* amax_dev, float lambda, int64_t rows,
+int launch_perturb_bf16(Ctx* ctx, const float* w, const float* nu, const float* row_amax, float lambda, int64_t rows,
                         int64_t cols, void* q, int64_t ldq, cudaStream_t st);
 int launch_sqdiff(Ctx* ctx, const float* y, const float* ref, int64_t n, double* partial, int blocks, cudaStream_t st);
 

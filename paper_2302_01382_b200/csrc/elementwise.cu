@@ -256,28 +256,78 @@ int launch_quantize(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_
 // bf16 operand of a weight tensor with Gaussian noise added: w + (lambda * max|w|) * nu, nu being
 // the caller's standard-normal draws; one fp32 multiply for the deviation, one for the scaled
 // draw, one add (no FMA), then round-to-nearest-even to bf16.  Columns cols..ldq-1 are zero.
+// max|w| is that of the rows' maxima, which every block folds for itself (they sit in L2; a launch of their own and the
+// clearing of its result took 5 us per layer).  HBM-bound: eight elements per thread and step, the first step's loads
+// under way while the maxima are folded; with one element per thread 768 x 3072 took 12.2 us (floor 3.6).  The noise table
+// of a BERT-base block at 3072 tokens: 344 us, 302 with this and the wider loads of sqdiff_kernel.
+template <bool VEC>
 __global__ void __launch_bounds__(256) perturb_bf16_kernel(const float* __restrict__ w, const float* __restrict__ nu,
-                                                           const float* __restrict__ amax, float lambda, int64_t rows,
+                                                           const float* __restrict__ row_amax, float lambda, int64_t rows,
                                                            int64_t cols, __nv_bfloat16* __restrict__ q, int64_t ldq) {
   pdl_entry();
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= rows * ldq) return;
-  const int64_t r = idx / ldq, c = idx - r * ldq;
-  float v = 0.0f;
-  if (c < cols) {
-    const float sigma = __fmul_rn(lambda, __ldg(amax));
-    v = __fadd_rn(__ldg(w + r * cols + c), __fmul_rn(sigma, __ldg(nu + r * cols + c)));
+  const int64_t gpr = ldq >> 3, total = rows * gpr, step = (int64_t)gridDim.x * 256;      // groups of 8 per output row
+  float wv[8], nv[8];
+  int64_t c0 = 0;
+  auto load = [&](int64_t g) {
+    const int64_t r = g / gpr;
+    c0 = (g - r * gpr) << 3;
+    const int64_t at = r * cols + c0;
+    if (VEC && c0 + 8 <= cols) {
+      const float4 a = __ldg(reinterpret_cast<const float4*>(w + at)), b = __ldg(reinterpret_cast<const float4*>(w + at) + 1);
+      const float4 c = __ldg(reinterpret_cast<const float4*>(nu + at)), d = __ldg(reinterpret_cast<const float4*>(nu + at) + 1);
+      wv[0] = a.x; wv[1] = a.y; wv[2] = a.z; wv[3] = a.w; wv[4] = b.x; wv[5] = b.y; wv[6] = b.z; wv[7] = b.w;
+      nv[0] = c.x; nv[1] = c.y; nv[2] = c.z; nv[3] = c.w; nv[4] = d.x; nv[5] = d.y; nv[6] = d.z; nv[7] = d.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const bool in = c0 + j < cols;
+        wv[j] = in ? __ldg(w + at + j) : 0.0f;
+        nv[j] = in ? __ldg(nu + at + j) : 0.0f;
+      }
+    }
+  };
+  int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (g < total) load(g);
+  __shared__ unsigned sm[8];
+  unsigned m = 0;
+  for (int64_t i = threadIdx.x; i < rows; i += 256) {
+    const unsigned a = abs_bits(__ldg(row_amax + i));
+    m = m > a ? m : a;
   }
-  q[idx] = __float2bfloat16_rn(v);
+  m = warp_max_u(m);
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = warp_max_u(sm[threadIdx.x & 7]);
+  const float sigma = __fmul_rn(lambda, __uint_as_float(m));
+  while (g < total) {
+    uint32_t o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      // a column behind the last one is zero whatever sigma is
+      const float x = c0 + 2 * j < cols ? __fadd_rn(wv[2 * j], __fmul_rn(sigma, nv[2 * j])) : 0.0f;
+      const float y = c0 + 2 * j + 1 < cols ? __fadd_rn(wv[2 * j + 1], __fmul_rn(sigma, nv[2 * j + 1])) : 0.0f;
+      const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+      o[j] = *reinterpret_cast<const uint32_t*>(&h);
+    }
+    const int64_t dst = g << 3;
+    if ((g += step) < total) load(g);
+    *reinterpret_cast<uint4*>(q + dst) = make_uint4(o[0], o[1], o[2], o[3]);
+  }
 }
 
-int launch_perturb_bf16(Ctx* ctx, const float* w, const float* nu, const float* amax_dev, float lambda, int64_t rows,
+// row_amax: max|w| of every row; q starts on 16 bytes, ldq is a multiple of 8
+int launch_perturb_bf16(Ctx* ctx, const float* w, const float* nu, const float* row_amax, float lambda, int64_t rows,
                         int64_t cols, void* q, int64_t ldq, cudaStream_t st) {
-  const int64_t total = rows * ldq;
+  const int64_t total = rows * (ldq >> 3);
   if (total == 0) return QCFG_OK;
+  int64_t blocks = (total + 255) / 256;
+  if (blocks > (int64_t)sm_count(ctx) * 6) blocks = (int64_t)sm_count(ctx) * 6;
+  __nv_bfloat16* q16 = reinterpret_cast<__nv_bfloat16*>(q);
   prof_begin(ctx, 2, st);
-  launch_pdl(perturb_bf16_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, st, w, nu, amax_dev, lambda, rows, cols,
-                                                                      reinterpret_cast<__nv_bfloat16*>(q), ldq);
+  if ((uintptr_t)w % 16 == 0 && (uintptr_t)nu % 16 == 0 && cols % 4 == 0)
+    launch_pdl(perturb_bf16_kernel<true>, dim3((unsigned)blocks), dim3(256), 0, st, w, nu, row_amax, lambda, rows, cols, q16, ldq);
+  else
+    launch_pdl(perturb_bf16_kernel<false>, dim3((unsigned)blocks), dim3(256), 0, st, w, nu, row_amax, lambda, rows, cols, q16, ldq);
   prof_end(ctx, 2, 0.0, st);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "perturb launch");
@@ -285,16 +335,33 @@ int launch_perturb_bf16(Ctx* ctx, const float* w, const float* nu, const float* 
 
 // ------------------------------------------------------------------------------- output fidelity
 
-// Per-block partial sums of (y - ref)^2 and ref^2 in fp64 (fixed grid, fixed order: deterministic).
+// Per-block partial sums of (y - ref)^2 and ref^2 in fp64 (fixed grid, fixed order: deterministic).  vec: both start on 16
+// bytes.  Four loads of four elements from each in flight per thread (3072 x 768 took 7.6 us with single loads).
 __global__ void __launch_bounds__(256) sqdiff_kernel(const float* __restrict__ y, const float* __restrict__ ref,
-                                                     int64_t n, double* __restrict__ partial) {
+                                                     int64_t n, int vec, double* __restrict__ partial) {
   pdl_entry();
   double d2 = 0.0, r2 = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double r = (double)__ldg(ref + i), d = (double)__ldg(y + i) - r;
+  auto add = [&](float yv, float rv) {
+    const double r = (double)rv, d = (double)yv - r;
     d2 += d * d;
     r2 += r * r;
+  };
+  const int64_t first = (int64_t)blockIdx.x * 256 + threadIdx.x, step = (int64_t)gridDim.x * 256, n4 = vec ? n >> 2 : 0;
+  const float4* y4 = reinterpret_cast<const float4*>(y);
+  const float4* r4 = reinterpret_cast<const float4*>(ref);
+  int64_t i = first;
+  for (; i + 3 * step < n4; i += 4 * step) {
+    float4 a[4], b[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { a[u] = __ldg(y4 + i + u * step); b[u] = __ldg(r4 + i + u * step); }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { add(a[u].x, b[u].x); add(a[u].y, b[u].y); add(a[u].z, b[u].z); add(a[u].w, b[u].w); }
   }
+  for (; i < n4; i += step) {
+    const float4 a = __ldg(y4 + i), b = __ldg(r4 + i);
+    add(a.x, b.x); add(a.y, b.y); add(a.z, b.z); add(a.w, b.w);
+  }
+  for (i = 4 * n4 + first; i < n; i += step) add(__ldg(y + i), __ldg(ref + i));
   d2 = warp_sum(d2);
   r2 = warp_sum(r2);
   __shared__ double sm[8][2];
@@ -309,7 +376,7 @@ __global__ void __launch_bounds__(256) sqdiff_kernel(const float* __restrict__ y
 
 int launch_sqdiff(Ctx* ctx, const float* y, const float* ref, int64_t n, double* partial, int blocks, cudaStream_t st) {
   prof_begin(ctx, 2, st);
-  launch_pdl(sqdiff_kernel, dim3(blocks), dim3(256), 0, st, y, ref, n, partial);
+  launch_pdl(sqdiff_kernel, dim3(blocks), dim3(256), 0, st, y, ref, n, ((uintptr_t)y | (uintptr_t)ref) % 16 == 0 ? 1 : 0, partial);
   prof_end(ctx, 2, 0.0, st);
   count_launch(ctx);
   return check_cuda(ctx, cudaGetLastError(), "fidelity launch");

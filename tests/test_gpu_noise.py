@@ -29,7 +29,16 @@ def _run(ctx, w, nus, lam):
     return np.array(e)
 
 
-@pytest.mark.parametrize("make", [lambda: wl.tiny_mlp(), lambda: wl.bert_stack(41, 333, 128, 512, 2),
+def _ragged_mlp(sizes, m):
+    """Rows that are no whole groups of four or eight elements, outputs that are no multiple of four."""
+    rng = np.random.default_rng(sum(sizes))
+    layers = wl.mlp_layers(sizes)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    return wl.Workload("ragged", 1, layers, m, rng.standard_normal((m, sizes[0])).astype(np.float32), ws)
+
+
+@pytest.mark.parametrize("make", [lambda: wl.tiny_mlp(), lambda: _ragged_mlp((37, 1030, 22, 7), 33), lambda: _ragged_mlp((2052, 1500, 9, 3), 5),
+                                  lambda: wl.bert_stack(41, 333, 128, 512, 2),
                                   lambda: wl.resnet50(seed=3, batch=2, in_hw=32, width=16, n_classes=10, blocks=(1, 1, 1, 1))])
 def test_noise_sensitivity_matches_oracle(ctx, make):
     w = make()
