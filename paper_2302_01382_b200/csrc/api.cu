@@ -566,9 +566,32 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
           if (rc) return rc;
           pooled->pre_ptr = (const float*)pooled->prebuf.p;
         }
+        // the readers' int8 codes of the pooled tensor leave with it, one matrix per grid
+        CodeSlot codes[kStemSlots] = {};
+        for (int c : S.consumers) {
+          LayerState& C = M->L[c];
+          if (!pooled || calibrate || !ctx->fuse || !dirty[c] || C.d.pool_before != QCFG_POOL_MAX3S2 || C.d.src_h != oh || C.d.src_w != ow) continue;
+          const bool rows = C.d.kh == 0 || (C.d.kh == 1 && C.d.kw == 1 && C.d.stride == 1 && C.d.pad == 0);
+          const int64_t prows = m * ((oh - 1) / 2 + 1) * ((ow - 1) / 2 + 1);
+          if (!rows || C.d.src_col0 != 0 || C.d.k_in != d.n_out || !bits_int(bits[c]) || layer_rows(M, c, m) != prows || codes_kept(c)) continue;
+          float csc = 1.0f, cinv = 1.0f;
+          act_scales(C, bits[c], &csc, &cinv);
+          int at = 0;
+          while (at < kStemSlots && codes[at].kind && !(codes[at].inv_scale == cinv && codes[at].qmax == qmax_of(bits[c]) && codes[at].ld == C.ldk)) ++at;
+          if (at == kStemSlots) continue;              // this reader quantizes for itself
+          if (!codes[at].kind) {
+            rc = C.abuf.ensure(ctx, (size_t)(prows * C.ldk) * 2);
+            if (rc) return rc;
+            codes[at] = CodeSlot{C.abuf.p, C.ldk, cinv, qmax_of(bits[c]), 1};
+          }
+          C.a_ptr = codes[at].ptr;
+          C.a_ready = true;
+          C.bits = bits[c];
+          C.pre_ptr = pooled->pre_ptr;
+        }
         if (y_out || pooled)
           rc = launch_stem(ctx, sp, m, d.in_h, d.in_w, d.in_c, S.wc[16].codes.p, S.ldk, d.n_out, d.kh, d.kw, d.pad, d.act, y_out,
-                           pooled ? (float*)pooled->prebuf.p : nullptr, st);
+                           pooled ? (float*)pooled->prebuf.p : nullptr, codes, st);
         if (!rc && tmp)
           rc = check_cuda(ctx, cudaMemcpyAsync(tmp, y_out, (size_t)(S.rows * d.n_out) * 4, cudaMemcpyDeviceToDevice, st), "stem output copy");
         if (rc) return rc;

@@ -103,14 +103,6 @@ int launch_weight_alpha(Ctx* ctx, const float* dwq, int parts, const float* w, c
 // s[i] = float(double(s[i]) - lr * g[i])
 int launch_sgd(Ctx* ctx, float* s, const double* g, double lr, int64_t n, cudaStream_t st);
 
-// ----- stem.cu -------------------------------------------------------------------------
-int stem_init(Ctx* ctx);   // per-device kernel attributes
-// Whether a 16-bit convolution runs as the stem kernel: stride 2, up to four channels, 16..64 output channels
-bool stem_capable(int64_t n, int in_h, int in_w, int in_c, int kh, int kw, int stride, int pad, int act);
-// y = act(conv(bf16(x), w)) [images*OH*OW x n] and/or pool = its 3x3/2 max-pool (padding 1); either may be null
-int launch_stem(Ctx* ctx, const float* x, int64_t images, int H, int W, int C, const void* w_bf16, int64_t ldk, int64_t n, int kh, int kw,
-                int pad, int act, float* y, float* pool, cudaStream_t st);
-
 // ----- gemm.cu ------------------------------------------------------------------------
 constexpr int kMaxSlots = 3;
 struct CodeSlot {          // one fused re-quantize output of a GEMM epilogue
@@ -152,6 +144,16 @@ int gemm_chain_flush(Ctx* ctx);
 int gemm_chain_close(Ctx* ctx);
 int gemm_chain_reset(Ctx* ctx);
 int launch_wait_timeout(Ctx* ctx, uint64_t limit_ns, cudaStream_t st);
+
+// ----- stem.cu -------------------------------------------------------------------------
+constexpr int kStemSlots = 2;
+int stem_init(Ctx* ctx);   // per-device kernel attributes
+// Whether a 16-bit convolution runs as the stem kernel: stride 2, up to four channels, 16..64 output channels
+bool stem_capable(int64_t n, int in_h, int in_w, int in_c, int kh, int kw, int stride, int pad, int act);
+// codes[kStemSlots]: int8 codes of the pooled tensor (rows of ld bytes, on 4-byte boundaries); used ones first, only with pool.
+// y = act(conv(bf16(x), w)) [images*OH*OW x n] and/or pool = its 3x3/2 max-pool (padding 1); either may be null
+int launch_stem(Ctx* ctx, const float* x, int64_t images, int H, int W, int C, const void* w_bf16, int64_t ldk, int64_t n, int kh, int kw,
+                int pad, int act, float* y, float* pool, const CodeSlot* codes, cudaStream_t st);
 
 // Programmatic dependent launch of the element-wise kernels: the kernel is scheduled while its predecessor in the
 // stream drains and orders itself with pdl_entry(), its first statement, which waits until the predecessor

@@ -17,7 +17,7 @@
 //   warp  8     MMA issuer: one of two patch tiles into one of four accumulators.
 //   warps 9..12 epilogue: activation, running maximum over output rows in registers; every second row the
 //               maxima of the row triple cross lanes through shared memory, and the pooled row leaves in 16-byte
-//               stores.
+//               stores, with its readers' int8 codes beside it (a quantize launch per reader took 19 us each).
 // What bounds it: the two phases of a row in the producers (store two input rows, meet, build the tile) and the
 // epilogue's pooled rows share the issue slots and wait on shared memory in turn; leaving any one of them
 // out saves 30 to 60 us, leaving all three out 210.
@@ -51,6 +51,7 @@ struct StemParams {
   float* y;                    // [images * OH * OW, n] or null
   float* pool;                 // [images * PH * PW, n] or null
   int32_t H, W, C, kh, kw, pad, OH, OW, PH, PW, n, ldk, act;
+  CodeSlot codes[kStemSlots];  // int8 codes of the pooled tensor for its readers (kind 1; 0: unused)
   int32_t bands, band_rows, items;
   unsigned* err;
   unsigned long long* stamp;
@@ -359,6 +360,16 @@ __global__ void __launch_bounds__(kStemThreads, 1) stem_kernel(const __grid_cons
               r.x = fmaxf(r.x, 0.0f); r.y = fmaxf(r.y, 0.0f); r.z = fmaxf(r.z, 0.0f); r.w = fmaxf(r.w, 0.0f);
             }
             *reinterpret_cast<float4*>(dst + (int64_t)i * 4) = r;
+#pragma unroll
+            for (int s = 0; s < kStemSlots; ++s) {         // as the quantize kernel rounds: clamp, half to even
+              const CodeSlot& o = p.codes[s];
+              if (!o.kind) break;
+              auto code = [&](float x) {
+                return __float_as_uint(__fadd_rn(fminf(fmaxf(__fmul_rn(x, o.inv_scale), -o.qmax), o.qmax), 12582912.0f));
+              };
+              const uint32_t lo = __byte_perm(code(r.x), code(r.y), 0x0040), hi = __byte_perm(code(r.z), code(r.w), 0x0040);
+              *reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(o.ptr) + (((int64_t)b.img * p.PH + q) * p.PW + j) * o.ld + c) = __byte_perm(lo, hi, 0x5410);
+            }
           }
         }
         ++emitted;
@@ -392,9 +403,10 @@ bool stem_capable(int64_t n, int in_h, int in_w, int in_c, int kh, int kw, int s
 }
 
 int launch_stem(Ctx* ctx, const float* x, int64_t images, int H, int W, int C, const void* w_bf16, int64_t ldk, int64_t n, int kh, int kw,
-                int pad, int act, float* y, float* pool, cudaStream_t st) {
+                int pad, int act, float* y, float* pool, const CodeSlot* codes, cudaStream_t st) {
   if (images == 0) return QCFG_OK;
   StemParams p{};
+  for (int s = 0; s < kStemSlots; ++s) p.codes[s] = codes[s];
   p.x = x; p.w = reinterpret_cast<const __nv_bfloat16*>(w_bf16); p.y = y; p.pool = pool;
   p.H = H; p.W = W; p.C = C; p.kh = kh; p.kw = kw; p.pad = pad; p.n = (int32_t)n; p.ldk = (int32_t)ldk; p.act = act;
   p.OH = (H + 2 * pad - kh) / 2 + 1; p.OW = (W + 2 * pad - kw) / 2 + 1;

@@ -553,3 +553,47 @@ def test_convolution_by_slabs_matches_the_patch_matrix(ctx, c, n, h, wd, pad, ba
         assert torch.equal(codes[0], codes[1]) and torch.equal(outs[0], outs[1])
         assert codes[0].any()
     model.close()
+
+
+def test_stem_writes_the_codes_of_its_pooled_readers(ctx):
+    """Five readers of a pooled stem on four grids, one of them 16 bit: two int8 grids leave with the pooled tensor, the
+    others quantize for themselves; outputs and codes are those of a run in which every reader does.  Then one reader's
+    width at a time changes under prefix reuse."""
+    L = wl.Layer
+    h, wd, batch, n = 37, 62, 3, 48
+    oh, ow = (h - 1) // 2 + 1, (wd - 1) // 2 + 1
+    ph, pw = (oh - 1) // 2 + 1, (ow - 1) // 2 + 1
+    reader = dict(src=0, kh=1, kw=1, stride=1, in_h=ph, in_w=pw, in_c=n, pool_before=wl.POOL_MAX3S2, src_h=oh, src_w=ow)
+    layers = [L("stem", n, 147, src=-1, act=orc.ACT_RELU, kh=7, kw=7, stride=2, pad=3, in_h=h, in_w=wd, in_c=3, src_h=h, src_w=wd)]
+    layers += [L(f"r{i}", 16 + 8 * i, n, **reader) for i in range(5)]
+    rng = np.random.default_rng(11)
+    x = rng.standard_normal((batch, h, wd, 3)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    model, xd = build(ctx, wl.Workload("stem", 1, layers, batch, x, ws))
+    rows = batch * ph * pw
+
+    def run(bits):
+        ys = [None] + [torch.full((rows, l.n_out), float("nan"), device="cuda") for l in layers[1:]]
+        model.eval_config(bits, xd, batch, ys)
+        codes = []
+        for l in range(1, 6):
+            q = torch.zeros((rows, n), dtype=torch.int8, device="cuda")
+            if bits[l] != 16:
+                model.debug_dump(l, q, None, None)
+            codes.append(q)
+        ctx.check_sync()
+        return ys[1:] + codes
+
+    want = {}
+    steps = ([16, 8, 5, 16, 3, 8], [16, 8, 5, 16, 3, 4], [16, 6, 5, 16, 3, 4], [16, 6, 5, 8, 3, 4], [16, 8, 5, 16, 3, 8])
+    ctx.set_fusion(False)
+    for bits in steps:
+        want[tuple(bits)] = run(bits)
+    ctx.set_fusion(True)
+    for reuse in (False, True):
+        ctx.set_prefix_reuse(reuse)
+        for bits in steps:
+            for a, b in zip(run(bits), want[tuple(bits)]):
+                assert torch.equal(a, b)
+    ctx.set_prefix_reuse(False)
+    model.close()
