@@ -627,7 +627,28 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
         if (b != 16) act_scales(S, b, &sc, &inv);
         if (S.implicit)      // the input tensor's own codes, NHWC; the GEMM gathers the patches
           rc = launch_quantize(ctx, sp, srows, d.in_c, sld, nullptr, inv, QCFG_PER_TENSOR, b, S.abuf.p, d.in_c, st);
-        else if (direct)
+        else if (direct && !calibrate && !layer_ev) {
+          // layers behind this one that read the same tensor on other grids get their operands from the same pass
+          CodeSlot grids[kMaxSlots] = {};
+          int count = 0;
+          grids[count++] = CodeSlot{S.abuf.p, S.ldk, inv, b == 16 ? 0.0f : qmax_of(b), b == 16 ? 2 : 1, b};
+          for (int j = l + 1; j < n && count < kMaxSlots; ++j) {
+            LayerState& T = M->L[j];
+            if (!dirty[j] || T.a_ready || T.implicit || T.rows != S.rows || !same_input(T.d, d) || is_stem(T.d, T.bits)) continue;
+            float tsc = 1.0f, tinv = 1.0f;
+            if (T.bits != 16) act_scales(T, T.bits, &tsc, &tinv);
+            bool known = false;
+            for (int i = 0; i < count; ++i) known = known || (grids[i].bits == T.bits && grids[i].inv_scale == tinv);
+            if (known) continue;                       // shares the codes of an earlier layer when its turn comes
+            rc = T.abuf.ensure(ctx, (size_t)(T.rows * T.ldk) * 2);
+            if (rc) return rc;
+            grids[count++] = CodeSlot{T.abuf.p, T.ldk, tinv, T.bits == 16 ? 0.0f : qmax_of(T.bits), T.bits == 16 ? 2 : 1, T.bits};
+            T.a_ptr = T.abuf.p;
+            T.a_ready = true;
+            T.pre_ptr = S.pre_ptr;
+          }
+          rc = launch_quantize_multi(ctx, tp, S.rows, d.k_in, sld, grids, count, S.ldk, st);
+        } else if (direct)
           rc = launch_quantize(ctx, tp, S.rows, d.k_in, sld, nullptr, inv, QCFG_PER_TENSOR, b, S.abuf.p, S.ldk, st,
                                range_pending ? (float*)M->act_absmax_dev.p + l : nullptr);
         else
@@ -1444,6 +1465,7 @@ int adjust_pass(qcfg_ctx* h, Model* M, const uint8_t* bits, const float* x_dev, 
     else { *p = M->L[d.src].yact_ptr + d.src_col0; *ld = M->L[d.src].d.n_out; }
   };
   int rc = QCFG_OK;
+  std::vector<char> ready((size_t)n, 0);            // the operand was written along with an earlier layer's
   for (int l = 0; l < n && !rc; ++l) {
     LayerState& S = M->L[l];
     const qcfg_layer& d = S.d;
@@ -1459,9 +1481,26 @@ int adjust_pass(qcfg_ctx* h, Model* M, const uint8_t* bits, const float* x_dev, 
     S.a_ptr = nullptr;
     for (int j = 0; j < l && !S.a_ptr; ++j)          // layers that read the same input with the same grid share its codes
       if (same_input(M->L[j].d, d) && bits[j] == b && (b == 16 || act_inv(M->L[j], b) == ix)) S.a_ptr = M->L[j].a_ptr;
+    if (!S.a_ptr && ready[l]) S.a_ptr = S.abuf.p;
     if (!S.a_ptr) {
-      rc = S.abuf.ensure(c, (size_t)(m * S.ldk) * 2);
-      if (!rc) rc = launch_quantize(c, xin, m, d.k_in, ldx, nullptr, ix, QCFG_PER_TENSOR, b, S.abuf.p, S.ldk, st);
+      // this layer's operand, and those of layers behind it that read the same tensor on other grids
+      CodeSlot grids[kMaxSlots] = {};
+      int count = 0;
+      for (int j = l; j < n && count < kMaxSlots && !rc; ++j) {
+        LayerState& T = M->L[j];
+        if (!same_input(T.d, d)) continue;
+        float tsc = 1.0f, tinv = 1.0f;
+        if (bits[j] != 16) act_scales(T, bits[j], &tsc, &tinv);
+        bool known = false;
+        for (int i = 0; i < count; ++i) known = known || (grids[i].bits == bits[j] && grids[i].inv_scale == tinv);
+        for (int i = 0; i < l; ++i)
+          known = known || (same_input(M->L[i].d, d) && bits[i] == bits[j] && (bits[j] == 16 || act_inv(M->L[i], bits[i]) == tinv));
+        if (known || ready[j]) continue;
+        rc = T.abuf.ensure(c, (size_t)(m * T.ldk) * 2);
+        grids[count++] = CodeSlot{T.abuf.p, T.ldk, tinv, bits[j] == 16 ? 0.0f : qmax_of(bits[j]), bits[j] == 16 ? 2 : 1, bits[j]};
+        ready[j] = 1;
+      }
+      if (!rc) rc = launch_quantize_multi(c, xin, m, d.k_in, ldx, grids, count, S.ldk, st);
       if (rc) break;
       S.a_ptr = S.abuf.p;
     }

@@ -52,6 +52,10 @@ int launch_quantize(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_
                     const float* inv_scale_ptr, float inv_scale_val, int granularity, int bits,
                     void* q, int64_t ldq, cudaStream_t st, float* absmax = nullptr);
 
+// the operands of layers on up to kMaxSlots grids, in one pass (CodeSlot::ld is not read: all have row pitch ldq)
+struct CodeSlot;
+int launch_quantize_multi(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_t ld, const CodeSlot* outs, int count, int64_t ldq, cudaStream_t st);
+
 int launch_perturb_bf16(Ctx* ctx, const float* w, const float* nu, const float* row_amax, float lambda, int64_t rows,
                         int64_t cols, void* q, int64_t ldq, cudaStream_t st);
 int launch_sqdiff(Ctx* ctx, const float* y, const float* ref, int64_t n, double* partial, int blocks, cudaStream_t st);
@@ -111,6 +115,7 @@ struct CodeSlot {          // one fused re-quantize output of a GEMM epilogue
   float inv_scale;         // consumer's calibrated pre-rounding scale
   float qmax;              // consumer's grid limit
   int kind;                // 0 = unused
+  int bits = 0;            // the grid's width (launch_quantize_multi)
 };
 struct GemmArgs {
   const void* a; int64_t lda;   // [m x lda] int8 or bf16, K-major

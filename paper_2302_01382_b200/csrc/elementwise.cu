@@ -217,6 +217,72 @@ __global__ void __launch_bounds__(256) quantize_kernel(const float* __restrict__
   }
 }
 
+// Scheduled early only up to 64 MB of input: behind a GEMM a long one streams more slowly that way, probably because its
+// blocks arrive while the SM is set up for the GEMM's shared memory and keep that set-up, with little L1, to the
+// end.  Evaluations that quantize behind a GEMM, early / not: 100352 x 1536 220.3 / 205.9 us, 100352 x 768 141.2 / 135.6,
+// 25088 x 1024 58.6 / 55.8; 12288 x 768 45.0 / 46.1.
+static bool quantize_early(int64_t rows, int64_t cols) { return rows * cols * 4 <= (int64_t)64 << 20; }
+
+// The operands of up to three layers that read one tensor on different grids, in one pass over it (columns cols..ldq-1 zero).
+// HBM-bound; a launch per grid reads the tensor again.  An evaluation of a mixed 4/8/16-bit BERT-base block at 3072 tokens,
+// two grids of its input: 58.4 us with a launch each, 55.4 this way.
+struct QuantOuts { CodeSlot o[kMaxSlots]; };
+template <int N>
+__global__ void __launch_bounds__(256) quantize_multi_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, const QuantOuts outs,
+                                                             int64_t ldq, int vec) {
+  pdl_entry();
+  const int64_t gpr = ldq >> 3, idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= rows * gpr) return;
+  const int64_t row = idx / gpr, c0 = (idx - row * gpr) << 3;
+  float v[8];
+  const float* p = x + row * ld + c0;
+  if (vec && c0 + 8 <= cols) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = (c0 + j < cols) ? __ldg(p + j) : 0.0f;
+  }
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    const CodeSlot& o = outs.o[n];
+    if (o.kind == 2) {
+      uint32_t w[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+        w[j] = *reinterpret_cast<const uint32_t*>(&h);
+      }
+      *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(o.ptr) + row * ldq + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+      uint32_t lo = 0, hi = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        lo |= (uint32_t)(quant_code(v[j], o.inv_scale, o.qmax) & 0xff) << (8 * j);
+        hi |= (uint32_t)(quant_code(v[j + 4], o.inv_scale, o.qmax) & 0xff) << (8 * j);
+      }
+      *reinterpret_cast<uint2*>(reinterpret_cast<int8_t*>(o.ptr) + row * ldq + c0) = make_uint2(lo, hi);
+    }
+  }
+}
+
+int launch_quantize_multi(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_t ld, const CodeSlot* outs, int count, int64_t ldq, cudaStream_t st) {
+  if (count == 1)
+    return launch_quantize(ctx, x, rows, cols, ld, nullptr, outs[0].inv_scale, QCFG_PER_TENSOR, outs[0].bits, outs[0].ptr, ldq, st);
+  if (count < 1 || count > kMaxSlots) return set_error(ctx, QCFG_EINVAL, "quantize: %d grids", count);
+  if (rows == 0 || ldq == 0) return QCFG_OK;
+  const int vec = ((uintptr_t)x % 16 == 0 && ld % 4 == 0) ? 1 : 0;
+  const unsigned blocks = (unsigned)((rows * (ldq >> 3) + 255) / 256);
+  QuantOuts q{};
+  for (int i = 0; i < count; ++i) q.o[i] = outs[i];
+  prof_begin(ctx, 2, st);
+  launch_pdl_if(quantize_early(rows, cols), count == 2 ? quantize_multi_kernel<2> : quantize_multi_kernel<3>, dim3(blocks), dim3(256), 0, st, x, rows, cols, ld,
+                q, ldq, vec);
+  prof_end(ctx, 2, 0.0, st);
+  count_launch(ctx);
+  return check_cuda(ctx, cudaGetLastError(), "quantize launch");
+}
+
 int launch_quantize(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_t ld,
                     const float* inv_scale_ptr, float inv_scale_val, int granularity, int bits, void* q,
                     int64_t ldq, cudaStream_t st, float* absmax) {
@@ -230,11 +296,7 @@ int launch_quantize(Ctx* ctx, const float* x, int64_t rows, int64_t cols, int64_
   const int vec = ((uintptr_t)x % 16 == 0 && ld % 4 == 0) ? 1 : 0;
   const int64_t total = rows * (ldq >> 3);
   const unsigned blocks = (unsigned)((total + 255) / 256);
-  // Scheduled early only up to 64 MB of input: behind a GEMM a long one streams more slowly that way, probably because its
-  // blocks arrive while the SM is set up for the GEMM's shared memory and keep that set-up, with little L1, to the
-  // end.  Evaluations that quantize behind a GEMM, early / not: 100352 x 1536 220.3 / 205.9 us, 100352 x 768 141.2 / 135.6,
-  // 25088 x 1024 58.6 / 55.8; 12288 x 768 45.0 / 46.1.
-  const bool early = rows * cols * 4 <= (int64_t)64 << 20;
+  const bool early = quantize_early(rows, cols);
   if (bits == 16) {
     prof_begin(ctx, 2, st);
     launch_pdl_if(early, quantize_kernel<true>, dim3(blocks), dim3(256), 0, st, x, rows, cols, ld, nullptr, 1.0f, 0, 0.0f, q, ldq, vec,

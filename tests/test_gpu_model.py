@@ -597,3 +597,25 @@ def test_stem_writes_the_codes_of_its_pooled_readers(ctx):
                 assert torch.equal(a, b)
     ctx.set_prefix_reuse(False)
     model.close()
+
+
+@pytest.mark.parametrize("m,k,off", [(33, 75, 0), (400, 96, 1), (5, 1030, 0)])
+def test_operands_on_several_grids_come_from_one_pass(ctx, m, k, off):
+    """Six layers on five grids (more than one pass writes) that read the same rows of the external input, next to one that
+    reads other columns: codes, accumulators and outputs against the oracle, rows on and off 16 bytes."""
+    import paper_2302_01382_b200 as q
+    L = wl.Layer
+    layers = [L(f"l{i}", 24 + i, k, src=-1) for i in range(6)] + [L("slice", 16, 32, src=-1, src_col0=16)]
+    rng = np.random.default_rng(m + k)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("grids", 1, layers, m, rng.standard_normal((m, k)).astype(np.float32), ws)
+    model = q.Model(ctx, layers, [dev(a) for a in ws])
+    buf = torch.zeros(m * k + 4, device="cuda")
+    x = buf[off:off + m * k].reshape(m, k)
+    x.copy_(dev(w.x))
+    model.calibrate_model(x, m)
+    act_g, w_amax = check_calibration(model, w)
+    for bits in ([8, 4, 16, 4, 5, 3, 8], [16, 16, 8, 2, 8, 6, 16]):
+        ys = run_eval(ctx, model, w, x, bits)
+        teacher_forced_check(ctx, model, w, x, bits, ys, act_g, w_amax)
+    model.close()
