@@ -790,6 +790,66 @@ __device__ __forceinline__ void epilogue_slab(const GroupDesc& G, uint32_t tbase
   }
 }
 
+// 256-column tiles of an fp32 matrix whose row pitch TMA cannot write (the only output).  The four warps of a lane quadrant
+// turn 32 rows x 128 columns together, 32 columns each, and every warp writes eight of the rows, cut where 128-byte lines
+// begin: of a row's seventeen sectors only the first and the last are written in part.  With 32 columns at a time two of five
+// were, and L2 takes those slowly (12000 x 4001 x 500 with its quantize: 99 us, 83 this way).
+// The warps meet at a named barrier, so after a wait that gave up (ok false) they go through the motions.
+template <bool BF16, bool PAIR>
+__device__ __forceinline__ void epilogue_rows(const GroupDesc& G, uint32_t tbase, const float* cs, uint32_t stage, uint32_t slot0, uint32_t slot_step, int quad,
+                                              int colgrp, int m, int row0, int col0, int lane, uint32_t tempty_bar, bool ok) {
+  const OutDesc& o = G.outs[1];
+  const int act = G.act;
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    uint32_t v[32];
+    if (ok) {
+      tmem_ld32_issue(tbase + 32 * (4 * h + colgrp), v);
+      tmem_ld_wait();
+      if (h == 1) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) { if (PAIR) mbar_arrive_leader(tempty_bar); else mbar_arrive(tempty_bar); }
+      }
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + quad) : "memory");      // the rows turned last have been read
+    if (ok) {
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        uint32_t part[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) part[i] = v[16 * p + i];
+        float2 y[8];
+        sub_values<BF16>(y, part, cs + 32 * h + 16 * p, act);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          st_shared_v4(stage + lane * 128 + (((4 * p + j) ^ (lane & 7)) << 4), __float_as_uint(y[2 * j].x), __float_as_uint(y[2 * j].y),
+                       __float_as_uint(y[2 * j + 1].x), __float_as_uint(y[2 * j + 1].y));
+      }
+    }
+    asm volatile("bar.sync %0, 128;" ::"r"(1 + quad) : "memory");
+    const int left = G.n - col0 - 128 * h, ncols = left < 128 ? left : 128;
+    if (!ok || ncols <= 0) continue;
+#pragma unroll 2
+    for (int i = 0; i < 8; ++i) {
+      const int r = 8 * colgrp + i;
+      if (row0 + r >= m) break;
+      uint32_t* out = reinterpret_cast<uint32_t*>(o.ptr) + (int64_t)(row0 + r) * o.ld + col0 + 128 * h;
+      const int c0 = lane - (int)(((uintptr_t)out >> 2) & 31);          // lanes count from the line's beginning
+      const uint32_t src = slot0 + r * 128;
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        const int c = c0 + 32 * j;
+        if (c >= 0 && c < ncols) {
+          uint32_t x;
+          asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(src + (c >> 5) * slot_step + ((((c >> 2) & 7) ^ (r & 7)) << 4) + (c & 3) * 4) : "memory");
+          out[c] = x;
+        }
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------- the kernel
 
 // One launch runs one GEMM record or, in the CHAIN flavour, up to kChainMax records one after the
@@ -807,7 +867,7 @@ __device__ __forceinline__ void epilogue_slab(const GroupDesc& G, uint32_t tbase
 // FL: what the single-GEMM flavours carry besides the plain matrix product.  Convolutions and shortcut layers have
 // instantiations of their own: their code inside the plain kernel slowed its short launches by a tenth to a fifth
 // (100352 x 128 x 512: 20.0 -> 24.5 us).
-enum : int { FL_PLAIN = 0, FL_CONV = 1, FL_SHORTCUT = 2, FL_SLAB = 3, FL_SLAB64 = 4 };
+enum : int { FL_PLAIN = 0, FL_CONV = 1, FL_SHORTCUT = 2, FL_SLAB = 3, FL_SLAB64 = 4, FL_ROWS = 5 };
 template <bool BF16, bool PAIR, bool GROUPED, bool CHAIN, int FL = FL_PLAIN>
 __global__ void __launch_bounds__(FL == FL_CONV || CHAIN ? kGemmThreadsConv : kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
@@ -1370,6 +1430,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     while (inflight > 0) landed();
   } else {
     // ------------------------------------------------------------------ epilogue
+    constexpr bool kRowsOut = FL == FL_ROWS;
     const int ew = warp - 2;
     const int quad = warp & 3;                 // TMEM lanes 32*quad .. 32*quad+31 belong to this warp
     const bool alternate = !PAIR && !GROUPED && !CHAIN && FL != FL_SHORTCUT && p.alternate;
@@ -1403,10 +1464,10 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
       const int gi = GROUPED ? (int)(tile_tn >= qq->grp[1].tn_begin) + (int)(tile_tn >= qq->grp[2].tn_begin) : 0;
       const GroupDesc& G = qq->grp[gi];
       if (!G.need_y) return;
-      const int cb = (GROUPED ? tile_tn - G.tn_begin : tile_tn) * p.bn + c_begin * 32;
+      const int cb = (GROUPED ? tile_tn - G.tn_begin : tile_tn) * p.bn + (kRowsOut ? colgrp : c_begin) * 32;
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        const int col = cb + j * 32 + lane;
+        const int col = cb + j * (kRowsOut ? 128 : 32) + lane;
         if (c_begin + j < c_end && col < G.n) w[j] = __ldg(G.scale_w + col);
       }
     };
@@ -1440,7 +1501,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
     } else {
       load_scales(q, tile < num_tiles, tn, sw_next);
     }
-    for (; tile < total_tiles && ok; tile += e_step, t += alternate ? 2 : 1) {
+    for (; tile < total_tiles && (ok || kRowsOut); tile += e_step, t += alternate ? 2 : 1) {
       if (CHAIN) {     // record of this tile, column tile fastest inside it
         cur_seek(cur, tile); q = cur.q; mp = cur.mp;
         int gi_;
@@ -1497,13 +1558,26 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
         cs_tab[32 + lane] = cs[1];
         __syncwarp();
       }
-      if (!mbar_wait(tfull0 + 8 * a, a_ph, abort_flag, p.err)) { ok = false; break; }
+      if (!mbar_wait(tfull0 + 8 * a, a_ph, abort_flag, p.err)) { ok = false; if (!kRowsOut) break; }
       tc_fence_after();
       const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(a * kAccCols + c_begin * 32);
       const int nch = c_end - c_begin;           // 0, 1 or 2
       const int64_t row = (int64_t)row0 + lane;
       const uint32_t tempty_bar = tempty0 + 8 * a;
-      if (kSlab) {
+      if (kRowsOut) {
+        ok = __all_sync(0xffffffffu, ok);
+        cs_tab[lane] = cs[0];
+        cs_tab[32 + lane] = cs[1];
+        __syncwarp();
+        if (row0 < q->m)
+          epilogue_rows<BF16, PAIR>(G, tbase - (uint32_t)(c_begin * 32), cs_tab, stage, smem_u32(epi_stage + (ew & 3) * p.epi_bytes), (uint32_t)(4 * p.epi_bytes), quad,
+                                    colgrp, q->m, row0, tn * p.bn, lane, tempty_bar, ok);
+        else if (ok) {
+          __syncwarp();
+          if (lane == 0) { if (PAIR) mbar_arrive_leader(tempty_bar); else mbar_arrive(tempty_bar); }
+        }
+        __syncwarp();
+      } else if (kSlab) {
         if (nch == 0 || col_base >= G.n) {
           __syncwarp();
           if (lane == 0) { if (PAIR) mbar_arrive_leader(tempty_bar); else mbar_arrive(tempty_bar); }
@@ -1860,7 +1934,7 @@ int gemm_init(Ctx* ctx) {
     g_encode = reinterpret_cast<EncodeTiledFn>(fn);
   }
   cudaError_t e = cudaSuccess;
-  const void* kernels[18] = {
+  const void* kernels[22] = {
       (const void*)gemm_kernel<false, false, false, false>, (const void*)gemm_kernel<false, false, true, false>,
       (const void*)gemm_kernel<false, true, false, false>,  (const void*)gemm_kernel<false, true, true, false>,
       (const void*)gemm_kernel<true, false, false, false>,  (const void*)gemm_kernel<true, false, true, false>,
@@ -1870,8 +1944,10 @@ int gemm_init(Ctx* ctx) {
       (const void*)gemm_kernel<true, false, false, false, FL_CONV>,  (const void*)gemm_kernel<true, true, false, false, FL_CONV>,
       (const void*)gemm_kernel<false, false, false, false, FL_SHORTCUT>,
       (const void*)gemm_kernel<false, false, false, false, FL_SLAB>, (const void*)gemm_kernel<false, true, false, false, FL_SLAB>,
-      (const void*)gemm_kernel<false, false, false, false, FL_SLAB64>};
-  for (int i = 0; i < 18 && e == cudaSuccess; ++i)
+      (const void*)gemm_kernel<false, false, false, false, FL_SLAB64>,
+      (const void*)gemm_kernel<false, false, false, false, FL_ROWS>, (const void*)gemm_kernel<false, true, false, false, FL_ROWS>,
+      (const void*)gemm_kernel<true, false, false, false, FL_ROWS>,  (const void*)gemm_kernel<true, true, false, false, FL_ROWS>};
+  for (int i = 0; i < 22 && e == cudaSuccess; ++i)
     e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
   if (e != cudaSuccess) return check_cuda(ctx, e, "gemm smem attribute");
   ChainState* cs = new (std::nothrow) ChainState();
@@ -2227,6 +2303,9 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
     ops += 2.0 * (double)g.m * (double)g.n * (double)g.k;
   }
   p.tiles_n = tn_total;
+  // an fp32 matrix that TMA cannot write, in whole 256-column tiles, and nothing else (narrower tiles keep the general body)
+  const bool rows_out = count == 1 && bn == 256 && g0.conv_kh == 0 && !g0.residual && !g0.amax && !p.grp[0].outs[0].kind && p.grp[0].outs[1].kind &&
+                        !p.grp[0].outs[1].tma && !p.grp[0].outs[2].kind && !p.grp[0].outs[3].kind && !p.grp[0].outs[4].kind;
   const bool conv = g0.conv_kh > 0;
   if (conv) {
     ConvDesc& cv = p.conv;
@@ -2251,7 +2330,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   ChainState* cs = static_cast<ChainState*>(chain_slot(ctx));
   // (a GEMM with fewer tiles than CTA pairs has nothing to overlap with: the wait for its
   // producer's rows would cost more than the launch boundary it saves)
-  const bool chainable = cs && cs->open && ctx_chain_enabled(ctx) && pair && !conv && bn == 256 && prof_mode(ctx) != 1 && p.tiles_m <= kChainMaxTilesM &&
+  const bool chainable = cs && cs->open && ctx_chain_enabled(ctx) && pair && !conv && !rows_out && bn == 256 && prof_mode(ctx) != 1 && p.tiles_m <= kChainMaxTilesM &&
                          2 * p.tiles_m * p.tiles_n >= sm_count(ctx);
   p.alternate = !pair && bn == 64 && (slab || p.grp[0].mode == EPI_CODES32);
   p.epi_bytes = slab ? 0 : shortcut ? kShortcutBytes : (wide || chainable) ? 4096 : 2048;
@@ -2437,7 +2516,9 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
       gemm_kernel<true, false, false, false, FL_CONV>,  gemm_kernel<true, true, false, false, FL_CONV>};
   static const Kern slab_kernels[3] = {gemm_kernel<false, false, false, false, FL_SLAB64>, gemm_kernel<false, false, false, false, FL_SLAB>,
                                        gemm_kernel<false, true, false, false, FL_SLAB>};
-  const Kern kern = slab ? slab_kernels[sd.chunk == 64 ? 0 : pair ? 2 : 1] : shortcut ? gemm_kernel<false, false, false, false, FL_SHORTCUT>
+  static const Kern rows_kernels[4] = {gemm_kernel<false, false, false, false, FL_ROWS>, gemm_kernel<false, true, false, false, FL_ROWS>,
+                                       gemm_kernel<true, false, false, false, FL_ROWS>, gemm_kernel<true, true, false, false, FL_ROWS>};
+  const Kern kern = rows_out ? rows_kernels[(g0.is_bf16 ? 2 : 0) + (pair ? 1 : 0)] : slab ? slab_kernels[sd.chunk == 64 ? 0 : pair ? 2 : 1] : shortcut ? gemm_kernel<false, false, false, false, FL_SHORTCUT>
                     : conv   ? conv_kernels[(g0.is_bf16 ? 2 : 0) + (pair ? 1 : 0)]
                              : kernels[(g0.is_bf16 ? 4 : 0) + (pair ? 2 : 0) + (count > 1 ? 1 : 0)];
   p.stamp = prof_stamp(ctx, g0.is_bf16 ? 1 : 0, ops);

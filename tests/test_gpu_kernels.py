@@ -341,6 +341,47 @@ def test_gemm_row_pitch_without_16_byte_alignment(ctx, m, n, k):
         assert (host(out)[:guard] == 7).all() and (host(out)[-guard:] == 7).all()
 
 
+@pytest.mark.parametrize("m,n,k,off", [(4099, 1001, 48, 0), (6401, 259, 32, 1), (6399, 385, 80, 2), (3000, 1030, 16, 3), (38001, 255, 16, 1), (128 * 151, 257, 96, 0)])
+@pytest.mark.parametrize("pair", [True, False])
+def test_wide_rows_without_16_byte_pitch_are_written_line_by_line(ctx, m, n, k, off, pair):
+    """256-column tiles of fp32 matrices TMA cannot write, with and without CTA pairs: row starts at every place of a
+    128-byte line, last column tiles of one to 255 columns, a last row tile of one row; bit-exact against the same
+    product into an aligned matrix, and nothing outside is written.  16-bit operands and GELU likewise."""
+    import ctypes as C
+    import paper_2302_01382_b200 as q
+    rng = np.random.default_rng(m + n + k)
+    ld, na = (k + 15) // 16 * 16, (n + 3) // 4 * 4
+    qx, qw = _codes(rng, m, k, ld), np.zeros((na, ld), np.int8)
+    qw[:n] = _codes(rng, n, k, ld)
+    sw = np.ones(na, np.float32)
+    sw[:n] = (10.0 ** rng.uniform(-4, -2, n)).astype(np.float32)
+    st = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    ctx.set_pair_tiles(pair)
+    try:
+        for bf16 in (False, True):
+            x, w = dev(qx), dev(qw)
+            if bf16:
+                x, w = x.to(torch.bfloat16) * 0.37, w.to(torch.bfloat16)
+            swd = dev(sw)
+            for act in (0, 2):
+                res = []
+                for cols, guard in ((na, 64), (n, 64 + off)):        # aligned, then the odd pitch
+                    y = torch.full((m * cols + 256,), 7.0, device="cuda")
+                    p = C.c_void_p(y.data_ptr() + 4 * guard)
+                    xp, wp = C.c_void_p(x.data_ptr()), C.c_void_p(w.data_ptr())
+                    if bf16:
+                        rc = ctx.lib.qcfg_gemm_bf16(ctx.h, xp, ld, wp, ld, m, cols, k, act, p, st)
+                    else:
+                        rc = ctx.lib.qcfg_gemm_i8(ctx.h, xp, ld, wp, ld, m, cols, k, 0.0173, C.c_void_p(swd.data_ptr()), act, p, None, st)
+                    assert rc == q.OK
+                    ctx.check_sync()
+                    assert (y[:guard] == 7).all() and (y[guard + m * cols:] == 7).all()
+                    res.append(y[guard:guard + m * cols].reshape(m, cols)[:, :n])
+                assert torch.equal(res[0].contiguous().view(torch.int32), res[1].contiguous().view(torch.int32))
+    finally:
+        ctx.set_pair_tiles(True)
+
+
 def test_gemm_i8_worst_case_magnitude(ctx):
     k = 4608
     qx = np.full((128, k), 127, np.int8)
