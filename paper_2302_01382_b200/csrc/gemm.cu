@@ -73,12 +73,13 @@ constexpr int kPoolAll = kMaxGroups * kMapsPerGroup;   // a launch of its own: e
 constexpr int kPoolChain = 8;                          // a record of a chain: the (distinct) maps it really uses
 // Epilogue bodies.  The general one handles any combination of outputs with run-time branches; the
 // two common combinations have straight-line bodies (same arithmetic, same order).
-enum : int32_t { EPI_GENERAL = 0, EPI_CODES1 = 1, EPI_Y = 2, EPI_SHORTCUT = 3, EPI_CODES32 = 4, EPI_BF16 = 5 };
+enum : int32_t { EPI_GENERAL = 0, EPI_CODES1 = 1, EPI_Y = 2, EPI_SHORTCUT = 3, EPI_CODES32 = 4, EPI_BF16 = 5, EPI_Y32 = 6 };
 // Fast bodies (256-column tiles only): EPI_CODES1 writes each warp's 32 x 64 int8 block with one
 // TMA store (64-byte rows, 64B swizzle), EPI_Y each 32 x 32 fp32 block with one (128-byte rows,
 // 128B swizzle), EPI_BF16 each warp's 32 x 64 bf16 block with one (128-byte rows, 128B swizzle), taking the maximum
 // of what it writes along in the calibration forward.  EPI_SHORTCUT (int8, one CTA per tile, at most 128 columns): fp32 shortcut in, fp32 matrix and
 // up to two int8 code matrices out.  EPI_CODES32 (one CTA per tile, fewer than 256 columns): one int8 code matrix.
+// EPI_Y32 (int8, fewer than 256 columns): the fp32 matrix.
 struct GroupDesc {
   int32_t n, tn_begin;        // columns; first column-tile index of the group in the launch's numbering
   int32_t act;
@@ -687,6 +688,38 @@ __device__ __forceinline__ void epilogue_codes32(const GroupDesc& G, const CUten
   __syncwarp();
   st_shared_v4(stage + lane * 32, w[0], w[1], w[2], w[3]);
   st_shared_v4(stage + lane * 32 + 16, w[4], w[5], w[6], w[7]);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  if (lane == 0 && inside) tma_store_2d(map, stage, col0, row0);
+}
+
+// One warp's 32 x 32 block of an int8 layer whose only output is the fp32 matrix, in tiles narrower than 256 columns (launches
+// of one tile per CTA, whose epilogue nothing hides): broadcast scales, one TMA store of 128-byte rows.  The general body
+// shuffles a scale per element and stores twice; 3072 x 768 x 3072 took 2.7 us there from the last product to the last store.
+// Two blocks of 768 at 384 rows: 60.5 us there, 59.1 here; ResNet-50 of 16 images of 64 x 64 225.8 / 221.8.  16-bit layers
+// need no scales and gain nothing.
+template <bool PAIR>
+__device__ __forceinline__ void epilogue_y32(const GroupDesc& G, const CUtensorMap* map, uint32_t tbase, const float* cs, uint32_t stage,
+                                             int row0, int col0, bool inside, int lane, uint32_t tempty_bar) {
+  uint32_t v[32];
+  tmem_ld32_issue(tbase, v);
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the last tile's store has read the slot
+  tmem_ld_wait();
+  tc_fence_before();
+  __syncwarp();
+  if (lane == 0) { if (PAIR) mbar_arrive_leader(tempty_bar); else mbar_arrive(tempty_bar); }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t part[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) part[i] = v[16 * h + i];
+    float2 y[8];
+    sub_values<false>(y, part, cs + 16 * h, G.act);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      st_shared_v4(stage + lane * 128 + (((4 * h + j) ^ (lane & 7)) << 4), __float_as_uint(y[2 * j].x), __float_as_uint(y[2 * j].y),
+                   __float_as_uint(y[2 * j + 1].x), __float_as_uint(y[2 * j + 1].y));
+  }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncwarp();
   if (lane == 0 && inside) tma_store_2d(map, stage, col0, row0);
@@ -1607,6 +1640,16 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
           }
           epilogue_codes32<BF16>(G, &mp[q->mi[0][MAP_OUT + 2]], tbase, cs_tab, stage, row0, col_base, row0 < q->m && col_base < G.n, lane, tempty_bar);
         }
+      } else if (!BF16 && FL == FL_PLAIN && !CHAIN && G.mode == EPI_Y32) {
+        if (nch == 0) {
+          __syncwarp();
+          if (lane == 0) { if (PAIR) mbar_arrive_leader(tempty_bar); else mbar_arrive(tempty_bar); }
+        } else {
+          cs_tab[lane] = cs[0];
+          __syncwarp();
+          epilogue_y32<PAIR>(G, &mp[q->mi[g][MAP_FAST]], tbase, cs_tab, stage, row0, col_base, row0 < q->m && col_base < G.n, lane, tempty_bar);
+        }
+        prev_fast = true;
       } else if (G.mode != EPI_GENERAL) {
         // fast bodies: 256-column tiles, so this warp owns 64 columns starting at col_base
         if (!fast_inside) {
@@ -2288,6 +2331,9 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
       if (!G.outs[1].kind && G.outs[2].kind == 1 && make_fast_map(&maps[i * kMapsPerGroup + MAP_FAST], G.outs[2], g.m, g.n)) G.mode = EPI_CODES1;
       else if (G.outs[1].kind && !G.outs[2].kind && make_fast_map(&maps[i * kMapsPerGroup + MAP_FAST], G.outs[1], g.m, g.n)) { G.mode = EPI_Y; wide = true; }
     }
+    if (bn < 256 && !shortcut && !g.is_bf16 && g.conv_kh == 0 && !G.residual && !G.amax && !G.outs[0].kind && G.outs[1].kind && !G.outs[2].kind && !G.outs[3].kind &&
+        !G.outs[4].kind && make_fast_map(&maps[i * kMapsPerGroup + MAP_FAST], G.outs[1], g.m, g.n))
+      G.mode = EPI_Y32;
     if (shortcut) {      // MAP_OUT, the raw accumulators' place, holds the shortcut's map
       OutDesc in{};
       in.kind = 3; in.ptr = const_cast<float*>(g.residual); in.ld = g.ldr;
