@@ -15,7 +15,7 @@
 //               channel count known every address of a pixel is an immediate (12 instructions per pixel and warp;
 //               with 16-bit loads and computed addresses the kernel took 358 us, 302 us this way).
 //   warp  8     MMA issuer: one of two patch tiles into one of four accumulators.
-//   warps 9..12 epilogue: activation, running maximum over output rows in registers; every second row the
+//   warps 9..16 epilogue: activation, running maximum over output rows in registers; every second row the
 //               maxima of the row triple cross lanes through shared memory, and the pooled row leaves in 16-byte
 //               stores, with its readers' int8 codes beside it (a quantize launch per reader took 19 us each).
 // What bounds it: the two phases of a row in the producers (store two input rows, meet, build the tile) and the
@@ -30,7 +30,11 @@ namespace qcfg {
 namespace {
 
 constexpr int kProducers = 8;                 // warps
-constexpr int kStemThreads = 32 * (kProducers + 1 + 4);
+// Two epilogue warps per lane quadrant, 32 channels each.  With one (64 running maxima in registers, spilled) an output row
+// took the epilogue 4200 of the 5500 cycles between rows and the producers waited for it: an evaluation of ResNet-50 at
+// batch 128 2272 us, 2201 with two.
+constexpr int kEpiWarps = 8;
+constexpr int kStemThreads = 32 * (kProducers + 1 + kEpiWarps);
 constexpr int kRows = 16;                     // input rows held (power of two)
 constexpr int kMaxKh = 8, kMaxW = 256;
 constexpr int kMaxK = 192, kKBlocks = kMaxK / 64;      // 128-byte k-blocks of 64 elements
@@ -92,7 +96,7 @@ __global__ void __launch_bounds__(kStemThreads, 1) stem_kernel(const __grid_cons
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kTiles; ++i) { mbar_init(full0 + 8 * i, kProducers); mbar_init(empty0 + 8 * i, 1); }
-    for (int i = 0; i < kAccs; ++i) { mbar_init(tfull0 + 8 * i, 1); mbar_init(tempty0 + 8 * i, 4); }
+    for (int i = 0; i < kAccs; ++i) { mbar_init(tfull0 + 8 * i, 1); mbar_init(tempty0 + 8 * i, kEpiWarps); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -284,9 +288,10 @@ __global__ void __launch_bounds__(kStemThreads, 1) stem_kernel(const __grid_cons
     }
   } else {
     // ------------------------------------------------------------------ epilogue
-    // The four warps meet at a named barrier, so none of them may leave early: after a wait that gave up
+    // The warps meet at a named barrier, so none of them may leave early: after a wait that gave up
     // they go through the motions without touching memory.
-    const int quad = warp & 3;
+    constexpr int kThreadsE = 32 * kEpiWarps;
+    const int quad = warp & 3, h = (warp - kProducers - 1) >> 2;      // lane quadrant and half of the channels
     const int ow = quad * 32 + lane;
     const int et = (warp - kProducers - 1) * 32 + lane;
     const float ninf = __int_as_float(0xff800000);
@@ -295,9 +300,9 @@ __global__ void __launch_bounds__(kStemThreads, 1) stem_kernel(const __grid_cons
     bool ok = true;
     for (int item = blockIdx.x; item < p.items; item += gridDim.x) {
       const Band b = band_of(p, item);
-      float m[2][32];                                     // maximum over the rows of the open triple
+      float m[32];                                        // maximum over the rows of the open triple
 #pragma unroll
-      for (int c = 0; c < 32; ++c) m[0][c] = m[1][c] = ninf;
+      for (int c = 0; c < 32; ++c) m[c] = ninf;
       for (int oh = b.oh0; oh <= b.oh1; ++oh, ++t) {
         const uint32_t a = t & (kAccs - 1);
         if (ok && !mbar_wait(tfull0 + 8 * a, (t / kAccs) & 1u, abort_flag, p.err)) ok = false;
@@ -308,49 +313,44 @@ __global__ void __launch_bounds__(kStemThreads, 1) stem_kernel(const __grid_cons
         const int q = oh >> 1;
         const bool emit = p.pool && (odd || oh == p.OH - 1) && q >= b.p0 && q < b.p1;
         float* stage = pool_rows + (emitted & 1u) * (128 * kPoolPitch) + ow * kPoolPitch;
+        uint32_t v[32];
+        if (ok) {
+          tmem_ld32_issue(tmem_base + ((uint32_t)(quad * 32) << 16) + a * 64 + 32 * h, v);
+          tmem_ld_wait();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty0 + 8 * a);
+        } else {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t v[32];
-          if (ok) {
-            tmem_ld32_issue(tmem_base + ((uint32_t)(quad * 32) << 16) + a * 64 + 32 * h, v);
-            tmem_ld_wait();
-          } else {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) v[c] = 0u;
-          }
-          if (h == 1 && ok) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty0 + 8 * a);
-          }
-          if (p.y && ok && ow < p.OW) {
-            if (p.act == QCFG_ACT_RELU) {
-#pragma unroll
-              for (int c = 0; c < 32; ++c) v[c] = __float_as_uint(fmaxf(__uint_as_float(v[c]), 0.0f));
-            }
-            float* dst = p.y + (((int64_t)b.img * p.OH + oh) * p.OW + ow) * p.n + 32 * h;
-#pragma unroll
-            for (int c = 0; c < 32; c += 4)
-              if (32 * h + c < p.n) *reinterpret_cast<uint4*>(dst + c) = make_uint4(v[c], v[c + 1], v[c + 2], v[c + 3]);
-          }
-          if (emit && ow < p.OW) {
-#pragma unroll
-            for (int c = 0; c < 32; c += 4)
-              if (32 * h + c < p.n)
-                *reinterpret_cast<float4*>(stage + 32 * h + c) =
-                    make_float4(fmaxf(m[h][c], __uint_as_float(v[c])), fmaxf(m[h][c + 1], __uint_as_float(v[c + 1])),
-                                fmaxf(m[h][c + 2], __uint_as_float(v[c + 2])), fmaxf(m[h][c + 3], __uint_as_float(v[c + 3])));
-          }
-#pragma unroll
-          for (int c = 0; c < 32; ++c) m[h][c] = odd ? __uint_as_float(v[c]) : fmaxf(m[h][c], __uint_as_float(v[c]));
+          for (int c = 0; c < 32; ++c) v[c] = 0u;
         }
+        if (p.y && ok && ow < p.OW) {
+          if (p.act == QCFG_ACT_RELU) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) v[c] = __float_as_uint(fmaxf(__uint_as_float(v[c]), 0.0f));
+          }
+          float* dst = p.y + (((int64_t)b.img * p.OH + oh) * p.OW + ow) * p.n + 32 * h;
+#pragma unroll
+          for (int c = 0; c < 32; c += 4)
+            if (32 * h + c < p.n) *reinterpret_cast<uint4*>(dst + c) = make_uint4(v[c], v[c + 1], v[c + 2], v[c + 3]);
+        }
+        if (emit && ow < p.OW) {
+#pragma unroll
+          for (int c = 0; c < 32; c += 4)
+            if (32 * h + c < p.n)
+              *reinterpret_cast<float4*>(stage + 32 * h + c) =
+                  make_float4(fmaxf(m[c], __uint_as_float(v[c])), fmaxf(m[c + 1], __uint_as_float(v[c + 1])),
+                              fmaxf(m[c + 2], __uint_as_float(v[c + 2])), fmaxf(m[c + 3], __uint_as_float(v[c + 3])));
+        }
+#pragma unroll
+        for (int c = 0; c < 32; ++c) m[c] = odd ? __uint_as_float(v[c]) : fmaxf(m[c], __uint_as_float(v[c]));
         if (!emit) continue;
         // two stages in turn: whoever writes a stage again has passed the barrier that follows its last reads
-        asm volatile("bar.sync 1, 128;" ::: "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(kThreadsE) : "memory");
         if (ok) {
           const float* row = pool_rows + (emitted & 1u) * (128 * kPoolPitch);
           float* dst = p.pool + ((int64_t)b.img * p.PH + q) * p.PW * p.n;
-          for (int i = et; i < pooled4; i += 128) {
+          for (int i = et; i < pooled4; i += kThreadsE) {
             const int j = i / n4, c = (i - j * n4) * 4;
             float4 r = *reinterpret_cast<const float4*>(row + 2 * j * kPoolPitch + c);
             if (j > 0) {
