@@ -826,7 +826,7 @@ __device__ __forceinline__ void epilogue_slab(const GroupDesc& G, uint32_t tbase
 // 256-column tiles of an fp32 matrix whose row pitch TMA cannot write (the only output).  The four warps of a lane quadrant
 // turn 32 rows x 128 columns together, 32 columns each, and every warp writes eight of the rows, cut where 128-byte lines
 // begin: of a row's seventeen sectors only the first and the last are written in part.  With 32 columns at a time two of five
-// were, and L2 takes those slowly (12000 x 4001 x 500 with its quantize: 99 us, 83 this way).
+// were, and L2 takes those slowly (12000 x 4001 x 500 with its quantize: 99.5 us, 64 this way).
 // The warps meet at a named barrier, so after a wait that gave up (ok false) they go through the motions.
 template <bool BF16, bool PAIR>
 __device__ __forceinline__ void epilogue_rows(const GroupDesc& G, uint32_t tbase, const float* cs, uint32_t stage, uint32_t slot0, uint32_t slot_step, int quad,
@@ -863,21 +863,31 @@ __device__ __forceinline__ void epilogue_rows(const GroupDesc& G, uint32_t tbase
     asm volatile("bar.sync %0, 128;" ::"r"(1 + quad) : "memory");
     const int left = G.n - col0 - 128 * h, ncols = left < 128 ? left : 128;
     if (!ok || ncols <= 0) continue;
-#pragma unroll 2
-    for (int i = 0; i < 8; ++i) {
-      const int r = 8 * colgrp + i;
-      if (row0 + r >= m) break;
-      uint32_t* out = reinterpret_cast<uint32_t*>(o.ptr) + (int64_t)(row0 + r) * o.ld + col0 + 128 * h;
-      const int c0 = lane - (int)(((uintptr_t)out >> 2) & 31);          // lanes count from the line's beginning
-      const uint32_t src = slot0 + r * 128;
+    // Two rows at a time: all their reads, then all their stores (a store behind every read waited for the read each time:
+    // 83 us for the matrix above)
+    constexpr int kBatch = 2;
+#pragma unroll 1
+    for (int i = 8 * colgrp; i < 8 * colgrp + 8; i += kBatch) {
+      uint32_t x[kBatch][5];
+      // a lane's words of a row are 32 apart, counted from the line's beginning: one place in each of the four warps' slots,
+      // begun in the slot before for lanes whose first word lies in front of the row
+      uint32_t* out = reinterpret_cast<uint32_t*>(o.ptr) + (int64_t)(row0 + i) * o.ld + col0 + 128 * h;
 #pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        const int c = c0 + 32 * j;
-        if (c >= 0 && c < ncols) {
-          uint32_t x;
-          asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x) : "r"(src + (c >> 5) * slot_step + ((((c >> 2) & 7) ^ (r & 7)) << 4) + (c & 3) * 4) : "memory");
-          out[c] = x;
-        }
+      for (int b = 0; b < kBatch; ++b) {
+        const int c0 = lane - (int)(((uintptr_t)(out + b * o.ld) >> 2) & 31), w = c0 & 31;
+        const uint32_t src = slot0 + (i + b) * 128 + (((w >> 2) ^ ((i + b) & 7)) << 4) + (w & 3) * 4 - (c0 < 0 ? slot_step : 0u);
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+          if (j == 0 ? c0 >= 0 : j < 4 || c0 < 0) asm volatile("ld.shared.b32 %0, [%1];" : "=r"(x[b][j]) : "r"(src + j * slot_step));
+      }
+#pragma unroll
+      for (int b = 0; b < kBatch; ++b) {
+        if (row0 + i + b >= m) break;
+        const int c0 = lane - (int)(((uintptr_t)(out + b * o.ld) >> 2) & 31);
+        uint32_t* at = out + b * o.ld + c0;
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+          if (c0 + 32 * j >= 0 && c0 + 32 * j < ncols) at[32 * j] = x[b][j];
       }
     }
   }
