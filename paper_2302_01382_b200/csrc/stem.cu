@@ -18,9 +18,10 @@
 //   warps 9..16 epilogue: activation, running maximum over output rows in registers; every second row the
 //               maxima of the row triple cross lanes through shared memory, and the pooled row leaves in 16-byte
 //               stores, with its readers' int8 codes beside it (a quantize launch per reader took 19 us each).
-// What bounds it: the two phases of a row in the producers (store two input rows, meet, build the tile) and the
-// epilogue's pooled rows share the issue slots and wait on shared memory in turn; leaving any one of them
-// out saves 30 to 60 us, leaving all three out 210.
+// What bounds it (128 images of 224 x 224 x 3: 238 us, 299 before the row pitch and the second epilogue warp per
+// quadrant): the producers, 3500 cycles per output row: 2000 for the patch copies through shared memory, 900 in which the
+// next rows' loads wait for the registers the stores of the last ones still read, 300 waiting for the tensor core.  The
+// epilogue takes 2400.  Seven pixels per batch, predicated loads and an unrolled MMA loop changed nothing.
 // Work items are bands of pooled rows of one image; a band repeats one output row of its neighbour.
 #include "common.cuh"
 #include "ptx.cuh"
