@@ -283,10 +283,13 @@ bool implicit_capable(const qcfg_layer& d) { return d.kh > 0 && !reads_rows_dire
 bool is_stem(const qcfg_layer& d, int bits) {
   return bits == 16 && d.kh > 0 && d.residual_from < 0 && stem_capable(d.n_out, d.in_h, d.in_w, d.in_c, d.kh, d.kw, d.stride, d.pad, d.act);
 }
+// The source's size counts where it is read as an image: it decides what a pool gives, and it is checked in the layer's turn,
+// which a layer that takes another one's operand does not have.
 bool same_input(const qcfg_layer& a, const qcfg_layer& b) {
+  const bool image = a.kh > 0 || a.pool_before != QCFG_POOL_NONE;
   return a.src == b.src && a.src_col0 == b.src_col0 && a.k_in == b.k_in && a.kh == b.kh && a.kw == b.kw &&
          a.stride == b.stride && a.pad == b.pad && a.pool_before == b.pool_before && a.in_h == b.in_h &&
-         a.in_w == b.in_w && a.in_c == b.in_c;
+         a.in_w == b.in_w && a.in_c == b.in_c && (!image || (a.src_h == b.src_h && a.src_w == b.src_w));
 }
 
 // Weight codes and per-row scales for (layer, bits); computed once and kept.

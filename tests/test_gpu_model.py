@@ -619,3 +619,30 @@ def test_operands_on_several_grids_come_from_one_pass(ctx, m, k, off):
         ys = run_eval(ctx, model, w, x, bits)
         teacher_forced_check(ctx, model, w, x, bits, ys, act_g, w_amax)
     model.close()
+
+
+def test_readers_of_one_source_in_two_geometries_have_operands_of_their_own(ctx):
+    """Two pooling readers that declare one source with transposed sizes: each pools it as it says, at equal and at different
+    widths, and a size that is not the source's is refused whatever the widths of its neighbours."""
+    import paper_2302_01382_b200 as q
+    L = wl.Layer
+    reader = dict(src=0, kh=1, kw=1, stride=1, in_h=5, in_w=7, in_c=32, pool_before=wl.POOL_MAX3S2)
+    layers = [L("in", 32, 16, src=-1, kh=1, kw=1, stride=1, in_h=10, in_w=14, in_c=16, src_h=10, src_w=14),
+              L("a", 24, 32, src_h=10, src_w=14, **reader), L("b", 20, 32, src_h=14, src_w=10, **reader),
+              L("c", 16, 32, src_h=14, src_w=10, **reader)]
+    rng = np.random.default_rng(7)
+    x = rng.standard_normal((3, 10, 14, 16)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("geometries", 1, layers, 3, x, ws)
+    model, xd = build(ctx, w)
+    act_g, w_amax = check_calibration(model, w)
+    for bits in ([8, 8, 8, 8], [8, 8, 4, 4], [8, 4, 8, 6], [16, 16, 8, 8], [8, 8, 16, 16]):
+        teacher_forced_check(ctx, model, w, xd, bits, run_eval(ctx, model, w, xd, bits), act_g, w_amax)
+    model.close()
+    for i in (1, 2, 3):
+        bad = [L(**{**vars(l), "src_w": l.src_w + 1}) if j == i else l for j, l in enumerate(layers)]
+        model = q.Model(ctx, bad, [dev(a) for a in ws])
+        with pytest.raises(q.QcfgError) as e:
+            model.calibrate_model(xd, 3)
+        assert e.value.status == q.ESHAPE
+        model.close()
