@@ -361,6 +361,20 @@ int qcfg_model_reset_scales(qcfg_model* model);
 int qcfg_debug_dump(qcfg_ctx* ctx, qcfg_model* model, int32_t layer, int8_t* qx_dev,
                     int8_t* qw_dev, int32_t* acc_dev, void* stream);
 
+/* How many GEMM launches of the context took each of these forms since it was created (HOST array
+ * of QCFG_FORMS values), so that a test can see that a case ran in the form it is meant for.   */
+enum {
+  QCFG_FORM_CONV_GATHER = 0,   /* convolution, patches copied by warps                          */
+  QCFG_FORM_CONV_IM2COL,       /* convolution, TMA im2col loads                                 */
+  QCFG_FORM_CONV_SLAB,         /* convolution by slabs, weights resident in shared memory       */
+  QCFG_FORM_CONV_STREAMED,     /* convolution by slabs, weights streamed                        */
+  QCFG_FORM_SHORTCUT,          /* shortcut layer in a body of its own                           */
+  QCFG_FORM_ROWS,              /* fp32 rows TMA cannot write, line by line                      */
+  QCFG_FORM_NARROW_FP32,       /* int8 layers with fp32 output in narrow tiles (groups count)   */
+  QCFG_FORMS
+};
+int qcfg_debug_launch_forms(qcfg_ctx* ctx, int64_t* counts_host);
+
 #ifdef __cplusplus
 }
 #endif

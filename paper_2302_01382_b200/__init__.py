@@ -18,6 +18,7 @@ OK = 0
 PER_TENSOR, PER_ROW = 0, 1
 ACT_NONE, ACT_RELU, ACT_GELU_TANH = 0, 1, 2
 SEARCH_BISECTION, SEARCH_GREEDY = 0, 1
+FORMS = ("conv_gather", "conv_im2col", "conv_slab", "conv_streamed", "shortcut", "rows", "narrow_fp32")
 STATUS_NAMES = {0: "OK", 1: "EINVAL", 2: "EBITS", 3: "ESHAPE", 4: "EALIGN", 5: "ENOMEM", 6: "ENONFINITE", 7: "EARCH",
                 8: "ECUDA", 9: "ETIMEOUT", 11: "ESTATE"}
 EINVAL, EBITS, ESHAPE, EALIGN, ENOMEM, ENONFINITE, EARCH, ECUDA, ETIMEOUT = range(1, 10)
@@ -28,7 +29,7 @@ EXPORTS = ["qcfg_create", "qcfg_destroy", "qcfg_sync_status", "qcfg_selftest_wai
            "qcfg_quant_error_sweep", "qcfg_quant_error_sweep_static", "qcfg_gemm_i8", "qcfg_gemm_i8_requant", "qcfg_gemm_bf16", "qcfg_model_create",
            "qcfg_model_destroy", "qcfg_calibrate_model", "qcfg_model_act_absmax",
            "qcfg_model_weight_absmax", "qcfg_eval_config", "qcfg_latency_table", "qcfg_config_cost", "qcfg_noise_sensitivity", "qcfg_search", "qcfg_adjust_scales", "qcfg_scale_gradients", "qcfg_model_scales",
-           "qcfg_model_reset_scales", "qcfg_debug_dump"]
+           "qcfg_model_reset_scales", "qcfg_debug_dump", "qcfg_debug_launch_forms"]
 
 
 class QcfgError(RuntimeError):
@@ -86,6 +87,7 @@ def load_library() -> C.CDLL:
         "qcfg_model_weight_absmax": [vp, i32, C.POINTER(f32)],
         "qcfg_eval_config": [vp, vp, C.POINTER(C.c_uint8), vp, i64, C.POINTER(vp), vp],
         "qcfg_debug_dump": [vp, vp, i32, vp, vp, vp, vp],
+        "qcfg_debug_launch_forms": [vp, C.POINTER(i64)],
         "qcfg_search": [vp, vp, ci, C.POINTER(i32), C.POINTER(C.c_uint8), i32, C.c_double, vp, i64, C.POINTER(C.c_uint8),
                         C.POINTER(C.c_uint8), C.POINTER(C.c_double), i32, C.POINTER(i32), vp],
         "qcfg_noise_sensitivity": [vp, vp, vp, i64, C.POINTER(C.c_void_p), C.c_float, C.POINTER(C.c_double), vp],
@@ -157,6 +159,12 @@ class Context:
 
     def launch_count(self) -> int:
         return int(self.lib.qcfg_launch_count(self.h))
+
+    def launch_forms(self) -> dict:
+        """GEMM launches of the context by the form they took (FORMS), since it was created."""
+        counts = (C.c_int64 * len(FORMS))()
+        self._check(self.lib.qcfg_debug_launch_forms(self.h, counts))
+        return dict(zip(FORMS, counts))
 
     def sync_status(self, stream=None) -> int:
         return int(self.lib.qcfg_sync_status(self.h, _stream(stream)))

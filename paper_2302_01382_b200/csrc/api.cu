@@ -21,6 +21,7 @@ struct Ctx {
   char* pin_buf = nullptr;          // pinned host memory for small results; the error word's copy comes first
   size_t pin_bytes = 0;
   int64_t launches = 0;
+  int64_t forms[QCFG_FORMS] = {0};  // GEMM launches by form
   int fuse = 1;
   int pair = 1;                     // two-CTA GEMM tiles where they apply
   int group = 1;                    // independent GEMMs of equal shape share a launch
@@ -110,6 +111,7 @@ void prof_end(Ctx* ctx, int cls, double ops, cudaStream_t st) {
 }
 
 void count_launch(Ctx* ctx, int n) { ctx->launches += n; }
+void count_form(Ctx* ctx, int form) { ctx->forms[form] += 1; }
 unsigned* err_word(Ctx* ctx) { return ctx->err_dev; }
 int sm_count(Ctx* ctx) { return ctx->sms; }
 bool ctx_pair_enabled(Ctx* ctx) { return ctx->pair != 0; }
@@ -835,6 +837,12 @@ int qcfg_selftest_wait_timeout(qcfg_ctx* ctx, uint64_t limit_ns, void* stream) {
 
 const char* qcfg_last_error(qcfg_ctx* ctx) { return ctx ? ctx->c.msg : "null context"; }
 int64_t qcfg_launch_count(qcfg_ctx* ctx) { return ctx ? ctx->c.launches : 0; }
+int qcfg_debug_launch_forms(qcfg_ctx* ctx, int64_t* counts_host) {
+  if (!ctx) return QCFG_EINVAL;
+  if (!counts_host) return set_error(&ctx->c, QCFG_EINVAL, "launch_forms: counts is null");
+  memcpy(counts_host, ctx->c.forms, sizeof(ctx->c.forms));
+  return QCFG_OK;
+}
 int qcfg_profile_enable(qcfg_ctx* ctx, int enabled) {
   if (!ctx) return QCFG_EINVAL;
   Ctx* c = &ctx->c;

@@ -16,6 +16,7 @@ struct Ctx;  // defined in api.cu
 
 // ----- context services (api.cu) ------------------------------------------------------
 void count_launch(Ctx* ctx, int n = 1);
+void count_form(Ctx* ctx, int form);     // QCFG_FORM_*
 int set_error(Ctx* ctx, int code, const char* fmt, ...);
 int check_cuda(Ctx* ctx, cudaError_t e, const char* what);
 unsigned* err_word(Ctx* ctx);

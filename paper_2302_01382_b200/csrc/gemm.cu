@@ -2175,6 +2175,20 @@ static bool shortcut_body_pays(const GemmArgs& g, int bn, int sms) {
   return g.k <= 1280 && g.m * g.k <= (g.k <= 1024 ? (int64_t)32 << 20 : (int64_t)16 << 20);
 }
 
+// The body that writes fp32 rows line by line turns whole 128-column halves of a tile and has its warps meet twice per half; the
+// general one works in 32-column chunks, with a shuffle per element at int8, and leaves more sectors half written, which costs
+// most once the output no longer fits in L2.  us per launch, general / line by line:
+//   int8    38001 x 131, k = 64: 14.2 / 16.0    75719 x 150: 20.9 / 22.5    75719 x 177: 22.5 / 22.2    38001 x 201: 16.5 / 16.5    38001 x 255: 18.4 / 16.2
+//           12000 x 513: 14.4 / 12.4    12000 x 2049: 34.5 / 30.2    12000 x 4001: 89.2 / 51.8
+//   16 bit  38001 x 131, k = 500: 15.1 / 17.5    38001 x 201: 17.2 / 17.8    38001 x 255: 18.8 / 18.4
+//           6000 x 3999 (96 MB), k = 64: 24.9 / 26.5    256: 29.6 / 31.4    500: 41.0 / 39.5    1024: 63.1 / 59.5
+//           12000 x 2049 (98 MB), k = 64: 25.2 / 26.6    256: 30.9 / 31.7    500: 45.0 / 40.8    1024: 68.4 / 60.0
+//           8231 x 3999 (132 MB), k = 64: 54.7 / 42.3    12000 x 4001 (192 MB), k = 64: 89.4 / 47.1    500: 91.7 / 74.7
+static bool rows_body_pays(const GemmArgs& g) {
+  if (g.n <= (g.is_bf16 ? 208 : 176)) return false;      // few columns of the second half
+  return !g.is_bf16 || g.k >= 500 || 4 * g.m * g.n > (int64_t)96 << 20;
+}
+
 // Whether a convolution goes by slabs (and how it is cut).  Integer widths only: the reduction runs chunk by chunk, tap by
 // tap inside, and only integer sums do not depend on the order.
 // By slabs / by im2col loads, us of a launch between two small ones, channels x channels, side, images:
@@ -2360,7 +2374,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   }
   p.tiles_n = tn_total;
   // an fp32 matrix that TMA cannot write, in whole 256-column tiles, and nothing else (narrower tiles keep the general body)
-  const bool rows_out = count == 1 && bn == 256 && g0.conv_kh == 0 && !g0.residual && !g0.amax && !p.grp[0].outs[0].kind && p.grp[0].outs[1].kind &&
+  const bool rows_out = count == 1 && bn == 256 && rows_body_pays(g0) && g0.conv_kh == 0 && !g0.residual && !g0.amax && !p.grp[0].outs[0].kind && p.grp[0].outs[1].kind &&
                         !p.grp[0].outs[1].tma && !p.grp[0].outs[2].kind && !p.grp[0].outs[3].kind && !p.grp[0].outs[4].kind;
   const bool conv = g0.conv_kh > 0;
   if (conv) {
@@ -2577,6 +2591,10 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   const Kern kern = rows_out ? rows_kernels[(g0.is_bf16 ? 2 : 0) + (pair ? 1 : 0)] : slab ? slab_kernels[sd.chunk == 64 ? 0 : pair ? 2 : 1] : shortcut ? gemm_kernel<false, false, false, false, FL_SHORTCUT>
                     : conv   ? conv_kernels[(g0.is_bf16 ? 2 : 0) + (pair ? 1 : 0)]
                              : kernels[(g0.is_bf16 ? 4 : 0) + (pair ? 2 : 0) + (count > 1 ? 1 : 0)];
+  if (conv) count_form(ctx, p.conv.on == CONV_GATHER ? QCFG_FORM_CONV_GATHER : !slab ? QCFG_FORM_CONV_IM2COL : sd.resident ? QCFG_FORM_CONV_SLAB : QCFG_FORM_CONV_STREAMED);
+  if (shortcut) count_form(ctx, QCFG_FORM_SHORTCUT);
+  if (rows_out) count_form(ctx, QCFG_FORM_ROWS);
+  for (int i = 0; i < count; ++i) if (p.grp[i].mode == EPI_Y32) count_form(ctx, QCFG_FORM_NARROW_FP32);
   p.stamp = prof_stamp(ctx, g0.is_bf16 ? 1 : 0, ops);
   static thread_local LaunchArgs<false> one;
   memcpy(one.rec[0].m, maps, sizeof(maps));

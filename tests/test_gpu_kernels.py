@@ -382,6 +382,28 @@ def test_wide_rows_without_16_byte_pitch_are_written_line_by_line(ctx, m, n, k, 
         ctx.set_pair_tiles(True)
 
 
+@pytest.mark.parametrize("m,n,k,bf16,rows", [
+    (10001, 175, 48, False, False), (10001, 177, 48, False, True), (10001, 207, 500, True, False), (10001, 209, 500, True, True),
+    (10001, 209, 499, True, False), (12093, 2081, 16, True, False), (12100, 2081, 16, True, True)])
+def test_rows_written_line_by_line_where_that_pays(ctx, m, n, k, bf16, rows):
+    """Both sides of the rule that chooses the body for fp32 rows TMA cannot write: the body it names runs, with the bits of
+    the same product into an aligned matrix."""
+    rng = np.random.default_rng(n + k)
+    ld, na = (k + 15) // 16 * 16, (n + 3) // 4 * 4
+    x, w = dev(_codes(rng, m, k, ld)), torch.zeros((na, ld), dtype=torch.int8, device="cuda")
+    w[:n] = dev(_codes(rng, n, k, ld))
+    sw = torch.linspace(1e-4, 1e-2, na, device="cuda")
+    if bf16:
+        x, w = x.to(torch.bfloat16) * 0.37, w.to(torch.bfloat16)
+    res = []
+    for cols in (na, n):
+        before = ctx.launch_forms()["rows"]
+        res.append(ctx.gemm_bf16(x, w[:cols], k) if bf16 else ctx.gemm_i8(x, w[:cols], k, 0.0173, sw[:cols])[0])
+        ctx.check_sync()
+        assert ctx.launch_forms()["rows"] - before == (1 if rows and cols == n else 0)
+    assert torch.equal(res[0][:, :n].contiguous().view(torch.int32), res[1].view(torch.int32))
+
+
 def test_gemm_i8_worst_case_magnitude(ctx):
     k = 4608
     qx = np.full((128, k), 127, np.int8)
