@@ -123,6 +123,7 @@ struct SlabDesc {
   int32_t resident;                     // one chunk, one column tile: all weights stay in shared memory, a stage (and barrier) per tap
 };
 constexpr int kMaxSlabs = 4;
+constexpr int kSlabRoom = kSmemMax - kSmemHeader - kCsBytes - 1024;      // shared memory for slabs and weights
 constexpr int kMaxDeps = 4;
 struct GemmParams {
   int32_t m, k_blocks, bn, tiles_m, tiles_n, stages, is_bf16;   // tiles_n: column tiles of all groups together
@@ -2195,6 +2196,8 @@ static bool rows_body_pays(const GemmArgs& g) {
 //   weights resident   64 56 128: 128 / 163   128 28 128: 52 / 61   64 8 128: 10.5 / 11.3   128 8 128: 12.9 / 14.0   128 28 8: 13.9 / 12.5 (56 tiles)
 //   weights streamed   256 14 128: 28.4 / 31.2   512 7 128: 25 / 27.7   512 6 128: 24.2 / 25.4 (64 tiles, 36 runs)   256 9 128: 21.3 / 21.7
 //                      256 8 128: 19.0 / 18.3 (128 tiles, 64 runs)   256 12 128: 26.2 / 21.7 (two rounds of CTA pairs in place of one)   256 14 8: 16.0 / 14.4
+//   ... of 128 columns or fewer (three slabs of the cut leave the weights no room): 128 40 32: 38.5 / 35.2   128 40 128: 110.0 / 104.6   128 -> 96 40 64: 67.6 / 65.9
+//   so such a convolution goes by slabs only with its weights resident.  Streamed without CTA pairs: 256 14 128: 39.1 / 38.7   256 40 16: 40.6 / 40.4   512 7 128: 31.6 / 30.9
 static bool slab_pays(const GemmArgs& g, int sms, SlabDesc* sd) {
   if (g.conv_kh != 3 || g.conv_kw != 3 || g.conv_stride != 1 || g.is_bf16 || g.conv_c % 64 || g.n % 32 || g.residual || g.amax || g.acc || g.y ||
       g.slots[0].kind != 1 || g.slots[1].kind || g.slots[2].kind || ((uintptr_t)g.slots[0].ptr & 15) || g.slots[0].ld % 16)
@@ -2204,7 +2207,14 @@ static bool slab_pays(const GemmArgs& g, int sms, SlabDesc* sd) {
   if (!slab_plan(g, g.m / ((int64_t)OH * OW), OH, OW, sd)) return false;
   const int64_t tiles = (int64_t)sd->tiles_w * sd->tiles_h * ((sd->images + sd->imgs - 1) / sd->imgs), runs = (g.m + BM - 1) / BM;
   if (sd->bytes > 40 * 1024) return false;
-  if (sd->chunks == 1 && g.n <= 128) return 2 * tiles > sms && tiles <= 2 * runs;
+  sd->count = 3;
+  sd->resident = sd->chunks == 1 && g.n <= 128;
+  if (sd->resident) {      // one column tile of the width tile_n_of gives: 2 * tiles > sms leaves it as it is
+    const int weights = 9 * tile_n_of(g.n) * sd->chunk;
+    if (3 * sd->bytes + weights > kSlabRoom) return false;
+    if (4 * sd->bytes + weights <= kSlabRoom) sd->count = kMaxSlabs;
+    return 2 * tiles > sms && tiles <= 2 * runs;
+  }
   const int64_t cols = (g.n + 255) / 256;
   auto rounds = [&](int64_t t) { return ((t + 1) / 2 * cols + sms / 2 - 1) / (sms / 2); };
   return g.n > 128 && sms > 1 && tiles * ((g.n + 127) / 128) > sms && rounds(tiles) <= rounds(runs) && 5 * tiles <= 9 * runs;
@@ -2405,13 +2415,9 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   p.alternate = !pair && bn == 64 && (slab || p.grp[0].mode == EPI_CODES32);
   p.epi_bytes = slab ? 0 : shortcut ? kShortcutBytes : (wide || chainable) ? 4096 : 2048;
   if (slab) {
-    // three slabs, all weights if they fit beside them (they are then loaded once per CTA), else a ring of stages
-    const int room = kSmemMax - kSmemHeader - kCsBytes - 1024, blocks = 9 * sd.chunks;
-    sd.count = 3;
-    sd.resident = !pair && p.tiles_n == 1 && sd.chunks == 1 && 3 * sd.bytes + blocks * stage_bytes <= room;
-    if (sd.resident && 4 * sd.bytes + blocks * stage_bytes <= room) sd.count = kMaxSlabs;
+    if (sd.resident && (pair || p.tiles_n != 1)) return set_error(ctx, QCFG_ESHAPE, "gemm: resident weights need one column tile");
     p.slab = sd;
-    p.k_blocks = blocks;
+    p.k_blocks = 9 * sd.chunks;
   }
   int stages = (kSmemMax - kSmemHeader - kCsBytes - 1024 - kEpiWarps * p.epi_bytes - (slab ? sd.count * sd.bytes : 0)) / stage_bytes;
   if (stages > kMaxStages) stages = kMaxStages;

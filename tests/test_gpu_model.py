@@ -646,3 +646,48 @@ def test_readers_of_one_source_in_two_geometries_have_operands_of_their_own(ctx)
             model.calibrate_model(xd, 3)
         assert e.value.status == q.ESHAPE
         model.close()
+
+
+def _conv_both_ways(ctx, c, n, h, wd, pad, batch, widths=((8, 8, 8), (8, 5, 4))):
+    """A stride-1 3x3 convolution between a 1x1 layer and a reader of its codes: codes and output with implicit convolutions
+    are those of the patch matrix, bit for bit.  Returns the forms of the implicit runs' launches."""
+    L = wl.Layer
+    oh, ow = h + 2 * pad - 2, wd + 2 * pad - 2
+    layers = [L("in", c, 16, src=-1, kh=1, kw=1, stride=1, in_h=h, in_w=wd, in_c=16, src_h=h, src_w=wd),
+              L("conv", n, 9 * c, src=0, act=orc.ACT_RELU, kh=3, kw=3, stride=1, pad=pad, in_h=h, in_w=wd, in_c=c, src_h=h, src_w=wd),
+              L("out", 16, n, src=1, kh=1, kw=1, stride=1, in_h=oh, in_w=ow, in_c=n, src_h=oh, src_w=ow)]
+    rng = np.random.default_rng(c + n + h)
+    x = rng.standard_normal((batch, h, wd, 16)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    model, xd = build(ctx, wl.Workload("conv", 1, layers, batch, x, ws))
+    rows = batch * oh * ow
+    forms = []
+    try:
+        for bits in widths:
+            got = []
+            for implicit in (True, False):
+                ctx.set_implicit_conv(implicit)
+                y = torch.full((rows, 16), float("nan"), device="cuda")
+                before = ctx.launch_forms()
+                model.eval_config(list(bits), xd, batch, [None, None, y])
+                if implicit:
+                    forms += [f for f, v in ctx.launch_forms().items() if f.startswith("conv") for _ in range(v - before[f])]
+                qx = torch.zeros((rows, n), dtype=torch.int8, device="cuda")
+                model.debug_dump(2, qx, None, None)
+                ctx.check_sync()
+                got.append((qx, y))
+            assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+            assert got[0][0].any()
+    finally:
+        ctx.set_implicit_conv(True)
+    model.close()
+    return forms
+
+
+@pytest.mark.parametrize("c,n,h,wd,batch,form", [
+    (128, 128, 40, 40, 8, "conv_im2col"), (128, 96, 40, 40, 8, "conv_im2col"), (128, 64, 40, 40, 8, "conv_slab"), (64, 128, 40, 40, 8, "conv_slab"),
+    (128, 128, 44, 44, 8, "conv_slab")])
+def test_slab_weights_of_one_column_tile_are_resident(ctx, c, n, h, wd, batch, form):
+    """A convolution of up to 128 columns goes by slabs only where its weights fit beside them: 40 x 40 x 128 is cut into slabs
+    of 27 KB, three of which leave no room for 144 KB of weights."""
+    assert _conv_both_ways(ctx, c, n, h, wd, 1, batch) == [form] * 2
