@@ -2248,6 +2248,21 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   const GemmArgs* gs = ordered;
   const GemmArgs& g0 = gs[0];
   const int esz = g0.is_bf16 ? 2 : 1;
+  for (int i = 0; i < count; ++i) {
+    const GemmArgs& g = gs[i];
+    if (g.m <= 0 || g.n <= 0 || g.k <= 0) return set_error(ctx, QCFG_ESHAPE, "gemm: m, n, k must be positive");
+    if (((uintptr_t)g.a & 15) || ((uintptr_t)g.b & 15) || (g.lda * esz) % 16 || (g.ldb * esz) % 16)
+      return set_error(ctx, QCFG_EALIGN, "gemm: operands need 16-byte aligned pointers and row strides");
+    if (g.conv_kh > 0) {
+      if (count > 1) return set_error(ctx, QCFG_EINVAL, "gemm: convolutions are launched alone");
+      if ((g.conv_c * esz) % 16 || g.lda != g.conv_c || g.k != (int64_t)g.conv_kh * g.conv_kw * g.conv_c || g.conv_stride < 1)
+        return set_error(ctx, QCFG_ESHAPE, "gemm: convolution needs channels in whole 16-byte chunks and k = kh*kw*c");
+      if (g.ldb < g.k) return set_error(ctx, QCFG_ESHAPE, "gemm: leading dimension below k");
+    } else if (g.lda < g.k || g.ldb < g.k) return set_error(ctx, QCFG_ESHAPE, "gemm: leading dimension below k");
+    if (g.m > 0x7fffffff || g.n > 0x7fffffff) return set_error(ctx, QCFG_ESHAPE, "gemm: dimension too large");
+    if (i && !gemm_groupable(g0, g)) return set_error(ctx, QCFG_EINVAL, "gemm: grouped launches need equal m, k, type and tile width");
+  }
+
   // Tile width: by the output's width, then halved while every CTA of the launch still has one tile at
   // most: a launch that fills half of the SMs or fewer is as long as one tile, and half a tile is
   // shorter (a mixed 4/8/16-bit block of 768 x 3072 at 3072 tokens: 76.6 -> 74.1 us; the results do not
@@ -2277,21 +2292,6 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
       if (g0.slots[i].kind) shortcut = shortcut && g0.slots[i].kind == 1 && aligned(g0.slots[i].ptr, g0.slots[i].ld);
     if (shortcut && bn > 128) bn = 128;
   }
-  for (int i = 0; i < count; ++i) {
-    const GemmArgs& g = gs[i];
-    if (g.m <= 0 || g.n <= 0 || g.k <= 0) return set_error(ctx, QCFG_ESHAPE, "gemm: m, n, k must be positive");
-    if (((uintptr_t)g.a & 15) || ((uintptr_t)g.b & 15) || (g.lda * esz) % 16 || (g.ldb * esz) % 16)
-      return set_error(ctx, QCFG_EALIGN, "gemm: operands need 16-byte aligned pointers and row strides");
-    if (g.conv_kh > 0) {
-      if (count > 1) return set_error(ctx, QCFG_EINVAL, "gemm: convolutions are launched alone");
-      if ((g.conv_c * esz) % 16 || g.lda != g.conv_c || g.k != (int64_t)g.conv_kh * g.conv_kw * g.conv_c || g.conv_stride < 1)
-        return set_error(ctx, QCFG_ESHAPE, "gemm: convolution needs channels in whole 16-byte chunks and k = kh*kw*c");
-      if (g.ldb < g.k) return set_error(ctx, QCFG_ESHAPE, "gemm: leading dimension below k");
-    } else if (g.lda < g.k || g.ldb < g.k) return set_error(ctx, QCFG_ESHAPE, "gemm: leading dimension below k");
-    if (g.m > 0x7fffffff || g.n > 0x7fffffff) return set_error(ctx, QCFG_ESHAPE, "gemm: dimension too large");
-    if (i && !gemm_groupable(g0, g)) return set_error(ctx, QCFG_EINVAL, "gemm: grouped launches need equal m, k, type and tile width");
-  }
-
   GemmParams p{};
   p.m = (int32_t)g0.m;
   const int64_t kbytes = g0.k * esz;
