@@ -1753,8 +1753,20 @@ struct ChainState {
   int64_t m = 0;
   size_t smem = 0;
   cudaStream_t st = nullptr;
+  const void* ready[32];          // kernels whose shared-memory limit this context has raised (make_ready)
+  int n_ready = 0;
   ChainState() { memset(&args, 0, sizeof(args)); memset(&solo, 0, sizeof(solo)); }
 };
+
+// Raises a kernel's shared-memory limit when a context first launches it, which also loads the kernel.  With all 22 flavours
+// loaded when a context is made, the first one of a process took 12.0 ms, 6.4 this way; with a block's noise table (8.9 ms in
+// place of 4.7), calibration and evaluation behind it 23.1, 21.8 this way.
+cudaError_t make_ready(ChainState* cs, const void* kern) {
+  for (int i = 0; i < cs->n_ready; ++i) if (cs->ready[i] == kern) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+  if (e == cudaSuccess && cs->n_ready < 32) cs->ready[cs->n_ready++] = kern;
+  return e;
+}
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -1987,26 +1999,9 @@ int gemm_init(Ctx* ctx) {
     else (void)cudaGetLastError();        // convolutions then keep the gather warps
     g_encode = reinterpret_cast<EncodeTiledFn>(fn);
   }
-  cudaError_t e = cudaSuccess;
-  const void* kernels[22] = {
-      (const void*)gemm_kernel<false, false, false, false>, (const void*)gemm_kernel<false, false, true, false>,
-      (const void*)gemm_kernel<false, true, false, false>,  (const void*)gemm_kernel<false, true, true, false>,
-      (const void*)gemm_kernel<true, false, false, false>,  (const void*)gemm_kernel<true, false, true, false>,
-      (const void*)gemm_kernel<true, true, false, false>,   (const void*)gemm_kernel<true, true, true, false>,
-      (const void*)gemm_kernel<false, true, true, true>,    (const void*)gemm_kernel<true, true, true, true>,
-      (const void*)gemm_kernel<false, false, false, false, FL_CONV>, (const void*)gemm_kernel<false, true, false, false, FL_CONV>,
-      (const void*)gemm_kernel<true, false, false, false, FL_CONV>,  (const void*)gemm_kernel<true, true, false, false, FL_CONV>,
-      (const void*)gemm_kernel<false, false, false, false, FL_SHORTCUT>,
-      (const void*)gemm_kernel<false, false, false, false, FL_SLAB>, (const void*)gemm_kernel<false, true, false, false, FL_SLAB>,
-      (const void*)gemm_kernel<false, false, false, false, FL_SLAB64>,
-      (const void*)gemm_kernel<false, false, false, false, FL_ROWS>, (const void*)gemm_kernel<false, true, false, false, FL_ROWS>,
-      (const void*)gemm_kernel<true, false, false, false, FL_ROWS>,  (const void*)gemm_kernel<true, true, false, false, FL_ROWS>};
-  for (int i = 0; i < 22 && e == cudaSuccess; ++i)
-    e = cudaFuncSetAttribute(kernels[i], cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-  if (e != cudaSuccess) return check_cuda(ctx, e, "gemm smem attribute");
   ChainState* cs = new (std::nothrow) ChainState();
   if (!cs) return set_error(ctx, QCFG_ENOMEM, "gemm: host allocation failed");
-  e = cudaMalloc(&cs->ring, kFlagRingBytes);
+  cudaError_t e = cudaMalloc(&cs->ring, kFlagRingBytes);
   if (e == cudaSuccess) e = cudaMemset(cs->ring, 0, kFlagRingBytes);
   if (e == cudaSuccess) e = cudaMalloc(&cs->zero, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMemset(cs->zero, 0, sizeof(unsigned));
@@ -2057,11 +2052,10 @@ int gemm_chain_flush(Ctx* ctx) {
     cfg.numAttrs = 2;
     cs->solo.rec[0].p.stamp = prof_stamp(ctx, cs->bf16 ? 1 : 0, cs->ops);
     cs->ops = 0.0;
-    cudaError_t le;
-    if (cs->bf16) le = cs->solo_grouped ? cudaLaunchKernelEx(&cfg, gemm_kernel<true, true, true, false>, cs->solo)
-                                        : cudaLaunchKernelEx(&cfg, gemm_kernel<true, true, false, false>, cs->solo);
-    else le = cs->solo_grouped ? cudaLaunchKernelEx(&cfg, gemm_kernel<false, true, true, false>, cs->solo)
-                               : cudaLaunchKernelEx(&cfg, gemm_kernel<false, true, false, false>, cs->solo);
+    const auto kern = cs->bf16 ? cs->solo_grouped ? gemm_kernel<true, true, true, false> : gemm_kernel<true, true, false, false>
+                               : cs->solo_grouped ? gemm_kernel<false, true, true, false> : gemm_kernel<false, true, false, false>;
+    cudaError_t le = make_ready(cs, (const void*)kern);
+    if (le == cudaSuccess) le = cudaLaunchKernelEx(&cfg, kern, cs->solo);
     if (le != cudaSuccess) return check_cuda(ctx, le, "gemm launch");
     count_launch(ctx);
     return check_cuda(ctx, cudaGetLastError(), "gemm launch");
@@ -2105,8 +2099,9 @@ int gemm_chain_flush(Ctx* ctx) {
   attr[2].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 3;
-  const cudaError_t le = cs->bf16 ? cudaLaunchKernelEx(&cfg, gemm_kernel<true, true, true, true>, A)
-                                  : cudaLaunchKernelEx(&cfg, gemm_kernel<false, true, true, true>, A);
+  const auto kern = cs->bf16 ? gemm_kernel<true, true, true, true> : gemm_kernel<false, true, true, true>;
+  cudaError_t le = make_ready(cs, (const void*)kern);
+  if (le == cudaSuccess) le = cudaLaunchKernelEx(&cfg, kern, A);
   A.n = 0;
   if (le == cudaErrorCooperativeLaunchTooLarge || le == cudaErrorNotSupported) {
     // The device cannot keep the whole grid resident right now (or does not take cooperative
@@ -2124,8 +2119,9 @@ int gemm_chain_flush(Ctx* ctx) {
       for (int d = 0; d < kMaxDeps; ++d) cs->solo.rec[0].p.deps[d] = -1;
       cs->solo.n = 1;
       cs->solo.total_tiles = A.rec[i].p.tiles_m * A.rec[i].p.tiles_n;
-      const cudaError_t se = cs->bf16 ? cudaLaunchKernelEx(&one, gemm_kernel<true, true, true, false>, cs->solo)
-                                      : cudaLaunchKernelEx(&one, gemm_kernel<false, true, true, false>, cs->solo);
+      const auto apart = cs->bf16 ? gemm_kernel<true, true, true, false> : gemm_kernel<false, true, true, false>;
+      cudaError_t se = make_ready(cs, (const void*)apart);
+      if (se == cudaSuccess) se = cudaLaunchKernelEx(&one, apart, cs->solo);
       if (se != cudaSuccess) return check_cuda(ctx, se, "gemm launch");
       count_launch(ctx);
     }
@@ -2408,9 +2404,10 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   // Launches that may join a chain all take the larger staging size, so any sequence of them
   // shares one shared-memory layout.
   ChainState* cs = static_cast<ChainState*>(chain_slot(ctx));
+  if (!cs) return set_error(ctx, QCFG_ESTATE, "gemm: context not initialised");
   // (a GEMM with fewer tiles than CTA pairs has nothing to overlap with: the wait for its
   // producer's rows would cost more than the launch boundary it saves)
-  const bool chainable = cs && cs->open && ctx_chain_enabled(ctx) && pair && !conv && !rows_out && bn == 256 && prof_mode(ctx) != 1 && p.tiles_m <= kChainMaxTilesM &&
+  const bool chainable = cs->open && ctx_chain_enabled(ctx) && pair && !conv && !rows_out && bn == 256 && prof_mode(ctx) != 1 && p.tiles_m <= kChainMaxTilesM &&
                          2 * p.tiles_m * p.tiles_n >= sm_count(ctx);
   p.alternate = !pair && bn == 64 && (slab || p.grp[0].mode == EPI_CODES32);
   p.epi_bytes = slab ? 0 : shortcut ? kShortcutBytes : (wide || chainable) ? 4096 : 2048;
@@ -2439,8 +2436,9 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
       qa[0].val.clusterDim.x = 2; qa[0].val.clusterDim.y = 1; qa[0].val.clusterDim.z = 1;
       q.attrs = qa; q.numAttrs = 1;
       int n = 0;
-      cudaError_t oe = g0.is_bf16 ? cudaOccupancyMaxActiveClusters(&n, gemm_kernel<true, true, true, true>, &q)
-                                  : cudaOccupancyMaxActiveClusters(&n, gemm_kernel<false, true, true, true>, &q);
+      const auto probe = g0.is_bf16 ? gemm_kernel<true, true, true, true> : gemm_kernel<false, true, true, true>;
+      cudaError_t oe = make_ready(cs, (const void*)probe);
+      if (oe == cudaSuccess) oe = cudaOccupancyMaxActiveClusters(&n, probe, &q);
       if (oe != cudaSuccess || n < 1) { (void)cudaGetLastError(); n = grid / 2; }
       if (n > grid / 2) n = grid / 2;
       *cached = n;
@@ -2483,7 +2481,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
         for (int j = 0; j < kMapsPerGroup; ++j) p.mi[i][j] = (uint8_t)(i * kMapsPerGroup + j);
   }
   const bool chained = chainable && fits;
-  if (cs && cs->args.n > 0 &&
+  if (cs->args.n > 0 &&
       (!chained || cs->args.n == kChainMax || cs->st != st || cs->bf16 != (g0.is_bf16 != 0) || cs->grid != grid ||
        cs->smem != smem || cs->m != g0.m)) {
     const int rc = gemm_chain_flush(ctx);
@@ -2607,7 +2605,8 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
   one.rec[0].p = p;
   one.n = 1; one.total_tiles = num_tiles; one.flag_stride = 0; one.flags = nullptr;
   prof_begin(ctx, g0.is_bf16 ? 1 : 0, st);
-  const cudaError_t le = cudaLaunchKernelEx(&cfg, kern, one);
+  cudaError_t le = make_ready(cs, (const void*)kern);
+  if (le == cudaSuccess) le = cudaLaunchKernelEx(&cfg, kern, one);
   prof_end(ctx, g0.is_bf16 ? 1 : 0, ops, st);
   if (le != cudaSuccess) return check_cuda(ctx, le, "gemm launch");
   count_launch(ctx);

@@ -404,6 +404,37 @@ def test_rows_written_line_by_line_where_that_pays(ctx, m, n, k, bf16, rows):
     assert torch.equal(res[0][:, :n].contiguous().view(torch.int32), res[1].view(torch.int32))
 
 
+FIRST_GEMMS = r"""
+import sys
+sys.path.insert(0, {root!r})
+import torch
+import paper_2302_01382_b200 as q
+ctx = q.Context(0)
+gen = torch.Generator(device="cuda")
+gen.manual_seed(1)
+for m, n, k in ((64, 32, 64), (1000, 1024, 256), (9000, 259, 64), (3000, 96, 64)):
+    x, w = (torch.randint(-9, 10, (r, k), dtype=torch.int8, device="cuda", generator=gen) for r in (m, n))
+    xb, wb, sw = x.to(torch.bfloat16), w.to(torch.bfloat16), torch.full((n,), 0.01, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        y, z = ctx.gemm_i8(x, w, k, 0.5, sw)[0], ctx.gemm_bf16(xb, wb, k)
+    graph.replay()
+    assert torch.equal(z, (x.double() @ w.double().T).float())
+    assert torch.equal(y, ctx.gemm_i8(x, w, k, 0.5, sw)[0]) and y.any()
+    ctx.check_sync()
+"""
+
+
+def test_first_gemms_of_a_process_can_be_captured():
+    """Kernels are set up when a context first launches them; that may be while a stream is captured."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    run = subprocess.run([sys.executable, "-c", FIRST_GEMMS.format(root=root)], capture_output=True, text=True, timeout=300)
+    assert run.returncode == 0, run.stderr
+
+
 def test_gemm_i8_worst_case_magnitude(ctx):
     k = 4608
     qx = np.full((128, k), 127, np.int8)
