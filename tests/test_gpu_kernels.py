@@ -404,6 +404,30 @@ def test_rows_written_line_by_line_where_that_pays(ctx, m, n, k, bf16, rows):
     assert torch.equal(res[0][:, :n].contiguous().view(torch.int32), res[1].view(torch.int32))
 
 
+@pytest.mark.parametrize("m,n,k", [(1, 32, 16), (129, 132, 48), (300, 36, 771), (3072, 768, 96), (3001, 764, 130), (6300, 132, 64), (2048, 1028, 3072)])
+@pytest.mark.parametrize("pair", [True, False])
+def test_narrow_fp32_tiles(ctx, m, n, k, pair):
+    """Launches of one narrow tile per CTA (or CTA pair: 3072 x 768, 3001 x 764, 6300 x 132, 2048 x 1028) with fp32 output: the bits
+    of the general body, which a raw-accumulator output asks for."""
+    import paper_2302_01382_b200 as q
+    rng = np.random.default_rng(m + n + k)
+    ld = (k + 15) // 16 * 16
+    x, w = dev(_codes(rng, m, k, ld)), dev(_codes(rng, n, k, ld))
+    sw = dev((10.0 ** rng.uniform(-4, -2, n)).astype(np.float32))
+    ctx.set_pair_tiles(pair)
+    try:
+        for act in (q.ACT_NONE, q.ACT_RELU, q.ACT_GELU_TANH):
+            before = ctx.launch_forms()["narrow_fp32"]
+            y = ctx.gemm_i8(x, w, k, 0.0173, sw, act)[0]
+            assert ctx.launch_forms()["narrow_fp32"] == before + 1
+            general, acc = ctx.gemm_i8(x, w, k, 0.0173, sw, act, want_acc=True)
+            assert ctx.launch_forms()["narrow_fp32"] == before + 1
+            ctx.check_sync()
+            assert torch.equal(y.view(torch.int32), general.view(torch.int32)) and acc.any()
+    finally:
+        ctx.set_pair_tiles(True)
+
+
 FIRST_GEMMS = r"""
 import sys
 sys.path.insert(0, {root!r})

@@ -368,6 +368,50 @@ def test_shortcut_layers_at_tile_edges(ctx, m, n):
     model.close()
 
 
+@pytest.mark.parametrize("m,n", [(9001, 516), (2500, 1156), (20000, 132)])
+def test_shortcut_tiles_column_tile_fastest(ctx, m, n):
+    """Shortcut layers of several column tiles and more tiles than SMs, so that a CTA's steps wrap in both coordinates: output
+    and codes of the body of their own are those of the general one (which a raw-accumulator tap asks for) on every row."""
+    L = wl.Layer
+    layers = [L("a", n, 32, src=-1), L("b", n, 64, src=-1, src_col0=32, act=orc.ACT_RELU, residual_from=0), L("c", 16, n, src=1)]
+    rng = np.random.default_rng(m + n)
+    x = rng.standard_normal((m, 96)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("shortcut", 1, layers, m, x, ws)
+    model, xd = build(ctx, w)
+    act_g, w_amax = check_calibration(model, w)
+    before = ctx.launch_forms()["shortcut"]
+    ys = run_eval(ctx, model, w, xd, [8, 6, 8])
+    assert ctx.launch_forms()["shortcut"] == before + 1
+    teacher_forced_check(ctx, model, w, xd, [8, 6, 8], ys, act_g, w_amax)
+    model.close()
+
+
+@pytest.mark.parametrize("pair", [True, False])
+@pytest.mark.parametrize("m,hidden", [(3072, 256), (2900, 200), (300, 64)])
+def test_narrow_fp32_groups_beside_a_general_body(ctx, m, hidden, pair):
+    """Projections in one grouped launch of narrow tiles: those that only return fp32 run in the straight-line body, the one
+    that also feeds a reader in the general one, with and without CTA pairs."""
+    L = wl.Layer
+    layers = [L("q", hidden, 96, src=-1), L("k", hidden, 96, src=-1), L("v", hidden, 96, src=-1), L("o", hidden, hidden, src=2)]
+    rng = np.random.default_rng(m)
+    x = rng.standard_normal((m, 96)).astype(np.float32)
+    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("groups", 1, layers, m, x, ws)
+    model, xd = build(ctx, w)
+    act_g, w_amax = check_calibration(model, w)
+    ctx.set_pair_tiles(pair)
+    try:
+        for bits in ([8, 8, 8, 8], [4, 8, 6, 3]):
+            before = ctx.launch_forms()["narrow_fp32"]
+            ys = run_eval(ctx, model, w, xd, bits)
+            assert ctx.launch_forms()["narrow_fp32"] == before + 3
+            teacher_forced_check(ctx, model, w, xd, bits, ys, act_g, w_amax)
+    finally:
+        ctx.set_pair_tiles(True)
+    model.close()
+
+
 @pytest.mark.parametrize("m,n,k,act", [(300, 200, 768, 2), (300, 200, 784, 2), (257, 132, 2064, 2), (9000, 260, 1280, 2), (9000, 260, 1296, 1),
                                        (33000, 36, 1024, 2), (130, 48, 64, 2)])
 def test_shortcut_layers_of_long_reductions(ctx, m, n, k, act):
@@ -517,42 +561,64 @@ def test_stem_and_its_pool_match_the_oracle(ctx, c, n, h, wd, k, pad, batch, act
     model.close()
 
 
-@pytest.mark.parametrize("c,n,h,wd,pad,batch", [
-    (64, 64, 56, 56, 1, 4), (64, 64, 9, 9, 1, 80), (64, 32, 11, 7, 1, 90), (128, 128, 28, 28, 1, 13), (128, 96, 5, 5, 2, 230), (64, 64, 130, 6, 1, 13),
-    (64, 32, 8, 8, 0, 160), (256, 256, 14, 14, 1, 128), (256, 256, 14, 14, 1, 77), (512, 512, 7, 7, 1, 129), (192, 288, 13, 17, 0, 30), (64, 320, 6, 140, 1, 8),
-    (128, 160, 28, 28, 1, 11), (64, 256, 64, 64, 1, 5), (256, 224, 14, 14, 2, 70), (128, 128, 28, 28, 1, 2)])
-def test_convolution_by_slabs_matches_the_patch_matrix(ctx, c, n, h, wd, pad, batch):
-    """Stride-1 3x3 convolutions whose only output is their reader's int8 codes load their input once per tile.  Tiles that
-    are whole rows, parts of rows and whole images, halos shared and not, 64- and 128-byte chunks, weights resident and
-    streamed, one and several column tiles, CTA pairs with an odd last tile; few tiles stay with the other kernel: codes
-    bit for bit."""
+def _conv_both_ways(ctx, c, n, h, wd, pad, batch, widths=((8, 8, 8), (8, 5, 4))):
+    """A stride-1 3x3 convolution between a 1x1 layer and a reader of its codes: codes and output with implicit convolutions
+    are those of the patch matrix, bit for bit.  Returns the forms of the implicit runs' launches."""
     L = wl.Layer
-    kh = kw = 3
-    oh, ow = h + 2 * pad - kh + 1, wd + 2 * pad - kw + 1
+    oh, ow = h + 2 * pad - 2, wd + 2 * pad - 2
     layers = [L("in", c, 16, src=-1, kh=1, kw=1, stride=1, in_h=h, in_w=wd, in_c=16, src_h=h, src_w=wd),
-              L("conv", n, kh * kw * c, src=0, act=orc.ACT_RELU, kh=kh, kw=kw, stride=1, pad=pad, in_h=h, in_w=wd, in_c=c, src_h=h, src_w=wd),
+              L("conv", n, 9 * c, src=0, act=orc.ACT_RELU, kh=3, kw=3, stride=1, pad=pad, in_h=h, in_w=wd, in_c=c, src_h=h, src_w=wd),
               L("out", 16, n, src=1, kh=1, kw=1, stride=1, in_h=oh, in_w=ow, in_c=n, src_h=oh, src_w=ow)]
     rng = np.random.default_rng(c + n + h)
     x = rng.standard_normal((batch, h, wd, 16)).astype(np.float32)
     ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
-    w = wl.Workload("conv", 1, layers, batch, x, ws)
-    model, xd = build(ctx, w)
+    model, xd = build(ctx, wl.Workload("conv", 1, layers, batch, x, ws))
     rows = batch * oh * ow
-    for bits in ([8, 8, 8], [8, 5, 4]):
-        outs, codes = [], []
-        for implicit in (True, False):
-            ctx.set_implicit_conv(implicit)
-            y = torch.full((rows, 16), float("nan"), device="cuda")
-            model.eval_config(bits, xd, batch, [None, None, y])
-            qx = torch.zeros((rows, n), dtype=torch.int8, device="cuda")
-            model.debug_dump(2, qx, None, None)
-            ctx.check_sync()
-            outs.append(y)
-            codes.append(qx)
+    forms = []
+    try:
+        for bits in widths:
+            got = []
+            for implicit in (True, False):
+                ctx.set_implicit_conv(implicit)
+                y = torch.full((rows, 16), float("nan"), device="cuda")
+                before = ctx.launch_forms()
+                model.eval_config(list(bits), xd, batch, [None, None, y])
+                if implicit:
+                    forms += [f for f, v in ctx.launch_forms().items() if f.startswith("conv") for _ in range(v - before[f])]
+                qx = torch.zeros((rows, n), dtype=torch.int8, device="cuda")
+                model.debug_dump(2, qx, None, None)
+                ctx.check_sync()
+                got.append((qx, y))
+            assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+            assert got[0][0].any()
+    finally:
         ctx.set_implicit_conv(True)
-        assert torch.equal(codes[0], codes[1]) and torch.equal(outs[0], outs[1])
-        assert codes[0].any()
     model.close()
+    return forms
+
+
+@pytest.mark.parametrize("c,n,h,wd,pad,batch,form", [
+    (64, 64, 56, 56, 1, 4, "slab"), (64, 64, 9, 9, 1, 80, "slab"), (64, 32, 11, 7, 1, 90, "slab"), (128, 128, 28, 28, 1, 13, "slab"),
+    (128, 96, 5, 5, 2, 230, "slab"), (64, 64, 130, 6, 1, 13, "slab"), (64, 32, 8, 8, 0, 160, "slab"), (256, 256, 14, 14, 1, 128, "streamed"),
+    (256, 256, 14, 14, 1, 77, "im2col"), (512, 512, 7, 7, 1, 129, "streamed"), (192, 288, 13, 17, 0, 30, "streamed"), (64, 320, 6, 140, 1, 8, "streamed"),
+    (128, 160, 28, 28, 1, 11, "streamed"), (64, 256, 64, 64, 1, 5, "streamed"), (256, 224, 14, 14, 2, 70, "streamed"), (128, 128, 28, 28, 1, 2, "im2col"),
+    (64, 64, 20, 20, 3, 20, "slab"), (128, 256, 20, 20, 3, 20, "streamed"), (64, 96, 12, 30, 5, 20, "slab")])
+def test_convolution_by_slabs_matches_the_patch_matrix(ctx, c, n, h, wd, pad, batch, form):
+    """Stride-1 3x3 convolutions whose only output is their reader's int8 codes load their input once per tile.  Tiles that
+    are whole rows, parts of rows and whole images, halos shared and not, padding up to and beyond what a tap reaches, 64- and
+    128-byte chunks, weights resident and streamed, one and several column tiles, CTA pairs with an odd last tile; few tiles
+    stay with the other kernel: the form it names (on 148 SMs), codes bit for bit."""
+    assert _conv_both_ways(ctx, c, n, h, wd, pad, batch) == ["conv_" + form] * 2
+
+
+@pytest.mark.parametrize("c,n,h,wd,batch", [(256, 256, 14, 14, 128), (128, 256, 28, 28, 20), (128, 128, 28, 28, 13)])
+def test_convolution_by_slabs_without_cta_pairs(ctx, c, n, h, wd, batch):
+    """128-byte chunks with one CTA per tile, weights streamed and resident."""
+    ctx.set_pair_tiles(False)
+    try:
+        assert _conv_both_ways(ctx, c, n, h, wd, 1, batch) == ["conv_streamed" if n > 128 else "conv_slab"] * 2
+    finally:
+        ctx.set_pair_tiles(True)
 
 
 def test_stem_writes_the_codes_of_its_pooled_readers(ctx):
@@ -586,16 +652,19 @@ def test_stem_writes_the_codes_of_its_pooled_readers(ctx):
 
     want = {}
     steps = ([16, 8, 5, 16, 3, 8], [16, 8, 5, 16, 3, 4], [16, 6, 5, 16, 3, 4], [16, 6, 5, 8, 3, 4], [16, 8, 5, 16, 3, 8])
-    ctx.set_fusion(False)
-    for bits in steps:
-        want[tuple(bits)] = run(bits)
-    ctx.set_fusion(True)
-    for reuse in (False, True):
-        ctx.set_prefix_reuse(reuse)
+    try:
+        ctx.set_fusion(False)
         for bits in steps:
-            for a, b in zip(run(bits), want[tuple(bits)]):
-                assert torch.equal(a, b)
-    ctx.set_prefix_reuse(False)
+            want[tuple(bits)] = run(bits)
+        ctx.set_fusion(True)
+        for reuse in (False, True):
+            ctx.set_prefix_reuse(reuse)
+            for bits in steps:
+                for a, b in zip(run(bits), want[tuple(bits)]):
+                    assert torch.equal(a, b)
+    finally:
+        ctx.set_fusion(True)
+        ctx.set_prefix_reuse(False)
     model.close()
 
 
@@ -646,42 +715,6 @@ def test_readers_of_one_source_in_two_geometries_have_operands_of_their_own(ctx)
             model.calibrate_model(xd, 3)
         assert e.value.status == q.ESHAPE
         model.close()
-
-
-def _conv_both_ways(ctx, c, n, h, wd, pad, batch, widths=((8, 8, 8), (8, 5, 4))):
-    """A stride-1 3x3 convolution between a 1x1 layer and a reader of its codes: codes and output with implicit convolutions
-    are those of the patch matrix, bit for bit.  Returns the forms of the implicit runs' launches."""
-    L = wl.Layer
-    oh, ow = h + 2 * pad - 2, wd + 2 * pad - 2
-    layers = [L("in", c, 16, src=-1, kh=1, kw=1, stride=1, in_h=h, in_w=wd, in_c=16, src_h=h, src_w=wd),
-              L("conv", n, 9 * c, src=0, act=orc.ACT_RELU, kh=3, kw=3, stride=1, pad=pad, in_h=h, in_w=wd, in_c=c, src_h=h, src_w=wd),
-              L("out", 16, n, src=1, kh=1, kw=1, stride=1, in_h=oh, in_w=ow, in_c=n, src_h=oh, src_w=ow)]
-    rng = np.random.default_rng(c + n + h)
-    x = rng.standard_normal((batch, h, wd, 16)).astype(np.float32)
-    ws = [(rng.standard_normal((l.n_out, l.k_in)) / np.sqrt(l.k_in)).astype(np.float32) for l in layers]
-    model, xd = build(ctx, wl.Workload("conv", 1, layers, batch, x, ws))
-    rows = batch * oh * ow
-    forms = []
-    try:
-        for bits in widths:
-            got = []
-            for implicit in (True, False):
-                ctx.set_implicit_conv(implicit)
-                y = torch.full((rows, 16), float("nan"), device="cuda")
-                before = ctx.launch_forms()
-                model.eval_config(list(bits), xd, batch, [None, None, y])
-                if implicit:
-                    forms += [f for f, v in ctx.launch_forms().items() if f.startswith("conv") for _ in range(v - before[f])]
-                qx = torch.zeros((rows, n), dtype=torch.int8, device="cuda")
-                model.debug_dump(2, qx, None, None)
-                ctx.check_sync()
-                got.append((qx, y))
-            assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
-            assert got[0][0].any()
-    finally:
-        ctx.set_implicit_conv(True)
-    model.close()
-    return forms
 
 
 @pytest.mark.parametrize("c,n,h,wd,batch,form", [

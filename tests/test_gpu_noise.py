@@ -90,3 +90,30 @@ def test_noise_sensitivity_zero_lambda_and_errors(ctx):
         model.noise_sensitivity(x, w.m, [None] * 3, -1.0)
     assert e.value.status == q.EINVAL
     model.close()
+
+
+@pytest.mark.parametrize("k,cols", [(37, 19), (64, 32)])
+def test_noise_beyond_the_range_of_32_bits(ctx, k, cols):
+    """A deviation that overflows makes every perturbed weight infinite and nothing else: with positive weights, inputs and
+    draws the output is infinite, not NaN, which a deviation that reached the zeros behind a row's last column would give."""
+    rng = np.random.default_rng(k)
+    layers = wl.mlp_layers((k, cols))
+    ws = [rng.uniform(0.5, 1.5, (l.n_out, l.k_in)).astype(np.float32) for l in layers]
+    w = wl.Workload("range", 1, layers, 33, rng.uniform(0.5, 1.5, (33, k)).astype(np.float32), ws)
+    nus = [rng.uniform(1.0, 2.0, a.shape).astype(np.float32) for a in ws]
+    assert np.isfinite(_run(ctx, w, nus, 1.0)).all()
+    assert np.isposinf(_run(ctx, w, nus, 3.4e38)).all()
+
+
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+def test_non_finite_weight_reaches_every_row_through_the_deviation(ctx, value):
+    """The tensor's maximum is folded from the rows' maxima as an integer, where an infinity or a NaN in one row wins: with draws
+    of zero every perturbed weight of the layer is NaN.  ReLU turns its outputs into zeros, so the last output is zero and its
+    distance is exactly 1, unless the unperturbed output is infinite itself."""
+    w = _ragged_mlp((37, 1030, 22, 7), 33)
+    w.weights[1][20, 1029] = value
+    nus = [np.zeros_like(a) for a in w.weights]
+    nus[0] = nus[2] = None
+    e = _run(ctx, w, nus, 0.05)
+    assert e[0] == 0.0 and e[2] == 0.0
+    assert e[1] == 1.0 if np.isnan(value) else not np.isfinite(e[1])
