@@ -578,7 +578,7 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
           if (!pooled || calibrate || !ctx->fuse || !dirty[c] || C.d.pool_before != QCFG_POOL_MAX3S2 || C.d.src_h != oh || C.d.src_w != ow) continue;
           const bool rows = C.d.kh == 0 || (C.d.kh == 1 && C.d.kw == 1 && C.d.stride == 1 && C.d.pad == 0);
           const int64_t prows = m * ((oh - 1) / 2 + 1) * ((ow - 1) / 2 + 1);
-          if (!rows || C.d.src_col0 != 0 || C.d.k_in != d.n_out || !bits_int(bits[c]) || layer_rows(M, c, m) != prows || codes_kept(c)) continue;
+          if (!rows || C.d.src_col0 != 0 || C.d.k_in != d.n_out || !bits_int(bits[c]) || layer_rows(M, c, m) != prows) continue;
           float csc = 1.0f, cinv = 1.0f;
           act_scales(C, bits[c], &csc, &cinv);
           int at = 0;
@@ -639,7 +639,7 @@ int forward(Ctx* ctx, Model* M, const uint8_t* bits, const float* x_dev, int64_t
           grids[count++] = CodeSlot{S.abuf.p, S.ldk, inv, b == 16 ? 0.0f : qmax_of(b), b == 16 ? 2 : 1, b};
           for (int j = l + 1; j < n && count < kMaxSlots; ++j) {
             LayerState& T = M->L[j];
-            if (!dirty[j] || T.a_ready || T.implicit || T.rows != S.rows || !same_input(T.d, d) || is_stem(T.d, T.bits)) continue;
+            if (!dirty[j] || T.a_ready || T.rows != S.rows || !same_input(T.d, d)) continue;
             float tsc = 1.0f, tinv = 1.0f;
             if (T.bits != 16) act_scales(T, T.bits, &tsc, &tinv);
             bool known = false;

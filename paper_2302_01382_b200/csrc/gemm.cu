@@ -72,7 +72,7 @@ enum : int { MAP_A = 0, MAP_B = 1, MAP_FAST = 2, MAP_OUT = 3 };
 constexpr int kPoolAll = kMaxGroups * kMapsPerGroup;   // a launch of its own: every map has its place
 constexpr int kPoolChain = 8;                          // a record of a chain: the (distinct) maps it really uses
 // Epilogue bodies.  The general one handles any combination of outputs with run-time branches; the
-// two common combinations have straight-line bodies (same arithmetic, same order).
+// common combinations have straight-line bodies (same arithmetic, same order).
 enum : int32_t { EPI_GENERAL = 0, EPI_CODES1 = 1, EPI_Y = 2, EPI_SHORTCUT = 3, EPI_CODES32 = 4, EPI_BF16 = 5, EPI_Y32 = 6 };
 // Fast bodies (256-column tiles only): EPI_CODES1 writes each warp's 32 x 64 int8 block with one
 // TMA store (64-byte rows, 64B swizzle), EPI_Y each 32 x 32 fp32 block with one (128-byte rows,
