@@ -2159,12 +2159,16 @@ bool gemm_groupable(const GemmArgs& a, const GemmArgs& b) {
 
 // The body for shortcut layers leaves room for a ring of two stages, stages twice the operand bytes of a 256-column pair
 // tile and joins no chain, so it pays while the reduction is short against the blocks it moves.  us for such a
-// layer between two small ones, this body / the general one:
-//   12288 x 768    k = 768 50.5 / 57.2    1280 68.9 / 69.2    1536 77.1 / 73.7
-//   25088 x 1024   k = 768 104 / 119      1024 121 / 127      1280 138 / 134
-//   50176 x 512    k = 768 131 / 139      1024 155 / 152      (the left operand no longer stays in L2 between column tiles)
-//   3072 x 768     k = 1536 28.6 / 31.5   2048 30.7 / 33.0    3072 38.6 / 37.5     (one tile per CTA: no ring to keep full)
-// Twelve transformer blocks of 768 with shortcuts (k = 768 and 3072) at 12288 rows: 1875 us with every shortcut in this body.
+// layer between three small ones, this body / the general one:
+//   12288 x 768    k = 768 39.3 / 48.6    1024 43.1 / 53.3    1280 48.1 / 55.6    1536 53.4 / 57.3    2048 66.4 / 64.2
+//   25088 x 1024   k = 768 95.7 / 107.7   1024 110.3 / 111.0  1280 124.1 / 116.5
+//   50176 x 512    k = 768 113.5 / 119.3  1024 128.2 / 125.5
+//   6144 x 1024    k = 1280 36.7 / 44.3   1536 40.0 / 47.6    2048 45.4 / 48.9
+//   3072 x 768     k = 1536 25.2 / 31.0   2048 26.9 / 32.2    3072 31.1 / 35.5     (one tile per CTA: no ring to keep full)
+// Alone it would also pay at 1536 in few rounds of tiles and at 3072 with one tile per CTA.  In a stack it does not, where the
+// general body's launches overlap their neighbours or join a chain: four transformer blocks with shortcuts, hidden / ffn,
+// 768 / 1536 at 12288 rows 441 / 404, 1024 / 1536 at 6144 rows 337 / 305, 768 / 3072 at 3072 rows 242 / 236, 1024 / 4096 at 1500 rows
+// 249 / 224; 768 / 1024 at 12288 rows 395 / 379 and at 6144 rows 254 / 288.
 static bool shortcut_body_pays(const GemmArgs& g, int bn, int sms) {
   const int64_t width = bn > 128 ? 128 : bn;
   if (g.k <= 768) return true;

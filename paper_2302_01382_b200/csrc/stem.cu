@@ -18,10 +18,12 @@
 //   warps 9..16 epilogue: activation, running maximum over output rows in registers; every second row the
 //               maxima of the row triple cross lanes through shared memory, and the pooled row leaves in 16-byte
 //               stores, with its readers' int8 codes beside it (a quantize launch per reader took 19 us each).
-// What bounds it (128 images of 224 x 224 x 3: 238 us, 299 before the row pitch and the second epilogue warp per
-// quadrant): the producers, 3500 cycles per output row: 2000 for the patch copies through shared memory, 900 in which the
-// next rows' loads wait for the registers the stores of the last ones still read, 300 waiting for the tensor core.  The
-// epilogue takes 2400.  Seven pixels per batch, predicated loads and an unrolled MMA loop changed nothing.
+// What bounds it (128 images of 224 x 224 x 3: 233 us from the end of the kernel in front to the last CTA's end, 299 before the
+// row pitch and the second epilogue warp per quadrant): the producers.  With clocks read in the kernel (243 us, 1.84 GHz) a
+// CTA of 105 output rows takes 446000 cycles: 220000 patch copies through shared memory, 126000 storing the two rows an
+// output row adds and issuing the next loads, 24000 waiting for the tensor core, 34000 first rows of bands, 40000 weights,
+// barriers and exit.  The epilogue is busy for 2250 of the 4100 cycles per output row.  Seven pixels per batch, predicated
+// loads and an unrolled MMA loop changed nothing.
 // Work items are bands of pooled rows of one image; a band repeats one output row of its neighbour.
 #include "common.cuh"
 #include "ptx.cuh"
@@ -31,9 +33,8 @@ namespace qcfg {
 namespace {
 
 constexpr int kProducers = 8;                 // warps
-// Two epilogue warps per lane quadrant, 32 channels each.  With one (64 running maxima in registers, spilled) an output row
-// took the epilogue 4200 of the 5500 cycles between rows and the producers waited for it: an evaluation of ResNet-50 at
-// batch 128 2272 us, 2201 with two.
+// Two epilogue warps per lane quadrant, 32 channels each.  With one (64 running maxima in registers, spilled) the producers
+// waited for it: an evaluation of ResNet-50 at batch 128 2272 us, 2201 with two.
 constexpr int kEpiWarps = 8;
 constexpr int kStemThreads = 32 * (kProducers + 1 + kEpiWarps);
 constexpr int kRows = 16;                     // input rows held (power of two)
