@@ -79,7 +79,7 @@ enum : int32_t { EPI_GENERAL = 0, EPI_CODES1 = 1, EPI_Y = 2, EPI_SHORTCUT = 3, E
 // 128B swizzle), EPI_BF16 each warp's 32 x 64 bf16 block with one (128-byte rows, 128B swizzle), taking the maximum
 // of what it writes along in the calibration forward.  EPI_SHORTCUT (int8, one CTA per tile, at most 128 columns): fp32 shortcut in, fp32 matrix and
 // up to two int8 code matrices out.  EPI_CODES32 (one CTA per tile, fewer than 256 columns): one int8 code matrix.
-// EPI_Y32 (int8, fewer than 256 columns): the fp32 matrix.
+// EPI_Y32 (int8, fewer than 256 columns, not a lone GEMM in CTA pairs): the fp32 matrix.
 struct GroupDesc {
   int32_t n, tn_begin;        // columns; first column-tile index of the group in the launch's numbering
   int32_t act;
@@ -698,7 +698,10 @@ __device__ __forceinline__ void epilogue_codes32(const GroupDesc& G, const CUten
 // of one tile per CTA, whose epilogue nothing hides): broadcast scales, one TMA store of 128-byte rows.  The general body
 // shuffles a scale per element and stores twice; 3072 x 768 x 3072 took 2.7 us there from the last product to the last store.
 // Two blocks of 768 at 384 rows: 60.5 us there, 59.1 here; ResNet-50 of 16 images of 64 x 64 225.8 / 221.8.  16-bit layers
-// need no scales and gain nothing.
+// need no scales and gain nothing.  A lone GEMM in CTA pairs keeps the general body: it gains 0.05 us from this one, whose code
+// in that kernel, the one of the plain 256-column launches, cost every launch 0.25 (4096 x 1024 x 1024 with its quantize 12.97
+// and 12.62 us, three such layers 28.1 and 27.2).  In groups of pairs it stays (a block at 3072 rows with its q and k
+// outputs: 45.6 us without, 45.3 with).
 template <bool PAIR>
 __device__ __forceinline__ void epilogue_y32(const GroupDesc& G, const CUtensorMap* map, uint32_t tbase, const float* cs, uint32_t stage,
                                              int row0, int col0, bool inside, int lane, uint32_t tempty_bar) {
@@ -1651,7 +1654,7 @@ gemm_kernel(const __grid_constant__ LaunchArgs<CHAIN> L) {
           }
           epilogue_codes32<BF16>(G, &mp[q->mi[0][MAP_OUT + 2]], tbase, cs_tab, stage, row0, col_base, row0 < q->m && col_base < G.n, lane, tempty_bar);
         }
-      } else if (!BF16 && FL == FL_PLAIN && !CHAIN && G.mode == EPI_Y32) {
+      } else if (!BF16 && FL == FL_PLAIN && !CHAIN && (!PAIR || GROUPED) && G.mode == EPI_Y32) {
         if (nch == 0) {
           __syncwarp();
           if (lane == 0) { if (PAIR) mbar_arrive_leader(tempty_bar); else mbar_arrive(tempty_bar); }
@@ -2365,7 +2368,7 @@ int launch_gemm_group(Ctx* ctx, const GemmArgs* gs_in, int count, cudaStream_t s
       if (!G.outs[1].kind && G.outs[2].kind == 1 && make_fast_map(&maps[i * kMapsPerGroup + MAP_FAST], G.outs[2], g.m, g.n)) G.mode = EPI_CODES1;
       else if (G.outs[1].kind && !G.outs[2].kind && make_fast_map(&maps[i * kMapsPerGroup + MAP_FAST], G.outs[1], g.m, g.n)) { G.mode = EPI_Y; wide = true; }
     }
-    if (bn < 256 && !shortcut && !g.is_bf16 && g.conv_kh == 0 && !G.residual && !G.amax && !G.outs[0].kind && G.outs[1].kind && !G.outs[2].kind && !G.outs[3].kind &&
+    if (bn < 256 && (!pair || count > 1) && !shortcut && !g.is_bf16 && g.conv_kh == 0 && !G.residual && !G.amax && !G.outs[0].kind && G.outs[1].kind && !G.outs[2].kind && !G.outs[3].kind &&
         !G.outs[4].kind && make_fast_map(&maps[i * kMapsPerGroup + MAP_FAST], G.outs[1], g.m, g.n))
       G.mode = EPI_Y32;
     if (shortcut) {      // MAP_OUT, the raw accumulators' place, holds the shortcut's map
